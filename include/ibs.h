@@ -366,13 +366,16 @@ ibs_status ibs_kernel_info(ibs_ctx* ctx, int64_t out[4]);
 
 /* The pair kernel ibs_compute runs on this context for an n_samples x
  * n_variants matrix, written to *out: 0 POPC plain, 1 POPC carry-save,
- * 2 tensor core with one persistent CTA per SM, 3 tensor core with the
- * two-SM kernel (clusters of two CTAs, tcgen05 cta_group::2), 4 tensor core
- * with one CTA per tile (square output).  The two-SM kernel runs for E2M1
- * operands, triangle output and 129 or more samples when the matrix has at
- * least 65,536 variants (1,024 chunks of 64), where it is the faster one;
- * IBS_TC_PAIR=1 in the environment selects it for every size, IBS_TC_PAIR=0
- * never.  Host only, no device work; IBS_EINVAL for sizes ibs_compute
+ * 2 tensor core, 3 tensor core with 129 or more samples and at least 65,536
+ * variants (E2M1 operands, triangle output), 4 tensor core with square output.
+ * E2M1 triangles of both classes run on the two-SM kernel that sweeps the
+ * markers once per product (clusters of two CTAs, tcgen05 cta_group::2); where
+ * its workspace does not fit, with 2^21 or more variants and with E4M3
+ * operands, class 2 runs one persistent CTA per SM and class 3 the two-SM
+ * kernel over 256 x 128 tiles.
+ * IBS_TC_PAIR=1 in the environment reports class 3 for every size of 129 or
+ * more samples, IBS_TC_PAIR=0 runs (and reports) one CTA per SM always.  Host
+ * only, no device work; IBS_EINVAL for sizes ibs_compute
  * refuses or out == NULL. */
 ibs_status ibs_compute_kernel(ibs_ctx* ctx, int64_t n_samples, int64_t n_variants, int64_t* out);
 

@@ -207,6 +207,101 @@ static bool tc_tile_kernel_forced() {
   return v;
 }
 
+// The sweep kernel (ibs_sweep.cu) computes the E2M1 triangle: at every size the
+// faster one (256 x 4,096: 31 us a call against 82 on the kernels below; 4,096 x
+// 100,000: 1,076 against 1,564; 20,000 x 500,000: 82 against 142 ms).
+static bool use_sweep(const ibs_ctx* ctx, int64_t n, int64_t m, bool square) {
+  return !square && tc_format_for(ctx) == kTcFp4 && tc_pair_mode() >= 0 && !tc_tile_kernel_forced() &&
+         sweep_usable(n, m) && ctx->sweep_refused != std::vector<int64_t>{n, m, square ? 1 : 0};
+}
+
+// ibs_compute on the sweep kernel: operand planes, the sweeps over the shape's
+// work list (kept for the last shape), the sums of split tiles.
+static ibs_status compute_sweep(ibs_ctx* ctx, const uint8_t* packed, int64_t n, int64_t m, int32_t* out_counts,
+                                double* out_dist, bool square, cudaStream_t st) {
+  const int clusters = sweep_clusters();
+  const std::vector<int64_t> key = {n, m, clusters, tc_pair_sync_setting(0).x, tc_pair_sync_setting(0).y};
+  if (ctx->sweep_key != key) {
+    ctx->sweep_key.clear();
+    SweepPlan pl = sweep_plan(n, m, clusters);
+    const size_t ib = pl.items.size() * sizeof(SweepItem), fb = pl.first.size() * sizeof(int32_t);
+    const size_t gb = std::max<size_t>(1, pl.groups.size()) * sizeof(SweepGroup);
+    if (ibs_status s = ensure_buf(ctx, ctx->sweep_items, ib)) return s;
+    if (ibs_status s = ensure_buf(ctx, ctx->sweep_first, fb)) return s;
+    if (ibs_status s = ensure_buf(ctx, ctx->sweep_groups, gb)) return s;
+    // pageable sources: the copies are staged before return
+    IBS_CUDA_TRY(cudaMemcpyAsync(ctx->sweep_items.p, pl.items.data(), ib, cudaMemcpyHostToDevice, st));
+    IBS_CUDA_TRY(cudaMemcpyAsync(ctx->sweep_first.p, pl.first.data(), fb, cudaMemcpyHostToDevice, st));
+    if (!pl.groups.empty())
+      IBS_CUDA_TRY(cudaMemcpyAsync(ctx->sweep_groups.p, pl.groups.data(), pl.groups.size() * sizeof(SweepGroup),
+                                   cudaMemcpyHostToDevice, st));
+    ctx->sweep_stages = pl.stages;
+    ctx->sweep_clusters = pl.clusters;
+    ctx->sweep_waves = pl.waves;
+    ctx->sweep_slots = pl.slots;
+    ctx->sweep_has_whole = pl.scratch;
+    ctx->sweep_n_groups = (int64_t)pl.groups.size();
+    ctx->sweep_key = key;
+  }
+  if (ibs_status s = ensure_buf(ctx, ctx->planes, sweep_planes_bytes(n, m))) return s;
+  if (ctx->sweep_has_whole)
+    if (ibs_status s = ensure_buf(ctx, ctx->sweep_scratch, sweep_scratch_bytes(ctx->sweep_clusters))) return s;
+  if (ibs_status s = ensure_buf(ctx, ctx->partial, (size_t)ctx->sweep_slots * sweep_slot_bytes())) return s;
+  SweepSync sync;
+  size_t sync_bytes = 0;
+  const int2 ss = tc_pair_sync_setting(0);  // in chunks of 64 markers
+  if (ss.x > 0 && ctx->sweep_waves > 0) {
+    sync.seg = std::max(1, ss.x * 64 / 288);
+    sync.lag = ss.y;
+    sync.n_seg = (4 * ctx->sweep_stages + sync.seg - 1) / sync.seg;
+    sync_bytes = (size_t)ctx->sweep_waves * sync.n_seg * sizeof(int);
+    if (ibs_status s = ensure_buf(ctx, ctx->single_sync, sync_bytes)) return s;
+    sync.ctr = static_cast<int*>(ctx->single_sync.p);
+  }
+  const bool timing = (ctx->flags & IBS_TIMING) != 0, split = ctx->sweep_n_groups > 0;
+  ibs_ctx::TimingRec rec;
+  if (timing) {
+    if (!ctx->timing_free.empty()) {
+      rec = ctx->timing_free.back();
+      ctx->timing_free.pop_back();
+    } else {
+      for (auto& e : rec.ev) IBS_CUDA_TRY(cudaEventCreate(&e));
+    }
+    rec.n = split ? 4 : 3;
+    IBS_CUDA_TRY(cudaEventRecord(rec.ev[0], st));
+  }
+  IBS_CUDA_TRY(launch_sweep_planes(packed, n, m, static_cast<uint8_t*>(ctx->planes.p), st));
+  if (timing) IBS_CUDA_TRY(cudaEventRecord(rec.ev[1], st));
+  SweepLaunch l;
+  l.a_planes = l.b_planes = static_cast<const uint8_t*>(ctx->planes.p);
+  l.a_half = l.b_half = (n + 63) / 64;
+  l.n = n;
+  l.counts = out_counts;
+  l.dist = out_dist;
+  l.square = square;
+  l.items = static_cast<const SweepItem*>(ctx->sweep_items.p);
+  l.first = static_cast<const int32_t*>(ctx->sweep_first.p);
+  l.stages = ctx->sweep_stages;
+  l.clusters = ctx->sweep_clusters;
+  l.scratch = static_cast<float*>(ctx->sweep_scratch.p);
+  l.part = static_cast<float*>(ctx->partial.p);
+  l.status = ctx->status_dev;
+  l.wait_ns = ctx->wait_ns > 0 ? ctx->wait_ns : kWaitLimitNs;
+  l.sync = sync;
+  if (sync_bytes > 0) IBS_CUDA_TRY(cudaMemsetAsync(sync.ctr, 0, sync_bytes, st));
+  IBS_CUDA_TRY(launch_sweep(l, st));
+  if (timing) IBS_CUDA_TRY(cudaEventRecord(rec.ev[2], st));
+  IBS_CUDA_TRY(launch_sweep_finalize(l, static_cast<const SweepGroup*>(ctx->sweep_groups.p), ctx->sweep_n_groups, st));
+  if (timing) {
+    if (split) IBS_CUDA_TRY(cudaEventRecord(rec.ev[3], st));
+    ctx->timing_used.push_back(rec);
+  }
+  ctx->last_info[0] = split ? 3 : 2;
+  ctx->last_info[1] = tc_tiles(n);
+  ctx->last_info[2] = split ? 2 : 1;
+  return IBS_OK;
+}
+
 ibs_status ibs_compute(ibs_ctx* ctx, const uint8_t* packed, int64_t n, int64_t m, int32_t* out_counts,
                        double* out_dist, void* stream) {
   clear_error();
@@ -224,6 +319,18 @@ ibs_status ibs_compute(ibs_ctx* ctx, const uint8_t* packed, int64_t n, int64_t m
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   const bool tc = use_tc(ctx);
   const int fmt = tc_format_for(ctx);
+  if (tc && use_sweep(ctx, n, m, square)) {
+    const ibs_status s = compute_sweep(ctx, packed, n, m, out_counts, out_dist, square, st);
+    if (s != IBS_ENOMEM) return s;
+    // no room for its scratch and parts: nothing is enqueued, and the kernels
+    // below take the call with the memory that they always needed
+    for (DevBuf* b : {&ctx->planes, &ctx->partial, &ctx->sweep_scratch, &ctx->sweep_items, &ctx->sweep_first,
+                      &ctx->sweep_groups, &ctx->single_sync})
+      free_buf(ctx, *b);
+    ctx->sweep_key.clear();
+    ctx->sweep_refused = {n, m, square ? 1 : 0};
+    clear_error();
+  }
   // Tensor-core form, triangle output: the persistent kernel over a work list
   // (tail wave split over K).  Square output, or IBS_TC_TILE_KERNEL set: one
   // CTA per tile (or tile piece).
@@ -1519,7 +1626,8 @@ extern "C" ibs_status ibs_shutdown(ibs_ctx* ctx) {
     free_buf(ctx, ctx->planes);
     free_buf(ctx, ctx->partial);
     free_buf(ctx, ctx->tile_list);
-    for (DevBuf* b : {&ctx->single_items, &ctx->single_split, &ctx->single_counter, &ctx->single_sync, &ctx->ld_planes, &ctx->ld_diff,
+    for (DevBuf* b : {&ctx->single_items, &ctx->single_split, &ctx->single_counter, &ctx->single_sync, &ctx->sweep_items,
+                      &ctx->sweep_first, &ctx->sweep_groups, &ctx->sweep_scratch, &ctx->ld_planes, &ctx->ld_diff,
                       &ctx->ld_items, &ctx->ld_counter, &ctx->cluster_work, &ctx->grm_work,
                       &ctx->grm_items, &ctx->grm_splits, &ctx->grm_part, &ctx->grm_counter})
       free_buf(ctx, *b);

@@ -142,6 +142,12 @@ struct ibs_ctx {
   int64_t single_n_sync = 0;  // pair items in full waves of equal length (the K-lockstep's items)
   int single_clusters = 0;
   bool single_pair = false;  // single_items holds PairItem (two-SM kernel), else WorkItem
+  // sweep kernel: work list of the last (n, m, clusters), scratch of whole tiles
+  std::vector<int64_t> sweep_key, sweep_refused;  // refused: the shape that found no room last
+  ibs::DevBuf sweep_items, sweep_first, sweep_groups, sweep_scratch;
+  int sweep_stages = 0, sweep_clusters = 0, sweep_waves = 0, sweep_slots = 0;
+  int64_t sweep_n_groups = 0;
+  bool sweep_has_whole = false;
   int* status_host = nullptr;     // mapped pinned status word
   int* status_dev = nullptr;
   // device-side bound of the pipeline waits of ibs_compute's persistent pair

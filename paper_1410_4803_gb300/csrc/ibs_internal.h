@@ -256,6 +256,70 @@ cudaError_t launch_tc_pair_cross(const uint8_t* panel, int64_t n_panel, int64_t 
                                  int64_t q_blocks_cap, int32_t* const* row_out, int64_t n_rows, const PairItem* items,
                                  int64_t n_items, int* status, cudaStream_t st, const PairSync& sync = PairSync{});
 int tc_block_samples();  // 128
+
+// Pair counts in marker sweeps (ibs_sweep.cu): the two-SM kernel over 256 x
+// 384 tiles, one product at a time.  A work item: block rows I and I + 1 (one
+// per CTA of the cluster), block columns J .. J + w - 1, ring stages q0 .. q1 - 1
+// of the tile's four sweeps; slot < 0: a whole tile, else the first part slot
+// of a piece (one slot per product it touches); wave: the wave of a whole
+// tile that streams in lockstep with the other clusters, or -1.
+struct SweepItem {
+  int32_t I, J, w;
+  int32_t q0, q1;
+  int32_t slot, wave;
+  int32_t pad;
+};
+// A split tile: its parts are slots slot, slot + 1, ..., pieces[0] of V V^T,
+// then pieces[1] of U U^T, then pieces[2] of Q R^T + R Q^T.
+struct SweepGroup {
+  int32_t I, J, w, slot;
+  int32_t pieces[3];
+  int32_t pad;
+};
+struct SweepPlan {
+  int stages = 0;    // ring stages per sweep
+  int clusters = 0;  // clusters that have work
+  int waves = 0;     // waves of whole tiles
+  int slots = 0;     // part slots
+  bool scratch = false;  // some tile runs whole
+  std::vector<SweepItem> items;   // cluster by cluster
+  std::vector<int32_t> first;     // [clusters + 1] offsets into items
+  std::vector<SweepGroup> groups;  // the split tiles
+};
+// Lockstep of the waves of whole tiles: the copy warp of every CTA counts each
+// seg-stage segment it starts in ctr[wave * n_seg + segment] and, before
+// segment s, waits (bounded) until every CTA has started segment s - lag.
+struct SweepSync {
+  int* ctr = nullptr;
+  int32_t n_seg = 0, seg = 0, lag = 0;
+};
+struct SweepLaunch {
+  const uint8_t* a_planes = nullptr;  // rows' planes, a_half half-blocks
+  const uint8_t* b_planes = nullptr;  // columns' planes, b_half half-blocks
+  int64_t a_half = 0, b_half = 0;
+  int64_t n = 0;  // samples of the triangle or square
+  int32_t* counts = nullptr;
+  double* dist = nullptr;
+  bool square = false;
+  const SweepItem* items = nullptr;
+  const int32_t* first = nullptr;
+  int stages = 0, clusters = 0;
+  float* scratch = nullptr;
+  float* part = nullptr;
+  int* status = nullptr;
+  unsigned long long wait_ns = 0;
+  SweepSync sync;
+};
+int sweep_stages(int64_t m);
+int sweep_clusters();  // clusters of two that fit on the current device (0: the kernel cannot run)
+bool sweep_usable(int64_t n, int64_t m);
+size_t sweep_planes_bytes(int64_t n, int64_t m);
+size_t sweep_scratch_bytes(int clusters);
+size_t sweep_slot_bytes();
+SweepPlan sweep_plan(int64_t n, int64_t m, int clusters);
+cudaError_t launch_sweep_planes(const uint8_t* packed, int64_t n, int64_t m, uint8_t* planes, cudaStream_t st);
+cudaError_t launch_sweep(const SweepLaunch& l, cudaStream_t st);
+cudaError_t launch_sweep_finalize(const SweepLaunch& l, const SweepGroup* groups, int64_t n_groups, cudaStream_t st);
 // LD correlation (ibs_ld.cu): operand planes of the markers (128-marker
 // blocks, 64-sample chunks, planes X, V, H), the band's work items and the
 // launch sequence (operand builder with per-marker allele balance, persistent

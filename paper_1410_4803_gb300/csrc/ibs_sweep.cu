@@ -1,0 +1,805 @@
+// Pair counts in marker sweeps: the two-SM tensor-core kernel of ibs_compute.
+//
+// The indicator products are those of ibs_tc.cu: per sample and marker V = 1
+// present, U = +1 homozygous / -1 heterozygous, Q = 1 homozygous A2, R = 1
+// homozygous A1 (0 when missing), N = V V^T, IBS1 = (N - U U^T) / 2,
+// IBS0 = Q R^T + R Q^T, all exact integers in FP32.  That kernel streams all
+// four planes of a tile together into three accumulators of 128 columns.  Here
+// a tile is swept over the marker axis four times, one plane pair at a time,
+//   sweep 0: V V^T    sweep 1: U U^T    sweep 2: Q R^T    sweep 3: + R Q^T,
+// and the 384 accumulator columns of tensor memory hold one product of a tile
+// three times as wide: a cluster of two CTAs computes 256 x 384 pairs.  Per SM
+// and 96 markers of one product that is 6 KiB of A and 9 KiB of B for three
+// 128 x 128 results, 13.3 KiB per result, plane set and 64 markers against 24
+// KiB for 256 x 128 tiles with all planes together.  Between sweeps the
+// accumulators go to a scratch buffer (three values per pair, in L2).
+//
+// The MMAs are kind::mxf4 with K = 96 (sm_103a; bit 31 of the instruction
+// descriptor), M = 256, N = 192 over the CTA pair.  Measured back to back from
+// shared memory on all SMs: 96 cycles each, 14.5 PFLOP/s; N = 256: 128 cycles,
+// the same rate; N = 128: 76 cycles, 12.2 PFLOP/s; K = 64: 9.7 PFLOP/s for
+// every N.  One CTA's MMAs (cta_group::1) reach 9.7 at K = 96, N = 128 and
+// 12.9 at N = 256.
+//
+// Operand planes: [plane][64-sample half-block][32-marker column][64 rows][16
+// bytes], E2M1, so a column of a half-block is 1 KiB in the canonical K-major
+// layout without swizzle (8-row x 16-byte core matrices 128 bytes apart), and
+// a K step of 96 markers is three columns.  One tensor map box copies any
+// number of half-blocks over kSwCols columns into [column][half-block][1 KiB],
+// an operand whose rows are one contiguous run per column.
+#include <algorithm>
+#include <atomic>
+#include <cstdio>
+#include <cstdlib>
+#include <cstring>
+#include <type_traits>
+#include <vector>
+
+#include "ibs_tc_common.cuh"
+
+namespace ibs {
+
+namespace {
+
+// A ring stage is kSwCols columns (three K steps): 18 KiB of A and up to 27
+// KiB of B.  A stage costs about 500 cycles whatever its size (barrier wait,
+// two copies, release; measured with copies alone: 31, 62 and 95 B/clk per SM
+// for stages of 3, 6 and 9 columns, 95 B/clk also for 12), and the MMAs of
+// three K steps take 576, so this is the smallest stage that does not bind.
+constexpr int kSwCols = 9;
+constexpr int kSwMarkers = 32 * kSwCols;  // 288
+constexpr int kSwStages = 4;
+constexpr int kSwABytes = kSwCols * 2048, kSwBBytes = kSwCols * 3072;
+constexpr int kSwStageBytes = kSwABytes + kSwBBytes;
+constexpr int kSwEpiWarps = 8;  // two per tensor-memory lane quarter
+constexpr int kSwThreads = 128 + 32 * kSwEpiWarps;
+constexpr int kSwTransBytes = 32 * 17 * 8;  // per epilogue warp: the counts of 32 x 16 pairs, packed
+constexpr size_t kSwSmem = (size_t)kSwStages * kSwStageBytes + kSwEpiWarps * kSwTransBytes + 1024;
+static_assert(kSwSmem <= 227 * 1024, "ring exceeds shared memory");
+constexpr int kSwTileCols = 384;
+constexpr size_t kSwHalfTile = (size_t)kSwTileCols * kTB;  // values of one product of one CTA's 128 x 384 tile
+constexpr int kSwEpiBar = 1, kSwBar = 2;  // hardware barriers: epilogue warps; ring slots 0 .. kSwStages - 1
+
+// The waiter warp's release of ring slot s to the MMA warp: one hardware barrier
+// per slot, on which the waiter arrives without blocking and the MMA warp
+// waits.  The waiter cannot arrive on a slot's barrier again before the MMA
+// warp has passed it: the slot is filled again only after its MMAs.
+__device__ __forceinline__ void sweep_release(uint32_t s) {
+  asm volatile("barrier.cta.arrive %0, 64;" ::"r"(kSwBar + s) : "memory");
+}
+__device__ __forceinline__ void sweep_acquire(uint32_t s) {
+  asm volatile("barrier.cta.sync %0, 64;" ::"r"(kSwBar + s) : "memory");
+}
+
+// kind::mxf4, E2M1 x E2M1 -> F32, UE8M0 scale factors, K = 96, M = 256.
+template <int N>
+constexpr uint32_t kIdescSweep = (1u << 7) | (1u << 10) | ((uint32_t)(N >> 3) << 17) | (1u << 23) |
+                                 ((uint32_t)(256 >> 4) << 24) | (1u << 31);
+
+template <int N>
+__device__ __forceinline__ void umma_sweep(uint32_t tmem, uint64_t a, uint64_t b, uint32_t acc, uint32_t sf) {
+  asm volatile(
+      "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
+      "tcgen05.mma.cta_group::2.kind::mxf4.block_scale.block32 [%0], %1, %2, %3, [%5], [%6], p;\n\t}" ::"r"(tmem),
+      "l"(a), "l"(b), "r"(kIdescSweep<N>), "r"(acc), "r"(sf), "r"(sf + 64u)
+      : "memory");
+}
+
+// Operand of rows 16 bytes apart in columns `col` bytes apart (K core matrices).
+__device__ __forceinline__ uint64_t sweep_desc(uint32_t saddr, uint32_t col) {
+  return (uint64_t)((saddr >> 4) & 0x3FFF) | (uint64_t)(col >> 4) << 16 | (uint64_t)(128 >> 4) << 32 |
+         (uint64_t)1 << 46;
+}
+
+// ---------------------------------------------------------------------------
+// Packed .bed rows -> operand planes.  Warp = one column of one half-block: lane
+// t reads the 16 bytes (64 samples) of marker row t, and each of the four
+// 16-sample words is transposed by warp shuffles; then lanes 2s and 2s + 1
+// hold the low and the high code bits of sample s at the 32 markers, exchange
+// them, and write 16 bytes of V and U (even lanes) or Q and R (odd lanes).  The
+// eight warps of a CTA take neighbouring half-blocks, so the CTA reads whole
+// 128-byte lines of the rows, and every store of a warp is 256 contiguous bytes
+// per plane.  HBM-bound: 0.25 B read and 2 B written per genotype.
+__global__ void __launch_bounds__(256) sweep_planes_kernel(const uint8_t* __restrict__ packed, int64_t row_bytes,
+                                                           int64_t n, int64_t m, uint8_t* __restrict__ planes,
+                                                           int64_t n_half, int64_t n_cols) {
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int64_t c = blockIdx.x, h = (int64_t)blockIdx.y * 8 + warp;
+  if (h >= n_half) return;
+  const int64_t marker = c * 32 + lane, byte0 = h * 16;
+  uint32_t w[4] = {0x55555555u, 0x55555555u, 0x55555555u, 0x55555555u};  // missing
+  if (marker < m) {
+    const uint8_t* p = packed + marker * row_bytes + byte0;
+    const int64_t left = row_bytes - byte0;  // bytes of the row from here on
+    const uintptr_t at = reinterpret_cast<uintptr_t>(p);
+    if (left >= 16 && (at & 15) == 0) {
+      const uint4 v = __ldg(reinterpret_cast<const uint4*>(p));
+      w[0] = v.x;
+      w[1] = v.y;
+      w[2] = v.z;
+      w[3] = v.w;
+    } else if (left >= 16 && marker > 0 && marker + 1 < m) {
+      // any alignment: five aligned words, all inside the matrix (the row is
+      // neither its first nor its last), shifted into place
+      const uint32_t* q = reinterpret_cast<const uint32_t*>(at & ~(uintptr_t)3);
+      const int sh = 8 * (int)(at & 3);
+      uint32_t v[5];
+#pragma unroll
+      for (int i = 0; i < 4; ++i) v[i] = __ldg(q + i);
+      v[4] = sh ? __ldg(q + 4) : 0u;
+#pragma unroll
+      for (int i = 0; i < 4; ++i) w[i] = __funnelshift_r(v[i], v[i + 1], sh);
+    } else {
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        uint32_t v = 0;
+#pragma unroll
+        for (int b = 0; b < 4; ++b)
+          v |= (uint32_t)(4 * i + b < left ? __ldg(p + 4 * i + b) : (uint8_t)0x55) << (8 * b);
+        w[i] = v;
+      }
+    }
+  }
+  const bool odd = (lane & 1) != 0;
+  const size_t plane_stride = (size_t)n_half * n_cols * 1024;
+  uint8_t* base = planes + (size_t)(odd ? 2 : 0) * plane_stride + ((size_t)h * n_cols + c) * 1024;
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    const uint32_t x = tc_transpose32(w[i], lane);
+    const uint32_t y = __shfl_xor_sync(0xffffffffu, x, 1);
+    const uint32_t L = odd ? y : x, H = odd ? x : y;
+    const int s = i * 16 + (lane >> 1);
+    const uint32_t mask = h * 64 + s < n ? 0xFFFFFFFFu : 0u;
+    const uint32_t a = (odd ? H & L : H | ~L) & mask;    // Q, or V
+    const uint32_t b = (odd ? ~H & ~L : H & ~L) & mask;  // R, or heterozygous
+    uint32_t wa[4], wb[4];
+#pragma unroll
+    for (int g = 0; g < 4; ++g) {
+      const uint32_t na = nib8(a >> (8 * g)) << 1, nb = nib8(b >> (8 * g));
+      wa[g] = na;
+      wb[g] = odd ? nb << 1 : na | (nb << 3);  // R, or U with the sign bit of heterozygous calls
+    }
+    *reinterpret_cast<uint4*>(base + s * 16) = make_uint4(wa[0], wa[1], wa[2], wa[3]);
+    *reinterpret_cast<uint4*>(base + plane_stride + s * 16) = make_uint4(wb[0], wb[1], wb[2], wb[3]);
+  }
+}
+
+// ---------------------------------------------------------------------------
+// Outputs of a tile.
+
+// Where the counts go: the triangle or the full square of n samples.
+struct SweepOut {
+  int64_t n;
+  int32_t* counts;
+  double* dist;
+  int32_t square;
+};
+
+// Write one piece of a tile, 32 rows from gi0 by 16 columns from gj0, from its
+// three products: load(pr, v) sets v[j] to product pr of (row gi0 + lane, column
+// gj0 + j).
+// The counts are packed into 64 bits (each below 2^21) and
+// transposed through `sm`, so that a half-warp stores 16 consecutive pairs of a
+// row (256 bytes of counts) at a time; a square's mirror image is contiguous
+// down the column as it is loaded.
+template <class Load>
+__device__ __forceinline__ void sweep_store(const SweepOut& o, int64_t gi0, int64_t gj0, const Load& load,
+                                            uint64_t* sm) {
+  const int lane = threadIdx.x & 31;
+  const int64_t n = o.n;
+  if (gi0 >= n || gj0 >= n || gj0 + 15 < gi0) return;
+  float vn[16], vu[16], vz[16];
+  load(0, vn);
+  load(1, vu);
+  load(2, vz);
+  __syncwarp();  // the warp's previous piece has been read
+#pragma unroll
+  for (int j = 0; j < 16; ++j) {
+    const uint32_t nn = (uint32_t)__float2int_rn(vn[j]), i0 = (uint32_t)__float2int_rn(vz[j]);
+    const uint32_t i1 = (nn - (uint32_t)__float2int_rn(vu[j])) >> 1;
+    sm[lane * 17 + j] = (uint64_t)nn << 42 | (uint64_t)i0 << 21 | i1;
+  }
+  __syncwarp();
+  auto put = [&](int64_t p, uint64_t v) {
+    const int32_t nn = (int32_t)(v >> 42), i0 = (int32_t)(v >> 21 & 0x1FFFFF), i1 = (int32_t)(v & 0x1FFFFF);
+    reinterpret_cast<int4*>(o.counts)[p] = make_int4(i0, i1, nn - i0 - i1, nn);
+    if (o.dist) o.dist[p] = ibs_dist(i0, i1, nn);
+  };
+  const int64_t gj = gj0 + (lane & 15);
+#pragma unroll 4
+  for (int r = lane >> 4; r < 32; r += 2) {
+    const int64_t gi = gi0 + r;
+    if (gi < n && gj < n && gj >= gi) put(o.square ? gi * n + gj : tri_index(gi, gj, n), sm[r * 17 + (lane & 15)]);
+  }
+  if (o.square) {
+    const int64_t gi = gi0 + lane;
+#pragma unroll 4
+    for (int j = 0; j < 16; ++j)
+      if (gi < n && gj0 + j < n && gj0 + j > gi) put((gj0 + j) * n + gi, sm[lane * 17 + j]);
+  }
+}
+
+// ---------------------------------------------------------------------------
+// The kernel.
+
+// A ring barrier's wait: one probe on the usual path; past it, bounded by
+// limit_ns and ended by another role's abort.
+__device__ __noinline__ bool sweep_wait_slow(uint64_t* bar, uint32_t parity, unsigned long long limit_ns,
+                                             const int* abort_flag) {
+  const unsigned long long t0 = globaltimer_ns();
+  for (;;) {
+    if (limit_ns < 1000000ull) {  // short bounds (tests): a blocking probe could outlast them
+      if (mbar_test_wait(bar, parity)) return true;
+    } else {
+      for (int i = 0; i < 64; ++i)
+        if (mbar_try_wait(bar, parity)) return true;
+    }
+    if (*(volatile const int*)abort_flag != 0 || globaltimer_ns() - t0 > limit_ns) return false;
+  }
+}
+__device__ __forceinline__ bool sweep_wait(uint64_t* bar, uint32_t parity, unsigned long long limit_ns,
+                                           const int* abort_flag) {
+  if (limit_ns >= 1000000ull && mbar_try_wait(bar, parity)) return true;
+  return sweep_wait_slow(bar, parity, limit_ns, abort_flag);
+}
+
+struct SweepArgs {
+  SweepOut out;
+  const SweepItem* items;
+  const int32_t* first;  // items of cluster c: first[c] .. first[c + 1] - 1
+  int32_t stages;        // ring stages per sweep
+  float* scratch;        // [CTA][3][384][128]: products of the CTA's whole item
+  float* part;           // [slot][2][384][128]: products of split items
+  int* status;
+  unsigned long long wait_ns;
+  SweepSync sync;
+};
+
+// Warps: 0 and 3 copies of A and of B, 1 MMAs (even CTA), 2 the MMA warp's waits
+// (even CTA), 4..11 epilogue.  Roles and barriers as in ibs_tc.cu's two-SM kernel: both CTAs'
+// copies complete on the even CTA's `full`; its MMA warp never waits on memory
+// itself (warp 2 does, and releases it once per stage through a hardware
+// barrier) and commits each stage to both CTAs' `empty` and each finished
+// product to both CTAs' `tfull`; the epilogue warps of both arrive on the even
+// CTA's `tempty` once the product is read.  Every wait is bounded.
+//
+// An item is a tile and a range [q0, q1) of the 4 * stages ring stages of its
+// sweeps.  A whole tile (slot < 0) keeps its products in the CTA's scratch and
+// is written after its last sweep, while the next item's first sweep runs; a
+// piece writes each product it has a part of to a slot of its own, which the
+// finalisation adds up.
+__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kSwThreads, 1)
+    sweep_kernel(const __grid_constant__ CUtensorMap amap, const __grid_constant__ CUtensorMap bmap1,
+                 const __grid_constant__ CUtensorMap bmap2, const __grid_constant__ CUtensorMap bmap3,
+                 const SweepArgs args) {
+  extern __shared__ __align__(1024) uint8_t smem_raw[];
+  uint8_t* ring = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
+  __shared__ __align__(8) uint64_t full[kSwStages], empty[kSwStages], tfull, tempty, drain;
+  __shared__ uint32_t tmem_slot;
+  __shared__ uint32_t issued[2];  // ring stages this CTA's copy warps issued
+  __shared__ int abort_flag;
+  __shared__ int s_dead;  // the waiter has stopped: the MMA warp does too
+  __shared__ int s_ok[2];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const uint32_t rank = cluster_rank();
+  const uint32_t cid = cluster_index();
+  const int S = args.stages;
+  int* status = args.status;
+  const unsigned long long wait_ns = args.wait_ns;
+  const int it0 = args.first[cid], it1 = args.first[cid + 1];
+  if (threadIdx.x == 0) {
+    for (int s = 0; s < kSwStages; ++s) {
+      mbar_init(&full[s], 1);  // the even CTA's: both CTAs' copies complete on it
+      mbar_init(&empty[s], 1);
+    }
+    mbar_init(&tfull, 1);
+    mbar_init(&tempty, 2 * kSwEpiWarps);
+    mbar_init(&drain, 1);
+    mbar_fence_init();
+    abort_flag = 0;
+    s_dead = 0;
+  }
+  if (warp == 0) {
+    asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_addr(&tmem_slot)),
+                 "r"(kTmemCols)
+                 : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
+  }
+  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+  __syncthreads();
+  asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+  const uint32_t tmem = tmem_slot;
+  if (warp >= 4 && warp < 8) tmem_fill_unit_scales(tmem, warp - 4);
+  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+  cluster_sync_all();  // both CTAs' barriers initialised and scale factors stored
+  asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+
+  // a product ends with sweep 0, 1 or 3, or with the item
+  auto product_end = [&](int q, int q1) { return min(q1, q < S ? S : (q < 2 * S ? 2 * S : 4 * S)); };
+
+  if (warp == 0 || warp == 3) {
+    // Copies: lane 0 of warp 0 streams the A operand, lane 0 of warp 3 the B
+    // operand, one box per ring stage each.
+    if (lane == 0) {
+      const bool is_b = warp == 3;
+      const uint32_t full0 = cluster_addr(&full[0], 0);  // the even CTA's ring barriers
+      uint8_t* dst0 = ring + (is_b ? kSwABytes : 0);
+      uint32_t g = 0, s = 0, ph = 1;  // stages issued, ring slot, parity of the slot's previous release
+      bool stop = false;
+      for (int e = it0; e < it1 && !stop; ++e) {
+        const SweepItem it = args.items[e];
+        const int h = is_b ? 2 * it.J + it.w * (int)rank : 2 * (it.I + (int)rank);
+        const CUtensorMap* map = !is_b ? &amap : (it.w == 3 ? &bmap3 : (it.w == 2 ? &bmap2 : &bmap1));
+        const uint32_t bytes = 2u * (uint32_t)(kSwABytes + kSwCols * 1024 * it.w);
+        // lockstep: warp 0 announces every segment and holds back until the
+        // whole wave has started the segment `lag` back (warp 3 follows
+        // through the ring)
+        int* ctr = !is_b && args.sync.seg > 0 && it.wave >= 0 ? args.sync.ctr + (int64_t)it.wave * args.sync.n_seg : nullptr;
+        int left = 0, sg = 0;
+        int q = it.q0;
+        while (q < it.q1 && !stop) {
+          const int sw = q < 2 * S ? (q < S ? 0 : 1) : (q < 3 * S ? 2 : 3);
+          const int plane = is_b && sw >= 2 ? 5 - sw : sw;  // sweep 2: Q R^T, sweep 3: R Q^T
+          const int end = min(it.q1, (sw + 1) * S);
+          for (int col = (q - sw * S) * kSwCols; q < end; ++q, col += kSwCols) {
+            if (ctr != nullptr && left-- == 0) {
+              left = args.sync.seg - 1;
+              atomicAdd(ctr + sg, 1);
+              if (sg >= args.sync.lag && !wait_ready(ctr + sg - args.sync.lag, 2 * (int)cluster_total(), wait_ns)) {
+                stop = true;
+                break;
+              }
+              ++sg;
+            }
+            if (g >= (uint32_t)kSwStages && !sweep_wait(&empty[s], ph, wait_ns, &abort_flag)) {
+              stop = true;
+              break;
+            }
+            const uint32_t bar = full0 + s * 8u;
+            if (!is_b && rank == 0) mbar_arrive_expect_tx(&full[s], bytes);
+            tma_load_4d_pair(dst0 + s * kSwStageBytes, map, 0, h, col, plane, bar);
+            ++g;
+            if (++s == kSwStages) {
+              s = 0;
+              ph ^= 1u;
+            }
+          }
+        }
+      }
+      if (stop && *(volatile int*)&abort_flag == 0) {
+        atomicExch(status, kDevTimeout);
+        atomicExch(&abort_flag, 1);
+      }
+      // the last stages' releases (commits of the even CTA) have landed here
+      for (uint32_t j = g > (uint32_t)kSwStages ? g - kSwStages : 0; j < g && !stop; ++j)
+        if (!mbar_wait_bounded(&empty[j % kSwStages], (j / kSwStages) & 1u)) {
+          atomicExch(status, kDevTimeout);
+          atomicExch(&abort_flag, 1);
+          break;
+        }
+      issued[is_b ? 1 : 0] = g;
+    }
+    __syncwarp();
+  } else if (warp == 1 && rank == 0) {
+    // The tensor core queues only a few MMAs, so what lies between one stage's
+    // last MMA and the next one's first is kept short.
+    uint32_t s = 0;
+    const uint32_t sf = tmem + kSfCol, ring0 = smem_addr(ring);
+    bool dead = false;
+    // the stages [q, end) of one product, kN columns per MMA, kM MMAs per K step
+    auto product = [&](auto width, int stages) {
+      constexpr int w = decltype(width)::value;
+      constexpr int kN = w == 3 ? 192 : 128 * w;
+      uint32_t acc = 0;  // the first K step overwrites
+      for (int k = 0; k < stages; ++k) {
+        sweep_acquire(s);
+        if (*(volatile int*)&s_dead != 0) {
+          dead = true;
+          return;
+        }
+        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+        if (lane == 0) {
+          const uint32_t st0 = ring0 + s * kSwStageBytes;
+          const uint64_t a = sweep_desc(st0, 2048), b = sweep_desc(st0 + kSwABytes, 1024 * w);
+#pragma unroll
+          for (int t = 0; t < kSwCols / 3; ++t) {
+            umma_sweep<kN>(tmem, a + t * (3 * 2048 / 16), b + t * (3 * 1024 * w / 16), acc, sf);
+            if constexpr (w == 3)
+              umma_sweep<kN>(tmem + 192, a + t * (3 * 2048 / 16), b + t * (3 * 1024 * w / 16) + 96 * 16 / 16, acc, sf);
+            acc = 1;
+          }
+          umma_commit_both(&empty[s]);
+        }
+        acc = 1;
+        s = s + 1 == kSwStages ? 0 : s + 1;
+      }
+      if (lane == 0) umma_commit_both(&tfull);
+    };
+    for (int e = it0; e < it1 && !dead; ++e) {
+      const SweepItem it = args.items[e];
+      for (int q = it.q0; q < it.q1 && !dead;) {
+        const int end = product_end(q, it.q1);
+        if (it.w == 3)
+          product(std::integral_constant<int, 3>{}, end - q);
+        else if (it.w == 2)
+          product(std::integral_constant<int, 2>{}, end - q);
+        else
+          product(std::integral_constant<int, 1>{}, end - q);
+        q = end;
+      }
+    }
+    __syncwarp();
+    if (lane == 0) umma_commit_local2(&drain);
+    __syncwarp();
+    const bool drained = mbar_wait_bounded(&drain, 0);
+    if (lane == 0 && !drained) atomicExch(status, kDevTimeout);
+  } else if (warp == 2 && rank == 0) {
+    // After a failed wait or another role's abort the waiter and the MMA warp
+    // stop together: nothing is issued or released any more, and the copy and
+    // epilogue warps of both CTAs come to the end of their own bounds.
+    uint32_t s = 0, ph = 0, p = 0;  // ring slot and its parity, products
+    bool dead = false, wrapped = false;
+    for (int e = it0; e < it1 && !dead; ++e) {
+      const SweepItem it = args.items[e];
+      for (int q = it.q0; q < it.q1 && !dead; ++p) {
+        const int end = product_end(q, it.q1);
+        bool ok = lane != 0 || p == 0 || mbar_wait_cluster_bounded(&tempty, (p - 1) & 1u, wait_ns);
+        for (; q < end; ++q) {
+          // every lane of the warp goes on, or none
+          if (lane == 0 && ok) ok = sweep_wait(&full[s], ph, wait_ns, &abort_flag);
+          if (__any_sync(0xffffffffu, !ok)) {
+            dead = true;
+            break;
+          }
+          asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+          sweep_release(s);
+          s = s + 1 == kSwStages ? 0 : s + 1;
+          ph ^= s == 0 ? 1u : 0u;
+          wrapped |= s == 0;
+        }
+      }
+    }
+    if (dead) {
+      if (lane == 0) {
+        if (*(volatile int*)&abort_flag == 0) {
+          atomicExch(status, kDevTimeout);
+          atomicExch(&abort_flag, 1);
+        }
+        *(volatile int*)&s_dead = 1;
+        // the slot's previous release has been taken once its stage is
+        // committed: two arrivals before the MMA warp's would pair up
+        if (wrapped) mbar_wait_bounded(&empty[s], ph ^ 1u);
+      }
+      __syncwarp();
+      sweep_release(s);  // the MMA warp finds s_dead
+    }
+  } else if (warp >= 4) {
+    const int quarter = warp & 3, part = (warp - 4) >> 2, row = quarter * 32 + lane;
+    const uint32_t lane_base = tmem + ((uint32_t)(quarter * 32) << 16);
+    const uint32_t tempty_addr = cluster_addr(&tempty, 0);
+    float* scratch = args.scratch + (size_t)(2 * cid + rank) * 3 * kSwHalfTile;
+    uint64_t* sm = reinterpret_cast<uint64_t*>(ring + (size_t)kSwStages * kSwStageBytes + (warp - 4) * kSwTransBytes);
+    uint32_t p = 0;
+    bool stop = false;
+    for (int e = it0; e < it1 && !stop; ++e) {
+      const SweepItem it = args.items[e];
+      int slot = it.slot;
+      for (int q = it.q0; q < it.q1;) {
+        const int pr = q < S ? 0 : (q < 2 * S ? 1 : 2);
+        const int end = pr == 2 ? 4 * S : (pr + 1) * S;
+        q = end < it.q1 ? end : it.q1;
+        // one thread waits for the product and decides for all eight warps
+        // (alternating slots: a warp that is late still reads its own decision)
+        if (threadIdx.x == 128)
+          s_ok[p & 1] = mbar_wait_bounded(&tfull, p & 1u, wait_ns) && *(volatile int*)&abort_flag == 0;
+        asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+        asm volatile("bar.sync %0, %1;" ::"n"(kSwEpiBar), "n"(32 * kSwEpiWarps) : "memory");
+        if (*(volatile int*)&s_ok[p & 1] == 0) {
+          if (threadIdx.x == 128 && *(volatile int*)&abort_flag == 0) {
+            atomicExch(status, kDevTimeout);
+            atomicExch(&abort_flag, 1);
+          }
+          stop = true;
+          break;
+        }
+        ++p;
+        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+        float* dst = it.slot < 0 ? scratch + pr * kSwHalfTile : args.part + (size_t)(2 * slot + (int)rank) * kSwHalfTile;
+        ++slot;
+        // 32-column groups part, part + 2, ...; three in flight
+        const int ng = 4 * it.w;
+        for (int g0 = part; g0 < ng; g0 += 6) {
+          uint32_t v[3][32];
+#pragma unroll
+          for (int u = 0; u < 3; ++u) tmem_ld32(lane_base + (g0 + 2 * u) * 32, v[u]);  // past ng: columns unused
+          asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+          if (g0 + 6 >= ng) {  // the last of this warp's columns are in registers: hand tensor memory back
+            asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+            __syncwarp();
+            if (lane == 0) mbar_arrive_cluster(tempty_addr);
+          }
+#pragma unroll
+          for (int u = 0; u < 3; ++u) {
+            const int gr = g0 + 2 * u;
+            if (gr < ng) {
+              // w = 3: two MMAs of 192 columns, each 96 of the even CTA's B
+              // rows and 96 of the odd CTA's
+              const int c0 = it.w == 3 ? (gr % 6) / 3 * 192 + gr / 6 * 96 + gr % 3 * 32 : gr * 32;
+#pragma unroll
+              for (int j = 0; j < 32; ++j) dst[(size_t)(c0 + j) * kTB + row] = __uint_as_float(v[u][j]);
+            }
+          }
+        }
+      }
+      if (stop || it.slot >= 0) continue;
+      // whole tile: every product is in the scratch; 32 x 16 pieces by warps
+      asm volatile("bar.sync %0, %1;" ::"n"(kSwEpiBar), "n"(32 * kSwEpiWarps) : "memory");
+      const int64_t gi0 = (int64_t)(it.I + (int)rank) * kTB + quarter * 32;
+      for (int ct = part; ct < 8 * it.w; ct += 2) {
+        const float* src = scratch + (size_t)ct * 16 * kTB + row;
+        sweep_store(args.out, gi0, (int64_t)it.J * kTB + ct * 16,
+                    [&](int pr, float (&v)[16]) {
+#pragma unroll
+                      for (int j = 0; j < 16; ++j) v[j] = __ldcg(src + pr * kSwHalfTile + (size_t)j * kTB);
+                    },
+                    sm);
+      }
+    }
+  }
+  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+  __syncthreads();
+  cluster_sync_all();  // both CTAs have issued their last copy and the even CTA's MMAs are drained
+  if (rank == 0 && warp == 0) {
+    // Every copy of either CTA completes on the even CTA's `full`.  After a
+    // stop some issued stages were never consumed, so wait (bounded) for the
+    // last ring's worth that either CTA issued before either CTA may exit.
+    uint32_t p0 = 0, p1 = 0;
+    asm volatile("ld.shared::cluster.u32 %0, [%1];" : "=r"(p0) : "r"(cluster_addr(&issued[0], 1)) : "memory");
+    asm volatile("ld.shared::cluster.u32 %0, [%1];" : "=r"(p1) : "r"(cluster_addr(&issued[1], 1)) : "memory");
+    const uint32_t gmax = max(max(issued[0], issued[1]), max(p0, p1));
+    for (uint32_t j = gmax > (uint32_t)kSwStages ? gmax - kSwStages : 0; j < gmax; ++j) {
+      const bool ok = mbar_wait_bounded(&full[j % kSwStages], (j / kSwStages) & 1u);
+      if (__any_sync(0xffffffffu, !ok)) {
+        if (lane == 0) atomicExch(status, kDevTimeout);
+        break;
+      }
+    }
+  }
+  __syncthreads();
+  cluster_sync_all();  // no copy into either CTA and no arrival on either CTA's barriers is outstanding
+  asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+  if (warp == 0) {
+    asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(kTmemCols) : "memory");
+  }
+}
+
+// Split tiles: the parts of each product added up and written.  Warp = one 32 x
+// 16 piece of a tile, 32 loads of parts in flight per thread.
+__global__ void __launch_bounds__(128) sweep_finalize_kernel(const SweepGroup* __restrict__ groups,
+                                                             const float* __restrict__ part, const SweepOut out) {
+  __shared__ uint64_t sm[4][32 * 17];
+  const SweepGroup gr = groups[blockIdx.x];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int t = blockIdx.y * 4 + warp;  // 2 CTAs x 4 row quarters x 24 column pieces
+  const int ct = t % 24, quarter = (t / 24) & 3, rank = t / 96;
+  if (ct >= 8 * gr.w) return;
+  const float* src = part + (size_t)(2 * gr.slot + rank) * kSwHalfTile + (size_t)ct * 16 * kTB + quarter * 32 + lane;
+  const int first[3] = {0, gr.pieces[0], gr.pieces[0] + gr.pieces[1]};
+  sweep_store(out, (int64_t)(gr.I + rank) * kTB + quarter * 32, (int64_t)gr.J * kTB + ct * 16,
+              [&](int pr, float (&v)[16]) {
+                const float* p = src + (size_t)first[pr] * 2 * kSwHalfTile;
+#pragma unroll
+                for (int j = 0; j < 16; ++j) v[j] = 0.0f;
+#pragma unroll 2
+                for (int k = 0; k < gr.pieces[pr]; ++k, p += 2 * kSwHalfTile)
+#pragma unroll
+                  for (int j = 0; j < 16; ++j) v[j] += __ldg(p + (size_t)j * kTB);  // whole numbers: exact
+              },
+              sm[warp]);
+}
+
+// A view of the operand planes, a box `halves` half-blocks over kSwCols
+// columns of one plane, landing as [column][half-block][1 KiB]; half-blocks
+// past the last read as zeros.
+bool encode_sweep_map(CUtensorMap* map, const void* planes, int64_t n_half, int64_t n_cols, int halves) {
+  const EncodeTiledFn fn = encode_tiled_fn();
+  if (!fn) return false;
+  const cuuint64_t dims[4] = {128, (cuuint64_t)n_half, (cuuint64_t)n_cols, 4};
+  const cuuint64_t strides[3] = {(cuuint64_t)n_cols * 1024, 1024, (cuuint64_t)n_half * (cuuint64_t)n_cols * 1024};
+  const cuuint32_t box[4] = {128, (cuuint32_t)halves, kSwCols, 1};
+  const cuuint32_t elem[4] = {1, 1, 1, 1};
+  return fn(map, CU_TENSOR_MAP_DATA_TYPE_UINT64, 4, const_cast<void*>(planes), dims, strides, box, elem,
+            CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+            CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
+}  // namespace
+
+int sweep_stages(int64_t m) { return (int)((m + kSwMarkers - 1) / kSwMarkers); }
+
+size_t sweep_planes_bytes(int64_t n, int64_t m) {
+  return (size_t)((n + 63) / 64) * (size_t)sweep_stages(m) * kSwCols * 4096;
+}
+
+size_t sweep_scratch_bytes(int clusters) { return (size_t)clusters * 2 * 3 * kSwHalfTile * sizeof(float); }
+size_t sweep_slot_bytes() { return 2 * kSwHalfTile * sizeof(float); }
+
+cudaError_t launch_sweep_planes(const uint8_t* packed, int64_t n, int64_t m, uint8_t* planes, cudaStream_t st) {
+  const int64_t nh = (n + 63) / 64, nc = (int64_t)sweep_stages(m) * kSwCols;
+  if (nc > 2147483647LL || (nh + 7) / 8 > 65535) return cudaErrorInvalidValue;
+  sweep_planes_kernel<<<dim3((unsigned)nc, (unsigned)((nh + 7) / 8)), 256, 0, st>>>(packed, (n + 3) / 4, n, m, planes,
+                                                                                    nh, nc);
+  return cudaGetLastError();
+}
+
+// Clusters of two that fit at once, counted once per device ordinal.
+int sweep_clusters() {
+  constexpr int kDevs = 64;
+  static std::atomic<int> cache[kDevs];  // 0 = not yet counted, else count + 1
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kDevs) {
+    cudaGetLastError();
+    return 0;
+  }
+  if (const int c = cache[dev].load(std::memory_order_acquire)) return c - 1;
+  int n = 0, sms = 0;
+  if (cudaFuncSetAttribute(sweep_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSwSmem) == cudaSuccess &&
+      cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)std::max(2, sms & ~1));
+    cfg.blockDim = dim3(kSwThreads);
+    cfg.dynamicSmemBytes = kSwSmem;
+    if (cudaOccupancyMaxActiveClusters(&n, sweep_kernel, &cfg) != cudaSuccess) n = 0;
+  }
+  cudaGetLastError();
+  cache[dev].store(n + 1, std::memory_order_release);
+  return n;
+}
+
+// E2M1 form; a tile's counts below 2^21 (exact FP32 sums, and their packing in
+// sweep_store); the tensor map's coordinates.
+bool sweep_usable(int64_t n, int64_t m) {
+  if (m >= ((int64_t)1 << 21) || (n + 63) / 64 > 65535 * 8) return false;
+  return encode_tiled_fn() != nullptr && sweep_clusters() > 0;
+}
+
+// Work list of a triangle of n samples.  Tiles of two block rows by up to
+// three block columns, in bands of 16 block rows, column by column in a band, so
+// that the tiles in flight share operand blocks through L2.  The columns are
+// grouped from the right edge, the same for every row, and the group that
+// holds the diagonal starts at it.  The full-width tiles run whole, one per cluster and wave, as
+// many full waves as there are; the rest (the last partial wave and the
+// narrower tiles) are laid end to end, weighted by their cost per stage, and
+// cut into equal shares, one per cluster, each share a few pieces of
+// neighbouring tiles.
+SweepPlan sweep_plan(int64_t n, int64_t m, int clusters) {
+  SweepPlan pl;
+  const int S = sweep_stages(m);
+  pl.stages = S;
+  const int T = (int)((n + kTB - 1) / kTB), C = std::max(1, clusters);
+  struct Tile {
+    int I, J, w;
+  };
+  std::vector<Tile> full, rest;
+  constexpr int G = 16;
+  for (int g0 = 0; g0 < T; g0 += G)
+    for (int end = (T - g0 - 1) % 3 + 1 + g0; end <= T; end += 3)  // column groups end at T, T - 3, ...
+      for (int I = g0; I < std::min(T, g0 + G) && I < end; I += 2) {
+        const int J = std::max(I, end - 3);
+        (end - J == 3 ? full : rest).push_back({I, J, end - J});
+      }
+  const int waves = (int)(full.size() / (size_t)C);
+  const size_t whole = (size_t)waves * C;
+  rest.insert(rest.begin(), full.begin() + (long)whole, full.end());
+  // cost of one stage (cycles measured or, for narrow tiles, bound by the
+  // copies) and of a piece's start and end
+  auto cost = [](int w) { return w == 3 ? 620.0 : (w == 2 ? 520.0 : 500.0); };
+  double total = 0;
+  for (const Tile& t : rest) total += cost(t.w) * 4 * S;
+  // shares: one per cluster, but none shorter than a few stages (a piece costs
+  // about kMin stages of its own: pipeline fill, read-back, a part to add up)
+  constexpr double kMin = 8;
+  const int shares = (int)std::max(1.0, std::min((double)C, total / (620.0 * kMin)));
+  std::vector<std::vector<SweepItem>> own((size_t)C);
+  for (size_t t = 0; t < whole; ++t) {
+    SweepItem it{};
+    it.I = full[t].I;
+    it.J = full[t].J;
+    it.w = full[t].w;
+    it.q1 = 4 * S;
+    it.slot = -1;
+    it.wave = (int)(t / C);
+    own[t % C].push_back(it);
+  }
+  pl.waves = waves;
+  int share = 0;
+  double used = 0;  // cost laid so far
+  for (const Tile& t : rest) {
+    SweepGroup gr{};
+    gr.I = t.I;
+    gr.J = t.J;
+    gr.w = t.w;
+    gr.slot = pl.slots;
+    int q = 0;
+    while (q < 4 * S) {
+      // stages left in this share
+      const double left = total * (share + 1) / shares - used;
+      int k = (int)(left / cost(t.w) + 0.5);
+      if (share == shares - 1) k = 4 * S - q;
+      k = std::min(k, 4 * S - q);
+      if (4 * S - q - k > 0 && 4 * S - q - k < 3) k = 4 * S - q;  // no sliver left behind
+      if (k < 3 && k < 4 * S - q) {                              // nor one begun
+        ++share;
+        continue;
+      }
+      SweepItem it{};
+      it.I = t.I;
+      it.J = t.J;
+      it.w = t.w;
+      it.q0 = q;
+      it.q1 = q + k;
+      it.slot = pl.slots;
+      it.wave = -1;
+      if (q == 0 && k == 4 * S) {
+        it.slot = -1;  // a whole tile after all
+      } else {
+        for (int pr = 0; pr < 3; ++pr) {
+          const int a = pr == 0 ? 0 : pr * S, b = pr == 2 ? 4 * S : (pr + 1) * S;
+          if (it.q0 < b && it.q1 > a) {
+            ++gr.pieces[pr];
+            ++pl.slots;
+          }
+        }
+      }
+      own[(size_t)(share % C)].push_back(it);
+      used += cost(t.w) * k;
+      q += k;
+      if (used >= total * (share + 1) / shares - 1e-6 && share < shares - 1) ++share;
+    }
+    if (gr.pieces[0] + gr.pieces[1] + gr.pieces[2] > 0) pl.groups.push_back(gr);
+  }
+  pl.first.assign((size_t)C + 1, 0);
+  for (int c = 0; c < C; ++c) {
+    for (const SweepItem& it : own[(size_t)c]) {
+      if (it.slot < 0) pl.scratch = true;
+      pl.items.push_back(it);
+    }
+    pl.first[(size_t)c + 1] = (int32_t)pl.items.size();
+  }
+  // clusters without work are not launched
+  pl.clusters = C;
+  while (pl.clusters > 1 && pl.first[(size_t)pl.clusters - 1] == (int32_t)pl.items.size()) --pl.clusters;
+  return pl;
+}
+
+cudaError_t launch_sweep(const SweepLaunch& l, cudaStream_t st) {
+  CUtensorMap a, b1, b2, b3;
+  const int64_t nc = (int64_t)l.stages * kSwCols;
+  if (!encode_sweep_map(&a, l.a_planes, l.a_half, nc, 2) || !encode_sweep_map(&b1, l.b_planes, l.b_half, nc, 1) ||
+      !encode_sweep_map(&b2, l.b_planes, l.b_half, nc, 2) || !encode_sweep_map(&b3, l.b_planes, l.b_half, nc, 3))
+    return cudaErrorInvalidValue;
+  // function attributes are per device: set before every launch
+  cudaError_t e = cudaFuncSetAttribute(sweep_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSwSmem);
+  if (e != cudaSuccess) return e;
+  SweepArgs args{};
+  args.out = SweepOut{l.n, l.counts, l.dist, l.square ? 1 : 0};
+  args.items = l.items;
+  args.first = l.first;
+  args.stages = l.stages;
+  args.scratch = l.scratch;
+  args.part = l.part;
+  args.status = l.status;
+  args.wait_ns = l.wait_ns;
+  args.sync = l.sync;
+  sweep_kernel<<<2 * l.clusters, kSwThreads, kSwSmem, st>>>(a, b1, b2, b3, args);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_sweep_finalize(const SweepLaunch& l, const SweepGroup* groups, int64_t n_groups, cudaStream_t st) {
+  if (n_groups <= 0) return cudaSuccess;
+  sweep_finalize_kernel<<<dim3((unsigned)n_groups, 48), 128, 0, st>>>(
+      groups, l.part, SweepOut{l.n, l.counts, l.dist, l.square ? 1 : 0});
+  return cudaGetLastError();
+}
+
+}  // namespace ibs

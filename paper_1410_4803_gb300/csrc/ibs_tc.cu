@@ -46,8 +46,6 @@
 #include <cstring>
 #include <vector>
 
-#include <cuda.h>
-
 #include "ibs_tc_common.cuh"
 
 namespace ibs {
@@ -106,18 +104,6 @@ __device__ __forceinline__ void store_plane_row(uint8_t* base, uint32_t vb, uint
 // bits of its part of the row: FP8, lane 2k markers 0..15 and lane 2k+1
 // markers 16..31; FP4 (two groups), lane 2k markers 0..31 and lane 2k+1
 // markers 32..63.  Each lane writes 16 bytes of each of the sample's planes.
-__device__ __forceinline__ uint32_t tc_transpose32(uint32_t x, int lane) {
-  constexpr uint32_t kMask[5] = {0x0000FFFFu, 0x00FF00FFu, 0x0F0F0F0Fu, 0x33333333u, 0x55555555u};
-#pragma unroll
-  for (int r = 0; r < 5; ++r) {
-    const int j = 16 >> r;
-    const uint32_t m = kMask[r];
-    const uint32_t y = __shfl_xor_sync(0xffffffffu, x, j);
-    x = (lane & j) == 0 ? ((x & m) | ((y & m) << j)) : ((x & ~m) | ((y & ~m) >> j));
-  }
-  return x;
-}
-
 template <int F>
 __global__ void __launch_bounds__(256) tc_planes_kernel(const uint8_t* __restrict__ packed, int64_t row_bytes,
                                                         int64_t n, int64_t m, uint8_t* __restrict__ planes,
@@ -911,71 +897,6 @@ __global__ void __launch_bounds__(256, 1)
 // (tc_pair_mode).  A relay warp that forwarded each stage of the odd CTA with
 // a cluster-scope release arrive cost about 1.7 us per stage (2.8 ms).
 
-__device__ __forceinline__ uint32_t cluster_rank() {
-  uint32_t r;
-  asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
-  return r;
-}
-__device__ __forceinline__ uint32_t cluster_index() {
-  uint32_t r;
-  asm volatile("mov.u32 %0, %%clusterid.x;" : "=r"(r));
-  return r;
-}
-__device__ __forceinline__ uint32_t cluster_total() {
-  uint32_t r;
-  asm volatile("mov.u32 %0, %%nclusterid.x;" : "=r"(r));
-  return r;
-}
-// Every thread of both CTAs: release this CTA's prior writes, acquire the peer's.
-__device__ __forceinline__ void cluster_sync_all() {
-  asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
-}
-// Address of the same shared variable in cluster CTA `rank`.
-__device__ __forceinline__ uint32_t cluster_addr(const void* p, uint32_t rank) {
-  uint32_t r;
-  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(smem_addr(p)), "r"(rank));
-  return r;
-}
-__device__ __forceinline__ void mbar_arrive_cluster(uint32_t addr) {
-  asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(addr) : "memory");
-}
-// Waits on a barrier that the peer CTA also arrives on (acquire at cluster scope).
-__device__ __forceinline__ bool mbar_try_wait_cluster(uint64_t* bar, uint32_t parity) {
-  uint32_t ok;
-  asm volatile(
-      "{\n\t.reg .pred p;\n\t"
-      "mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n\t"
-      "selp.u32 %0, 1, 0, p;\n\t}"
-      : "=r"(ok)
-      : "r"(smem_addr(bar)), "r"(parity)
-      : "memory");
-  return ok != 0;
-}
-__device__ __forceinline__ bool mbar_wait_cluster_bounded(uint64_t* bar, uint32_t parity,
-                                                          unsigned long long limit_ns = kWaitLimitNs) {
-  if (limit_ns < 1000000ull) {  // short bounds (tests): non-blocking probes, clock read after each
-    const unsigned long long t0 = globaltimer_ns();
-    for (;;) {
-      uint32_t ok;
-      asm volatile(
-          "{\n\t.reg .pred p;\n\t"
-          "mbarrier.test_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n\t"
-          "selp.u32 %0, 1, 0, p;\n\t}"
-          : "=r"(ok)
-          : "r"(smem_addr(bar)), "r"(parity)
-          : "memory");
-      if (ok) return true;
-      if (globaltimer_ns() - t0 > limit_ns) return false;
-    }
-  }
-  if (mbar_try_wait_cluster(bar, parity)) return true;
-  const unsigned long long t0 = globaltimer_ns();
-  for (;;) {
-    for (int i = 0; i < 64; ++i)
-      if (mbar_try_wait_cluster(bar, parity)) return true;
-    if (globaltimer_ns() - t0 > limit_ns) return false;
-  }
-}
 // The same loads issued by either CTA of the pair, completing on the barrier
 // at `bar` (a shared::cluster address: the even CTA's barrier), so the even
 // CTA's MMA warp sees both CTAs' operands land on one barrier.
@@ -987,15 +908,6 @@ __device__ __forceinline__ void tma_load_3d_pair(void* dst, const CUtensorMap* m
       "l"(reinterpret_cast<uint64_t>(map)), "r"(x0), "r"(x1), "r"(x2), "r"(bar)
       : "memory");
 }
-__device__ __forceinline__ void tma_load_4d_pair(void* dst, const CUtensorMap* map, int x0, int x1, int x2, int x3,
-                                                 uint32_t bar) {
-  asm volatile(
-      "cp.async.bulk.tensor.4d.shared::cluster.global.tile.mbarrier::complete_tx::bytes.cta_group::2 [%0], [%1, {%2, "
-      "%3, %4, %5}], [%6];" ::"r"(smem_addr(dst)),
-      "l"(reinterpret_cast<uint64_t>(map)), "r"(x0), "r"(x1), "r"(x2), "r"(x3), "r"(bar)
-      : "memory");
-}
-
 // Block-scaled E2M1 x E2M1 -> F32, M = 256 over the CTA pair, N = 128.
 constexpr uint32_t kIdescFp4Pair =
     (1u << 7) | (1u << 10) | ((uint32_t)(128 >> 3) << 17) | (1u << 23) | ((uint32_t)(256 >> 4) << 24);
@@ -1006,18 +918,6 @@ __device__ __forceinline__ void umma_pair(uint32_t tmem, uint64_t a, uint64_t b,
           tmem),
       "l"(a), "l"(b), "r"(kIdescFp4Pair), "r"(acc), "r"(sf), "r"(sf + 64u)
       : "memory");
-}
-// Arrives on the barrier at this offset in both CTAs once the MMAs issued so far are done.
-__device__ __forceinline__ void umma_commit_both(uint64_t* bar) {
-  asm volatile(
-      "tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;" ::"r"(
-          smem_addr(bar)),
-      "h"((uint16_t)3)
-      : "memory");
-}
-__device__ __forceinline__ void umma_commit_local2(uint64_t* bar) {
-  asm volatile("tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(smem_addr(bar))
-               : "memory");
 }
 // The four MMAs of one chunk; b0 is this CTA's B half: [plane][64 rows].
 __device__ __forceinline__ void chunk_mmas_pair(uint32_t tmem, uint32_t a0, uint32_t b0, uint32_t acc) {
@@ -1089,18 +989,6 @@ __device__ __forceinline__ TriEpi pair_epi(const PW& w, const PairItem& pi, int3
 __device__ __forceinline__ CrossWork::Epi pair_epi(const PairCrossWork& w, const PairItem& pi, int32_t ib, int row) {
   const int64_t r = ib >= 0 ? (int64_t)ib * kTB + row : w.n_rows;
   return {r < w.n_rows ? w.row_out[r] : nullptr, (int64_t)pi.J * kTB, w.n_panel};
-}
-
-// Wait until *counter >= need (another CTA's gather units; bounded).
-__device__ __forceinline__ bool wait_ready(const int* counter, int need, unsigned long long limit_ns) {
-  const unsigned long long t0 = globaltimer_ns();
-  for (unsigned ns = 32;; ns = ns < 1024 ? 2 * ns : ns) {
-    int v;
-    asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(counter) : "memory");
-    if (v >= need) return true;
-    if (globaltimer_ns() - t0 > limit_ns) return false;
-    __nanosleep(ns);
-  }
 }
 
 // Hardware barrier of the pair kernel's four epilogue warps (the fused gather's lock step).
@@ -1816,25 +1704,6 @@ int tc_pair_clusters(int64_t chunks_per_item) {
   if (r.per == 4 && r.stages == 2) return pair_clusters_s<2, 4>();
   if (r.per == 3 && r.stages == 3) return pair_clusters_s<3, 3>();
   return 0;
-}
-
-// cuTensorMapEncodeTiled, from the driver through the runtime (no link-time
-// dependency on libcuda).
-using EncodeTiledFn = CUresult (*)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
-                                   const cuuint64_t*, const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave,
-                                   CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
-EncodeTiledFn encode_tiled_fn() {
-  static const EncodeTiledFn fn = [] {
-    void* p = nullptr;
-    cudaDriverEntryPointQueryResult q = cudaDriverEntryPointSymbolNotFound;
-    if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &p, 12000, cudaEnableDefault, &q) != cudaSuccess ||
-        q != cudaDriverEntryPointSuccess) {
-      cudaGetLastError();
-      return (EncodeTiledFn) nullptr;
-    }
-    return reinterpret_cast<EncodeTiledFn>(p);
-  }();
-  return fn;
 }
 
 // Two views of the operand planes as 64-bit elements.  A: [block * chunk]

@@ -1,0 +1,92 @@
+// Host-only check of the sweep kernel's work lists (sweep_plan), built by
+// tests/test_sweep_plan.py with nvcc and run on the CPU: no device call.  For
+// every shape and cluster count it checks that
+//   - every block of the triangle (rows in pairs, from the diagonal to the right
+//     edge) is covered once over the stages of all four sweeps;
+//   - a tile covered by several items is in the list of split tiles with one
+//     part slot per item and product it touches, all slots used exactly once;
+//   - items stay inside the triangle, and the waves of whole tiles have one tile
+//     per cluster.
+// Prints one line per failure and "checked N lists, F failures".
+#include "../paper_1410_4803_gb300/csrc/ibs_sweep.cu"
+
+#include <map>
+#include <utility>
+
+namespace {
+
+int failures = 0;
+void fail(const char* what, int64_t n, int64_t m, int c) {
+  ++failures;
+  printf("FAIL %s: n=%lld m=%lld clusters=%d\n", what, (long long)n, (long long)m, c);
+}
+
+void check(int64_t n, int64_t m, int C) {
+  using namespace ibs;
+  const int T = (int)((n + 127) / 128), S = sweep_stages(m);
+  const SweepPlan p = sweep_plan(n, m, C);
+  std::map<std::pair<int, int>, std::vector<std::pair<int, int>>> cover;
+  std::map<std::pair<int, int>, SweepGroup> groups;
+  std::vector<int> used((size_t)p.slots, 0), wave((size_t)p.waves, 0);
+  for (const SweepGroup& g : p.groups) groups[{g.I, g.J}] = g;
+  if (p.clusters < 1 || p.clusters > C || p.first.size() != (size_t)C + 1) fail("cluster count", n, m, C);
+  for (const SweepItem& it : p.items) {
+    if (it.w < 1 || it.w > 3 || it.I % 2 || it.I < 0 || it.J < it.I || it.J + it.w > T || it.q0 < 0 || it.q1 <= it.q0 ||
+        it.q1 > 4 * S)
+      fail("item", n, m, C);
+    for (int b = 0; b < it.w; ++b) cover[{it.I, it.J + b}].push_back({it.q0, it.q1});
+    if (it.wave >= 0) {
+      if (it.wave >= p.waves || it.slot >= 0) fail("wave", n, m, C);
+      else ++wave[(size_t)it.wave];
+    }
+    if (it.slot < 0) {
+      if (it.q0 != 0 || it.q1 != 4 * S || !p.scratch) fail("whole tile", n, m, C);
+      continue;
+    }
+    const auto g = groups.find({it.I, it.J});
+    if (g == groups.end()) {
+      fail("split tile without a group", n, m, C);
+      continue;
+    }
+    int slot = it.slot, base = g->second.slot;
+    for (int pr = 0; pr < 3; ++pr) {
+      const int a = pr * S, b = pr == 2 ? 4 * S : a + S;
+      if (it.q0 < b && it.q1 > a) {
+        if (slot < base || slot >= base + g->second.pieces[pr] || used[(size_t)slot]++) fail("part slot", n, m, C);
+        ++slot;
+      }
+      base += g->second.pieces[pr];
+    }
+  }
+  for (int u : used)
+    if (u != 1) fail("unused slot", n, m, C);
+  for (int u : wave)
+    if (u != C) fail("wave size", n, m, C);
+  size_t blocks = 0;
+  for (int I = 0; I < T; I += 2)
+    for (int J = I; J < T; ++J, ++blocks) {
+      auto v = cover[{I, J}];
+      std::sort(v.begin(), v.end());
+      int e = 0;
+      for (const auto& r : v) {
+        if (r.first != e) fail("stages not contiguous", n, m, C);
+        e = r.second;
+      }
+      if (e != 4 * S) fail("stages not covered", n, m, C);
+    }
+  if (cover.size() != blocks) fail("blocks", n, m, C);
+}
+
+}  // namespace
+
+int main() {
+  int lists = 0;
+  for (int64_t n : {1, 63, 64, 128, 129, 256, 257, 384, 385, 700, 1501, 4096, 5000, 9999, 20000})
+    for (int64_t m : {1, 288, 289, 1000, 30011, 100000, 500000, 2097151})
+      for (int c : {1, 5, 74, 76}) {
+        check(n, m, c);
+        ++lists;
+      }
+  printf("checked %d lists, %d failures\n", lists, failures);
+  return failures == 0 ? 0 : 1;
+}

@@ -1,0 +1,60 @@
+"""The sweep kernel (E2M1 triangles of ibs_compute) at its own edges, against the
+oracle: half-blocks of 64 samples, row pairs of 256, column groups of 384, ring
+stages of 288 markers, rows at every alignment, tiles split into parts and
+whole waves of tiles; and the call whose workspace has no room for it."""
+import numpy as np
+import pytest
+
+import oracle
+from helpers import assert_dist_close, gpu_compute, pack_codes, random_codes
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def ctx():
+    from paper_1410_4803_gb300 import ibs
+    c = ibs.ibs_init(0, flags=ibs.IBS_KERNEL_TC | ibs.IBS_TC_FP4)
+    yield c
+    ibs.ibs_shutdown(c)
+
+
+def _check(ctx, n, m, seed):
+    rng = np.random.default_rng(seed)
+    packed = pack_codes(random_codes(rng, n, m, miss=0.05), garbage_rng=rng)
+    want_c, want_d = oracle.ibs_triangle(packed, n, m)
+    got_c, got_d = gpu_compute(ctx, packed, n, m)
+    bad = np.flatnonzero((got_c != want_c).any(axis=1))
+    assert bad.size == 0, f"n={n} m={m}: {bad.size} pairs differ, first {bad[:5]}"
+    assert_dist_close(got_d, want_d)
+
+
+@pytest.mark.parametrize("n", [1, 64, 65, 192, 193, 255, 257, 384, 385, 511, 513, 639, 770])
+@pytest.mark.parametrize("m", [1, 31, 287, 288, 289, 577, 2593])
+def test_edges(ctx, n, m):
+    _check(ctx, n, m, 1000 * n + m)
+
+
+# parts only (few tiles, many markers); one full wave of whole tiles (76 clusters) and
+# a split rest; two waves, with more than one lockstep segment each
+@pytest.mark.parametrize("n,m", [(130, 60_000), (1100, 9_001), (3201, 2_000), (4500, 3_003)])
+def test_parts_and_waves(ctx, n, m):
+    _check(ctx, n, m, n + m)
+
+
+def test_no_room_for_the_workspace():
+    """A workspace bound that holds operand planes and partial counts but not
+    the sweep kernel's scratch and parts: the call still computes."""
+    from paper_1410_4803_gb300 import ibs
+    rng = np.random.default_rng(3)
+    n, m = 600, 20_000
+    packed = pack_codes(random_codes(rng, n, m))
+    want_c, want_d = oracle.ibs_triangle(packed, n, m)
+    c = ibs.ibs_init(0, workspace_bytes=32 << 20)  # planes 26 MB, partial counts 2.9 MB
+    try:
+        for _ in range(2):
+            got_c, got_d = gpu_compute(c, packed, n, m)
+            assert (got_c == want_c).all()
+            assert_dist_close(got_d, want_d)
+    finally:
+        ibs.ibs_shutdown(c)
