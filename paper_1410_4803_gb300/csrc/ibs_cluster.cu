@@ -12,14 +12,17 @@
 //
 // Here every active row i keeps its minimum (D[i][j], j) over active j > i,
 // compared lexicographically.  Each step is then O(n) parallel work:
-//   1. the global minimum over the row minima, (value, row), lexicographic;
-//   2. the merged row and column become the elementwise max of the two; the
-//      same pass finds the merged row's new minimum and lists the rows whose
-//      minimum is gone: it pointed at the cluster merged away, or at the
-//      merged cluster and that distance grew (distances only grow, so every
-//      other row's minimum stays);
-//   3. the listed rows (3.2 per merge on 4,096 unrelated samples) rescan
-//      their row, the CTA's warps divided evenly among them.
+//   1. the global minimum over the row minima, (value, row), lexicographic,
+//      gives the pair (i, j) to merge;
+//   2. the rows whose minimum may be gone are listed: it pointed at j, which
+//      disappears, or at i, whose distance may grow (distances only grow, so
+//      every other row's minimum stays);
+//   3. row and column i become the elementwise max of rows i and j, the same
+//      pass finds row i's new minimum, and the listed rows rescan their row,
+//      the CTA's warps divided evenly among them (3.2 rows per merge on 4,096
+//      unrelated samples).  A rescan needs nothing of the update: by symmetry
+//      row r holds both D[r][i] and D[r][j], whose max it takes in column i's
+//      place.  So a merge waits for memory once, for both together.
 // The steps form one persistent CTA of 1,024 threads (32 warps); phases are
 // separated by block barriers, which also order the memory updates.  Up to
 // kClSmemRows samples the row minima and flags sit in shared memory.  The
@@ -29,11 +32,12 @@
 // its FP32 rate, and redux.sync takes three instructions where a shuffle tree
 // over (double, index) pairs takes fifteen.
 //
-// What bounds it: latency.  The merges are a serial chain; each is three
-// dependent rounds of loads (about 700 cycles from L2) and block reductions.
-// Measured, n = 4,096 unrelated samples: 34.3 ms, 8.4 us per merge; 125.1 ms
-// with one warp per rescanned row, a check of every flag before the next load
-// of a row, FP64 shuffle trees and every row of a grown cluster rescanned.
+// What bounds it: latency.  The merges are a serial chain, each one round of
+// loads (700 cycles from L2, more from HBM) and four block barriers.
+// Measured, n = 4,096 unrelated samples: 31.3 ms, 7.6 us per merge (34.3 ms with the
+// rescans after the update); 125.1 ms with one warp per
+// rescanned row, a check of every flag before the next load of a row, FP64
+// shuffle trees and rescans after the update.
 #include <cstdint>
 
 #include "ibs_device.cuh"
@@ -57,6 +61,17 @@ __device__ __forceinline__ uint64_t cl_key(double d) {
 }
 __device__ __forceinline__ double cl_value(uint64_t k) {
   return __longlong_as_double((long long)((k >> 63) ? (k & 0x7fffffffffffffffull) : ~k));
+}
+
+// An entry that one thread of the CTA may read while another replaces it: either
+// the old or the new value is read.
+__device__ __forceinline__ uint64_t ld_shared_entry(const uint64_t* p) {
+  uint64_t v;
+  asm volatile("ld.relaxed.cta.global.u64 %0, [%1];" : "=l"(v) : "l"(p) : "memory");
+  return v;
+}
+__device__ __forceinline__ void st_shared_entry(uint64_t* p, uint64_t v) {
+  asm volatile("st.relaxed.cta.global.u64 [%0], %1;" ::"l"(p), "l"(v) : "memory");
 }
 
 // Smallest (key, index), lexicographic, over the warp's lanes (in every lane).
@@ -140,39 +155,45 @@ constexpr size_t cl_smem_bytes(int64_t n) { return n <= kClSmemRows ? (size_t)n 
 // CTA, or two batches of 8 for an eighth of it.
 constexpr int kClUpd = 4, kClScan = 8;
 
+template <bool kSmem>
 __global__ void __launch_bounds__(kClThreads, 1) cl_main_kernel(ClArgs a) {
   extern __shared__ __align__(16) uint8_t cl_smem[];
   constexpr int kWarps = kClThreads / 32;
   __shared__ uint64_t s_k[kWarps], s_uk[kWarps], s_sk[kWarps];
   __shared__ uint32_t s_i[kWarps], s_ui[kWarps], s_si[kWarps];
-  __shared__ uint32_t s_cnt;
-  const int64_t n = a.n;
+  __shared__ uint32_t s_cnt[2];
+  const int n = (int)a.n;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  if (n <= kClSmemRows) {
-    uint64_t* sk = reinterpret_cast<uint64_t*>(cl_smem);
-    uint32_t* sj = reinterpret_cast<uint32_t*>(cl_smem + (size_t)n * 8);
-    uint32_t* sl = reinterpret_cast<uint32_t*>(cl_smem + (size_t)n * 12);
-    uint8_t* sa = cl_smem + (size_t)n * 16;
-    for (int64_t r = tid; r < n; r += kClThreads) {
-      sk[r] = a.rk[r];
-      sj[r] = a.rj[r];
-      sa[r] = a.active[r];
+  uint64_t* rk;
+  uint32_t *rj, *list;
+  uint8_t* active;
+  if constexpr (kSmem) {
+    rk = reinterpret_cast<uint64_t*>(cl_smem);
+    rj = reinterpret_cast<uint32_t*>(cl_smem + (size_t)n * 8);
+    list = reinterpret_cast<uint32_t*>(cl_smem + (size_t)n * 12);
+    active = cl_smem + (size_t)n * 16;
+    for (int r = tid; r < n; r += kClThreads) {
+      rk[r] = a.rk[r];
+      rj[r] = a.rj[r];
+      active[r] = a.active[r];
     }
-    a.rk = sk;
-    a.rj = sj;
-    a.list = sl;
-    a.active = sa;
+  } else {
+    rk = a.rk;
+    rj = a.rj;
+    list = a.list;
+    active = a.active;
   }
-  if (tid == 0) s_cnt = 0;
+  if (tid < 2) s_cnt[tid] = 0;
   __syncthreads();
-  for (int64_t step = 0; step + 1 < n; ++step) {
+  for (int step = 0; step + 1 < n; ++step) {
     // 1. global minimum over the row minima: (value, row) lexicographic
     uint64_t k = kNoKey;
     uint32_t b = kNoIdx;
-    for (int64_t r = tid; r < n; r += kClThreads) {
-      const uint64_t rk = a.rk[r];
-      if (rk < k) {
-        k = rk;
+#pragma unroll 4
+    for (int r = tid; r < n; r += kClThreads) {
+      const uint64_t v = rk[r];
+      if (v < k) {
+        k = v;
         b = (uint32_t)r;
       }
     }
@@ -185,40 +206,96 @@ __global__ void __launch_bounds__(kClThreads, 1) cl_main_kernel(ClArgs a) {
     k = s_k[lane];
     b = s_i[lane];
     warp_best(k, b);  // every warp has the result
-    const int64_t i0 = b, j0 = a.rj[b];
-    // 2. the merged cluster's distances: elementwise max of the two rows; its
-    // new minimum; the rows that lost theirs
-    const uint64_t* Di = a.D + i0 * n;
-    const uint64_t* Dj = a.D + j0 * n;
-    uint64_t uk = kNoKey;
-    uint32_t ui = kNoIdx;
-    for (int64_t c0 = tid; c0 < n; c0 += kClUpd * kClThreads) {
-      uint64_t di[kClUpd], dj[kClUpd];
+    const int i0 = (int)b, j0 = (int)rj[b];
+    const uint64_t* Di = a.D + (size_t)i0 * n;
+    const uint64_t* Dj = a.D + (size_t)j0 * n;
+    // the update's first loads, in flight while the list is made
+    uint64_t di[kClUpd], dj[kClUpd];
+    auto load_update = [&](int c0) {
 #pragma unroll
       for (int q = 0; q < kClUpd; ++q) {
-        const int64_t c = c0 + q * kClThreads;
+        const int c = c0 + q * kClThreads;
         di[q] = dj[q] = kNoKey;
-        if (c < n && c != i0 && c != j0 && a.active[c]) {
+        if (c < n && c != i0 && c != j0 && active[c]) {
           di[q] = Di[c];
           dj[q] = Dj[c];
         }
       }
+    };
+    load_update(tid);
+    // 2. rows that may have lost their minimum
+    uint32_t* cnt = &s_cnt[step & 1];
+#pragma unroll 4
+    for (int c = tid; c < n; c += kClThreads) {
+      const int cj = (int)rj[c];
+      if ((cj == j0 && c != i0) || cj == i0) list[atomicAdd(cnt, 1u)] = (uint32_t)c;
+    }
+    __syncthreads();
+    const uint32_t L = *cnt;
+    if (tid == 0) s_cnt[(step + 1) & 1] = 0;
+    // 3a. rescan the listed rows: 8, 4, 2 or 1 warps each
+    const int gw = L <= 4 ? 8 : (L <= 8 ? 4 : (L <= 16 ? 2 : 1));
+    for (uint32_t t = (uint32_t)(warp / gw); t < L; t += kWarps / gw) {
+      const int r = (int)list[t];
+      const uint64_t* Dr = a.D + (size_t)r * n;
+      const int stride = 32 * gw;
+      uint64_t sk = kNoKey;
+      uint32_t si = kNoIdx;
+      if (r < i0 && warp % gw == 0 && lane == 0) {  // column i0 takes the max of columns i0 and j0
+        const uint64_t x = ld_shared_entry(Dr + i0), y = Dr[j0];
+        sk = x > y ? x : y;
+        si = (uint32_t)i0;
+      }
+      for (int c0 = r + 1 + lane + 32 * (warp % gw); c0 < n; c0 += kClScan * stride) {
+        uint64_t d[kClScan];
+#pragma unroll
+        for (int q = 0; q < kClScan; ++q) {
+          const int c = c0 + q * stride;
+          d[q] = c < n && c != i0 && c != j0 && active[c] ? Dr[c] : kNoKey;
+        }
+#pragma unroll
+        for (int q = 0; q < kClScan; ++q) {
+          const int c = c0 + q * stride;
+          if (d[q] < sk || (d[q] == sk && (uint32_t)c < si && sk != kNoKey)) {
+            sk = d[q];
+            si = (uint32_t)c;
+          }
+        }
+      }
+      warp_best(sk, si);
+      if (lane == 0) {
+        if (gw == 1) {
+          rk[r] = sk;
+          rj[r] = si;
+        } else {  // one row per group of warps
+          s_sk[warp] = sk;
+          s_si[warp] = si;
+        }
+      }
+    }
+    // 3b. the merged cluster's distances: elementwise max of the two rows, and
+    // its new minimum.  (A rescan reads its row's entry in column i0 before or
+    // after it is replaced here: the max with column j0's is the same.)
+    uint64_t uk = kNoKey;
+    uint32_t ui = kNoIdx;
+    for (int c0 = tid;;) {
 #pragma unroll
       for (int q = 0; q < kClUpd; ++q) {
         if (di[q] == kNoKey) continue;
-        const int64_t c = c0 + q * kClThreads;
+        const int c = c0 + q * kClThreads;
         const uint64_t d = di[q] > dj[q] ? di[q] : dj[q];
         if (d != di[q]) {
-          a.D[i0 * n + c] = d;
-          a.D[c * n + i0] = d;
+          a.D[(size_t)i0 * n + c] = d;
+          st_shared_entry(a.D + (size_t)c * n + i0, d);
         }
         if (c > i0 && d < uk) {
           uk = d;
           ui = (uint32_t)c;
         }
-        const int64_t cj = a.rj[c];
-        if ((c < j0 && cj == j0) || (c < i0 && cj == i0 && d != a.rk[c])) a.list[atomicAdd(&s_cnt, 1u)] = (uint32_t)c;
       }
+      c0 += kClUpd * kClThreads;
+      if (c0 - tid >= n) break;
+      load_update(c0);
     }
     warp_best(uk, ui);
     if (lane == 0) {
@@ -226,81 +303,45 @@ __global__ void __launch_bounds__(kClThreads, 1) cl_main_kernel(ClArgs a) {
       s_ui[warp] = ui;
     }
     __syncthreads();
-    // 3. rescan the listed rows: 8, 4, 2 or 1 warps each
-    const uint32_t L = s_cnt;
-    const int gw = L <= 4 ? 8 : (L <= 8 ? 4 : (L <= 16 ? 2 : 1));
-    if (warp == kWarps - 1) {  // the merged row's minimum, and the merge itself
+    // 4. the new minima
+    if (gw > 1 && (uint32_t)tid < L) {
+      uint64_t sk = s_sk[tid * gw];
+      uint32_t si = s_si[tid * gw];
+      for (int w = 1; w < gw; ++w) {
+        const uint64_t ok = s_sk[tid * gw + w];
+        const uint32_t oi = s_si[tid * gw + w];
+        if (ok < sk || (ok == sk && oi < si)) {
+          sk = ok;
+          si = oi;
+        }
+      }
+      const uint32_t r = list[tid];
+      rk[r] = sk;
+      rj[r] = si;
+    }
+    if (warp == kWarps - 1) {
       uk = s_uk[lane];
       ui = s_ui[lane];
       warp_best(uk, ui);
       if (lane == 0) {
-        a.rk[i0] = uk;
-        a.rj[i0] = ui;
-        a.rk[j0] = kNoKey;
-        a.active[j0] = 0;  // nobody reads j0's flag in this phase
-        const int32_t ia = a.id[i0], ib = a.id[j0], sz = a.size[i0] + a.size[j0];
-        double* z = a.Z + step * 4;
-        z[0] = (double)(ia < ib ? ia : ib);
-        z[1] = (double)(ia < ib ? ib : ia);
-        z[2] = cl_value(k);
-        z[3] = (double)sz;
-        a.id[i0] = (int32_t)(n + step);
-        a.size[i0] = sz;
+        rk[i0] = uk;
+        rj[i0] = ui;
+        rk[j0] = kNoKey;
+        rj[j0] = kNoIdx;
+        active[j0] = 0;
       }
-      __syncwarp();
     }
-    for (uint32_t t = warp / gw; t < L; t += kWarps / gw) {
-      const int64_t r = a.list[t];
-      const uint64_t* Dr = a.D + r * n;
-      const int64_t stride = 32 * gw;
-      uint64_t sk = kNoKey;
-      uint32_t si = kNoIdx;
-      for (int64_t c0 = r + 1 + lane + 32 * (warp % gw); c0 < n; c0 += kClScan * stride) {
-        uint64_t d[kClScan];
-#pragma unroll
-        for (int q = 0; q < kClScan; ++q) {
-          const int64_t c = c0 + q * stride;
-          d[q] = c < n && c != j0 && a.active[c] ? Dr[c] : kNoKey;
-        }
-#pragma unroll
-        for (int q = 0; q < kClScan; ++q)
-          if (d[q] < sk) {  // columns visited in increasing order per lane
-            sk = d[q];
-            si = (uint32_t)(c0 + q * stride);
-          }
-      }
-      warp_best(sk, si);
-      if (lane == 0) {
-        if (gw == 1) {
-          a.rk[r] = sk;
-          a.rj[r] = si;
-        } else {  // one row per group of warps
-          s_sk[warp] = sk;
-          s_si[warp] = si;
-        }
-      }
+    if (tid == kClThreads - 64) {  // the merge itself, off the critical path
+      const int32_t ia = a.id[i0], ib = a.id[j0], sz = a.size[i0] + a.size[j0];
+      double* z = a.Z + (size_t)step * 4;
+      z[0] = (double)(ia < ib ? ia : ib);
+      z[1] = (double)(ia < ib ? ib : ia);
+      z[2] = cl_value(k);
+      z[3] = (double)sz;
+      a.id[i0] = (int32_t)(n + step);
+      a.size[i0] = sz;
     }
     __syncthreads();
-    if (tid == 0) s_cnt = 0;
-    if (L > 0 && gw > 1) {
-      const uint32_t t = (uint32_t)tid;
-      if (t < L) {
-        uint64_t sk = s_sk[t * gw];
-        uint32_t si = s_si[t * gw];
-        for (int w = 1; w < gw; ++w) {
-          const uint64_t ok = s_sk[t * gw + w];
-          const uint32_t oi = s_si[t * gw + w];
-          if (ok < sk || (ok == sk && oi < si)) {
-            sk = ok;
-            si = oi;
-          }
-        }
-        const uint32_t r = a.list[t];
-        a.rk[r] = sk;
-        a.rj[r] = si;
-      }
-      __syncthreads();
-    }
   }
 }
 
@@ -346,11 +387,11 @@ cudaError_t launch_cluster_complete(const double* tri, int64_t n, double* Z, voi
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
   ClArgs args{D, n, rk, rj, active, list, id, size, Z};
   const size_t smem = cl_smem_bytes(n);
+  auto kern = n <= kClSmemRows ? cl_main_kernel<true> : cl_main_kernel<false>;
   if (smem > 48 * 1024 &&
-      (e = cudaFuncSetAttribute(cl_main_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) !=
-          cudaSuccess)
+      (e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) != cudaSuccess)
     return e;
-  cl_main_kernel<<<1, kClThreads, smem, st>>>(args);
+  kern<<<1, kClThreads, smem, st>>>(args);
   return cudaGetLastError();
 }
 
