@@ -185,7 +185,9 @@ typedef struct {
  *      (a subset with fewer tiles than SMs, and the tiles of a final partial
  *      wave, split over K; their tiles finalised at the end); subsets whose
  *      windows reach the two-SM size (see ibs_compute_kernel) run the two-SM
- *      kernel;
+ *      kernel.  With E2M1 operands, the sweep kernel allowed and no workspace
+ *      limit set, this policy is one gather and one sweep-kernel launch over
+ *      all subsets instead, and it is taken without timing the others;
  *   3  one two-SM persistent launch over every subset's two-SM work list,
  *      concatenated, with the gather fused: a concurrent gather kernel fills
  *      the operand planes unit by unit and per-subset readiness counters hold

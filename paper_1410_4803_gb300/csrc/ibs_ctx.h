@@ -83,6 +83,15 @@ struct BatchPlan {
   std::vector<int64_t> q_unit_off;
   DevBuf pair_sync;
   size_t pair_sync_bytes = 0;
+  // split policy 2 on the sweep kernel (E2M1): tc_planes holds sweep planes,
+  // units the subsets' tensor maps, counter the items' offsets per cluster,
+  // split_tiles the split tiles, planes the scratch of whole tiles, partial the
+  // parts, jobs the SweepPool, words its regrouped rows
+  bool sweep = false;
+  int sweep_clusters = 0;
+  int64_t sweep_groups = 0;
+  SweepSync sweep_sync;
+  DevBuf words;
   cudaStream_t side = nullptr;
   std::vector<cudaEvent_t> stage_ev;
   cudaEvent_t fork_ev = nullptr, join_ev = nullptr;  // policy 3: the side stream's gather
@@ -145,7 +154,7 @@ struct ibs_ctx {
   // sweep kernel: work list of the last (n, m, clusters), scratch of whole tiles
   std::vector<int64_t> sweep_key, sweep_refused;  // refused: the shape that found no room last
   ibs::DevBuf sweep_items, sweep_first, sweep_groups, sweep_scratch;
-  int sweep_stages = 0, sweep_clusters = 0, sweep_waves = 0, sweep_slots = 0;
+  int sweep_clusters = 0, sweep_waves = 0, sweep_wave_stages = 0, sweep_slots = 0;
   int64_t sweep_n_groups = 0;
   bool sweep_has_whole = false;
   int* status_host = nullptr;     // mapped pinned status word

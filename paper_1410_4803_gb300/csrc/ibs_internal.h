@@ -4,6 +4,7 @@
 
 #include <cstddef>
 #include <cstdint>
+#include <utility>
 #include <vector>
 
 #include <cuda_runtime.h>
@@ -96,6 +97,7 @@ struct CrossItem {
 struct RowSrc {
   const uint32_t* planes;   // the request's bit planes
   int64_t row;              // row within the request
+  int64_t n_half;           // sweep planes: the request's half-blocks
 };
 
 // Kernel launchers (ibs_planes.cu / ibs_pairs.cu / ibs_misc.cu).
@@ -267,19 +269,19 @@ struct SweepItem {
   int32_t I, J, w;
   int32_t q0, q1;
   int32_t slot, wave;
-  int32_t pad;
+  int32_t subset;  // batched launches: the subset the tile belongs to (0 otherwise)
 };
 // A split tile: its parts are slots slot, slot + 1, ..., pieces[0] of V V^T,
 // then pieces[1] of U U^T, then pieces[2] of Q R^T + R Q^T.
 struct SweepGroup {
   int32_t I, J, w, slot;
   int32_t pieces[3];
-  int32_t pad;
+  int32_t subset;
 };
 struct SweepPlan {
-  int stages = 0;    // ring stages per sweep
   int clusters = 0;  // clusters that have work
   int waves = 0;     // waves of whole tiles
+  int wave_stages = 0;  // ring stages of the longest of them
   int slots = 0;     // part slots
   bool scratch = false;  // some tile runs whole
   std::vector<SweepItem> items;   // cluster by cluster
@@ -293,33 +295,61 @@ struct SweepSync {
   int* ctr = nullptr;
   int32_t n_seg = 0, seg = 0, lag = 0;
 };
+// What every launch takes: the plan's lists on the device and its workspace.
 struct SweepLaunch {
-  const uint8_t* a_planes = nullptr;  // rows' planes, a_half half-blocks
-  const uint8_t* b_planes = nullptr;  // columns' planes, b_half half-blocks
-  int64_t a_half = 0, b_half = 0;
-  int64_t n = 0;  // samples of the triangle or square
-  int32_t* counts = nullptr;
-  double* dist = nullptr;
-  bool square = false;
   const SweepItem* items = nullptr;
   const int32_t* first = nullptr;
-  int stages = 0, clusters = 0;
+  const SweepGroup* groups = nullptr;
+  int64_t n_groups = 0;
+  int clusters = 0;
   float* scratch = nullptr;
   float* part = nullptr;
   int* status = nullptr;
   unsigned long long wait_ns = 0;
   SweepSync sync;
+  cudaEvent_t between = nullptr;  // recorded before the split tiles' sums, if any
 };
+constexpr size_t kSweepMapsBytes = 384;  // the tensor maps of one matrix
 int sweep_stages(int64_t m);
+int64_t sweep_cols(int64_t m);
 int sweep_clusters();  // clusters of two that fit on the current device (0: the kernel cannot run)
 bool sweep_usable(int64_t n, int64_t m);
 size_t sweep_planes_bytes(int64_t n, int64_t m);
 size_t sweep_scratch_bytes(int clusters);
 size_t sweep_slot_bytes();
+SweepSync sweep_sync(int waves, int stages, int2 setting);
 SweepPlan sweep_plan(int64_t n, int64_t m, int clusters);
+SweepPlan sweep_plan_batch(const std::vector<std::pair<int64_t, int64_t>>& shapes, int clusters);  // {n, m}
+SweepPlan sweep_plan_cross(int64_t row_blocks, const int64_t (&cols)[2][2], int64_t m, int clusters);
 cudaError_t launch_sweep_planes(const uint8_t* packed, int64_t n, int64_t m, uint8_t* planes, cudaStream_t st);
-cudaError_t launch_sweep(const SweepLaunch& l, cudaStream_t st);
-cudaError_t launch_sweep_finalize(const SweepLaunch& l, const SweepGroup* groups, int64_t n_groups, cudaStream_t st);
+// One matrix: the triangle or the square of n samples.
+cudaError_t launch_sweep_one(const uint8_t* planes, int64_t n, int64_t m, int32_t* counts, double* dist, bool square,
+                             const SweepLaunch& l, cudaStream_t st);
+// Subsets of a batch: their tensor maps (kSweepMapsBytes each, encoded on the
+// host by sweep_encode_maps) and descriptors (n_chunks = ring stages) in
+// device memory; the gather fills the planes (TcGatherJob::tc, nc = columns;
+// map entries {job, sample block, group of sweep_gather_cols() columns}).
+bool sweep_encode_maps(void* maps, const void* planes, int64_t n, int64_t m);
+int64_t sweep_gather_ctas(int64_t n, int64_t n_cols);
+int sweep_gather_cols();
+// Batched subsets: the pool's rows in use, regrouped by sample (cols == 0: not).
+struct SweepPool {
+  const uint8_t* packed = nullptr;
+  int64_t row_bytes = 0, n = 0, m = 0;  // of the whole pool
+  int64_t begin = 0, cols = 0;          // first marker in use; columns of 32 from there
+  uint32_t* words = nullptr;            // [cols][n]{low code bits, high code bits}
+};
+bool sweep_words_pay(int64_t pool_genotypes, int64_t gathered);
+cudaError_t launch_sweep_gather(const TcGatherJob* jobs, const int4* map, int64_t ctas, const SweepPool* pool,
+                                int num_sms, int* status, cudaStream_t st);
+cudaError_t launch_sweep_batch(const void* maps_dev, const SubsetDev* subs, const SweepLaunch& l, cudaStream_t st);
+// Serving: n_rows dense rows (planes of row_half half-blocks) against a panel.
+cudaError_t launch_sweep_gather_rows(const RowSrc* rows, int64_t n_rows, int64_t n_cols, uint8_t* dst,
+                                     int64_t dst_half, cudaStream_t st);
+cudaError_t launch_sweep_cross(const uint8_t* row_planes, int64_t row_half, const uint8_t* panel, int64_t n_panel,
+                               int64_t m, int32_t* const* row_out, int64_t n_rows, const SweepLaunch& l,
+                               cudaStream_t st);
+
 // LD correlation (ibs_ld.cu): operand planes of the markers (128-marker
 // blocks, 64-sample chunks, planes X, V, H), the band's work items and the
 // launch sequence (operand builder with per-marker allele balance, persistent

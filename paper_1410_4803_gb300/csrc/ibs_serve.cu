@@ -118,6 +118,10 @@ class ServeEngine {
   ibs_serve_stats stats{};
   int64_t cursor = 0;  // first panel block of the next step
   int grid_ctas = 0;   // persistent cross-kernel CTAs (SMs x 2)
+  bool sweep = false;  // the sweep kernel for every step (E2M1)
+  DevBuf sweep_scratch, sweep_part;  // the steps'
+  DevBuf sync_scratch, sync_part;    // the unbatched path's, one call at a time
+  std::mutex sync_mu;
   bool pair = false;   // two-SM kernel for steps of two or more query blocks
   int clusters = 0;    // its clusters of two CTAs
   DevBuf sync_ctr;     // the two-SM kernel's K-lockstep counters of a step
@@ -143,6 +147,7 @@ class ServeEngine {
   explicit ServeEngine(ibs_ctx* c) : ctx(c) {}
 
   Geo geo(int64_t n) const {
+    if (sweep) return {(n + kTcBlock - 1) / kTcBlock, sweep_cols(pg.m), sweep_planes_bytes(n, pg.m)};
     if (tc) return {(n + kTcBlock - 1) / kTcBlock, tc_chunks(pg.m, fmt), tc_planes_bytes(n, pg.m, fmt)};
     const PlaneGeom g = PlaneGeom::make(n, pg.m);
     return {g.n_blocks, g.n_chunks, g.bytes()};
@@ -151,6 +156,7 @@ class ServeEngine {
 
   // Planes of n samples from a packed device matrix, on stream s.
   cudaError_t build_planes(const uint8_t* packed, int64_t n, void* planes, cudaStream_t s) const {
+    if (sweep) return launch_sweep_planes(packed, n, pg.m, static_cast<uint8_t*>(planes), s);
     if (tc) return launch_tc_planes(packed, n, pg.m, static_cast<uint8_t*>(planes), fmt, s);
     BedSource src;
     src.packed = packed;
@@ -294,9 +300,55 @@ class ServeEngine {
     }
   }
 
+  // Rows against panel blocks [cols[0][0], cols[0][1]) and [cols[1][0], cols[1][1])
+  // on the sweep kernel: the plan's lists through `host` (pinned; or pageable,
+  // staged before return) into `dev`, the launches on s.  Both hold at least
+  // sweep_list_bytes(plan) bytes.
+  static size_t sweep_list_bytes(const SweepPlan& pl) {
+    return pl.items.size() * sizeof(SweepItem) + pl.groups.size() * sizeof(SweepGroup) +
+           (pl.first.size() + 8) * sizeof(int32_t);
+  }
+  cudaError_t run_sweep(const SweepPlan& pl, const uint8_t* row_planes, int64_t row_half, int32_t* const* row_out,
+                        int64_t n_rows, uint8_t* host, uint8_t* dev, float* scratch, float* part, DevBuf& ctr,
+                        bool library_buf, cudaStream_t s) {
+    const size_t ib = pl.items.size() * sizeof(SweepItem), gb = pl.groups.size() * sizeof(SweepGroup);
+    std::memcpy(host, pl.items.data(), ib);
+    if (gb > 0) std::memcpy(host + ib, pl.groups.data(), gb);
+    std::memcpy(host + ib + gb, pl.first.data(), pl.first.size() * sizeof(int32_t));
+    cudaError_t e = cudaMemcpyAsync(dev, host, ib + gb + pl.first.size() * sizeof(int32_t), cudaMemcpyHostToDevice, s);
+    if (e != cudaSuccess) return e;
+    SweepLaunch l;
+    l.items = reinterpret_cast<const SweepItem*>(dev);
+    l.groups = reinterpret_cast<const SweepGroup*>(dev + ib);
+    l.first = reinterpret_cast<const int32_t*>(dev + ib + gb);
+    l.n_groups = (int64_t)pl.groups.size();
+    l.clusters = pl.clusters;
+    l.scratch = scratch;
+    l.part = part;
+    l.status = ctx->status_dev;
+    l.wait_ns = kWaitLimitNs;
+    l.sync = sweep_sync(pl.waves, pl.wave_stages, tc_pair_sync_setting(0));
+    const size_t bytes = (size_t)pl.waves * l.sync.n_seg * sizeof(int);
+    if (bytes > 0) {
+      if (library_buf ? ensure_buf(ctx, ctr, bytes) != IBS_OK : alloc(ctr, bytes, s) != IBS_OK) {
+        l.sync = SweepSync{};
+      } else {
+        if ((e = cudaMemsetAsync(ctr.p, 0, bytes, s)) != cudaSuccess) return e;
+        l.sync.ctr = static_cast<int*>(ctr.p);
+      }
+    }
+    return launch_sweep_cross(row_planes, row_half, static_cast<const uint8_t*>(panel_planes.p), pg.n, pg.m, row_out,
+                              n_rows, l, s);
+  }
+
+  // Parts that a plan over C clusters can need: its shares meet at C - 1 cuts,
+  // each the end of one piece and the start of another, and a piece touches at
+  // most three products.
+  size_t sweep_part_bytes() const { return (size_t)6 * (size_t)std::max(1, clusters) * sweep_slot_bytes(); }
+
   void ensure_items(size_t n) {
     if (n <= items_cap) return;
-    const size_t each = std::max(sizeof(CrossItem), sizeof(PairItem));
+    const size_t each = std::max(std::max(sizeof(CrossItem), sizeof(PairItem)), sizeof(SweepItem));
     for (int s = 0; s < 2; ++s) {
       if (step_ev[s]) cudaEventSynchronize(step_ev[s]);
       if (items_dev[s].p) cudaFree(items_dev[s].p);
@@ -384,6 +436,7 @@ class ServeEngine {
       for (int64_t row = 0; row < r->q; ++row) {
         rows_host[slot][n_rows].planes = static_cast<const uint32_t*>(r->planes.p);
         rows_host[slot][n_rows].row = row;
+        rows_host[slot][n_rows].n_half = (r->q + 63) / 64;
         outs_host[slot][n_rows] = counts_ptr(*r) + (size_t)row * pg.n * 4;
         ++n_rows;
       }
@@ -392,13 +445,23 @@ class ServeEngine {
     // lone request costs one launch, as on the unbatched path); many rows ->
     // shorter steps that new requests can join between.
     const bool two_sm = pair && qblocks >= 2;
-    const int64_t units = two_sm ? (qblocks + 1) / 2 : qblocks;
-    const int64_t len = step_len(units, two_sm ? clusters : grid_ctas);
+    const int64_t units = two_sm || sweep ? (qblocks + 1) / 2 : qblocks;
+    const int64_t len = step_len(units, two_sm || sweep ? clusters : grid_ctas);
     const size_t n_items = (size_t)units * (size_t)len;
-    ensure_items(std::max<size_t>(n_items, 1));
+    SweepPlan pl;
+    if (sweep && n_rows > 0) {
+      const int64_t end = cursor + len;  // wraps around the panel at most once
+      const int64_t cols[2][2] = {{cursor, std::min(end, pgeo.blocks)}, {0, std::max<int64_t>(0, end - pgeo.blocks)}};
+      pl = sweep_plan_cross(qblocks, cols, pg.m, clusters);
+      ensure_items(std::max<size_t>(sweep_list_bytes(pl) / sizeof(SweepItem) + 1, n_items));
+    } else {
+      ensure_items(std::max<size_t>(n_items, 1));
+    }
     size_t t = 0;
     int32_t** outs_d = static_cast<int32_t**>(outs_dev[slot].p);
-    if (two_sm) {
+    if (sweep) {
+      t = pl.items.size();
+    } else if (two_sm) {
       PairItem* h = reinterpret_cast<PairItem*>(items_host[slot]);
       for (int64_t k = 0; k < len; ++k) {
         const int64_t pb = (cursor + k) % pgeo.blocks;  // wraps around the panel
@@ -431,7 +494,10 @@ class ServeEngine {
       if (gathered_version != set_version) {
         // the admitted set changed: pack its rows into the step planes again
         cudaMemcpyAsync(rows_dev[slot].p, rows_host[slot], n_rows * sizeof(RowSrc), cudaMemcpyHostToDevice, stream);
-        if (tc)
+        if (sweep)
+          launch_sweep_gather_rows(static_cast<const RowSrc*>(rows_dev[slot].p), n_rows, pgeo.chunks,
+                                   static_cast<uint8_t*>(step_planes.p), kMaxRows / 64, stream);
+        else if (tc)
           launch_tc_gather_rows(static_cast<const RowSrc*>(rows_dev[slot].p), n_rows, pgeo.chunks,
                                 static_cast<uint8_t*>(step_planes.p), stream);
         else
@@ -440,7 +506,11 @@ class ServeEngine {
         gathered_version = set_version;
       }
       cudaMemcpyAsync(outs_dev[slot].p, outs_host[slot], n_rows * sizeof(int32_t*), cudaMemcpyHostToDevice, stream);
-      if (two_sm) {
+      if (sweep) {
+        run_sweep(pl, static_cast<const uint8_t*>(step_planes.p), kMaxRows / 64, outs_d, n_rows, items_host[slot],
+                  static_cast<uint8_t*>(items_dev[slot].p), static_cast<float*>(sweep_scratch.p),
+                  static_cast<float*>(sweep_part.p), sync_ctr, true, stream);
+      } else if (two_sm) {
         cudaMemcpyAsync(items_dev[slot].p, items_host[slot], t * sizeof(PairItem), cudaMemcpyHostToDevice, stream);
         launch_tc_pair_cross(static_cast<const uint8_t*>(panel_planes.p), pg.n, pgeo.chunks,
                              static_cast<const uint8_t*>(step_planes.p), geo(kMaxRows).blocks, outs_d, n_rows,
@@ -584,6 +654,7 @@ class ServeEngine {
     free_buf(ctx, step_planes);
     free_buf(ctx, counter);
     free_buf(ctx, sync_ctr);
+    for (DevBuf* b : {&sweep_scratch, &sweep_part, &sync_scratch, &sync_part}) free_buf(ctx, *b);
     for (int s = 0; s < 2; ++s) {
       free_buf(ctx, topk_dev[s]);
       if (topk_host[s]) cudaFreeHost(topk_host[s]);
@@ -631,18 +702,50 @@ ibs_status serve_panel_load(ibs_ctx* ctx, const uint8_t* panel, int64_t n_panel,
   // integer-pipe kernels.
   eng->tc = ctx_use_tc(ctx) && tc_chunks(m, eng->fmt) <= tc_max_chunks(eng->fmt);
   eng->blk = eng->tc ? kTcBlock : kSB;
+  // The sweep kernel where it can run, unless the caller bounds the library's
+  // memory (its workspace would leave less of the bound to the requests); its
+  // planes have a layout of their own, so this is settled before the panel's
+  // are built.
+  auto no_sweep = [&] {
+    for (DevBuf* b : {&eng->sweep_scratch, &eng->sweep_part, &eng->sync_scratch, &eng->sync_part}) free_buf(ctx, *b);
+    eng->sweep = false;
+    eng->clusters = 0;
+    eng->pgeo = eng->geo(n_panel);
+  };
+  if (eng->tc && eng->fmt == kTcFp4 && ctx->ws_limit == 0 && tc_pair_mode() >= 0 && sweep_usable(std::max<int64_t>(n_panel, kMaxRows), m)) {
+    eng->clusters = sweep_clusters();
+    eng->sweep = true;
+    for (DevBuf* b : {&eng->sweep_scratch, &eng->sync_scratch})
+      eng->sweep = eng->sweep && ensure_buf(ctx, *b, sweep_scratch_bytes(eng->clusters)) == IBS_OK;
+    for (DevBuf* b : {&eng->sweep_part, &eng->sync_part})
+      eng->sweep = eng->sweep && ensure_buf(ctx, *b, eng->sweep_part_bytes()) == IBS_OK;
+    if (!eng->sweep) no_sweep();
+    clear_error();
+  }
   eng->pgeo = eng->geo(n_panel);
-  IBS_CUDA_TRY(cudaStreamCreateWithFlags(&eng->stream, cudaStreamNonBlocking));
+  if (cudaStreamCreateWithFlags(&eng->stream, cudaStreamNonBlocking) != cudaSuccess) {
+    cudaGetLastError();
+    no_sweep();
+    return fail(IBS_ECUDA, "engine stream could not be created");
+  }
   if (cudaStreamCreateWithFlags(&eng->side, cudaStreamNonBlocking) != cudaSuccess) {
     cudaGetLastError();
     cudaStreamDestroy(eng->stream);
+    no_sweep();
     return fail(IBS_ECUDA, "copy stream could not be created");
   }
-  if (ibs_status s = ensure_buf(ctx, eng->panel_planes, eng->pgeo.bytes)) {
+  ibs_status ps = ensure_buf(ctx, eng->panel_planes, eng->pgeo.bytes);
+  if (ps == IBS_ENOMEM && eng->sweep) {
+    no_sweep();
+    ps = ensure_buf(ctx, eng->panel_planes, eng->pgeo.bytes);
+  }
+  if (ps) {
     cudaStreamDestroy(eng->stream);
     cudaStreamDestroy(eng->side);
-    return s;
+    no_sweep();
+    return ps;
   }
+  clear_error();
   const size_t bytes = (size_t)m * (size_t)((n_panel + 3) / 4);
   const uint8_t* src_dev = panel;
   void* tmp = nullptr;
@@ -650,6 +753,7 @@ ibs_status serve_panel_load(ibs_ctx* ctx, const uint8_t* panel, int64_t n_panel,
     cudaError_t e = cudaMalloc(&tmp, bytes);
     if (e != cudaSuccess) {
       free_buf(ctx, eng->panel_planes);
+      no_sweep();
       cudaStreamDestroy(eng->stream);
       cudaStreamDestroy(eng->side);
       cudaGetLastError();
@@ -666,9 +770,22 @@ ibs_status serve_panel_load(ibs_ctx* ctx, const uint8_t* panel, int64_t n_panel,
     return st;
   }
   eng->grid_ctas = eng->tc ? ctx->num_sms : ctx->num_sms * pair_kernel_ctas_per_sm(pick_mode(ctx));
-  eng->pair = eng->tc && tc_pair_cross_usable(n_panel, eng->pgeo.chunks, eng->fmt);
-  eng->clusters = eng->pair ? tc_pair_clusters(eng->pgeo.chunks) : 0;
+  eng->pair = eng->tc && !eng->sweep && tc_pair_cross_usable(n_panel, eng->pgeo.chunks, eng->fmt);
+  if (!eng->sweep) eng->clusters = eng->pair ? tc_pair_clusters(eng->pgeo.chunks) : 0;
   if (eng->clusters < 1) eng->pair = false;
+  if (eng->sweep) {
+    // lockstep counters for the most waves of a step (all 4,096 rows, every
+    // panel block), so that a step never grows them while earlier steps run
+    const int64_t cols[2][2] = {{0, eng->pgeo.blocks}, {0, 0}};
+    const SweepPlan pl = sweep_plan_cross(kMaxRows / kTcBlock, cols, m, eng->clusters);
+    const SweepSync sy = sweep_sync(pl.waves + 1, 4 * sweep_stages(m), tc_pair_sync_setting(0));
+    const size_t bytes = (size_t)(pl.waves + 1) * sy.n_seg * sizeof(int);
+    if (bytes > 0)
+      if (ibs_status st = ensure_buf(ctx, eng->sync_ctr, bytes)) {
+        eng->shutdown();
+        return st;
+      }
+  }
   if (eng->pair) {
     // lockstep counters for the largest step (all 4,096 rows, every panel
     // block), so that a step never grows them while earlier steps run
@@ -693,9 +810,11 @@ ibs_status serve_panel_load(ibs_ctx* ctx, const uint8_t* panel, int64_t n_panel,
   {
     size_t free_b = 0, total_b = 0;
     cudaMemGetInfo(&free_b, &total_b);
-    eng->pool_budget = free_b > kMemMargin ? free_b - kMemMargin : 0;
+    // the sweep kernel's workspace comes out of the margin
+    const size_t held = eng->sweep ? std::min(kMemMargin / 2, 2 * (eng->sweep_scratch.cap + eng->sweep_part.cap)) : 0;
+    eng->pool_budget = free_b > kMemMargin - held ? free_b - (kMemMargin - held) : 0;
   }
-  eng->fixed_bytes = eng->panel_planes.cap + eng->step_planes.cap + eng->counter.cap +
+  eng->fixed_bytes = eng->panel_planes.cap + eng->step_planes.cap + eng->counter.cap + 2 * (eng->sweep_scratch.cap + eng->sweep_part.cap) +
                      2 * (eng->rows_dev[0].cap + eng->outs_dev[0].cap);
   eng->start();
   std::lock_guard<std::mutex> lk(ctx->mu);
@@ -849,10 +968,19 @@ ibs_status serve_query_sync(ibs_ctx* ctx, const uint8_t* q, int64_t nq, int k, i
   cudaError_t ce = cudaMallocAsync(&outs_d.p, outs.size() * sizeof(int32_t*), s);
   // the engine's kernel rule: two or more query blocks on the two-SM kernel
   const bool two_sm = e.pair && qg.blocks >= 2;
+  SweepPlan pl;
+  std::vector<uint8_t> sweep_host;
+  std::unique_lock<std::mutex> sync_lk(e.sync_mu, std::defer_lock);
+  if (e.sweep) {
+    sync_lk.lock();  // the scratch and parts, until the stream is waited for
+    const int64_t cols[2][2] = {{0, e.pgeo.blocks}, {0, 0}};
+    pl = sweep_plan_cross(qg.blocks, cols, pg.m, e.clusters);
+    sweep_host.resize(ServeEngine::sweep_list_bytes(pl));
+  }
   std::vector<CrossItem> items;
   std::vector<PairItem> pitems;
   const size_t qblock_bytes = (size_t)qg.chunks * e.chunk_block_bytes();
-  for (int64_t pb = 0; pb < e.pgeo.blocks; ++pb) {
+  for (int64_t pb = 0; !e.sweep && pb < e.pgeo.blocks; ++pb) {
     if (two_sm) {
       for (int64_t u = 0; 2 * u < qg.blocks; ++u) {
         PairItem it{};
@@ -873,7 +1001,7 @@ ibs_status serve_query_sync(ibs_ctx* ctx, const uint8_t* q, int64_t nq, int k, i
       items.push_back(it);
     }
   }
-  const size_t item_bytes = two_sm ? pitems.size() * sizeof(PairItem) : items.size() * sizeof(CrossItem);
+  const size_t item_bytes = e.sweep ? sweep_host.size() : two_sm ? pitems.size() * sizeof(PairItem) : items.size() * sizeof(CrossItem);
   const void* item_src = two_sm ? static_cast<const void*>(pitems.data()) : static_cast<const void*>(items.data());
   DevBuf items_dev, sync_d;
   if (ce == cudaSuccess) ce = cudaMallocAsync(&items_dev.p, item_bytes, s);
@@ -883,10 +1011,16 @@ ibs_status serve_query_sync(ibs_ctx* ctx, const uint8_t* q, int64_t nq, int k, i
     if (ptr_kind(q) == PtrKind::Device) ce = cudaMemcpyAsync(r.packed.p, q, pk, cudaMemcpyDeviceToDevice, s);
     else ce = cudaMemcpyAsync(r.packed.p, q, pk, cudaMemcpyHostToDevice, s);
   }
-  if (ce == cudaSuccess) ce = cudaMemcpyAsync(items_dev.p, item_src, item_bytes, cudaMemcpyHostToDevice, s);
+  if (ce == cudaSuccess && !e.sweep)
+    ce = cudaMemcpyAsync(items_dev.p, item_src, item_bytes, cudaMemcpyHostToDevice, s);
   if (ce == cudaSuccess) ce = e.build_planes(static_cast<const uint8_t*>(r.packed.p), nq, r.planes.p, s);
   if (ce == cudaSuccess) {
-    if (two_sm)
+    if (e.sweep)
+      ce = e.run_sweep(pl, static_cast<const uint8_t*>(r.planes.p), (nq + 63) / 64,
+                       static_cast<int32_t* const*>(outs_d.p), nq, sweep_host.data(),
+                       static_cast<uint8_t*>(items_dev.p), static_cast<float*>(e.sync_scratch.p),
+                       static_cast<float*>(e.sync_part.p), sync_d, false, s);
+    else if (two_sm)
       ce = launch_tc_pair_cross(static_cast<const uint8_t*>(e.panel_planes.p), pg.n, e.pgeo.chunks,
                                 static_cast<const uint8_t*>(r.planes.p), qg.blocks,
                                 static_cast<int32_t* const*>(outs_d.p), nq,

@@ -5,8 +5,10 @@
 // homozygous A1 (0 when missing), N = V V^T, IBS1 = (N - U U^T) / 2,
 // IBS0 = Q R^T + R Q^T, all exact integers in FP32.  That kernel streams all
 // four planes of a tile together into three accumulators of 128 columns.  Here
-// a tile is swept over the marker axis four times, one plane pair at a time,
-//   sweep 0: V V^T    sweep 1: U U^T    sweep 2: Q R^T    sweep 3: + R Q^T,
+// a tile is swept over the marker axis once per product, one plane pair at a
+// time: V V^T, then U U^T, then Q R^T and R Q^T in turn, ring stage by ring stage
+// (so that the second finds its planes in L2: one after the other they took a
+// third more HBM reads, 3.5 GB against 2.4 for 6,000 samples x 60,000 markers),
 // and the 384 accumulator columns of tensor memory hold one product of a tile
 // three times as wide: a cluster of two CTAs computes 256 x 384 pairs.  Per SM
 // and 96 markers of one product that is 6 KiB of A and 9 KiB of B for three
@@ -33,6 +35,7 @@
 #include <cstdlib>
 #include <cstring>
 #include <type_traits>
+#include <utility>
 #include <vector>
 
 #include "ibs_tc_common.cuh"
@@ -60,17 +63,6 @@ constexpr int kSwTileCols = 384;
 constexpr size_t kSwHalfTile = (size_t)kSwTileCols * kTB;  // values of one product of one CTA's 128 x 384 tile
 constexpr int kSwEpiBar = 1, kSwBar = 2;  // hardware barriers: epilogue warps; ring slots 0 .. kSwStages - 1
 
-// The waiter warp's release of ring slot s to the MMA warp: one hardware barrier
-// per slot, on which the waiter arrives without blocking and the MMA warp
-// waits.  The waiter cannot arrive on a slot's barrier again before the MMA
-// warp has passed it: the slot is filled again only after its MMAs.
-__device__ __forceinline__ void sweep_release(uint32_t s) {
-  asm volatile("barrier.cta.arrive %0, 64;" ::"r"(kSwBar + s) : "memory");
-}
-__device__ __forceinline__ void sweep_acquire(uint32_t s) {
-  asm volatile("barrier.cta.sync %0, 64;" ::"r"(kSwBar + s) : "memory");
-}
-
 // kind::mxf4, E2M1 x E2M1 -> F32, UE8M0 scale factors, K = 96, M = 256.
 template <int N>
 constexpr uint32_t kIdescSweep = (1u << 7) | (1u << 10) | ((uint32_t)(N >> 3) << 17) | (1u << 23) |
@@ -91,6 +83,45 @@ __device__ __forceinline__ uint64_t sweep_desc(uint32_t saddr, uint32_t col) {
          (uint64_t)1 << 46;
 }
 
+// The 16 bytes (64 samples) from byte0 on of marker row `marker` of `m`: any
+// alignment; beyond the row or the matrix, missing.
+__device__ __forceinline__ void sweep_row64(const uint8_t* __restrict__ packed, int64_t row_bytes, int64_t marker,
+                                            int64_t m, int64_t byte0, uint32_t (&w)[4]) {
+#pragma unroll
+  for (int i = 0; i < 4; ++i) w[i] = 0x55555555u;  // missing
+  if (marker >= m) return;
+  const uint8_t* p = packed + marker * row_bytes + byte0;
+  const int64_t left = row_bytes - byte0;  // bytes of the row from here on
+  const uintptr_t at = reinterpret_cast<uintptr_t>(p);
+  if (left >= 16 && (at & 15) == 0) {
+    const uint4 v = __ldg(reinterpret_cast<const uint4*>(p));
+    w[0] = v.x;
+    w[1] = v.y;
+    w[2] = v.z;
+    w[3] = v.w;
+  } else if (left >= 16 && marker > 0 && marker + 1 < m) {
+    // five aligned words, all inside the matrix (the row is neither its first
+    // nor its last), shifted into place
+    const uint32_t* q = reinterpret_cast<const uint32_t*>(at & ~(uintptr_t)3);
+    const int sh = 8 * (int)(at & 3);
+    uint32_t v[5];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) v[i] = __ldg(q + i);
+    v[4] = sh ? __ldg(q + 4) : 0u;
+#pragma unroll
+    for (int i = 0; i < 4; ++i) w[i] = __funnelshift_r(v[i], v[i + 1], sh);
+  } else {
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      uint32_t v = 0;
+#pragma unroll
+      for (int b = 0; b < 4; ++b)
+        v |= (uint32_t)(4 * i + b < left ? __ldg(p + 4 * i + b) : (uint8_t)0x55) << (8 * b);
+      w[i] = v;
+    }
+  }
+}
+
 // ---------------------------------------------------------------------------
 // Packed .bed rows -> operand planes.  Warp = one column of one half-block: lane
 // t reads the 16 bytes (64 samples) of marker row t, and each of the four
@@ -106,40 +137,9 @@ __global__ void __launch_bounds__(256) sweep_planes_kernel(const uint8_t* __rest
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int64_t c = blockIdx.x, h = (int64_t)blockIdx.y * 8 + warp;
   if (h >= n_half) return;
-  const int64_t marker = c * 32 + lane, byte0 = h * 16;
-  uint32_t w[4] = {0x55555555u, 0x55555555u, 0x55555555u, 0x55555555u};  // missing
-  if (marker < m) {
-    const uint8_t* p = packed + marker * row_bytes + byte0;
-    const int64_t left = row_bytes - byte0;  // bytes of the row from here on
-    const uintptr_t at = reinterpret_cast<uintptr_t>(p);
-    if (left >= 16 && (at & 15) == 0) {
-      const uint4 v = __ldg(reinterpret_cast<const uint4*>(p));
-      w[0] = v.x;
-      w[1] = v.y;
-      w[2] = v.z;
-      w[3] = v.w;
-    } else if (left >= 16 && marker > 0 && marker + 1 < m) {
-      // any alignment: five aligned words, all inside the matrix (the row is
-      // neither its first nor its last), shifted into place
-      const uint32_t* q = reinterpret_cast<const uint32_t*>(at & ~(uintptr_t)3);
-      const int sh = 8 * (int)(at & 3);
-      uint32_t v[5];
-#pragma unroll
-      for (int i = 0; i < 4; ++i) v[i] = __ldg(q + i);
-      v[4] = sh ? __ldg(q + 4) : 0u;
-#pragma unroll
-      for (int i = 0; i < 4; ++i) w[i] = __funnelshift_r(v[i], v[i + 1], sh);
-    } else {
-#pragma unroll
-      for (int i = 0; i < 4; ++i) {
-        uint32_t v = 0;
-#pragma unroll
-        for (int b = 0; b < 4; ++b)
-          v |= (uint32_t)(4 * i + b < left ? __ldg(p + 4 * i + b) : (uint8_t)0x55) << (8 * b);
-        w[i] = v;
-      }
-    }
-  }
+  const int64_t marker = c * 32 + lane;
+  uint32_t w[4];
+  sweep_row64(packed, row_bytes, marker, m, h * 16, w);
   const bool odd = (lane & 1) != 0;
   const size_t plane_stride = (size_t)n_half * n_cols * 1024;
   uint8_t* base = planes + (size_t)(odd ? 2 : 0) * plane_stride + ((size_t)h * n_cols + c) * 1024;
@@ -167,87 +167,130 @@ __global__ void __launch_bounds__(256) sweep_planes_kernel(const uint8_t* __rest
 // ---------------------------------------------------------------------------
 // Outputs of a tile.
 
+// Counts of one pair, packed (N, IBS0, IBS1, each below 2^21).
+struct SweepCounts {
+  int32_t i0, i1, n;
+};
+__device__ __forceinline__ uint64_t sweep_pack(float vn, float vu, float vz) {
+  const uint32_t nn = (uint32_t)__float2int_rn(vn), i0 = (uint32_t)__float2int_rn(vz);
+  const uint32_t i1 = (nn - (uint32_t)__float2int_rn(vu)) >> 1;
+  return (uint64_t)nn << 42 | (uint64_t)i0 << 21 | i1;
+}
+__device__ __forceinline__ SweepCounts sweep_unpack(uint64_t v) {
+  return {(int32_t)(v >> 21 & 0x1FFFFF), (int32_t)(v & 0x1FFFFF), (int32_t)(v >> 42)};
+}
+
 // Where the counts go: the triangle or the full square of n samples.
 struct SweepOut {
   int64_t n;
   int32_t* counts;
   double* dist;
   int32_t square;
+  __device__ bool none(int64_t gi0, int64_t gj0, int cols) const {
+    return gi0 >= n || gj0 >= n || gj0 + cols <= gi0;
+  }
+  __device__ bool has(int64_t gi, int64_t gj) const { return gi < n && gj < n && gj >= gi; }
+  __device__ bool mirrored() const { return square != 0; }
+  __device__ void store(int64_t p, uint64_t v) const {
+    const SweepCounts c = sweep_unpack(v);
+    reinterpret_cast<int4*>(counts)[p] = make_int4(c.i0, c.i1, c.n - c.i0 - c.i1, c.n);
+    if (dist) dist[p] = ibs_dist(c.i0, c.i1, c.n);
+  }
+  __device__ void put(int64_t gi, int64_t gj, uint64_t v) const {
+    store(square ? gi * n + gj : tri_index(gi, gj, n), v);
+  }
+  __device__ void put_mirror(int64_t gi, int64_t gj, uint64_t v) const { store(gj * n + gi, v); }
+};
+
+// Serving: counts only, step row r through its own output row [n_cols][4].
+struct SweepRows {
+  int32_t* const* row_out;
+  int64_t n_rows, n_cols;
+  __device__ bool none(int64_t gi0, int64_t gj0, int) const { return gi0 >= n_rows || gj0 >= n_cols; }
+  __device__ bool has(int64_t gi, int64_t gj) const { return gi < n_rows && gj < n_cols; }
+  __device__ bool mirrored() const { return false; }
+  __device__ void put(int64_t gi, int64_t gj, uint64_t v) const {
+    const SweepCounts c = sweep_unpack(v);
+    reinterpret_cast<int4*>(row_out[gi])[gj] = make_int4(c.i0, c.i1, c.n - c.i0 - c.i1, c.n);
+  }
+  __device__ void put_mirror(int64_t, int64_t, uint64_t) const {}
 };
 
 // Write one piece of a tile, 32 rows from gi0 by 16 columns from gj0, from its
 // three products: load(pr, v) sets v[j] to product pr of (row gi0 + lane, column
-// gj0 + j).
-// The counts are packed into 64 bits (each below 2^21) and
-// transposed through `sm`, so that a half-warp stores 16 consecutive pairs of a
-// row (256 bytes of counts) at a time; a square's mirror image is contiguous
-// down the column as it is loaded.
-template <class Load>
-__device__ __forceinline__ void sweep_store(const SweepOut& o, int64_t gi0, int64_t gj0, const Load& load,
-                                            uint64_t* sm) {
+// gj0 + j).  The packed counts are transposed through `sm`, so that a half-warp
+// stores 16 consecutive pairs of a row (256 bytes of counts) at a time; a
+// square's mirror image is contiguous down the column as it is loaded.
+template <class Out, class Load>
+__device__ __forceinline__ void sweep_store(const Out& o, int64_t gi0, int64_t gj0, const Load& load, uint64_t* sm) {
   const int lane = threadIdx.x & 31;
-  const int64_t n = o.n;
-  if (gi0 >= n || gj0 >= n || gj0 + 15 < gi0) return;
+  if (o.none(gi0, gj0, 16)) return;
   float vn[16], vu[16], vz[16];
   load(0, vn);
   load(1, vu);
   load(2, vz);
   __syncwarp();  // the warp's previous piece has been read
 #pragma unroll
-  for (int j = 0; j < 16; ++j) {
-    const uint32_t nn = (uint32_t)__float2int_rn(vn[j]), i0 = (uint32_t)__float2int_rn(vz[j]);
-    const uint32_t i1 = (nn - (uint32_t)__float2int_rn(vu[j])) >> 1;
-    sm[lane * 17 + j] = (uint64_t)nn << 42 | (uint64_t)i0 << 21 | i1;
-  }
+  for (int j = 0; j < 16; ++j) sm[lane * 17 + j] = sweep_pack(vn[j], vu[j], vz[j]);
   __syncwarp();
-  auto put = [&](int64_t p, uint64_t v) {
-    const int32_t nn = (int32_t)(v >> 42), i0 = (int32_t)(v >> 21 & 0x1FFFFF), i1 = (int32_t)(v & 0x1FFFFF);
-    reinterpret_cast<int4*>(o.counts)[p] = make_int4(i0, i1, nn - i0 - i1, nn);
-    if (o.dist) o.dist[p] = ibs_dist(i0, i1, nn);
-  };
   const int64_t gj = gj0 + (lane & 15);
 #pragma unroll 4
-  for (int r = lane >> 4; r < 32; r += 2) {
-    const int64_t gi = gi0 + r;
-    if (gi < n && gj < n && gj >= gi) put(o.square ? gi * n + gj : tri_index(gi, gj, n), sm[r * 17 + (lane & 15)]);
-  }
-  if (o.square) {
+  for (int r = lane >> 4; r < 32; r += 2)
+    if (o.has(gi0 + r, gj)) o.put(gi0 + r, gj, sm[r * 17 + (lane & 15)]);
+  if (o.mirrored()) {
     const int64_t gi = gi0 + lane;
 #pragma unroll 4
     for (int j = 0; j < 16; ++j)
-      if (gi < n && gj0 + j < n && gj0 + j > gi) put((gj0 + j) * n + gi, sm[lane * 17 + j]);
+      if (gj0 + j > gi && o.has(gi, gj0 + j)) o.put_mirror(gi, gj0 + j, sm[lane * 17 + j]);
   }
 }
 
 // ---------------------------------------------------------------------------
 // The kernel.
 
-// A ring barrier's wait: one probe on the usual path; past it, bounded by
-// limit_ns and ended by another role's abort.
-__device__ __noinline__ bool sweep_wait_slow(uint64_t* bar, uint32_t parity, unsigned long long limit_ns,
-                                             const int* abort_flag) {
-  const unsigned long long t0 = globaltimer_ns();
-  for (;;) {
-    if (limit_ns < 1000000ull) {  // short bounds (tests): a blocking probe could outlast them
-      if (mbar_test_wait(bar, parity)) return true;
-    } else {
-      for (int i = 0; i < 64; ++i)
-        if (mbar_try_wait(bar, parity)) return true;
-    }
-    if (*(volatile const int*)abort_flag != 0 || globaltimer_ns() - t0 > limit_ns) return false;
+// Views of one matrix's operand planes, boxes of 1, 2 and 3 half-blocks.
+struct SweepMaps {
+  CUtensorMap half1, half2, half3;
+  __device__ const CUtensorMap* of(int w) const { return w == 3 ? &half3 : (w == 2 ? &half2 : &half1); }
+};
+static_assert(sizeof(SweepMaps) == kSweepMapsBytes, "the host sizes arrays of them");
+
+// What a launch computes.  One matrix:
+struct SweepOne {
+  SweepMaps maps;
+  SweepOut result;
+  int32_t n_stages;
+  __device__ const CUtensorMap* a(const SweepItem&) const { return &maps.half2; }
+  __device__ const CUtensorMap* b(const SweepItem& it) const { return maps.of(it.w); }
+  __device__ int stages(int) const { return n_stages; }
+  __device__ SweepOut out(int) const { return result; }
+};
+// the subsets of a batch (SubsetDev::n_chunks counts ring stages here):
+struct SweepBatch {
+  const SweepMaps* maps;
+  const SubsetDev* subs;
+  __device__ const CUtensorMap* a(const SweepItem& it) const { return &maps[it.subset].half2; }
+  __device__ const CUtensorMap* b(const SweepItem& it) const { return maps[it.subset].of(it.w); }
+  __device__ int stages(int subset) const { return (int)subs[subset].n_chunks; }
+  __device__ SweepOut out(int subset) const {
+    return {subs[subset].n, subs[subset].out_counts, subs[subset].out_dist, 0};
   }
-}
-__device__ __forceinline__ bool sweep_wait(uint64_t* bar, uint32_t parity, unsigned long long limit_ns,
-                                           const int* abort_flag) {
-  if (limit_ns >= 1000000ull && mbar_try_wait(bar, parity)) return true;
-  return sweep_wait_slow(bar, parity, limit_ns, abort_flag);
-}
+};
+// the rows of a serving step against a panel.
+struct SweepCross {
+  SweepMaps maps;      // the panel's planes
+  CUtensorMap rows;    // the step rows' planes, boxes of 2
+  SweepRows result;
+  int32_t n_stages;
+  __device__ const CUtensorMap* a(const SweepItem&) const { return &rows; }
+  __device__ const CUtensorMap* b(const SweepItem& it) const { return maps.of(it.w); }
+  __device__ int stages(int) const { return n_stages; }
+  __device__ SweepRows out(int) const { return result; }
+};
 
 struct SweepArgs {
-  SweepOut out;
   const SweepItem* items;
   const int32_t* first;  // items of cluster c: first[c] .. first[c + 1] - 1
-  int32_t stages;        // ring stages per sweep
   float* scratch;        // [CTA][3][384][128]: products of the CTA's whole item
   float* part;           // [slot][2][384][128]: products of split items
   int* status;
@@ -268,10 +311,9 @@ struct SweepArgs {
 // is written after its last sweep, while the next item's first sweep runs; a
 // piece writes each product it has a part of to a slot of its own, which the
 // finalisation adds up.
+template <class W>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kSwThreads, 1)
-    sweep_kernel(const __grid_constant__ CUtensorMap amap, const __grid_constant__ CUtensorMap bmap1,
-                 const __grid_constant__ CUtensorMap bmap2, const __grid_constant__ CUtensorMap bmap3,
-                 const SweepArgs args) {
+    sweep_kernel(const __grid_constant__ W work, const SweepArgs args) {
   extern __shared__ __align__(1024) uint8_t smem_raw[];
   uint8_t* ring = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   __shared__ __align__(8) uint64_t full[kSwStages], empty[kSwStages], tfull, tempty, drain;
@@ -283,7 +325,6 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kSwThreads, 1)
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const uint32_t rank = cluster_rank();
   const uint32_t cid = cluster_index();
-  const int S = args.stages;
   int* status = args.status;
   const unsigned long long wait_ns = args.wait_ns;
   const int it0 = args.first[cid], it1 = args.first[cid + 1];
@@ -314,8 +355,9 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kSwThreads, 1)
   cluster_sync_all();  // both CTAs' barriers initialised and scale factors stored
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
 
-  // a product ends with sweep 0, 1 or 3, or with the item
-  auto product_end = [&](int q, int q1) { return min(q1, q < S ? S : (q < 2 * S ? 2 * S : 4 * S)); };
+  // S stages of V V^T, S of U U^T, 2 S of Q R^T + R Q^T: the end of stage q's
+  // product, or of the item
+  auto product_end = [](int S, int q, int q1) { return min(q1, q < S ? S : (q < 2 * S ? 2 * S : 4 * S)); };
 
   if (warp == 0 || warp == 3) {
     // Copies: lane 0 of warp 0 streams the A operand, lane 0 of warp 3 the B
@@ -329,7 +371,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kSwThreads, 1)
       for (int e = it0; e < it1 && !stop; ++e) {
         const SweepItem it = args.items[e];
         const int h = is_b ? 2 * it.J + it.w * (int)rank : 2 * (it.I + (int)rank);
-        const CUtensorMap* map = !is_b ? &amap : (it.w == 3 ? &bmap3 : (it.w == 2 ? &bmap2 : &bmap1));
+        const CUtensorMap* map = is_b ? work.b(it) : work.a(it);
+        const int S = work.stages(it.subset);
         const uint32_t bytes = 2u * (uint32_t)(kSwABytes + kSwCols * 1024 * it.w);
         // lockstep: warp 0 announces every segment and holds back until the
         // whole wave has started the segment `lag` back (warp 3 follows
@@ -338,10 +381,12 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kSwThreads, 1)
         int left = 0, sg = 0;
         int q = it.q0;
         while (q < it.q1 && !stop) {
-          const int sw = q < 2 * S ? (q < S ? 0 : 1) : (q < 3 * S ? 2 : 3);
-          const int plane = is_b && sw >= 2 ? 5 - sw : sw;  // sweep 2: Q R^T, sweep 3: R Q^T
-          const int end = min(it.q1, (sw + 1) * S);
-          for (int col = (q - sw * S) * kSwCols; q < end; ++q, col += kSwCols) {
+          // V V^T, then U U^T, then Q R^T and R Q^T in turn over the same markers
+          const int pr = q < S ? 0 : (q < 2 * S ? 1 : 2), q0 = pr * S, end = product_end(S, q, it.q1);
+          for (; q < end; ++q) {
+            const int odd = (q - q0) & 1;
+            const int plane = pr < 2 ? pr : (is_b ? 3 - odd : 2 + odd);
+            const int col = (pr < 2 ? q - q0 : (q - q0) >> 1) * kSwCols;
             if (ctr != nullptr && left-- == 0) {
               left = args.sync.seg - 1;
               atomicAdd(ctr + sg, 1);
@@ -351,7 +396,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kSwThreads, 1)
               }
               ++sg;
             }
-            if (g >= (uint32_t)kSwStages && !sweep_wait(&empty[s], ph, wait_ns, &abort_flag)) {
+            if (g >= (uint32_t)kSwStages && !ring_wait(&empty[s], ph, wait_ns, &abort_flag)) {
               stop = true;
               break;
             }
@@ -392,7 +437,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kSwThreads, 1)
       constexpr int kN = w == 3 ? 192 : 128 * w;
       uint32_t acc = 0;  // the first K step overwrites
       for (int k = 0; k < stages; ++k) {
-        sweep_acquire(s);
+        ring_acquire(kSwBar + s);
         if (*(volatile int*)&s_dead != 0) {
           dead = true;
           return;
@@ -417,8 +462,9 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kSwThreads, 1)
     };
     for (int e = it0; e < it1 && !dead; ++e) {
       const SweepItem it = args.items[e];
+      const int S = work.stages(it.subset);
       for (int q = it.q0; q < it.q1 && !dead;) {
-        const int end = product_end(q, it.q1);
+        const int end = product_end(S, q, it.q1);
         if (it.w == 3)
           product(std::integral_constant<int, 3>{}, end - q);
         else if (it.w == 2)
@@ -441,18 +487,19 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kSwThreads, 1)
     bool dead = false, wrapped = false;
     for (int e = it0; e < it1 && !dead; ++e) {
       const SweepItem it = args.items[e];
+      const int S = work.stages(it.subset);
       for (int q = it.q0; q < it.q1 && !dead; ++p) {
-        const int end = product_end(q, it.q1);
+        const int end = product_end(S, q, it.q1);
         bool ok = lane != 0 || p == 0 || mbar_wait_cluster_bounded(&tempty, (p - 1) & 1u, wait_ns);
         for (; q < end; ++q) {
           // every lane of the warp goes on, or none
-          if (lane == 0 && ok) ok = sweep_wait(&full[s], ph, wait_ns, &abort_flag);
+          if (lane == 0 && ok) ok = ring_wait(&full[s], ph, wait_ns, &abort_flag);
           if (__any_sync(0xffffffffu, !ok)) {
             dead = true;
             break;
           }
           asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-          sweep_release(s);
+          ring_release(kSwBar + s);
           s = s + 1 == kSwStages ? 0 : s + 1;
           ph ^= s == 0 ? 1u : 0u;
           wrapped |= s == 0;
@@ -471,7 +518,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kSwThreads, 1)
         if (wrapped) mbar_wait_bounded(&empty[s], ph ^ 1u);
       }
       __syncwarp();
-      sweep_release(s);  // the MMA warp finds s_dead
+      ring_release(kSwBar + s);  // the MMA warp finds s_dead
     }
   } else if (warp >= 4) {
     const int quarter = warp & 3, part = (warp - 4) >> 2, row = quarter * 32 + lane;
@@ -483,6 +530,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kSwThreads, 1)
     bool stop = false;
     for (int e = it0; e < it1 && !stop; ++e) {
       const SweepItem it = args.items[e];
+      const int S = work.stages(it.subset);
       int slot = it.slot;
       for (int q = it.q0; q < it.q1;) {
         const int pr = q < S ? 0 : (q < 2 * S ? 1 : 2);
@@ -534,10 +582,11 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kSwThreads, 1)
       if (stop || it.slot >= 0) continue;
       // whole tile: every product is in the scratch; 32 x 16 pieces by warps
       asm volatile("bar.sync %0, %1;" ::"n"(kSwEpiBar), "n"(32 * kSwEpiWarps) : "memory");
+      const auto out = work.out(it.subset);
       const int64_t gi0 = (int64_t)(it.I + (int)rank) * kTB + quarter * 32;
       for (int ct = part; ct < 8 * it.w; ct += 2) {
         const float* src = scratch + (size_t)ct * 16 * kTB + row;
-        sweep_store(args.out, gi0, (int64_t)it.J * kTB + ct * 16,
+        sweep_store(out, gi0, (int64_t)it.J * kTB + ct * 16,
                     [&](int pr, float (&v)[16]) {
 #pragma unroll
                       for (int j = 0; j < 16; ++j) v[j] = __ldcg(src + pr * kSwHalfTile + (size_t)j * kTB);
@@ -575,8 +624,10 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kSwThreads, 1)
 
 // Split tiles: the parts of each product added up and written.  Warp = one 32 x
 // 16 piece of a tile, 32 loads of parts in flight per thread.
+template <class W>
 __global__ void __launch_bounds__(128) sweep_finalize_kernel(const SweepGroup* __restrict__ groups,
-                                                             const float* __restrict__ part, const SweepOut out) {
+                                                             const float* __restrict__ part,
+                                                             const __grid_constant__ W work) {
   __shared__ uint64_t sm[4][32 * 17];
   const SweepGroup gr = groups[blockIdx.x];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -585,7 +636,7 @@ __global__ void __launch_bounds__(128) sweep_finalize_kernel(const SweepGroup* _
   if (ct >= 8 * gr.w) return;
   const float* src = part + (size_t)(2 * gr.slot + rank) * kSwHalfTile + (size_t)ct * 16 * kTB + quarter * 32 + lane;
   const int first[3] = {0, gr.pieces[0], gr.pieces[0] + gr.pieces[1]};
-  sweep_store(out, (int64_t)(gr.I + rank) * kTB + quarter * 32, (int64_t)gr.J * kTB + ct * 16,
+  sweep_store(work.out(gr.subset), (int64_t)(gr.I + rank) * kTB + quarter * 32, (int64_t)gr.J * kTB + ct * 16,
               [&](int pr, float (&v)[16]) {
                 const float* p = src + (size_t)first[pr] * 2 * kSwHalfTile;
 #pragma unroll
@@ -596,6 +647,146 @@ __global__ void __launch_bounds__(128) sweep_finalize_kernel(const SweepGroup* _
                   for (int j = 0; j < 16; ++j) v[j] += __ldg(p + (size_t)j * kTB);  // whole numbers: exact
               },
               sm[warp]);
+}
+
+// Batched subsets, when they read a good part of the pool: the pool's rows
+// [begin, end) regrouped by sample, words[c][sample] = the low and the high code
+// bits of markers begin + 32 c ...  The gather below then reads 8 bytes per
+// sample and column; out of the rows it reads single bytes of 32 lines, which
+// took 1.8 ms of a 4 ms batch (24 subsets of 100 to 4000 samples, 10,000 x
+// 200,000 pool).  Warp = one column of 64 samples, transposed by shuffles;
+// 512 neighbouring samples per CTA.  A fixed grid (the launch is in a graph and
+// the window is known per call); HBM-bound: the pool read once and written once.
+__global__ void __launch_bounds__(256) sweep_words_kernel(const SweepPool* __restrict__ pool) {
+  const SweepPool p = *pool;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int64_t n_half = (p.n + 63) / 64, groups = (n_half + 7) / 8, total = p.cols * groups;
+  for (int64_t i = blockIdx.x; i < total; i += gridDim.x) {
+    const int64_t c = i / groups, h = (i % groups) * 8 + warp;
+    if (h >= n_half) continue;
+    uint32_t w[4];
+    sweep_row64(p.packed, p.row_bytes, p.begin + c * 32 + lane, p.m, h * 16, w);
+    uint32_t* out = p.words + ((size_t)c * p.n + (size_t)h * 64) * 2;
+#pragma unroll
+    for (int i4 = 0; i4 < 4; ++i4) {
+      const uint32_t x = tc_transpose32(w[i4], lane);
+      if (h * 64 + i4 * 16 + (lane >> 1) < p.n) out[i4 * 32 + lane] = x;
+    }
+  }
+}
+
+// Batched subsets: sample sel[128 block + r] of the pool over 16 columns of the
+// subset's window, thread r = sample r of the block; 16 bytes of each plane per
+// column.  map[c] = {job, sample block, column group} of CTA c, in the order of
+// the pool variant it starts at, so that subsets with overlapping windows share
+// the pool through L2.  An index outside the pool is not read: the sample is
+// all-missing and the status word reports it.  Without words the thread reads
+// one byte of each of a column's 32 marker rows.
+constexpr int kSwGatherCols = 16;
+__device__ __forceinline__ void sweep_put_column(uint32_t H, uint32_t L, uint8_t* base, size_t plane) {
+  const uint32_t V = H | ~L, P = H & ~L, Q = H & L, R = ~H & ~L;
+  uint32_t wv[4], wu[4], wq[4], wr[4];
+#pragma unroll
+  for (int g = 0; g < 4; ++g) {
+    wv[g] = nib8(V >> (8 * g)) << 1;
+    wu[g] = wv[g] | (nib8(P >> (8 * g)) << 3);
+    wq[g] = nib8(Q >> (8 * g)) << 1;
+    wr[g] = nib8(R >> (8 * g)) << 1;
+  }
+  *reinterpret_cast<uint4*>(base) = make_uint4(wv[0], wv[1], wv[2], wv[3]);
+  *reinterpret_cast<uint4*>(base + plane) = make_uint4(wu[0], wu[1], wu[2], wu[3]);
+  *reinterpret_cast<uint4*>(base + 2 * plane) = make_uint4(wq[0], wq[1], wq[2], wq[3]);
+  *reinterpret_cast<uint4*>(base + 3 * plane) = make_uint4(wr[0], wr[1], wr[2], wr[3]);
+}
+__global__ void __launch_bounds__(kTB, 8) sweep_gather_kernel(const TcGatherJob* __restrict__ jobs,
+                                                           const int4* __restrict__ map,
+                                                           const SweepPool* __restrict__ pool, int* status) {
+  const int4 e = map[blockIdx.x];
+  const TcGatherJob& j = jobs[e.x];
+  const int r = threadIdx.x;
+  const int64_t s = (int64_t)e.y * kTB + r, nh = (j.n + 63) / 64, h = s >> 6;
+  if (h >= nh) return;
+  int64_t ps = -1;
+  if (s < j.n) {
+    ps = j.src.sel[s];
+    if (ps < 0 || ps >= j.src.n_src) {
+      atomicExch(status, 1);
+      ps = -1;
+    }
+  }
+  // (in registers: the stores below could alias the job)
+  const int64_t row_bytes = j.src.row_bytes, nc = j.nc, m = j.m;
+  uint8_t* const out = j.tc + (size_t)h * nc * 1024 + (size_t)(s & 63) * 16;
+  const size_t plane = (size_t)nh * nc * 1024;
+  const int64_t c0 = (int64_t)e.z * kSwGatherCols, c1 = min(nc, c0 + kSwGatherCols);
+  const int64_t first = j.src.var_begin - pool->begin;
+  if (pool->cols > 0 && ps >= 0) {
+    // words of pool columns c + first / 32 and the next one, shifted; past the
+    // last one the markers are outside the window
+    const int64_t cols = pool->cols, stride = pool->n;
+    const uint2* w = reinterpret_cast<const uint2*>(pool->words) + ps;
+    const int sh = (int)(first & 31);
+    int64_t pc = c0 + (first >> 5);
+    const uint2 none = make_uint2(~0u, 0u);
+    uint2 cur = pc < cols ? __ldg(w + pc * stride) : none;
+#pragma unroll 4
+    for (int64_t c = c0; c < c1; ++c, ++pc) {
+      const uint2 next = pc + 1 < cols ? __ldg(w + (pc + 1) * stride) : none;
+      uint32_t L = __funnelshift_r(cur.x, next.x, sh), H = __funnelshift_r(cur.y, next.y, sh);
+      const int64_t kn = m - c * 32;  // markers of the column inside the window
+      if (kn < 32) {
+        const uint32_t in = kn > 0 ? (1u << kn) - 1u : 0u;
+        H &= in;
+        L |= ~in;
+      }
+      sweep_put_column(H, L, out + (size_t)c * 1024, plane);
+      cur = next;
+    }
+    return;
+  }
+  const int sh = ps >= 0 ? 2 * (int)(ps & 3) : 0;
+  const uint8_t* col = j.src.packed + j.src.var_begin * row_bytes + (ps >= 0 ? (ps >> 2) : 0);
+#pragma unroll 1
+  for (int64_t c = c0; c < c1; ++c) {
+    const int64_t k0 = c * 32;
+    const int kn = (int)(m - k0 < 32 ? m - k0 : 32);  // markers of the column inside the window
+    uint32_t H = 0, L = ~0u;                              // all missing unless read
+    if (ps >= 0 && kn > 0) {
+      // the row stride is re-read in each column (an empty asm), or the
+      // compiler keeps 32 row offsets in registers across columns and spills
+      int64_t stride = row_bytes;
+      asm volatile("" : "+l"(stride));
+      const uint8_t* p = col + k0 * stride;
+      uint32_t byte[32];
+#pragma unroll
+      for (int k = 0; k < 32; ++k, p += stride) byte[k] = k < kn ? __ldg(p) : 0x55u;
+      H = 0;
+      L = 0;
+#pragma unroll
+      for (int k = 0; k < 32; ++k) {
+        const uint32_t code = (byte[k] >> sh) & 3u;
+        H |= (code >> 1) << k;
+        L |= (code & 1u) << k;
+      }
+    }
+    sweep_put_column(H, L, out + (size_t)c * 1024, plane);
+  }
+}
+
+// Serving: rows of the requests' planes packed densely into the step's planes.
+// CTA = (column, half-block); thread (row, plane).
+__global__ void __launch_bounds__(256) sweep_gather_rows_kernel(const RowSrc* __restrict__ rows, int64_t n_rows,
+                                                                int64_t n_cols, uint8_t* __restrict__ dst,
+                                                                int64_t dst_half) {
+  const int64_t c = blockIdx.x, h = blockIdx.y;
+  const int r = threadIdx.x & 63, plane = threadIdx.x >> 6;
+  const int64_t d = h * 64 + r;
+  if (d >= n_rows) return;
+  const RowSrc src = rows[d];
+  const uint8_t* from = reinterpret_cast<const uint8_t*>(src.planes) +
+                        (((size_t)plane * src.n_half + (src.row >> 6)) * n_cols + c) * 1024 + (src.row & 63) * 16;
+  *reinterpret_cast<uint4*>(dst + (((size_t)plane * dst_half + h) * n_cols + c) * 1024 + r * 16) =
+      *reinterpret_cast<const uint4*>(from);
 }
 
 // A view of the operand planes, a box `halves` half-blocks over kSwCols
@@ -612,137 +803,100 @@ bool encode_sweep_map(CUtensorMap* map, const void* planes, int64_t n_half, int6
             CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
             CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
-
-}  // namespace
-
-int sweep_stages(int64_t m) { return (int)((m + kSwMarkers - 1) / kSwMarkers); }
-
-size_t sweep_planes_bytes(int64_t n, int64_t m) {
-  return (size_t)((n + 63) / 64) * (size_t)sweep_stages(m) * kSwCols * 4096;
+bool encode_sweep_maps(SweepMaps* m, const void* planes, int64_t n_half, int64_t n_cols) {
+  return encode_sweep_map(&m->half1, planes, n_half, n_cols, 1) &&
+         encode_sweep_map(&m->half2, planes, n_half, n_cols, 2) &&
+         encode_sweep_map(&m->half3, planes, n_half, n_cols, 3);
 }
 
-size_t sweep_scratch_bytes(int clusters) { return (size_t)clusters * 2 * 3 * kSwHalfTile * sizeof(float); }
-size_t sweep_slot_bytes() { return 2 * kSwHalfTile * sizeof(float); }
+// A tile before it is scheduled.
+struct Tile {
+  int I, J, w, subset, stages;
+};
 
-cudaError_t launch_sweep_planes(const uint8_t* packed, int64_t n, int64_t m, uint8_t* planes, cudaStream_t st) {
-  const int64_t nh = (n + 63) / 64, nc = (int64_t)sweep_stages(m) * kSwCols;
-  if (nc > 2147483647LL || (nh + 7) / 8 > 65535) return cudaErrorInvalidValue;
-  sweep_planes_kernel<<<dim3((unsigned)nc, (unsigned)((nh + 7) / 8)), 256, 0, st>>>(packed, (n + 3) / 4, n, m, planes,
-                                                                                    nh, nc);
-  return cudaGetLastError();
-}
-
-// Clusters of two that fit at once, counted once per device ordinal.
-int sweep_clusters() {
-  constexpr int kDevs = 64;
-  static std::atomic<int> cache[kDevs];  // 0 = not yet counted, else count + 1
-  int dev = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kDevs) {
-    cudaGetLastError();
-    return 0;
-  }
-  if (const int c = cache[dev].load(std::memory_order_acquire)) return c - 1;
-  int n = 0, sms = 0;
-  if (cudaFuncSetAttribute(sweep_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSwSmem) == cudaSuccess &&
-      cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess) {
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)std::max(2, sms & ~1));
-    cfg.blockDim = dim3(kSwThreads);
-    cfg.dynamicSmemBytes = kSwSmem;
-    if (cudaOccupancyMaxActiveClusters(&n, sweep_kernel, &cfg) != cudaSuccess) n = 0;
-  }
-  cudaGetLastError();
-  cache[dev].store(n + 1, std::memory_order_release);
-  return n;
-}
-
-// E2M1 form; a tile's counts below 2^21 (exact FP32 sums, and their packing in
-// sweep_store); the tensor map's coordinates.
-bool sweep_usable(int64_t n, int64_t m) {
-  if (m >= ((int64_t)1 << 21) || (n + 63) / 64 > 65535 * 8) return false;
-  return encode_tiled_fn() != nullptr && sweep_clusters() > 0;
-}
-
-// Work list of a triangle of n samples.  Tiles of two block rows by up to
-// three block columns, in bands of 16 block rows, column by column in a band, so
-// that the tiles in flight share operand blocks through L2.  The columns are
-// grouped from the right edge, the same for every row, and the group that
-// holds the diagonal starts at it.  The full-width tiles run whole, one per cluster and wave, as
-// many full waves as there are; the rest (the last partial wave and the
-// narrower tiles) are laid end to end, weighted by their cost per stage, and
-// cut into equal shares, one per cluster, each share a few pieces of
-// neighbouring tiles.
-SweepPlan sweep_plan(int64_t n, int64_t m, int clusters) {
-  SweepPlan pl;
-  const int S = sweep_stages(m);
-  pl.stages = S;
-  const int T = (int)((n + kTB - 1) / kTB), C = std::max(1, clusters);
-  struct Tile {
-    int I, J, w;
-  };
-  std::vector<Tile> full, rest;
+// The tiles of a triangle of n samples: two block rows by up to three block
+// columns, in bands of 16 block rows, column by column in a band, so that the
+// tiles in flight share operand blocks through L2.  The columns are grouped from
+// the right edge, the same for every row, and the group that holds the
+// diagonal starts at it.
+void triangle_tiles(int64_t n, int stages, int subset, std::vector<Tile>& full, std::vector<Tile>& narrow) {
+  const int T = (int)((n + kTB - 1) / kTB);
   constexpr int G = 16;
   for (int g0 = 0; g0 < T; g0 += G)
     for (int end = (T - g0 - 1) % 3 + 1 + g0; end <= T; end += 3)  // column groups end at T, T - 3, ...
       for (int I = g0; I < std::min(T, g0 + G) && I < end; I += 2) {
         const int J = std::max(I, end - 3);
-        (end - J == 3 ? full : rest).push_back({I, J, end - J});
+        (end - J == 3 ? full : narrow).push_back({I, J, end - J, subset, stages});
       }
-  const int waves = (int)(full.size() / (size_t)C);
-  const size_t whole = (size_t)waves * C;
-  rest.insert(rest.begin(), full.begin() + (long)whole, full.end());
-  // cost of one stage (cycles measured or, for narrow tiles, bound by the
-  // copies) and of a piece's start and end
-  auto cost = [](int w) { return w == 3 ? 620.0 : (w == 2 ? 520.0 : 500.0); };
+}
+
+// Cost of a tile's ring stage: about 620 cycles measured at full width, the fixed
+// cost of a stage for the narrow tiles.
+double stage_cost(int w) { return w == 3 ? 620.0 : (w == 2 ? 520.0 : 500.0); }
+double tile_cost(const Tile& t) { return stage_cost(t.w) * 4 * t.stages; }
+
+SweepItem whole_item(const Tile& t, int wave) {
+  SweepItem it{};
+  it.I = t.I;
+  it.J = t.J;
+  it.w = t.w;
+  it.subset = t.subset;
+  it.q1 = 4 * t.stages;
+  it.slot = -1;
+  it.wave = wave;
+  return it;
+}
+
+// Lay the tiles of `rest` end to end and cut them so that every cluster's load
+// ends at the same time: each takes the next stretch, a few pieces of
+// neighbouring tiles.  A stretch has at least a few stages (a piece costs about
+// kMin stages of its own: pipeline fill, read-back, a part to add up), so a
+// small problem leaves clusters idle.  Then the lists, cluster by cluster.
+void cut_rest(const std::vector<Tile>& rest, std::vector<std::vector<SweepItem>>& own, std::vector<double>& load,
+              SweepPlan& pl) {
+  const int C = (int)own.size();
+  constexpr double kMin = 8 * 620.0;
   double total = 0;
-  for (const Tile& t : rest) total += cost(t.w) * 4 * S;
-  // shares: one per cluster, but none shorter than a few stages (a piece costs
-  // about kMin stages of its own: pipeline fill, read-back, a part to add up)
-  constexpr double kMin = 8;
-  const int shares = (int)std::max(1.0, std::min((double)C, total / (620.0 * kMin)));
-  std::vector<std::vector<SweepItem>> own((size_t)C);
-  for (size_t t = 0; t < whole; ++t) {
-    SweepItem it{};
-    it.I = full[t].I;
-    it.J = full[t].J;
-    it.w = full[t].w;
-    it.q1 = 4 * S;
-    it.slot = -1;
-    it.wave = (int)(t / C);
-    own[t % C].push_back(it);
+  for (const Tile& t : rest) total += tile_cost(t);
+  // the clusters that take part, the least loaded first, and the common end
+  std::vector<int> by((size_t)C);
+  for (int c = 0; c < C; ++c) by[(size_t)c] = c;
+  std::stable_sort(by.begin(), by.end(), [&](int a, int b) { return load[(size_t)a] < load[(size_t)b]; });
+  int shares = 0;
+  double held = 0, end = 0;
+  for (int k = 1; k <= C; ++k) {
+    held += load[(size_t)by[(size_t)k - 1]];
+    const double e = (held + total) / k;  // if k clusters share the rest
+    if (k > 1 && e - load[(size_t)by[(size_t)k - 1]] < kMin) break;
+    shares = k;
+    end = e;
   }
-  pl.waves = waves;
+  std::sort(by.begin(), by.begin() + shares);  // in order, so that neighbours work on neighbouring tiles
   int share = 0;
-  double used = 0;  // cost laid so far
+  auto room = [&] { return end - load[(size_t)by[(size_t)share]]; };
   for (const Tile& t : rest) {
+    const int S = t.stages;
+    const double cost = stage_cost(t.w);
     SweepGroup gr{};
     gr.I = t.I;
     gr.J = t.J;
     gr.w = t.w;
+    gr.subset = t.subset;
     gr.slot = pl.slots;
     int q = 0;
     while (q < 4 * S) {
-      // stages left in this share
-      const double left = total * (share + 1) / shares - used;
-      int k = (int)(left / cost(t.w) + 0.5);
-      if (share == shares - 1) k = 4 * S - q;
-      k = std::min(k, 4 * S - q);
+      const bool last = share == shares - 1;
+      int k = last ? 4 * S - q : (int)std::max(0.0, std::min((double)(4 * S - q), room() / cost + 0.5));
       if (4 * S - q - k > 0 && 4 * S - q - k < 3) k = 4 * S - q;  // no sliver left behind
-      if (k < 3 && k < 4 * S - q) {                              // nor one begun
+      if (k < 3 && k < 4 * S - q) {                               // nor one begun
         ++share;
         continue;
       }
-      SweepItem it{};
-      it.I = t.I;
-      it.J = t.J;
-      it.w = t.w;
+      SweepItem it = whole_item(t, -1);
       it.q0 = q;
       it.q1 = q + k;
-      it.slot = pl.slots;
-      it.wave = -1;
-      if (q == 0 && k == 4 * S) {
-        it.slot = -1;  // a whole tile after all
-      } else {
+      if (q != 0 || k != 4 * S) {
+        it.slot = pl.slots;
         for (int pr = 0; pr < 3; ++pr) {
           const int a = pr == 0 ? 0 : pr * S, b = pr == 2 ? 4 * S : (pr + 1) * S;
           if (it.q0 < b && it.q1 > a) {
@@ -751,10 +905,10 @@ SweepPlan sweep_plan(int64_t n, int64_t m, int clusters) {
           }
         }
       }
-      own[(size_t)(share % C)].push_back(it);
-      used += cost(t.w) * k;
+      own[(size_t)by[(size_t)share]].push_back(it);
+      load[(size_t)by[(size_t)share]] += cost * k;
       q += k;
-      if (used >= total * (share + 1) / shares - 1e-6 && share < shares - 1) ++share;
+      if (!last && room() < 0.5 * cost) ++share;
     }
     if (gr.pieces[0] + gr.pieces[1] + gr.pieces[2] > 0) pl.groups.push_back(gr);
   }
@@ -769,37 +923,208 @@ SweepPlan sweep_plan(int64_t n, int64_t m, int clusters) {
   // clusters without work are not launched
   pl.clusters = C;
   while (pl.clusters > 1 && pl.first[(size_t)pl.clusters - 1] == (int32_t)pl.items.size()) --pl.clusters;
+}
+
+// One matrix or one step: the full-width tiles run whole, one per cluster and
+// wave, as many full waves as there are; the last partial wave and the
+// narrower tiles are cut into equal shares.
+SweepPlan schedule(std::vector<Tile>& full, const std::vector<Tile>& narrow, int clusters) {
+  SweepPlan pl;
+  const size_t C = (size_t)std::max(1, clusters), whole = full.size() / C * C;
+  std::vector<std::vector<SweepItem>> own(C);
+  std::vector<double> load(C, 0.0);
+  for (size_t t = 0; t < whole; ++t) {
+    own[t % C].push_back(whole_item(full[t], (int)(t / C)));
+    load[t % C] += tile_cost(full[t]);
+    pl.wave_stages = std::max(pl.wave_stages, 4 * full[t].stages);
+  }
+  pl.waves = (int)(whole / C);
+  std::vector<Tile> rest(full.begin() + (long)whole, full.end());
+  rest.insert(rest.end(), narrow.begin(), narrow.end());
+  cut_rest(rest, own, load, pl);
   return pl;
 }
 
-cudaError_t launch_sweep(const SweepLaunch& l, cudaStream_t st) {
-  CUtensorMap a, b1, b2, b3;
-  const int64_t nc = (int64_t)l.stages * kSwCols;
-  if (!encode_sweep_map(&a, l.a_planes, l.a_half, nc, 2) || !encode_sweep_map(&b1, l.b_planes, l.b_half, nc, 1) ||
-      !encode_sweep_map(&b2, l.b_planes, l.b_half, nc, 2) || !encode_sweep_map(&b3, l.b_planes, l.b_half, nc, 3))
-    return cudaErrorInvalidValue;
+template <class W>
+cudaError_t launch_sweep_w(const W& work, const SweepLaunch& l, cudaStream_t st) {
   // function attributes are per device: set before every launch
-  cudaError_t e = cudaFuncSetAttribute(sweep_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSwSmem);
+  cudaError_t e = cudaFuncSetAttribute(sweep_kernel<W>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSwSmem);
   if (e != cudaSuccess) return e;
-  SweepArgs args{};
-  args.out = SweepOut{l.n, l.counts, l.dist, l.square ? 1 : 0};
-  args.items = l.items;
-  args.first = l.first;
-  args.stages = l.stages;
-  args.scratch = l.scratch;
-  args.part = l.part;
-  args.status = l.status;
-  args.wait_ns = l.wait_ns;
-  args.sync = l.sync;
-  sweep_kernel<<<2 * l.clusters, kSwThreads, kSwSmem, st>>>(a, b1, b2, b3, args);
+  const SweepArgs args{l.items, l.first, l.scratch, l.part, l.status, l.wait_ns, l.sync};
+  sweep_kernel<W><<<2 * l.clusters, kSwThreads, kSwSmem, st>>>(work, args);
+  if ((e = cudaGetLastError()) != cudaSuccess || l.n_groups <= 0) return e;
+  if (l.between) {
+    e = cudaEventRecord(l.between, st);
+    if (e != cudaSuccess) return e;
+  }
+  sweep_finalize_kernel<W><<<dim3((unsigned)l.n_groups, 48), 128, 0, st>>>(l.groups, l.part, work);
   return cudaGetLastError();
 }
 
-cudaError_t launch_sweep_finalize(const SweepLaunch& l, const SweepGroup* groups, int64_t n_groups, cudaStream_t st) {
-  if (n_groups <= 0) return cudaSuccess;
-  sweep_finalize_kernel<<<dim3((unsigned)n_groups, 48), 128, 0, st>>>(
-      groups, l.part, SweepOut{l.n, l.counts, l.dist, l.square ? 1 : 0});
+}  // namespace
+
+int sweep_stages(int64_t m) { return (int)((m + kSwMarkers - 1) / kSwMarkers); }
+int64_t sweep_cols(int64_t m) { return (int64_t)sweep_stages(m) * kSwCols; }
+
+size_t sweep_planes_bytes(int64_t n, int64_t m) { return (size_t)((n + 63) / 64) * (size_t)sweep_cols(m) * 4096; }
+
+size_t sweep_scratch_bytes(int clusters) { return (size_t)clusters * 2 * 3 * kSwHalfTile * sizeof(float); }
+size_t sweep_slot_bytes() { return 2 * kSwHalfTile * sizeof(float); }
+
+// Lockstep of `waves` waves of whole tiles of at most `stages` ring stages, by
+// the two-SM kernels' setting {chunks of 64 markers, lag}; off: no counters.
+SweepSync sweep_sync(int waves, int stages, int2 ss) {
+  SweepSync s;
+  if (ss.x <= 0 || waves < 1) return s;
+  s.seg = std::max(1, ss.x * 64 / kSwMarkers);
+  s.lag = ss.y;
+  s.n_seg = (stages + s.seg - 1) / s.seg;
+  return s;
+}
+
+cudaError_t launch_sweep_planes(const uint8_t* packed, int64_t n, int64_t m, uint8_t* planes, cudaStream_t st) {
+  const int64_t nh = (n + 63) / 64, nc = sweep_cols(m);
+  if (nc > 2147483647LL || (nh + 7) / 8 > 65535) return cudaErrorInvalidValue;
+  sweep_planes_kernel<<<dim3((unsigned)nc, (unsigned)((nh + 7) / 8)), 256, 0, st>>>(packed, (n + 3) / 4, n, m, planes,
+                                                                                    nh, nc);
   return cudaGetLastError();
+}
+
+int64_t sweep_gather_ctas(int64_t n, int64_t n_cols) {
+  return (n + kTB - 1) / kTB * ((n_cols + kSwGatherCols - 1) / kSwGatherCols);
+}
+int sweep_gather_cols() { return kSwGatherCols; }
+
+// Regrouping costs about 0.12 ps per genotype of the pool's rows in use and
+// saves 0.8 ps per gathered genotype.
+bool sweep_words_pay(int64_t pool_genotypes, int64_t gathered) { return gathered >= pool_genotypes / 4; }
+
+cudaError_t launch_sweep_gather(const TcGatherJob* jobs, const int4* map, int64_t ctas, const SweepPool* pool,
+                                int num_sms, int* status, cudaStream_t st) {
+  if (ctas <= 0) return cudaSuccess;
+  if (ctas > 2147483647LL) return cudaErrorInvalidValue;
+  sweep_words_kernel<<<8 * num_sms, 256, 0, st>>>(pool);
+  if (cudaError_t e = cudaGetLastError()) return e;
+  sweep_gather_kernel<<<(unsigned)ctas, kTB, 0, st>>>(jobs, map, pool, status);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_sweep_gather_rows(const RowSrc* rows, int64_t n_rows, int64_t n_cols, uint8_t* dst,
+                                     int64_t dst_half, cudaStream_t st) {
+  if (n_rows <= 0) return cudaSuccess;
+  sweep_gather_rows_kernel<<<dim3((unsigned)n_cols, (unsigned)((n_rows + 63) / 64)), 256, 0, st>>>(rows, n_rows, n_cols,
+                                                                                                 dst, dst_half);
+  return cudaGetLastError();
+}
+
+// Clusters of two that fit at once, counted once per device ordinal.
+int sweep_clusters() {
+  constexpr int kDevs = 64;
+  static std::atomic<int> cache[kDevs];  // 0 = not yet counted, else count + 1
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kDevs) {
+    cudaGetLastError();
+    return 0;
+  }
+  if (const int c = cache[dev].load(std::memory_order_acquire)) return c - 1;
+  int n = 0, sms = 0;
+  auto kern = sweep_kernel<SweepOne>;
+  if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSwSmem) == cudaSuccess &&
+      cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)std::max(2, sms & ~1));
+    cfg.blockDim = dim3(kSwThreads);
+    cfg.dynamicSmemBytes = kSwSmem;
+    if (cudaOccupancyMaxActiveClusters(&n, kern, &cfg) != cudaSuccess) n = 0;
+  }
+  cudaGetLastError();
+  cache[dev].store(n + 1, std::memory_order_release);
+  return n;
+}
+
+// E2M1 form; a tile's counts below 2^21 (exact FP32 sums, and their packing in
+// sweep_store); the tensor map's coordinates.
+bool sweep_usable(int64_t n, int64_t m) {
+  if (m >= ((int64_t)1 << 21) || (n + 63) / 64 > 65535 * 8) return false;
+  return encode_tiled_fn() != nullptr && sweep_clusters() > 0;
+}
+
+SweepPlan sweep_plan(int64_t n, int64_t m, int clusters) {
+  std::vector<Tile> full, narrow;
+  triangle_tiles(n, sweep_stages(m), 0, full, narrow);
+  return schedule(full, narrow, clusters);
+}
+
+// Batched subsets, by decreasing marker count: each tile in turn to the least
+// loaded cluster, so that a subset's tiles run at the same time over the same
+// markers and share its planes through L2 (in shares of tiles laid end to
+// end the clusters ran all subsets at once, from HBM: 3.8 ms for 24 subsets of
+// a 10,000 x 200,000 pool); the last tiles, about one per cluster, are cut to
+// even out the end.
+SweepPlan sweep_plan_batch(const std::vector<std::pair<int64_t, int64_t>>& shapes, int clusters) {
+  std::vector<size_t> order(shapes.size());
+  for (size_t k = 0; k < order.size(); ++k) order[k] = k;
+  std::stable_sort(order.begin(), order.end(), [&](size_t a, size_t b) { return shapes[a].second > shapes[b].second; });
+  std::vector<Tile> all;
+  for (size_t k : order) {
+    std::vector<Tile> full, narrow;
+    triangle_tiles(shapes[k].first, sweep_stages(shapes[k].second), (int)k, full, narrow);
+    all.insert(all.end(), full.begin(), full.end());
+    all.insert(all.end(), narrow.begin(), narrow.end());
+  }
+  SweepPlan pl;
+  const size_t C = (size_t)std::max(1, clusters), lead = all.size() > C ? all.size() - C : 0;
+  std::vector<std::vector<SweepItem>> own(C);
+  std::vector<double> load(C, 0.0);
+  for (size_t t = 0; t < lead; ++t) {
+    const size_t c = (size_t)(std::min_element(load.begin(), load.end()) - load.begin());
+    own[c].push_back(whole_item(all[t], -1));
+    load[c] += tile_cost(all[t]);
+  }
+  cut_rest(std::vector<Tile>(all.begin() + (long)lead, all.end()), own, load, pl);
+  return pl;
+}
+
+// Row pairs over two ranges of block columns [col0, col1) (the second may be
+// empty): columns in groups of three, the row pairs of a group together.
+SweepPlan sweep_plan_cross(int64_t row_blocks, const int64_t (&cols)[2][2], int64_t m, int clusters) {
+  std::vector<Tile> full, narrow;
+  const int S = sweep_stages(m);
+  for (const auto& r : cols)
+    for (int64_t J = r[0]; J < r[1]; J += 3) {
+      const int w = (int)std::min<int64_t>(3, r[1] - J);
+      for (int64_t I = 0; I < row_blocks; I += 2) (w == 3 ? full : narrow).push_back({(int)I, (int)J, w, 0, S});
+    }
+  return schedule(full, narrow, clusters);
+}
+
+bool sweep_encode_maps(void* maps, const void* planes, int64_t n, int64_t m) {
+  return encode_sweep_maps(static_cast<SweepMaps*>(maps), planes, (n + 63) / 64, sweep_cols(m));
+}
+
+cudaError_t launch_sweep_one(const uint8_t* planes, int64_t n, int64_t m, int32_t* counts, double* dist, bool square,
+                             const SweepLaunch& l, cudaStream_t st) {
+  SweepOne w{};
+  if (!encode_sweep_maps(&w.maps, planes, (n + 63) / 64, sweep_cols(m))) return cudaErrorInvalidValue;
+  w.result = SweepOut{n, counts, dist, square ? 1 : 0};
+  w.n_stages = sweep_stages(m);
+  return launch_sweep_w(w, l, st);
+}
+
+cudaError_t launch_sweep_batch(const void* maps_dev, const SubsetDev* subs, const SweepLaunch& l, cudaStream_t st) {
+  return launch_sweep_w(SweepBatch{static_cast<const SweepMaps*>(maps_dev), subs}, l, st);
+}
+
+cudaError_t launch_sweep_cross(const uint8_t* row_planes, int64_t row_half, const uint8_t* panel, int64_t n_panel,
+                               int64_t m, int32_t* const* row_out, int64_t n_rows, const SweepLaunch& l,
+                               cudaStream_t st) {
+  SweepCross w{};
+  if (!encode_sweep_maps(&w.maps, panel, (n_panel + 63) / 64, sweep_cols(m)) ||
+      !encode_sweep_map(&w.rows, row_planes, row_half, sweep_cols(m), 2))
+    return cudaErrorInvalidValue;
+  w.result = SweepRows{row_out, n_rows, n_panel};
+  w.n_stages = sweep_stages(m);
+  return launch_sweep_w(w, l, st);
 }
 
 }  // namespace ibs

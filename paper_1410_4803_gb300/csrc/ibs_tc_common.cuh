@@ -150,6 +150,38 @@ __device__ __forceinline__ uint32_t tc_transpose32(uint32_t x, int lane) {
   return x;
 }
 
+// A ring barrier's wait: one probe on the usual path; past it, bounded by
+// limit_ns and ended by another role's abort.
+__device__ __noinline__ bool ring_wait_slow(uint64_t* bar, uint32_t parity, unsigned long long limit_ns,
+                                             const int* abort_flag) {
+  const unsigned long long t0 = globaltimer_ns();
+  for (;;) {
+    if (limit_ns < 1000000ull) {  // short bounds (tests): a blocking probe could outlast them
+      if (mbar_test_wait(bar, parity)) return true;
+    } else {
+      for (int i = 0; i < 64; ++i)
+        if (mbar_try_wait(bar, parity)) return true;
+    }
+    if (*(volatile const int*)abort_flag != 0 || globaltimer_ns() - t0 > limit_ns) return false;
+  }
+}
+__device__ __forceinline__ bool ring_wait(uint64_t* bar, uint32_t parity, unsigned long long limit_ns,
+                                           const int* abort_flag) {
+  if (limit_ns >= 1000000ull && mbar_try_wait(bar, parity)) return true;
+  return ring_wait_slow(bar, parity, limit_ns, abort_flag);
+}
+
+// A waiter warp's release of a ring slot to the MMA warp: one hardware barrier
+// per slot, on which the waiter arrives without blocking and the MMA warp
+// waits.  The waiter cannot arrive on a slot's barrier again before the MMA
+// warp has passed it: the slot is filled again only after its MMAs.
+__device__ __forceinline__ void ring_release(uint32_t id) {
+  asm volatile("barrier.cta.arrive %0, 64;" ::"r"(id) : "memory");
+}
+__device__ __forceinline__ void ring_acquire(uint32_t id) {
+  asm volatile("barrier.cta.sync %0, 64;" ::"r"(id) : "memory");
+}
+
 // ---------------------------------------------------------------------------
 // Clusters of two CTAs (the two-SM kernels).
 __device__ __forceinline__ uint32_t cluster_rank() {

@@ -1,7 +1,8 @@
 """The sweep kernel (E2M1 triangles of ibs_compute) at its own edges, against the
 oracle: half-blocks of 64 samples, row pairs of 256, column groups of 384, ring
 stages of 288 markers, rows at every alignment, tiles split into parts and
-whole waves of tiles; and the call whose workspace has no room for it."""
+whole waves of tiles; the call whose workspace has no room for it; and the gather
+of batched subsets from both forms of the pool."""
 import numpy as np
 import pytest
 
@@ -58,3 +59,28 @@ def test_no_room_for_the_workspace():
             assert_dist_close(got_d, want_d)
     finally:
         ibs.ibs_shutdown(c)
+
+
+@pytest.mark.parametrize("pool_n,n,vb,vl", [
+    (1003, 1000, 0, 3001),   # the window regrouped by sample: from the first marker to the last
+    (1003, 300, 37, 2593),   # from inside a column of the pool
+    (1003, 251, 2968, 33),   # two columns, just above a quarter of the pool's samples
+    (1003, 250, 37, 2593),   # below a quarter: single bytes
+    (4096, 1, 0, 3001),
+])
+def test_batch_gather(ctx, pool_n, n, vb, vl):
+    import torch
+    from paper_1410_4803_gb300 import ibs
+    rng = np.random.default_rng(n + vl)
+    codes = random_codes(rng, pool_n, 3001, miss=0.05)
+    idx = rng.permutation(pool_n)[:n].astype(np.int64)
+    want_c, want_d = oracle.ibs_triangle(pack_codes(codes[idx][:, vb:vb + vl]), n, vl)
+    pool = torch.from_numpy(pack_codes(codes, garbage_rng=rng)).cuda()
+    dev_idx = torch.from_numpy(idx).cuda()
+    for _ in range(2):
+        out_c = torch.full((n * (n + 1) // 2, 4), -7, dtype=torch.int32, device="cuda")
+        out_d = torch.empty(n * (n + 1) // 2, dtype=torch.float64, device="cuda")
+        ibs.ibs_compute_batch(ctx, pool, pool_n, 3001, [(dev_idx, vb, vl, out_c, out_d)])
+        ibs.ibs_synchronize(ctx)
+        assert (out_c.cpu().numpy() == want_c).all()
+        assert_dist_close(out_d.cpu().numpy(), want_d)

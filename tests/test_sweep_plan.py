@@ -21,4 +21,4 @@ def test_sweep_plans_cover_the_triangle(tmp_path):
     assert build.returncode == 0, build.stdout + build.stderr
     run = subprocess.run([exe], capture_output=True, text=True, timeout=300)
     assert run.returncode == 0, run.stdout[-4000:]
-    assert "checked 480 lists, 0 failures" in run.stdout, run.stdout[-2000:]
+    assert "checked 600 lists, 0 failures" in run.stdout, run.stdout[-2000:]
