@@ -14,7 +14,9 @@ namespace {
 // (monotone as unsigned), NaN (N == 0) mapped above +inf, padding above NaN;
 // ties are broken by ascending panel index.
 constexpr int kTopkMax = 64;
-constexpr int kTopkThreads = 256;
+constexpr int kTopkThreads = 512;
+constexpr int kTopkGroups = 128;  // groups of neighbouring threads (at least kTopkMax)
+constexpr int kTopkCand = 512;    // candidates kept per row
 constexpr uint64_t kNanKey = 0x7FF8000000000000ull;
 constexpr uint64_t kPadKey = 0xFFFFFFFFFFFFFFFFull;
 
@@ -22,10 +24,21 @@ __device__ __forceinline__ bool key_less(uint64_t ka, int ia, uint64_t kb, int i
   return ka < kb || (ka == kb && ia < ib);
 }
 
-// One row's k nearest panel samples (one CTA of kTopkThreads threads):
-// counts c[n_panel] -> out_idx[k], out_dist[k].
-__device__ __forceinline__ void topk_row(const int4* __restrict__ c, int64_t n_panel, int k,
-                                         int32_t* __restrict__ out_idx, double* __restrict__ out_dist) {
+// FP32 quotient of a pair's distance, infinite without a common call: at most
+// five roundings to nearest, so within 2^-21 of the distance.
+__device__ __forceinline__ float topk_approx(const int4& q) {
+  if (q.w == 0) return __int_as_float(0x7F800000);
+  return __fmul_rn(__fmaf_rn(2.0f, (float)q.x, (float)q.y), __frcp_rn(2.0f * (float)q.w));
+}
+__device__ __forceinline__ uint64_t topk_key(const int4& q) {
+  if (q.w == 0) return kNanKey;
+  return (uint64_t)__double_as_longlong((double)((long long)q.y + 2 * (long long)q.x) / (2.0 * (double)q.w));
+}
+
+// One row's k nearest panel samples, each thread keeping a sorted list (rows with
+// too many candidates for topk_row).
+__device__ __noinline__ void topk_row_lists(const int4* __restrict__ c, int64_t n_panel, int k,
+                                            int32_t* __restrict__ out_idx, double* __restrict__ out_dist) {
   uint64_t key[kTopkMax];
   int idx[kTopkMax];
 #pragma unroll
@@ -38,25 +51,14 @@ __device__ __forceinline__ void topk_row(const int4* __restrict__ c, int64_t n_p
   // among equal keys.
   for (int64_t e = threadIdx.x; e < n_panel; e += kTopkThreads) {
     const int4 q = c[e];
-    uint64_t kk;
-    if (q.w == 0) {
-      kk = kNanKey;
-    } else {
-      // Cheap exact reject once the list is full of finite keys: the two
-      // integer-to-FP32 conversions and the FP32 division are each correctly
-      // rounded, so the FP32 quotient f is within 3 * 2^-24 (relative) of the
-      // rational r.  If f > t (1 + 2^-20), with t the list's k-th key, then
-      // r > t, and the double key (r rounded, a monotone map) is >= t: it
-      // would not be inserted (strict comparison below).  Only the others pay
-      // the FP64 division.
-      const uint64_t last = key[k - 1];
-      if (last < kNanKey) {
-        const float f = __fdiv_rn((float)(q.y + 2 * q.x), (float)(2 * q.w));
-        if ((double)f > __longlong_as_double((long long)last) * (1.0 + 0x1p-20)) continue;
-      }
-      const double d = (double)(q.y + 2 * q.x) / (2.0 * (double)q.w);
-      kk = (uint64_t)__double_as_longlong(d);
-    }
+    // Cheap exact reject once the list is full of finite keys: with f within
+    // 2^-21 of the distance r and f > t (1 + 2^-20), t the list's k-th key,
+    // r > t, and the double key (r rounded, a monotone map) is >= t: it would not
+    // be inserted (strict comparison below).  Only the others pay the FP64
+    // division.
+    const uint64_t last = key[k - 1];
+    if (last < kNanKey && (double)topk_approx(q) > __longlong_as_double((long long)last) * (1.0 + 0x1p-20)) continue;
+    const uint64_t kk = topk_key(q);
     if (kk < key[k - 1]) {
       int pos = k - 1;
 #pragma unroll 1
@@ -121,6 +123,76 @@ __device__ __forceinline__ void topk_row(const int4* __restrict__ c, int64_t n_p
     __syncthreads();
     if (threadIdx.x == winner) ++head;
     __syncthreads();
+  }
+}
+
+// One row's k nearest panel samples (one CTA of kTopkThreads threads): counts
+// c[n_panel] -> out_idx[k], out_dist[k].  Two passes over the row with the
+// FP32 quotient f of each distance.  First the least f of each of 128
+// groups of threads: k groups hold a sample with f <= T, T the k-th smallest of
+// these, so each of the k nearest has f <= T (1 + 2^-20).  The samples below that
+// bound, few more than k, are collected and ranked by their exact keys.  A
+// sorted list per thread instead (topk_row_lists) divides in FP64 for every
+// entry of a list, and its k block-wide rounds run one after the other: 138 us
+// for one row and 1.69 ms for 3,003 rows of 20,000 samples, k = 16, against 35
+// us and 0.37 ms.
+__device__ __forceinline__ void topk_row(const int4* __restrict__ c, int64_t n_panel, int k,
+                                         int32_t* __restrict__ out_idx, double* __restrict__ out_dist) {
+  __shared__ float least[kTopkGroups];
+  __shared__ uint64_t ckey[kTopkCand];
+  __shared__ int cidx[kTopkCand];
+  __shared__ float bound;
+  __shared__ int n_cand;
+  const int t = threadIdx.x;
+  const float inf = __int_as_float(0x7F800000);
+  if (t == 0) n_cand = 0;
+  float f = inf;
+#pragma unroll 8
+  for (int64_t e = t; e < n_panel; e += kTopkThreads) f = fminf(f, topk_approx(__ldg(c + e)));
+  constexpr int kPer = kTopkThreads / kTopkGroups;
+#pragma unroll
+  for (int off = 1; off < kPer; off <<= 1) f = fminf(f, __shfl_xor_sync(0xffffffffu, f, off));
+  if (t % kPer == 0) least[t / kPer] = f;
+  __syncthreads();
+  if (t < kTopkGroups) {
+    const float mine = least[t];
+    int rank = 0;
+#pragma unroll 8
+    for (int g = 0; g < kTopkGroups; ++g) rank += least[g] < mine || (least[g] == mine && g < t);
+    if (rank == k - 1) bound = __fmul_ru(mine, 1.0f + 0x1p-20f);  // infinite: every sample
+  }
+  __syncthreads();
+  const float limit = bound;
+#pragma unroll 8
+  for (int64_t e = t; e < n_panel; e += kTopkThreads) {
+    const int4 q = __ldg(c + e);
+    if (topk_approx(q) <= limit) {
+      const int at = atomicAdd(&n_cand, 1);
+      if (at < kTopkCand) {
+        cidx[at] = (int)e;
+        ckey[at] = topk_key(q);
+      }
+    }
+  }
+  __syncthreads();
+  const int n = n_cand;
+  if (n > kTopkCand) {
+    topk_row_lists(c, n_panel, k, out_idx, out_dist);
+    return;
+  }
+  for (int i = t; i < n; i += kTopkThreads) {
+    const uint64_t key = ckey[i];
+    const int idx = cidx[i];
+    int rank = 0;
+    for (int j = 0; j < n; ++j) rank += key_less(ckey[j], cidx[j], key, idx);
+    if (rank < k) {
+      out_idx[rank] = idx;
+      out_dist[rank] = __longlong_as_double(key == kNanKey ? 0x7ff8000000000000LL : (long long)key);
+    }
+  }
+  for (int r = n + t; r < k; r += kTopkThreads) {  // fewer samples than k
+    out_idx[r] = -1;
+    out_dist[r] = __longlong_as_double(0x7ff8000000000000LL);
   }
 }
 
