@@ -98,7 +98,16 @@ struct RowSrc {
   const uint32_t* planes;   // the request's bit planes
   int64_t row;              // row within the request
   int64_t n_half;           // sweep planes: the request's half-blocks
-};
+};                          // (launch_few_rows: its packed bytes, their row length)
+
+// Serving: few rows against the panel's words (ibs_rows.cu), panel samples
+// [samples[0][0], samples[0][1]) and [samples[1][0], samples[1][1]).  `words`
+// holds few_rows_bytes; `part` at least 12 bytes per row and panel sample.
+constexpr int kFewRows = 16;
+size_t few_rows_bytes(int64_t n_cols);
+cudaError_t launch_few_rows(const RowSrc* rows, int64_t n_rows, const uint32_t* panel_words, int64_t n_panel, int64_t m,
+                            const int64_t (&samples)[2][2], void* words, void* part, size_t part_bytes, int num_sms,
+                            int32_t* const* row_out, cudaStream_t st);
 
 // Kernel launchers (ibs_planes.cu / ibs_pairs.cu / ibs_misc.cu).
 cudaError_t launch_planes(const BedSource& src, int64_t n, int64_t m, const PlaneGeom& g, uint32_t* planes,
@@ -339,6 +348,7 @@ struct SweepPool {
   int64_t begin = 0, cols = 0;          // first marker in use; columns of 32 from there
   uint32_t* words = nullptr;            // [cols][n]{low code bits, high code bits}
 };
+cudaError_t launch_sweep_words(const SweepPool& pool, int num_sms, cudaStream_t st);
 bool sweep_words_pay(int64_t pool_genotypes, int64_t gathered);
 cudaError_t launch_sweep_gather(const TcGatherJob* jobs, const int4* map, int64_t ctas, const SweepPool* pool,
                                 int num_sms, int* status, cudaStream_t st);

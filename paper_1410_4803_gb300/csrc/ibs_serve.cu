@@ -70,6 +70,7 @@ struct Request {
   std::vector<uint8_t> host_packed;
   DevBuf packed, planes, counts, tidx, tdist;
   size_t reserved = 0;
+  bool planes_built = false;
   int64_t blocks_done = 0;  // panel blocks processed since admission
   cudaEvent_t done_ev = nullptr;  // recorded on the engine's copy stream after the request's last output
   ibs_status status = IBS_OK;
@@ -122,6 +123,8 @@ class ServeEngine {
   DevBuf sweep_scratch, sweep_part;  // the steps'
   DevBuf sync_scratch, sync_part;    // the unbatched path's, one call at a time
   std::mutex sync_mu;
+  DevBuf panel_words, few_words;     // sweep: the panel's code bits by sample, for steps of few rows; the rows'
+  std::mutex words_mu;               // panel_words in use or given back
   bool pair = false;   // two-SM kernel for steps of two or more query blocks
   int clusters = 0;    // its clusters of two CTAs
   DevBuf sync_ctr;     // the two-SM kernel's K-lockstep counters of a step
@@ -202,9 +205,19 @@ class ServeEngine {
     r.done_ev = nullptr;
   }
 
+  // The panel's words are an extra: a request that finds no memory has them
+  // given back (true if there were any; cudaFree waits for their last use).
+  bool give_back_words() {
+    std::lock_guard<std::mutex> lk(words_mu);
+    if (!panel_words.p) return false;
+    free_buf(ctx, panel_words);
+    return true;
+  }
+
   ibs_status alloc(DevBuf& b, size_t bytes, cudaStream_t s) {
     if (bytes == 0) return IBS_OK;
     cudaError_t e = cudaMallocAsync(&b.p, bytes, s);
+    if (e != cudaSuccess && give_back_words()) e = cudaMallocAsync(&b.p, bytes, s);
     if (e != cudaSuccess) {
       cudaGetLastError();
       b.p = nullptr;
@@ -245,7 +258,6 @@ class ServeEngine {
       return false;
     }
     cudaMemcpyAsync(r->packed.p, r->host_packed.data(), pk, cudaMemcpyHostToDevice, stream);
-    build_planes(static_cast<const uint8_t*>(r->packed.p), r->q, r->planes.p, stream);
     cudaEventCreateWithFlags(&r->done_ev, cudaEventDisableTiming);
     r->blocks_done = 0;
     r->state = RState::Active;
@@ -432,11 +444,19 @@ class ServeEngine {
     const int slot = (int)(step_no & 1);
     if (step_ev[slot]) cudaEventSynchronize(step_ev[slot]);  // slot's host tables are free again
     int64_t n_rows = 0;
+    for (auto& r : active) n_rows += r->q;
+    // Up to kFewRows rows: the panel's code bits instead of its operand planes
+    // (one row against a 20,000 x 100,000 panel: 0.35 ms a request against 1.15;
+    // 16 rows cost two passes of about 0.3 ms, the tensor-core step 1 ms).
+    std::unique_lock<std::mutex> words_lk(words_mu);
+    const bool few = n_rows > 0 && n_rows <= kFewRows && panel_words.p;
+    if (!few) words_lk.unlock();
+    n_rows = 0;
     for (auto& r : active)
       for (int64_t row = 0; row < r->q; ++row) {
-        rows_host[slot][n_rows].planes = static_cast<const uint32_t*>(r->planes.p);
+        rows_host[slot][n_rows].planes = static_cast<const uint32_t*>(few ? r->packed.p : r->planes.p);
         rows_host[slot][n_rows].row = row;
-        rows_host[slot][n_rows].n_half = (r->q + 63) / 64;
+        rows_host[slot][n_rows].n_half = few ? (r->q + 3) / 4 : (r->q + 63) / 64;
         outs_host[slot][n_rows] = counts_ptr(*r) + (size_t)row * pg.n * 4;
         ++n_rows;
       }
@@ -449,9 +469,9 @@ class ServeEngine {
     const int64_t len = step_len(units, two_sm || sweep ? clusters : grid_ctas);
     const size_t n_items = (size_t)units * (size_t)len;
     SweepPlan pl;
-    if (sweep && n_rows > 0) {
-      const int64_t end = cursor + len;  // wraps around the panel at most once
-      const int64_t cols[2][2] = {{cursor, std::min(end, pgeo.blocks)}, {0, std::max<int64_t>(0, end - pgeo.blocks)}};
+    const int64_t end = cursor + len;  // wraps around the panel at most once
+    const int64_t cols[2][2] = {{cursor, std::min(end, pgeo.blocks)}, {0, std::max<int64_t>(0, end - pgeo.blocks)}};
+    if (sweep && n_rows > 0 && !few) {
       pl = sweep_plan_cross(qblocks, cols, pg.m, clusters);
       ensure_items(std::max<size_t>(sweep_list_bytes(pl) / sizeof(SweepItem) + 1, n_items));
     } else {
@@ -459,7 +479,9 @@ class ServeEngine {
     }
     size_t t = 0;
     int32_t** outs_d = static_cast<int32_t**>(outs_dev[slot].p);
-    if (sweep) {
+    if (few) {
+      t = 1;
+    } else if (sweep) {
       t = pl.items.size();
     } else if (two_sm) {
       PairItem* h = reinterpret_cast<PairItem*>(items_host[slot]);
@@ -491,7 +513,14 @@ class ServeEngine {
       }
     }
     if (t > 0) {
-      if (gathered_version != set_version) {
+      if (few) {
+        cudaMemcpyAsync(rows_dev[slot].p, rows_host[slot], n_rows * sizeof(RowSrc), cudaMemcpyHostToDevice, stream);
+      } else if (gathered_version != set_version) {
+        for (auto& r : active) {
+          if (r->planes_built) continue;
+          build_planes(static_cast<const uint8_t*>(r->packed.p), r->q, r->planes.p, stream);
+          r->planes_built = true;
+        }
         // the admitted set changed: pack its rows into the step planes again
         cudaMemcpyAsync(rows_dev[slot].p, rows_host[slot], n_rows * sizeof(RowSrc), cudaMemcpyHostToDevice, stream);
         if (sweep)
@@ -506,7 +535,14 @@ class ServeEngine {
         gathered_version = set_version;
       }
       cudaMemcpyAsync(outs_dev[slot].p, outs_host[slot], n_rows * sizeof(int32_t*), cudaMemcpyHostToDevice, stream);
-      if (sweep) {
+      if (few) {
+        const int64_t samples[2][2] = {{cols[0][0] * blk, std::min<int64_t>(cols[0][1] * blk, pg.n)},
+                                       {0, std::min<int64_t>(cols[1][1] * blk, pg.n)}};
+        launch_few_rows(static_cast<const RowSrc*>(rows_dev[slot].p), n_rows,
+                        static_cast<const uint32_t*>(panel_words.p), pg.n, pg.m, samples, few_words.p, sweep_part.p,
+                        sweep_part.cap, ctx->num_sms, outs_d, stream);
+        words_lk.unlock();
+      } else if (sweep) {
         run_sweep(pl, static_cast<const uint8_t*>(step_planes.p), kMaxRows / 64, outs_d, n_rows, items_host[slot],
                   static_cast<uint8_t*>(items_dev[slot].p), static_cast<float*>(sweep_scratch.p),
                   static_cast<float*>(sweep_part.p), sync_ctr, true, stream);
@@ -654,7 +690,7 @@ class ServeEngine {
     free_buf(ctx, step_planes);
     free_buf(ctx, counter);
     free_buf(ctx, sync_ctr);
-    for (DevBuf* b : {&sweep_scratch, &sweep_part, &sync_scratch, &sync_part}) free_buf(ctx, *b);
+    for (DevBuf* b : {&sweep_scratch, &sweep_part, &sync_scratch, &sync_part, &panel_words, &few_words}) free_buf(ctx, *b);
     for (int s = 0; s < 2; ++s) {
       free_buf(ctx, topk_dev[s]);
       if (topk_host[s]) cudaFreeHost(topk_host[s]);
@@ -763,6 +799,26 @@ ibs_status serve_panel_load(ibs_ctx* ctx, const uint8_t* panel, int64_t n_panel,
     src_dev = static_cast<const uint8_t*>(tmp);
   }
   IBS_CUDA_TRY(eng->build_planes(src_dev, n_panel, eng->panel_planes.p, eng->stream));
+  if (eng->sweep) {
+    // The panel's words, where they take at most an eighth of the free memory
+    // and a step's parts have room for kFewRows rows.
+    const size_t wb = (size_t)((m + 31) / 32) * (size_t)n_panel * 8;
+    size_t free_b = 0, total_b = 0;
+    if ((size_t)kFewRows * n_panel * 12 <= eng->sweep_part.cap && cudaMemGetInfo(&free_b, &total_b) == cudaSuccess &&
+        wb <= free_b / 8 && ensure_buf(ctx, eng->few_words, few_rows_bytes((m + 31) / 32)) == IBS_OK &&
+        ensure_buf(ctx, eng->panel_words, wb) == IBS_OK) {
+      SweepPool sp;
+      sp.packed = src_dev;
+      sp.row_bytes = (n_panel + 3) / 4;
+      sp.n = n_panel;
+      sp.m = m;
+      sp.cols = (m + 31) / 32;
+      sp.words = static_cast<uint32_t*>(eng->panel_words.p);
+      IBS_CUDA_TRY(launch_sweep_words(sp, ctx->num_sms, eng->stream));
+    }
+    cudaGetLastError();
+    clear_error();
+  }
   IBS_CUDA_TRY(cudaStreamSynchronize(eng->stream));
   if (tmp) cudaFree(tmp);
   if (ibs_status st = eng->alloc_step_buffers()) {
@@ -812,6 +868,7 @@ ibs_status serve_panel_load(ibs_ctx* ctx, const uint8_t* panel, int64_t n_panel,
     cudaMemGetInfo(&free_b, &total_b);
     // the sweep kernel's workspace comes out of the margin
     const size_t held = eng->sweep ? std::min(kMemMargin / 2, 2 * (eng->sweep_scratch.cap + eng->sweep_part.cap)) : 0;
+    free_b += eng->panel_words.cap;  // given back when a request needs the room
     eng->pool_budget = free_b > kMemMargin - held ? free_b - (kMemMargin - held) : 0;
   }
   eng->fixed_bytes = eng->panel_planes.cap + eng->step_planes.cap + eng->counter.cap + 2 * (eng->sweep_scratch.cap + eng->sweep_part.cap) +

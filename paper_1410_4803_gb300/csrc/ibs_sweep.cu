@@ -657,8 +657,7 @@ __global__ void __launch_bounds__(128) sweep_finalize_kernel(const SweepGroup* _
 // 200,000 pool).  Warp = one column of 64 samples, transposed by shuffles;
 // 512 neighbouring samples per CTA.  A fixed grid (the launch is in a graph and
 // the window is known per call); HBM-bound: the pool read once and written once.
-__global__ void __launch_bounds__(256) sweep_words_kernel(const SweepPool* __restrict__ pool) {
-  const SweepPool p = *pool;
+__device__ __forceinline__ void sweep_words(const SweepPool& p) {
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int64_t n_half = (p.n + 63) / 64, groups = (n_half + 7) / 8, total = p.cols * groups;
   for (int64_t i = blockIdx.x; i < total; i += gridDim.x) {
@@ -674,6 +673,9 @@ __global__ void __launch_bounds__(256) sweep_words_kernel(const SweepPool* __res
     }
   }
 }
+
+__global__ void __launch_bounds__(256) sweep_words_kernel(const SweepPool* __restrict__ pool) { sweep_words(*pool); }
+__global__ void __launch_bounds__(256) panel_words_kernel(const SweepPool pool) { sweep_words(pool); }
 
 // Batched subsets: sample sel[128 block + r] of the pool over 16 columns of the
 // subset's window, thread r = sample r of the block; 16 bytes of each plane per
@@ -994,6 +996,12 @@ int64_t sweep_gather_ctas(int64_t n, int64_t n_cols) {
   return (n + kTB - 1) / kTB * ((n_cols + kSwGatherCols - 1) / kSwGatherCols);
 }
 int sweep_gather_cols() { return kSwGatherCols; }
+
+// (ungraphed: a serving panel's words)
+cudaError_t launch_sweep_words(const SweepPool& pool, int num_sms, cudaStream_t st) {
+  panel_words_kernel<<<8 * num_sms, 256, 0, st>>>(pool);
+  return cudaGetLastError();
+}
 
 // Regrouping costs about 0.12 ps per genotype of the pool's rows in use and
 // saves 0.8 ps per gathered genotype.
