@@ -61,7 +61,7 @@ constexpr size_t kSwSmem = (size_t)kSwStages * kSwStageBytes + kSwEpiWarps * kSw
 static_assert(kSwSmem <= 227 * 1024, "ring exceeds shared memory");
 constexpr int kSwTileCols = 384;
 constexpr size_t kSwHalfTile = (size_t)kSwTileCols * kTB;  // values of one product of one CTA's 128 x 384 tile
-constexpr int kSwEpiBar = 1, kSwBar = 2;  // hardware barriers: epilogue warps; ring slots 0 .. kSwStages - 1
+constexpr int kSwEpiBar = 1;  // hardware barrier of the epilogue warps
 
 // kind::mxf4, E2M1 x E2M1 -> F32, UE8M0 scale factors, K = 96, M = 256.
 template <int N>
@@ -298,13 +298,12 @@ struct SweepArgs {
   SweepSync sync;
 };
 
-// Warps: 0 and 3 copies of A and of B, 1 MMAs (even CTA), 2 the MMA warp's waits
-// (even CTA), 4..11 epilogue.  Roles and barriers as in ibs_tc.cu's two-SM kernel: both CTAs'
-// copies complete on the even CTA's `full`; its MMA warp never waits on memory
-// itself (warp 2 does, and releases it once per stage through a hardware
-// barrier) and commits each stage to both CTAs' `empty` and each finished
-// product to both CTAs' `tfull`; the epilogue warps of both arrive on the even
-// CTA's `tempty` once the product is read.  Every wait is bounded.
+// Warps: 0 and 3 copies of A and of B, 1 and 2 MMAs (even CTA), 4..11 epilogue.
+// Roles and barriers as in ibs_tc.cu's two-SM kernel: both CTAs' copies complete
+// on the even CTA's `full`; its MMA warps commit each stage to both CTAs' `empty`
+// and each finished product to both CTAs' `tfull`; the epilogue warps of both
+// arrive on the even CTA's `tempty` once the product is read.  Every wait is
+// bounded.
 //
 // An item is a tile and a range [q0, q1) of the 4 * stages ring stages of its
 // sweeps.  A whole tile (slot < 0) keeps its products in the CTA's scratch and
@@ -320,7 +319,6 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kSwThreads, 1)
   __shared__ uint32_t tmem_slot;
   __shared__ uint32_t issued[2];  // ring stages this CTA's copy warps issued
   __shared__ int abort_flag;
-  __shared__ int s_dead;  // the waiter has stopped: the MMA warp does too
   __shared__ int s_ok[2];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const uint32_t rank = cluster_rank();
@@ -331,14 +329,13 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kSwThreads, 1)
   if (threadIdx.x == 0) {
     for (int s = 0; s < kSwStages; ++s) {
       mbar_init(&full[s], 1);  // the even CTA's: both CTAs' copies complete on it
-      mbar_init(&empty[s], 1);
+      mbar_init(&empty[s], 2);  // both MMA warps' commits
     }
-    mbar_init(&tfull, 1);
+    mbar_init(&tfull, 2);
     mbar_init(&tempty, 2 * kSwEpiWarps);
-    mbar_init(&drain, 1);
+    mbar_init(&drain, 2);
     mbar_fence_init();
     abort_flag = 0;
-    s_dead = 0;
   }
   if (warp == 0) {
     asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_addr(&tmem_slot)),
@@ -425,101 +422,74 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kSwThreads, 1)
       issued[is_b ? 1 : 0] = g;
     }
     __syncwarp();
-  } else if (warp == 1 && rank == 0) {
-    // The tensor core queues only a few MMAs, so what lies between one stage's
-    // last MMA and the next one's first is kept short.
-    uint32_t s = 0;
-    const uint32_t sf = tmem + kSfCol, ring0 = smem_addr(ring);
-    bool dead = false;
-    // the stages [q, end) of one product, kN columns per MMA, kM MMAs per K step
-    auto product = [&](auto width, int stages) {
-      constexpr int w = decltype(width)::value;
-      constexpr int kN = w == 3 ? 192 : 128 * w;
-      uint32_t acc = 0;  // the first K step overwrites
-      for (int k = 0; k < stages; ++k) {
-        ring_acquire(kSwBar + s);
-        if (*(volatile int*)&s_dead != 0) {
-          dead = true;
-          return;
-        }
-        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-        if (lane == 0) {
+  } else if ((warp == 1 || warp == 2) && rank == 0) {
+    // Two MMA warps, each with its own half of the accumulator columns.  The
+    // tensor core queues hardly more than the MMA it runs, so whatever a warp
+    // does between two stages (commit, the next stage's wait) leaves it idle
+    // unless another warp's MMAs follow: with one MMA warp, released through a
+    // hardware barrier by a warp that waits on memory, a stage took 790 cycles
+    // for 576 of MMAs (20,000 samples x 500,000 markers: 81.4 ms against 76.9;
+    // 4,096 x 100,000: 1,074 us against 1,033).
+    if (lane == 0) {
+      uint32_t s = 0, ph = 0, p = 0;  // ring slot and its parity, products
+      const uint32_t half = warp - 1, sf = tmem + kSfCol, ring0 = smem_addr(ring);
+      bool ok = true;
+      // `stages` stages of one product; W > 1: N = 64 W columns from column
+      // 64 W half on; W = 1 has no halves, the first warp takes it all
+      auto product = [&](auto width, int stages) {
+        constexpr int w = decltype(width)::value;
+        constexpr int kN = w == 3 ? 192 : 128;
+        uint32_t acc = 0;  // the first K step overwrites
+        for (int k = 0; k < stages; ++k) {
+          if (!ring_wait(&full[s], ph, wait_ns, &abort_flag)) {
+            ok = false;
+            return;
+          }
+          asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
           const uint32_t st0 = ring0 + s * kSwStageBytes;
-          const uint64_t a = sweep_desc(st0, 2048), b = sweep_desc(st0 + kSwABytes, 1024 * w);
+          const uint64_t a = sweep_desc(st0, 2048), b = sweep_desc(st0 + kSwABytes + half * (kN / 2 * 16), 1024 * w);
+          if (w > 1 || half == 0) {
 #pragma unroll
-          for (int t = 0; t < kSwCols / 3; ++t) {
-            umma_sweep<kN>(tmem, a + t * (3 * 2048 / 16), b + t * (3 * 1024 * w / 16), acc, sf);
-            if constexpr (w == 3)
-              umma_sweep<kN>(tmem + 192, a + t * (3 * 2048 / 16), b + t * (3 * 1024 * w / 16) + 96 * 16 / 16, acc, sf);
-            acc = 1;
+            for (int t = 0; t < kSwCols / 3; ++t) {
+              umma_sweep<kN>(tmem + kN * half, a + t * (3 * 2048 / 16), b + t * (3 * 1024 * w / 16), acc, sf);
+              acc = 1;
+            }
           }
           umma_commit_both(&empty[s]);
+          if (++s == kSwStages) {
+            s = 0;
+            ph ^= 1u;
+          }
         }
-        acc = 1;
-        s = s + 1 == kSwStages ? 0 : s + 1;
+        umma_commit_both(&tfull);
+      };
+      for (int e = it0; e < it1 && ok; ++e) {
+        const SweepItem it = args.items[e];
+        const int S = work.stages(it.subset);
+        for (int q = it.q0; q < it.q1 && ok; ++p) {
+          const int end = product_end(S, q, it.q1);
+          if (p > 0) ok = mbar_wait_cluster_bounded(&tempty, (p - 1) & 1u, wait_ns);
+          if (!ok) break;
+          if (it.w == 3)
+            product(std::integral_constant<int, 3>{}, end - q);
+          else if (it.w == 2)
+            product(std::integral_constant<int, 2>{}, end - q);
+          else
+            product(std::integral_constant<int, 1>{}, end - q);
+          q = end;
+        }
       }
-      if (lane == 0) umma_commit_both(&tfull);
-    };
-    for (int e = it0; e < it1 && !dead; ++e) {
-      const SweepItem it = args.items[e];
-      const int S = work.stages(it.subset);
-      for (int q = it.q0; q < it.q1 && !dead;) {
-        const int end = product_end(S, q, it.q1);
-        if (it.w == 3)
-          product(std::integral_constant<int, 3>{}, end - q);
-        else if (it.w == 2)
-          product(std::integral_constant<int, 2>{}, end - q);
-        else
-          product(std::integral_constant<int, 1>{}, end - q);
-        q = end;
+      if (!ok && *(volatile int*)&abort_flag == 0) {
+        // nothing more is issued: the other roles of both CTAs stop at this
+        // flag or come to the end of their own bounds
+        atomicExch(status, kDevTimeout);
+        atomicExch(&abort_flag, 1);
       }
+      umma_commit_local2(&drain);
     }
-    __syncwarp();
-    if (lane == 0) umma_commit_local2(&drain);
     __syncwarp();
     const bool drained = mbar_wait_bounded(&drain, 0);
     if (lane == 0 && !drained) atomicExch(status, kDevTimeout);
-  } else if (warp == 2 && rank == 0) {
-    // After a failed wait or another role's abort the waiter and the MMA warp
-    // stop together: nothing is issued or released any more, and the copy and
-    // epilogue warps of both CTAs come to the end of their own bounds.
-    uint32_t s = 0, ph = 0, p = 0;  // ring slot and its parity, products
-    bool dead = false, wrapped = false;
-    for (int e = it0; e < it1 && !dead; ++e) {
-      const SweepItem it = args.items[e];
-      const int S = work.stages(it.subset);
-      for (int q = it.q0; q < it.q1 && !dead; ++p) {
-        const int end = product_end(S, q, it.q1);
-        bool ok = lane != 0 || p == 0 || mbar_wait_cluster_bounded(&tempty, (p - 1) & 1u, wait_ns);
-        for (; q < end; ++q) {
-          // every lane of the warp goes on, or none
-          if (lane == 0 && ok) ok = ring_wait(&full[s], ph, wait_ns, &abort_flag);
-          if (__any_sync(0xffffffffu, !ok)) {
-            dead = true;
-            break;
-          }
-          asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-          ring_release(kSwBar + s);
-          s = s + 1 == kSwStages ? 0 : s + 1;
-          ph ^= s == 0 ? 1u : 0u;
-          wrapped |= s == 0;
-        }
-      }
-    }
-    if (dead) {
-      if (lane == 0) {
-        if (*(volatile int*)&abort_flag == 0) {
-          atomicExch(status, kDevTimeout);
-          atomicExch(&abort_flag, 1);
-        }
-        *(volatile int*)&s_dead = 1;
-        // the slot's previous release has been taken once its stage is
-        // committed: two arrivals before the MMA warp's would pair up
-        if (wrapped) mbar_wait_bounded(&empty[s], ph ^ 1u);
-      }
-      __syncwarp();
-      ring_release(kSwBar + s);  // the MMA warp finds s_dead
-    }
   } else if (warp >= 4) {
     const int quarter = warp & 3, part = (warp - 4) >> 2, row = quarter * 32 + lane;
     const uint32_t lane_base = tmem + ((uint32_t)(quarter * 32) << 16);
@@ -570,9 +540,10 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kSwThreads, 1)
           for (int u = 0; u < 3; ++u) {
             const int gr = g0 + 2 * u;
             if (gr < ng) {
-              // w = 3: two MMAs of 192 columns, each 96 of the even CTA's B
-              // rows and 96 of the odd CTA's
-              const int c0 = it.w == 3 ? (gr % 6) / 3 * 192 + gr / 6 * 96 + gr % 3 * 32 : gr * 32;
+              // w = 2 and 3: two MMAs of 64 w columns, each half of the even
+              // CTA's B rows, then half of the odd CTA's
+              const int r = gr % (2 * it.w), odd = r / it.w;
+              const int c0 = it.w == 1 ? gr * 32 : odd * 64 * it.w + (gr / (2 * it.w) * it.w + r % it.w) * 32;
 #pragma unroll
               for (int j = 0; j < 32; ++j) dst[(size_t)(c0 + j) * kTB + row] = __uint_as_float(v[u][j]);
             }
