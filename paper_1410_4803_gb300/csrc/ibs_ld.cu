@@ -27,15 +27,15 @@
 // reciprocal square root and the products are rounded, in float-float
 // arithmetic on the FP32 pipe (see ld_r_value).
 //
-// One persistent CTA per SM, 12 warps: the copy warp claims (A block, B
+// One persistent CTA per SM, 20 warps: the copy warp claims (A block, B
 // half-block) items of the band |b - a| <= window from a counter and streams
-// each item's sample chunks through a ring of 3 stages x 4 chunks (one copy of
+// each item's sample chunks through a ring of 3 stages x 3 chunks (one copy of
 // the A block's 3 planes x 4 KiB per chunk, one of the B half-block's 3 planes
-// x 2 KiB per chunk, from a second copy of the planes laid out for it); the
-// MMA warp issues 6 MMAs (M = 128, N = 64, K = 64) per chunk into six FP32
-// accumulators (tensor-memory columns 0, 64, ..., 320; unit scale factors at
-// 384..511); warps 4..11 read the accumulators back (two warps per lane
-// quarter, 32 columns each) and store r.  Every wait is bounded (2 s of
+// x 2 KiB per chunk, from a second copy of the planes laid out for it); two
+// MMA warps issue 3 MMAs (M = 128, N = 192, 128 and 64, K = 64) per chunk into
+// six FP32 accumulators (64 tensor-memory columns each; unit scale factors at
+// 384..511); warps 4..19 read the accumulators back (four warps per lane
+// quarter, 16 columns each) and store r.  Every wait is bounded (2 s of
 // %globaltimer), as in the IBS kernels.
 #include <algorithm>
 #include <vector>
@@ -51,19 +51,25 @@ constexpr int kLdChunkBytes = kLdPlanes * kTileBytes;  // 12 KiB per (marker blo
 constexpr int kLdHalfBytes = kTileBytes / 2;         // 64 rows of a plane tile
 constexpr int kLdHalfChunkBytes = kLdPlanes * kLdHalfBytes;  // 6 KiB per (half-block, sample chunk)
 // A ring stage holds kLdPer chunks of the A block and of the B half-block, one
-// bulk copy each (the copy engine spends a fixed time per copy).
-constexpr int kLdPer = 4;
-constexpr int kLdStageBytes = kLdPer * (kLdChunkBytes + kLdHalfChunkBytes);  // 72 KiB
+// bulk copy each (the copy engine spends a fixed time per copy).  Beside the
+// ring, each epilogue warp has a piece of 32 rows x 8 columns of r and N to
+// transpose.
+constexpr int kLdPer = 3;
+constexpr int kLdStageBytes = kLdPer * (kLdChunkBytes + kLdHalfChunkBytes);  // 54 KiB
 constexpr int kLdStages = 3;
-constexpr size_t kLdSmem = (size_t)kLdStages * kLdStageBytes + 1024;
+constexpr int kLdEpiWarps = 16;
+constexpr int kLdTransBytes = 32 * 9 * 12;
+constexpr size_t kLdSmem = (size_t)kLdStages * kLdStageBytes + kLdEpiWarps * kLdTransBytes + 1024;
+static_assert(kLdSmem <= 227 * 1024, "ring exceeds shared memory");
 constexpr int kLdN = 64;                             // B rows (markers) per item
+// Accumulator columns.  A chunk's X, V and H rows of B are contiguous, so one MMA
+// multiplies a plane of A by two or three of them (N = 128 or 192): 3 MMAs per
+// chunk; 6 of N = 64, one per sum, took 1.79 ms a call against 1.74
+// (4,096 samples x 100,000 markers, window 1,000).
+constexpr uint32_t kLdSy = 0, kLdCnt = 64, kLdSyy = 128, kLdSxy = 192, kLdSx = 256, kLdSxx = 320;
 constexpr int kLdQueue = 8;
-// warps 0 (copies), 1 (MMAs), 2 (the MMA warp's waits), 3 idle, 4..11 epilogue: two warps per TMEM lane
-// quarter, each reading 32 of the item's 64 accumulator columns
-constexpr int kLdEpiWarps = 8;
-// Hardware barrier between the waiter warp (2) and the MMA warp (1); barrier
-// 0 is __syncthreads.
-constexpr int kLdBar = 1;
+// warps 0 (copies), 1 and 2 (MMAs), 3 idle, 4..19 epilogue: four warps per TMEM
+// lane quarter, each reading 16 of the item's 64 accumulator columns
 constexpr int kLdThreads = (4 + kLdEpiWarps) * 32;
 
 // Even bits of a 64-bit word packed into 32 bits (bit 2i -> bit i).
@@ -164,20 +170,67 @@ __device__ __forceinline__ FF ff_mul(FF a, FF b) {
   return {s, __fsub_rn(e, __fsub_rn(s, p))};
 }
 
+// The double hi + lo (2^-70 < |hi| < 2^70, |lo| at most half an ulp of hi),
+// rounded to 53 bits: lo is scaled to units of the last bit (half as large where
+// lo takes a power of two below itself) and added to hi's bit pattern.  Two
+// conversions of FP32 to FP64 and an FP64 addition would hold the FP64 pipe for
+// 12,000 cycles per 128 x 64 pairs, as long as their MMAs.
+__device__ __forceinline__ double ff_to_double(FF r) {
+  const int hb = __float_as_int(r.hi), lb = __float_as_int(r.lo), e = (hb >> 23) & 0xFF;
+  const int below = (hb & 0x7FFFFF) == 0 && (hb ^ lb) < 0;
+  const int k = __float2int_rn(__fmul_rn(r.lo, __int_as_float((306 - e + below) << 23)));
+  const long long mag =
+      ((long long)(e - 127 + 1023) << 52) + ((long long)(hb & 0x7FFFFF) << 29) + (hb < 0 ? -k : k);
+  return __longlong_as_double(mag | ((long long)hb & (long long)0x8000000000000000ull));
+}
+
+// r = num / sqrt(va vb) from exact float-float operands, va and vb positive.
+__device__ __forceinline__ double ld_r_quotient(FF num, FF va, FF vb) {
+  if (num.hi == 0.0f) return 0.0;
+  const FF P = ff_mul(va, vb);
+  const float y0 = rsqrtf(P.hi);
+  const float q = __fmul_rn(y0, y0);
+  const FF w = ff_mul(P, FF{q, __fmaf_rn(y0, y0, -q)});  // P y0^2, near 1
+  const float t = __fsub_rn(__fsub_rn(1.0f, w.hi), w.lo);  // 1 - P y0^2 (the first difference is exact)
+  const FF y = ff_two_sum(y0, __fmul_rn(__fmul_rn(y0, t), 0.5f));  // one Newton step
+  return ff_to_double(ff_mul(num, y));
+}
+
+// x (|x| < 2^30) as an exact float-float, without conversions (they issue at a
+// quarter of the rate): x = h 2^15 + l, both made floats by their bit patterns.
+__device__ __forceinline__ FF ff_from_i30(int x) {
+  const float h = __fsub_rn(__int_as_float(0x4B400000 + (x >> 15)), 12582912.0f);
+  const float l = __fsub_rn(__int_as_float(0x4B000000 | (x & 0x7FFF)), 8388608.0f);
+  const float s = __fmaf_rn(h, 32768.0f, l);
+  return {s, __fadd_rn(__fmaf_rn(h, 32768.0f, -s), l)};
+}
+
+// The six sums of a pair, each below 2^15 in magnitude (fewer than 2^15
+// samples), in three words.
+struct LdSums {
+  uint32_t a, b, c;
+};
+__device__ __forceinline__ uint32_t ld_pack(uint32_t lo, uint32_t hi) {
+  // adding 1.5 * 2^23 leaves the integer in the low bits of the pattern
+  return __byte_perm(__float_as_uint(__fadd_rn(__uint_as_float(lo), 12582912.0f)),
+                     __float_as_uint(__fadd_rn(__uint_as_float(hi), 12582912.0f)), 0x5410);
+}
+__device__ __forceinline__ double ld_r_small(const LdSums& p, int sign) {
+  const int N = (int)(p.a & 0xFFFF), sxx = (int)(p.a >> 16), syy = (int)(p.b & 0xFFFF);
+  const int sx = (int)p.b >> 16, sy = (int)(p.c << 16) >> 16, sxy = (int)p.c >> 16;
+  const int va = N * sxx - sx * sx, vb = N * syy - sy * sy;  // 0 <= . < 2^30
+  if (va == 0 || vb == 0) return __longlong_as_double(0x7ff8000000000000LL);
+  const int num = N * sxy - sx * sy;
+  return ld_r_quotient(ff_from_i30(sign < 0 ? -num : num), ff_from_i30(va), ff_from_i30(vb));
+}
+
 __device__ __forceinline__ double ld_r_value(int32_t N, int32_t sx, int32_t sy, int32_t sxx, int32_t syy,
                                              int32_t sxy, int sign) {
   const long long n = N;
   const long long va = n * sxx - (long long)sx * sx, vb = n * syy - (long long)sy * sy;
   if (N == 0 || va == 0 || vb == 0) return __longlong_as_double(0x7ff8000000000000LL);
   const long long num = n * sxy - (long long)sx * sy;
-  const FF P = ff_mul(ff_from_i48(va), ff_from_i48(vb));
-  const float y0 = rsqrtf(P.hi);
-  const float q = __fmul_rn(y0, y0);
-  const FF w = ff_mul(P, FF{q, __fmaf_rn(y0, y0, -q)});  // P y0^2, near 1
-  const float t = __fsub_rn(__fsub_rn(1.0f, w.hi), w.lo);  // 1 - P y0^2 (the first difference is exact)
-  const FF y = ff_two_sum(y0, __fmul_rn(__fmul_rn(y0, t), 0.5f));  // one Newton step
-  const FF r = ff_mul(ff_from_i48(sign * num), y);
-  return (double)r.hi + (double)r.lo;
+  return ld_r_quotient(ff_from_i48(sign * num), ff_from_i48(va), ff_from_i48(vb));
 }
 
 struct LdArgs {
@@ -193,13 +246,27 @@ struct LdArgs {
   int* status;
 };
 
+__device__ __forceinline__ void tmem_ld8(uint32_t taddr, uint32_t (&r)[8]) {
+  asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
+               : "r"(taddr));
+}
+
+// kSmall: fewer than 2^15 samples.  The epilogue then packs the six sums of its
+// 32 rows x 16 columns into registers and hands tensor memory back before it
+// computes, so that the next item's MMAs run beside the arithmetic; with more
+// samples the accumulators are held while the first half is computed.  The
+// arithmetic is integer and FP32 only, and the stores go through shared memory.
+// With FP64 arithmetic on held accumulators and one lane per marker row the
+// call took 2.33 ms (4,096 samples x 100,000 markers, window 1,000); 1.74 with
+// 8 epilogue warps, 1.67 with 16.
+template <bool kSmall>
 __global__ void __launch_bounds__(kLdThreads, 1) tc_ld_kernel(const LdArgs args) {
   extern __shared__ __align__(1024) uint8_t smem_raw[];
   uint8_t* ring = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   __shared__ __align__(8) uint64_t full[kLdStages], empty[kLdStages], tfull, tempty, drain;
   __shared__ __align__(8) uint64_t qfull[kLdQueue], qempty[kLdQueue];
   __shared__ int64_t q_item[kLdQueue];
-  __shared__ int64_t s_item[2];  // the waiter's hand-over of items to the MMA warp
   __shared__ uint32_t tmem_slot;
   __shared__ int abort_flag;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -207,15 +274,15 @@ __global__ void __launch_bounds__(kLdThreads, 1) tc_ld_kernel(const LdArgs args)
   if (threadIdx.x == 0) {
     for (int s = 0; s < kLdStages; ++s) {
       mbar_init(&full[s], 1);
-      mbar_init(&empty[s], 1);
+      mbar_init(&empty[s], 2);  // both MMA warps' commits
     }
     for (int s = 0; s < kLdQueue; ++s) {
       mbar_init(&qfull[s], 1);
-      mbar_init(&qempty[s], 1 + kLdEpiWarps);  // the waiter warp and the epilogue warps
+      mbar_init(&qempty[s], 2 + kLdEpiWarps);  // the MMA warps and the epilogue warps
     }
-    mbar_init(&tfull, 1);
+    mbar_init(&tfull, 2);
     mbar_init(&tempty, kLdEpiWarps);
-    mbar_init(&drain, 1);
+    mbar_init(&drain, 2);
     mbar_fence_init();
     abort_flag = 0;
   }
@@ -234,198 +301,198 @@ __global__ void __launch_bounds__(kLdThreads, 1) tc_ld_kernel(const LdArgs args)
   __syncthreads();
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
 
-  auto fail = [&](bool cond) {
-    if (lane == 0 && cond) {
+  auto fail = [&] {  // one thread
+    if (*(volatile int*)&abort_flag == 0) {
       atomicExch(status, kDevTimeout);
       atomicExch(&abort_flag, 1);
     }
   };
-  auto aborted = [&]() { return __any_sync(0xffffffffu, *(volatile int*)&abort_flag != 0); };
+  // one thread's next item: false after a failed wait
   auto queue_get = [&](uint32_t e, int64_t& it) {
     const int qs = (int)(e % kLdQueue);
-    const bool ok = mbar_wait_bounded(&qfull[qs], (e / kLdQueue) & 1u);
-    if (__any_sync(0xffffffffu, !ok)) return false;
+    if (!ring_wait(&qfull[qs], (e / kLdQueue) & 1u, kWaitLimitNs, &abort_flag)) return false;
     it = *(volatile int64_t*)&q_item[qs];
-    __syncwarp();
-    if (lane == 0) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_addr(&qempty[qs])) : "memory");
+    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_addr(&qempty[qs])) : "memory");
     return true;
   };
-  const int64_t nk = args.n_chunks;
+  const int64_t nk = args.n_chunks;  // whole stages
 
   if (warp == 0) {
-    uint32_t g = 0;
-    for (uint32_t e = 0;; ++e) {
-      int64_t it = 0;
-      if (lane == 0) it = atomicAdd(args.counter, 1);
-      it = __shfl_sync(0xffffffffu, it, 0);
-      const bool last = it >= args.n_items;
-      const int qs = (int)(e % kLdQueue);
-      const bool qok = e < (uint32_t)kLdQueue || mbar_wait_bounded(&qempty[qs], ((e / kLdQueue) - 1) & 1u);
-      if (__any_sync(0xffffffffu, !qok)) {
-        fail(true);
-        break;
-      }
-      if (aborted()) break;
-      if (lane == 0) {
-        q_item[qs] = last ? -1 : it;
+    if (lane == 0) {
+      uint32_t g = 0, s = 0, ph = 1;  // stages issued, ring slot, parity of the slot's previous release
+      bool ok = true;
+      for (uint32_t e = 0; ok; ++e) {
+        int64_t it = atomicAdd(args.counter, 1);
+        if (it >= args.n_items) it = -1;
+        const int qs = (int)(e % kLdQueue);
+        if (e >= (uint32_t)kLdQueue && !ring_wait(&qempty[qs], ((e / kLdQueue) - 1) & 1u, kWaitLimitNs, &abort_flag)) {
+          ok = false;
+          break;
+        }
+        q_item[qs] = it;
         asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_addr(&qfull[qs])) : "memory");
-      }
-      __syncwarp();
-      if (last) break;
-      const int2 item = args.items[it];
-      const uint8_t* ablk = args.planes + (size_t)item.x * nk * kLdChunkBytes;
-      const uint8_t* bblk = args.planes_b + (size_t)item.y * nk * kLdHalfChunkBytes;
-      bool stop = false;
-      for (int64_t k = 0; k < nk; k += kLdPer, ++g) {
-        const int s = (int)(g % kLdStages);
-        const bool ok = g < (uint32_t)kLdStages || mbar_wait_bounded(&empty[s], ((g / kLdStages) - 1) & 1u);
-        if (__any_sync(0xffffffffu, !ok)) {
-          fail(true);
-          stop = true;
-          break;
-        }
-        if (aborted()) {
-          stop = true;
-          break;
-        }
-        if (lane == 0) {
+        if (it < 0) break;
+        const int2 item = args.items[it];
+        const uint8_t* a = args.planes + (size_t)item.x * nk * kLdChunkBytes;
+        const uint8_t* b = args.planes_b + (size_t)item.y * nk * kLdHalfChunkBytes;
+        for (int64_t k = 0; k < nk; k += kLdPer, a += kLdPer * kLdChunkBytes, b += kLdPer * kLdHalfChunkBytes) {
+          if (g >= (uint32_t)kLdStages && !ring_wait(&empty[s], ph, kWaitLimitNs, &abort_flag)) {
+            ok = false;
+            break;
+          }
           uint8_t* dst = ring + (size_t)s * kLdStageBytes;
           mbar_arrive_expect_tx(&full[s], kLdStageBytes);
-          bulk_g2s(dst, ablk + (size_t)k * kLdChunkBytes, kLdPer * kLdChunkBytes, &full[s]);
-          bulk_g2s(dst + kLdPer * kLdChunkBytes, bblk + (size_t)k * kLdHalfChunkBytes, kLdPer * kLdHalfChunkBytes,
-                   &full[s]);
+          bulk_g2s(dst, a, kLdPer * kLdChunkBytes, &full[s]);
+          bulk_g2s(dst + kLdPer * kLdChunkBytes, b, kLdPer * kLdHalfChunkBytes, &full[s]);
+          ++g;
+          if (++s == kLdStages) {
+            s = 0;
+            ph ^= 1u;
+          }
         }
-        __syncwarp();
       }
-      if (stop) break;
+      if (!ok) fail();
+      // (after a stop: the copies in flight land before the CTA may exit)
+      for (uint32_t j = g > (uint32_t)kLdStages ? g - kLdStages : 0; j < g && !ok; ++j)
+        mbar_wait_bounded(&full[j % kLdStages], (j / kLdStages) & 1u);
     }
-  } else if (warp == 1) {
-    // MMA warp.  It never waits on memory itself: a thread with MMAs in flight
-    // that polls a barrier or loads from memory stalls until they complete,
-    // which would drain the tensor pipe at every ring stage.  Warp 2 takes the
-    // items from the queue and does every wait; it hands each item over
-    // through s_item and releases this warp once per stage through hardware
-    // barrier kLdBar (both warps execute bar.sync once per hand-over and once
-    // per stage, in the same order; every item covers all chunks).
-    uint32_t g = 0;
-    const uint32_t sf = tmem + kSfCol;
-    for (uint32_t e = 0;; ++e) {
-      asm volatile("bar.sync %0, 64;" ::"n"(kLdBar) : "memory");
-      const int64_t it = *(volatile int64_t*)&s_item[e & 1u];
-      if (it < 0) break;
-      for (int64_t k0 = 0; k0 < nk; k0 += kLdPer, ++g) {
-        asm volatile("bar.sync %0, 64;" ::"n"(kLdBar) : "memory");
-        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-        const int s = (int)(g % kLdStages);
-        if (lane == 0) {
-          const uint32_t st0 = smem_addr(ring + (size_t)s * kLdStageBytes);
+    __syncwarp();
+  } else if (warp == 1 || warp == 2) {
+    // Two MMA warps with accumulators and products of their own, of the same
+    // cost: V_a times the three planes of B, and X_a times two and H_a times one.
+    // One warp's MMAs run while the other commits a stage and waits for the
+    // next (the tensor core queues hardly more than the MMA it runs).  Each waits
+    // (bounded), at an item's start, until the epilogue has read the previous
+    // item's accumulators, and for each stage until its operands have landed;
+    // after a failed wait or another role's abort nothing more is issued.
+    if (lane == 0) {
+      uint32_t s = 0, ph = 0;
+      const uint32_t sf = tmem + kSfCol, ring0 = smem_addr(ring);
+      bool ok = true;
+      for (uint32_t e = 0; ok; ++e) {
+        int64_t it = -1;
+        ok = queue_get(e, it);
+        if (!ok || it < 0) break;
+        if (e > 0) ok = mbar_wait_bounded(&tempty, (e - 1) & 1u);
+        for (int64_t k0 = 0; k0 < nk && ok; k0 += kLdPer) {
+          if (!ring_wait(&full[s], ph, kWaitLimitNs, &abort_flag)) {
+            ok = false;
+            break;
+          }
+          asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+          const uint32_t st0 = ring0 + s * kLdStageBytes;
 #pragma unroll
           for (int c = 0; c < kLdPer; ++c) {
+            // X, V and H of a chunk, 4 KiB each of A and 2 KiB each of B
             const uint32_t a0 = st0 + c * kLdChunkBytes, b0 = st0 + kLdPer * kLdChunkBytes + c * kLdHalfChunkBytes;
-            const uint64_t aX = umma_desc(a0), aV = umma_desc(a0 + kTileBytes), aH = umma_desc(a0 + 2 * kTileBytes);
-            const uint64_t bX = umma_desc(b0), bV = umma_desc(b0 + kLdHalfBytes),
-                           bH = umma_desc(b0 + 2 * kLdHalfBytes);
             const uint32_t acc = k0 + c > 0 ? 1u : 0u;
-            umma<kTcFp4, kLdN>(tmem + 0 * kLdN, aV, bV, acc, sf);  // N
-            umma<kTcFp4, kLdN>(tmem + 1 * kLdN, aX, bV, acc, sf);  // Sx
-            umma<kTcFp4, kLdN>(tmem + 2 * kLdN, aV, bX, acc, sf);  // Sy
-            umma<kTcFp4, kLdN>(tmem + 3 * kLdN, aH, bV, acc, sf);  // Sxx
-            umma<kTcFp4, kLdN>(tmem + 4 * kLdN, aV, bH, acc, sf);  // Syy
-            umma<kTcFp4, kLdN>(tmem + 5 * kLdN, aX, bX, acc, sf);  // Sxy
+            if (warp == 1) {
+              umma<kTcFp4, 3 * kLdN>(tmem + kLdSy, umma_desc(a0 + kTileBytes), umma_desc(b0), acc, sf);
+            } else {
+              umma<kTcFp4, 2 * kLdN>(tmem + kLdSxy, umma_desc(a0), umma_desc(b0), acc, sf);
+              umma<kTcFp4, kLdN>(tmem + kLdSxx, umma_desc(a0 + 2 * kTileBytes), umma_desc(b0 + kLdHalfBytes), acc, sf);
+            }
           }
           umma_commit(&empty[s]);
+          if (++s == kLdStages) {
+            s = 0;
+            ph ^= 1u;
+          }
         }
-        __syncwarp();
+        umma_commit(&tfull);
       }
-      if (lane == 0) umma_commit(&tfull);
-      __syncwarp();
+      if (!ok) fail();
+      umma_commit(&drain);
     }
-    if (lane == 0) umma_commit(&drain);
     __syncwarp();
     const bool drained = mbar_wait_bounded(&drain, 0);
     if (lane == 0 && !drained) atomicExch(status, kDevTimeout);
-  } else if (warp == 2) {
-    // Waiter: for each item from the queue, hand it over; before its first
-    // stage wait (bounded) until the epilogue has read the previous item's
-    // accumulators, and before each stage until its operands have landed;
-    // then release the MMA warp.  After a failed wait or another role's abort
-    // it stops waiting but keeps releasing the current item's stages (the MMA
-    // warp runs them out on stale operands; the call reports IBS_ETIMEOUT),
-    // then hands over the end (-1).
-    uint32_t g = 0;
-    bool dead = false;
+  } else if (warp >= 4) {
+    const int quarter = warp & 3, colq = (warp - 4) >> 2;
+    const uint32_t lane_base = tmem + ((uint32_t)(quarter * 32) << 16) + 16 * colq;
+    uint8_t* trans = ring + (size_t)kLdStages * kLdStageBytes + (size_t)(warp - 4) * kLdTransBytes;
+    double* sr = reinterpret_cast<double*>(trans);
+    int32_t* sn = reinterpret_cast<int32_t*>(trans + 32 * 9 * 8);
     for (uint32_t e = 0;; ++e) {
       int64_t it = -1;
-      if (!dead && !queue_get(e, it)) {
-        fail(true);
-        dead = true;
-      }
-      if (dead) it = -1;
-      if (lane == 0) s_item[e & 1u] = it;
-      __syncwarp();
-      asm volatile("bar.sync %0, 64;" ::"n"(kLdBar) : "memory");
-      if (it < 0) break;
-      for (int64_t k0 = 0; k0 < nk; k0 += kLdPer, ++g) {
-        if (!dead) {
-          bool ok = k0 > 0 || e == 0 || mbar_wait_bounded(&tempty, (e - 1) & 1u);
-          if (ok) ok = mbar_wait_bounded(&full[(int)(g % kLdStages)], (g / kLdStages) & 1u);
-          if (__any_sync(0xffffffffu, !ok)) {
-            fail(true);
-            dead = true;
-          } else if (aborted()) {
-            dead = true;
-          }
-        }
-        asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-        asm volatile("bar.sync %0, 64;" ::"n"(kLdBar) : "memory");
-      }
-    }
-  } else if (warp >= 4) {
-    const int quarter = warp & 3, colhalf = (warp - 4) >> 2;
-    const int row = quarter * 32 + lane;
-    const uint32_t lane_base = tmem + ((uint32_t)(quarter * 32) << 16);
-    for (uint32_t e = 0;; ++e) {
-      int64_t it;
-      if (!queue_get(e, it)) {
-        fail(true);
+      bool ok = true;
+      if (lane == 0) ok = queue_get(e, it);
+      it = __shfl_sync(0xffffffffu, it, 0);
+      if (ok && it >= 0) ok = mbar_wait_bounded(&tfull, e & 1u) && *(volatile int*)&abort_flag == 0;
+      if (__any_sync(0xffffffffu, !ok)) {
+        if (lane == 0) fail();
         break;
       }
       if (it < 0) break;
-      const bool ok = mbar_wait_bounded(&tfull, e & 1u);
-      if (__any_sync(0xffffffffu, !ok) || aborted()) {
-        fail(true);
-        break;
-      }
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
       const int2 item = args.items[it];
-      const int64_t a = (int64_t)item.x * kTB + row;
-      const int sa = a < args.m ? (args.diff[a] >= 0 ? 1 : -1) : 1;
-#pragma unroll 1
-      for (int cg = 2 * colhalf; cg < 2 * colhalf + 2; ++cg) {
-        uint32_t v[6][16];
+      const int64_t a0 = (int64_t)item.x * kTB + quarter * 32, b0 = (int64_t)item.y * kLdN + 16 * colq;
+      // markers whose major allele is A2: this thread's row, the warp's 16 columns
+      const bool minus = a0 + lane < args.m && args.diff[a0 + lane] < 0;
+      const uint32_t bminus = __ballot_sync(0xffffffffu, lane < 16 && b0 + lane < args.m && args.diff[b0 + lane] < 0);
+      auto hand_back = [&] {
+        asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+        __syncwarp();
+        if (lane == 0) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_addr(&tempty)) : "memory");
+      };
+      // Columns u0 .. u0 + 7 of the warp's: r of (row, column u) from value(u), N
+      // from count(u); transposed through shared memory, so that 8 lanes store 8
+      // consecutive pairs of a marker.
+      auto put = [&](int u0, auto&& value, auto&& count) {
+        __syncwarp();
 #pragma unroll
-        for (int q = 0; q < 6; ++q) tmem_ld16(lane_base + q * kLdN + cg * 16, v[q]);
-        asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-        if (cg == 2 * colhalf + 1) {
-          asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-          __syncwarp();
-          if (lane == 0) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_addr(&tempty)) : "memory");
+        for (int u = 0; u < 8; ++u) {
+          sr[lane * 9 + u] = value(u, ((bminus >> (u0 + u)) & 1u) != (minus ? 1u : 0u) ? -1 : 1);
+          sn[lane * 9 + u] = count(u);
         }
-        if (a >= args.m) continue;
+        __syncwarp();
+        const int64_t b = b0 + u0 + (lane & 7), a1 = a0 + (lane >> 3);
+        int64_t d = b - a1 - 1, at = a1 * args.window + d;
 #pragma unroll
-        for (int u = 0; u < 16; ++u) {
-          const int64_t b = (int64_t)item.y * kLdN + cg * 16 + u;
-          const int64_t d = b - a - 1;
-          if (d < 0 || d >= args.window || b >= args.m) continue;
-          const int32_t N = __float2int_rn(__uint_as_float(v[0][u]));
-          const int sb = args.diff[b] >= 0 ? 1 : -1;
-          const double r = ld_r_value(N, __float2int_rn(__uint_as_float(v[1][u])),
-                                      __float2int_rn(__uint_as_float(v[2][u])),
-                                      __float2int_rn(__uint_as_float(v[3][u])),
-                                      __float2int_rn(__uint_as_float(v[4][u])),
-                                      __float2int_rn(__uint_as_float(v[5][u])), sa * sb);
-          args.out_r[a * args.window + d] = r;
-          if (args.out_n) args.out_n[a * args.window + d] = N;
+        for (int r = 0; r < 32; r += 4, d -= 4, at += 4 * args.window - 4) {
+          if (d < 0 || d >= args.window || b >= args.m) continue;  // (b > the row's marker: that is below m too)
+          const int from = (r + (lane >> 3)) * 9 + (lane & 7);
+          args.out_r[at] = sr[from];
+          if (args.out_n) args.out_n[at] = sn[from];
+        }
+      };
+      if constexpr (kSmall) {
+        LdSums p[16];
+        uint32_t lo[16], hi[16];
+        auto pair = [&](uint32_t ql, uint32_t qh) {
+          tmem_ld16(lane_base + ql, lo);
+          tmem_ld16(lane_base + qh, hi);
+          asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+        };
+        pair(kLdCnt, kLdSxx);
+#pragma unroll
+        for (int u = 0; u < 16; ++u) p[u].a = ld_pack(lo[u], hi[u]);
+        pair(kLdSyy, kLdSx);
+#pragma unroll
+        for (int u = 0; u < 16; ++u) p[u].b = ld_pack(lo[u], hi[u]);
+        pair(kLdSy, kLdSxy);
+        hand_back();
+#pragma unroll
+        for (int u = 0; u < 16; ++u) p[u].c = ld_pack(lo[u], hi[u]);
+#pragma unroll
+        for (int u0 = 0; u0 < 16; u0 += 8)
+          put(u0, [&](int u, int sign) { return ld_r_small(p[u0 + u], sign); },
+              [&](int u) { return (int)(p[u0 + u].a & 0xFFFF); });
+      } else {
+#pragma unroll 1
+        for (int u0 = 0; u0 < 16; u0 += 8) {
+          constexpr uint32_t col[6] = {kLdCnt, kLdSx, kLdSy, kLdSxx, kLdSyy, kLdSxy};
+          uint32_t v[6][8];
+#pragma unroll
+          for (int q = 0; q < 6; ++q) tmem_ld8(lane_base + col[q] + u0, v[q]);
+          asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+          if (u0 == 8) hand_back();
+          auto sum = [&](int q, int u) { return __float2int_rn(__uint_as_float(v[q][u])); };
+          put(u0,
+              [&](int u, int sign) {
+                return ld_r_value(sum(0, u), sum(1, u), sum(2, u), sum(3, u), sum(4, u), sum(5, u), sign);
+              },
+              [&](int u) { return sum(0, u); });
         }
       }
     }
@@ -484,12 +551,12 @@ cudaError_t launch_ld(const uint8_t* packed, int64_t n, int64_t m, int64_t windo
                                                                       diff);
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
   if ((e = cudaMemsetAsync(counter, 0, sizeof(int), st)) != cudaSuccess) return e;
-  if ((e = cudaFuncSetAttribute(tc_ld_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kLdSmem)) !=
-      cudaSuccess)
+  auto kern = n < (1 << 15) ? tc_ld_kernel<true> : tc_ld_kernel<false>;
+  if ((e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kLdSmem)) != cudaSuccess)
     return e;
   LdArgs args{planes, planes_b, nc, m, window, items, n_items, diff, out_r, out_n, counter, status};
   if (n_items > 0) {
-    tc_ld_kernel<<<(int)std::min<int64_t>(num_sms, n_items), kLdThreads, kLdSmem, st>>>(args);
+    kern<<<(int)std::min<int64_t>(num_sms, n_items), kLdThreads, kLdSmem, st>>>(args);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
   }
   ld_fill_tail_kernel<<<64, 256, 0, st>>>(m, window, out_r, out_n);

@@ -70,6 +70,17 @@ def test_larger_case(ctx):
     _check(ctx, codes, 300)
 
 
+# the largest sample count whose sums the epilogue packs into 16 bits, and the next
+@pytest.mark.parametrize("n", [32_767, 32_768])
+def test_packed_sums_limit(ctx, n):
+    rng = np.random.default_rng(n)
+    codes = random_codes(rng, n, 70, miss=0.01)
+    codes[:, 3] = 0                                             # monomorphic: sums of n
+    codes[:, 4] = np.where(np.arange(n) % 2 == 0, 0, 3)         # variance n^2 / 4 ...
+    codes[:, 5] = np.where(codes[:, 4] == 0, 3, 0)              # ... and r = -1 (before orientation)
+    _check(ctx, codes, 69)
+
+
 def test_repeat_and_rejects(ctx):
     import torch
     from paper_1410_4803_gb300 import ibs
