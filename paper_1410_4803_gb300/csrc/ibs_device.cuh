@@ -137,21 +137,47 @@ constexpr int kLutAndOr = 0xEA;   // (a & b) | c
 constexpr int kLutXor3 = 0x96;    // a ^ b ^ c
 constexpr int kLutMaj = 0xE8;     // majority(a, b, c)
 
-// IBS distance (IBS1 + 2 IBS0) / (2N) in FP64, NaN when N = 0.  FP64
-// division is slow on this part, so the quotient is seeded in FP32 and
-// corrected once in FP64 (a Newton-Raphson step in residual form,
-// q1 = q0 + (a - q0 b) r0 with r0 ~ 1/b): the seed is within ~2^-22 of a/b and
-// r0 within 2^-24 of 1/b, so q1 is within ~2^-46 (about 1.1e-14) relative of
-// the exact quotient, well inside the 1e-12 bound.  Every kernel that writes a
-// distance uses this function, so all paths give identical doubles for
-// identical counts.
+// IBS distance (IBS1 + 2 IBS0) / (2N), NaN when N = 0: the correctly rounded
+// double quotient a / b of two integers, by integer arithmetic.  GB300 issues 2
+// FP64 operations per clock and SM against 64 integer multiplies, and the
+// distance of every pair is needed, so no FP64 operation is used.  With a and
+// b normalised to A, D in [2^30, 2^31), the leading bit of A / D is taken first
+// (r < D is what is left) and 52 more bits follow as two digits of 26:
+//   V ~ 2^61 / D, at most 4 below: an FP32 reciprocal (24 bits) and one Newton
+//   step in 64-bit integers;
+//   digit = floor(r V / 2^35), which is floor(r 2^26 / D) or one less, since
+//   r V / 2^35 is short of r 2^26 / D by less than 4 r / 2^35 < 1/4; the
+//   remainder r 2^26 - digit D < 5/4 D < 2^32 is exact modulo 2^32.
+// The last remainder rounds to nearest; a tie would need D to divide 2^53 times
+// an odd number, impossible for D < 2^31 with a remainder.  N >= 2^30 (b would
+// not fit) takes the FP64 division.
+// Measured with the FP64 form (two conversions, two FMAs; 1e-14 off): a call on
+// 1,501 x 30,011 112 us against 99, 24 batched subsets 2.90 ms against 2.61.
 __device__ __forceinline__ double ibs_dist(int32_t i0, int32_t i1, int32_t n) {
   if (n == 0) return __longlong_as_double(0x7ff8000000000000LL);
-  const long long ai = (long long)i1 + 2 * (long long)i0, bi = 2 * (long long)n;
-  const double a = (double)ai, b = (double)bi;
-  const float r0 = __frcp_rn((float)bi);
-  const double q0 = (double)((float)ai * r0);
-  return fma(fma(-q0, b, a), (double)r0, q0);
+  if (n >= (1 << 30)) return __ddiv_rn((double)((long long)i1 + 2 * (long long)i0), 2.0 * (double)n);
+  const uint32_t a = (uint32_t)i1 + 2u * (uint32_t)i0, b = 2u * (uint32_t)n;
+  if (a == 0) return 0.0;
+  const int sa = __clz((int)a) - 1, sb = __clz((int)b) - 1;
+  const uint32_t A = a << sa, D = b << sb;
+  uint32_t v0 = __float2uint_rz(__fmul_rn(__frcp_rn(__uint2float_rn(D)), 0x1p61f));
+  v0 -= v0 >> 31;  // 2^31 (D = 2^30, or just above it) does not fit the signed product
+  const long long e = (long long)((1ull << 61) - (unsigned long long)v0 * D);
+  const uint32_t v = v0 + (uint32_t)(__mulhi((int)(e >> 8), (int)v0) >> 21) - 2u;
+  const bool ge = A >= D;
+  const uint32_t r = ge ? A - D : 2u * A - D;
+  uint32_t d1 = __umulhi(r, v) >> 3, r1 = (r << 26) - d1 * D;
+  if (r1 >= D) {
+    r1 -= D;
+    ++d1;
+  }
+  uint32_t d2 = __umulhi(r1, v) >> 3, r2 = (r1 << 26) - d2 * D;
+  if (r2 >= D) {
+    r2 -= D;
+    ++d2;
+  }
+  const unsigned long long m = ((unsigned long long)d1 << 26 | d2) + (r2 > D - r2 ? 1u : 0u);
+  return __longlong_as_double((long long)(((unsigned long long)(1023 + sb - sa - (ge ? 0 : 1)) << 52) + m));
 }
 
 // Triangle index of pair (i, j), i <= j.
