@@ -207,11 +207,12 @@ static bool tc_tile_kernel_forced() {
   return v;
 }
 
-// The sweep kernel (ibs_sweep.cu) computes the E2M1 triangle: at every size the
-// faster one (256 x 4,096: 31 us a call against 82 on the kernels below; 4,096 x
-// 100,000: 1,076 against 1,564; 20,000 x 500,000: 82 against 142 ms).
+// The sweep kernel (ibs_sweep.cu) computes E2M1 inputs, triangle or square: at
+// every size the faster one (256 x 4,096: 33 us a call against 82 on the kernels
+// below; 4,096 x 100,000: 979 against 1,564; 20,000 x 500,000: 77 against 142
+// ms; the square of 3,001 x 60,000: 583 us against 786).
 static bool use_sweep(const ibs_ctx* ctx, int64_t n, int64_t m, bool square) {
-  return !square && tc_format_for(ctx) == kTcFp4 && tc_pair_mode() >= 0 && !tc_tile_kernel_forced() &&
+  return tc_format_for(ctx) == kTcFp4 && tc_pair_mode() >= 0 && !tc_tile_kernel_forced() &&
          sweep_usable(n, m) && ctx->sweep_refused != std::vector<int64_t>{n, m, square ? 1 : 0};
 }
 
@@ -277,7 +278,7 @@ static ibs_status compute_sweep(ibs_ctx* ctx, const uint8_t* packed, int64_t n, 
   l.scratch = static_cast<float*>(ctx->sweep_scratch.p);
   l.part = static_cast<float*>(ctx->partial.p);
   l.status = ctx->status_dev;
-  l.wait_ns = ctx->wait_ns > 0 ? ctx->wait_ns : kWaitLimitNs;
+  l.wait_ns = !square && ctx->wait_ns > 0 ? ctx->wait_ns : kWaitLimitNs;
   l.sync = sync;
   l.between = timing ? rec.ev[2] : nullptr;
   IBS_CUDA_TRY(launch_sweep_one(static_cast<const uint8_t*>(ctx->planes.p), n, m, out_counts, out_dist, square, l, st));

@@ -84,3 +84,26 @@ def test_batch_gather(ctx, pool_n, n, vb, vl):
         ibs.ibs_synchronize(ctx)
         assert (out_c.cpu().numpy() == want_c).all()
         assert_dist_close(out_d.cpu().numpy(), want_d)
+
+
+# the mirror image at the edges of row pairs, column groups and pieces; parts and
+# whole tiles.  The distances are the IEEE quotients.
+@pytest.mark.parametrize("n,m", [(1, 31), (129, 289), (257, 1000), (385, 2593), (513, 577), (1100, 9_001), (3201, 600)])
+def test_square(ctx, n, m):
+    from paper_1410_4803_gb300 import ibs
+    rng = np.random.default_rng(n + m)
+    packed = pack_codes(random_codes(rng, n, m, miss=0.05))
+    tri_c, tri_d = gpu_compute(ctx, packed, n, m)
+    sq = ibs.ibs_init(0, flags=ibs.IBS_KERNEL_TC | ibs.IBS_TC_FP4 | ibs.IBS_OUT_SQUARE)
+    try:
+        got_c, got_d = gpu_compute(sq, packed, n, m, square=True)
+    finally:
+        ibs.ibs_shutdown(sq)
+    got_c, got_d = got_c.reshape(n, n, 4), got_d.reshape(n, n)
+    i, j = np.triu_indices(n)
+    for c, d in ((got_c[i, j], got_d[i, j]), (got_c[j, i], got_d[j, i])):
+        assert (c == tri_c).all()
+        np.testing.assert_array_equal(d, tri_d)
+    c = tri_c.astype(np.float64)
+    with np.errstate(invalid="ignore"):
+        np.testing.assert_array_equal(tri_d, (c[:, 1] + 2 * c[:, 0]) / (2 * c[:, 3]))
