@@ -105,9 +105,13 @@ struct RowSrc {
 // holds few_rows_bytes; `part` at least 12 bytes per row and panel sample.
 constexpr int kFewRows = 16;
 size_t few_rows_bytes(int64_t n_cols);
-cudaError_t launch_few_rows(const RowSrc* rows, int64_t n_rows, const uint32_t* panel_words, int64_t n_panel, int64_t m,
+struct FewTables {  // by value: no copies in front of the kernels
+  RowSrc rows[kFewRows];
+  int32_t* out[kFewRows];
+};
+cudaError_t launch_few_rows(const FewTables& tab, int64_t n_rows, const uint32_t* panel_words, int64_t n_panel, int64_t m,
                             const int64_t (&samples)[2][2], void* words, void* part, size_t part_bytes, int num_sms,
-                            int32_t* const* row_out, cudaStream_t st);
+                            cudaStream_t st);
 
 // Kernel launchers (ibs_planes.cu / ibs_pairs.cu / ibs_misc.cu).
 cudaError_t launch_planes(const BedSource& src, int64_t n, int64_t m, const PlaneGeom& g, uint32_t* planes,
@@ -140,6 +144,8 @@ struct TopkRow {
   int32_t pad;
 };
 cudaError_t launch_topk_rows(const TopkRow* rows, int64_t n_rows, int64_t n_panel, cudaStream_t st);
+// At most kFewRows rows, the table from host memory.
+cudaError_t launch_topk_few(const TopkRow* rows, int64_t n_rows, int64_t n_panel, cudaStream_t st);
 cudaError_t launch_topk(const int32_t* counts, int64_t q, int64_t n_panel, int k, int32_t* out_idx,
                         double* out_dist, cudaStream_t st);
 int pair_kernel_ctas_per_sm(int mode);

@@ -1,5 +1,6 @@
 // Serving-side helper kernels (top-k nearest panel samples) and the
 // integer-pipe microbenchmark used to derive the pair loop's roofline.
+#include <algorithm>
 #include <cstdio>
 
 #include "ibs_device.cuh"
@@ -211,6 +212,14 @@ __global__ void __launch_bounds__(kTopkThreads) topk_rows_kernel(const TopkRow* 
   topk_row(reinterpret_cast<const int4*>(t.counts), n_panel, t.k, t.out_idx, t.out_dist);
 }
 
+struct TopkFew {
+  TopkRow row[kFewRows];
+};
+__global__ void __launch_bounds__(kTopkThreads) topk_few_kernel(const TopkFew rows, int64_t n_panel) {
+  const TopkRow t = rows.row[blockIdx.x];
+  topk_row(reinterpret_cast<const int4*>(t.counts), n_panel, t.k, t.out_idx, t.out_dist);
+}
+
 // ---------------------------------------------------------------------------
 // Integer-pipe microbenchmark: 8 independent dependency chains per thread.
 template <int OP>
@@ -304,6 +313,15 @@ cudaError_t launch_topk_rows(const TopkRow* rows, int64_t n_rows, int64_t n_pane
   if (n_rows <= 0) return cudaSuccess;
   if (n_rows > 2147483647LL) return cudaErrorInvalidValue;
   topk_rows_kernel<<<(unsigned)n_rows, kTopkThreads, 0, st>>>(rows, n_panel);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_topk_few(const TopkRow* rows, int64_t n_rows, int64_t n_panel, cudaStream_t st) {
+  if (n_rows <= 0) return cudaSuccess;
+  if (n_rows > kFewRows) return cudaErrorInvalidValue;
+  TopkFew t{};
+  std::copy(rows, rows + n_rows, t.row);
+  topk_few_kernel<<<(unsigned)n_rows, kTopkThreads, 0, st>>>(t, n_panel);
   return cudaGetLastError();
 }
 

@@ -35,13 +35,13 @@ constexpr int kFewCols = 64;               // columns of the rows' words staged 
 // The rows' words from their requests' packed bytes: thread = column c of row r,
 // {V, hom, H, 0}; rows past the last and markers past m count as missing.
 template <int kQ>
-__global__ void __launch_bounds__(256) few_words_kernel(const RowSrc* __restrict__ rows, int64_t n_rows, int64_t m,
-                                                        int64_t n_cols, uint4* __restrict__ words) {
+__global__ void __launch_bounds__(256) few_words_kernel(const FewTables tab, int64_t n_rows, int64_t m, int64_t n_cols,
+                                                        uint4* __restrict__ words) {
   const int64_t c = (int64_t)blockIdx.x * 256 + threadIdx.x, r = blockIdx.y;
   if (c >= n_cols) return;
   uint32_t H = 0, L = ~0u;
   if (r < n_rows) {
-    const RowSrc src = rows[r];
+    const RowSrc src = tab.rows[r];
     const int64_t stride = src.n_half, left = m - c * 32;
     const uint8_t* p = reinterpret_cast<const uint8_t*>(src.planes) + c * 32 * stride + (src.row >> 2);
     const int sh = 2 * (int)(src.row & 3);
@@ -113,7 +113,7 @@ __global__ void __launch_bounds__(kFewThreads) few_pairs_kernel(const FewArgs a)
   }
 }
 
-__global__ void __launch_bounds__(256) few_sum_kernel(const FewArgs a, int splits, int32_t* const* __restrict__ row_out) {
+__global__ void __launch_bounds__(256) few_sum_kernel(const FewArgs a, int splits, const FewTables tab) {
   const int64_t i = (int64_t)blockIdx.x * 256 + threadIdx.x, r = blockIdx.y;
   if (i >= a.count) return;
   int32_t sum[3] = {0, 0, 0};
@@ -123,20 +123,19 @@ __global__ void __launch_bounds__(256) few_sum_kernel(const FewArgs a, int split
 #pragma unroll
     for (int v = 0; v < 3; ++v) sum[v] += p[v * a.count];
   }
-  reinterpret_cast<int4*>(row_out[r])[few_sample(a, i)] = make_int4(sum[0], sum[1], sum[2] - sum[0] - sum[1], sum[2]);
+  reinterpret_cast<int4*>(tab.out[r])[few_sample(a, i)] = make_int4(sum[0], sum[1], sum[2] - sum[0] - sum[1], sum[2]);
 }
 
 template <int kQ>
-cudaError_t few(const RowSrc* rows, int64_t m, uint4* words, int splits, const FewArgs& a, int32_t* const* row_out,
-                cudaStream_t st) {
+cudaError_t few(const FewTables& tab, int64_t m, uint4* words, int splits, const FewArgs& a, cudaStream_t st) {
   const unsigned groups = (unsigned)((a.n_rows + kQ - 1) / kQ);
-  few_words_kernel<kQ><<<dim3((unsigned)((a.n_cols + 255) / 256), groups * kQ), 256, 0, st>>>(rows, a.n_rows, m,
+  few_words_kernel<kQ><<<dim3((unsigned)((a.n_cols + 255) / 256), groups * kQ), 256, 0, st>>>(tab, a.n_rows, m,
                                                                                              a.n_cols, words);
   if (cudaError_t e = cudaGetLastError()) return e;
   few_pairs_kernel<kQ><<<dim3((unsigned)((a.count + kFewSpan - 1) / kFewSpan), (unsigned)splits, groups), kFewThreads, 0,
                          st>>>(a);
   if (cudaError_t e = cudaGetLastError()) return e;
-  few_sum_kernel<<<dim3((unsigned)((a.count + 255) / 256), (unsigned)a.n_rows), 256, 0, st>>>(a, splits, row_out);
+  few_sum_kernel<<<dim3((unsigned)((a.count + 255) / 256), (unsigned)a.n_rows), 256, 0, st>>>(a, splits, tab);
   return cudaGetLastError();
 }
 
@@ -144,9 +143,9 @@ cudaError_t few(const RowSrc* rows, int64_t m, uint4* words, int splits, const F
 
 size_t few_rows_bytes(int64_t n_cols) { return (size_t)kFewRows * n_cols * sizeof(uint4); }
 
-cudaError_t launch_few_rows(const RowSrc* rows, int64_t n_rows, const uint32_t* panel_words, int64_t n_panel, int64_t m,
+cudaError_t launch_few_rows(const FewTables& tab, int64_t n_rows, const uint32_t* panel_words, int64_t n_panel, int64_t m,
                             const int64_t (&samples)[2][2], void* words, void* part, size_t part_bytes, int num_sms,
-                            int32_t* const* row_out, cudaStream_t st) {
+                            cudaStream_t st) {
   FewArgs a;
   a.panel = reinterpret_cast<const uint2*>(panel_words);
   a.rows = static_cast<const uint4*>(words);
@@ -167,10 +166,10 @@ cudaError_t launch_few_rows(const RowSrc* rows, int64_t n_rows, const uint32_t* 
   if (splits < 1) return cudaErrorInvalidValue;
   a.split_cols = (a.n_cols + splits - 1) / splits;
   splits = (a.n_cols + a.split_cols - 1) / a.split_cols;
-  if (n_rows > 4) return few<8>(rows, m, static_cast<uint4*>(words), (int)splits, a, row_out, st);
-  if (n_rows > 2) return few<4>(rows, m, static_cast<uint4*>(words), (int)splits, a, row_out, st);
-  if (n_rows > 1) return few<2>(rows, m, static_cast<uint4*>(words), (int)splits, a, row_out, st);
-  return few<1>(rows, m, static_cast<uint4*>(words), (int)splits, a, row_out, st);
+  if (n_rows > 4) return few<8>(tab, m, static_cast<uint4*>(words), (int)splits, a, st);
+  if (n_rows > 2) return few<4>(tab, m, static_cast<uint4*>(words), (int)splits, a, st);
+  if (n_rows > 1) return few<2>(tab, m, static_cast<uint4*>(words), (int)splits, a, st);
+  return few<1>(tab, m, static_cast<uint4*>(words), (int)splits, a, st);
 }
 
 }  // namespace ibs

@@ -30,6 +30,7 @@
 // device step by step on a second stream (the panel columns each step wrote),
 // so those copies overlap the following steps instead of trailing them.  The
 // top-k of all requests that finish in a step runs as one launch.
+#include <shared_mutex>
 #include <algorithm>
 #include <atomic>
 #include <chrono>
@@ -71,6 +72,10 @@ struct Request {
   DevBuf packed, planes, counts, tidx, tdist;
   size_t reserved = 0;
   bool planes_built = false;
+  int32_t* map_idx = nullptr;  // pinned top-k outputs as the device sees them
+  double* map_dist = nullptr;
+  bool topk_direct = false;    // written there by the kernel
+  bool early = false;  // reserved and on the device since ibs_query
   int64_t blocks_done = 0;  // panel blocks processed since admission
   cudaEvent_t done_ev = nullptr;  // recorded on the engine's copy stream after the request's last output
   ibs_status status = IBS_OK;
@@ -88,6 +93,16 @@ PtrKind ptr_kind(const void* p) {
   if (a.type == cudaMemoryTypeDevice || a.type == cudaMemoryTypeManaged) return PtrKind::Device;
   if (a.type == cudaMemoryTypeHost) return PtrKind::PinnedHost;
   return PtrKind::Pageable;
+}
+
+// The device's address of pinned host memory, or null.
+void* mapped(void* p) {
+  cudaPointerAttributes a;
+  if (cudaPointerGetAttributes(&a, p) != cudaSuccess) {
+    cudaGetLastError();
+    return nullptr;
+  }
+  return a.type == cudaMemoryTypeHost ? a.devicePointer : nullptr;
 }
 
 }  // namespace
@@ -108,6 +123,9 @@ class ServeEngine {
   Geo pgeo{};            // the panel's geometry
   DevBuf panel_planes, counter;
   cudaStream_t stream = nullptr;
+  cudaStream_t in = nullptr;  // ibs_query's copies
+  std::shared_mutex in_mu;    // in used, or destroyed
+  int64_t early_rows = 0;     // rows of the unfinished requests copied to the device by ibs_query (mu)
   std::thread worker;
   std::mutex mu;
   std::condition_variable cv_work, cv_done;
@@ -189,12 +207,16 @@ class ServeEngine {
   // (cudaMallocAsync / cudaFreeAsync on the stream that uses them): no
   // device-wide synchronisation when a request's memory is returned, so the
   // step pipeline never stalls on a free.
-  void release(Request& r, cudaStream_t s) {
+  void free_async(Request& r, bool packed_too, cudaStream_t s) {
     for (DevBuf* b : {&r.packed, &r.planes, &r.counts, &r.tidx, &r.tdist}) {
+      if (b == &r.packed && !packed_too) continue;
       if (b->p) cudaFreeAsync(b->p, s);
       b->p = nullptr;
       b->cap = 0;
     }
+  }
+  void release(Request& r, cudaStream_t s) {
+    free_async(r, true, s);
     if (r.reserved) {
       release_bytes(ctx, r.reserved);
       std::lock_guard<std::mutex> lk(budget_mu);
@@ -244,20 +266,47 @@ class ServeEngine {
     return true;
   }
 
+  // The samples of a request from the caller's memory into device memory
+  // (caller's thread; done on return).  Device memory is read in the legacy
+  // stream's order, as by a plain copy.  The calls are allowed while a thread
+  // captures a graph elsewhere.
+  bool copy_in(Request& r, const uint8_t* q, size_t bytes, size_t need) {
+    std::shared_lock<std::shared_mutex> in_lk(in_mu);
+    if (!in) return false;
+    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+    cudaThreadExchangeStreamCaptureMode(&mode);
+    bool ok = reserve_request(r, need);
+    if (ok && alloc(r.packed, bytes, in) == IBS_OK) {
+      const cudaStream_t s = ptr_kind(q) == PtrKind::Device ? cudaStreamLegacy : in;
+      ok = cudaStreamSynchronize(in) == cudaSuccess &&
+           cudaMemcpyAsync(r.packed.p, q, bytes, cudaMemcpyDefault, s) == cudaSuccess &&
+           cudaStreamSynchronize(s) == cudaSuccess;
+      if (!ok) cudaGetLastError();
+    } else {
+      ok = false;
+    }
+    if (!ok) release(r, in);
+    cudaThreadExchangeStreamCaptureMode(&mode);
+    return ok;
+  }
+
   // Try to admit r (engine thread).  Returns false if it must wait.
   bool admit(const std::shared_ptr<Request>& r, int64_t active_rows) {
     if (active_rows + r->q > kMaxRows && active_rows > 0) return false;
     const size_t need = mem_need(r->q, r->k, r->counts_on_dev, r->topk_on_dev);
-    if (!reserve_request(*r, need)) return false;
+    if (!r->early && !reserve_request(*r, need)) return false;
     const size_t pk = (size_t)pg.m * (size_t)((r->q + 3) / 4);
-    if (alloc(r->packed, pk, stream) || alloc(r->planes, geo(r->q).bytes, stream) ||
+    if ((!r->early && alloc(r->packed, pk, stream)) || alloc(r->planes, geo(r->q).bytes, stream) ||
         (!r->counts_on_dev && alloc(r->counts, (size_t)r->q * pg.n * 16, stream)) ||
         (!r->topk_on_dev && r->k > 0 &&
          (alloc(r->tidx, (size_t)r->q * r->k * 4, stream) || alloc(r->tdist, (size_t)r->q * r->k * 8, stream)))) {
-      release(*r, stream);
+      if (r->early)
+        free_async(*r, false, stream);  // it keeps its reservation and its samples
+      else
+        release(*r, stream);
       return false;
     }
-    cudaMemcpyAsync(r->packed.p, r->host_packed.data(), pk, cudaMemcpyHostToDevice, stream);
+    if (!r->early) cudaMemcpyAsync(r->packed.p, r->host_packed.data(), pk, cudaMemcpyHostToDevice, stream);
     cudaEventCreateWithFlags(&r->done_ev, cudaEventDisableTiming);
     r->blocks_done = 0;
     r->state = RState::Active;
@@ -285,16 +334,24 @@ class ServeEngine {
     // every row of every finishing request in one launch (at most kMaxRows
     // rows: the admitted set never holds more)
     int64_t n = 0;
+    for (auto& rp : done) n += rp->k > 0 ? rp->q : 0;
+    // few rows: the table goes as an argument and the lists straight to mapped
+    // pinned memory, instead of three small copies
+    const bool few = n <= kFewRows;
+    n = 0;
     for (auto& rp : done) {
       Request& r = *rp;
       if (r.k <= 0) continue;
-      int32_t* oi = r.topk_on_dev ? r.user_idx : static_cast<int32_t*>(r.tidx.p);
-      double* od = r.topk_on_dev ? r.user_dist : static_cast<double*>(r.tdist.p);
+      r.topk_direct = few && r.map_idx && r.map_dist;
+      int32_t* oi = r.topk_on_dev ? r.user_idx : r.topk_direct ? r.map_idx : static_cast<int32_t*>(r.tidx.p);
+      double* od = r.topk_on_dev ? r.user_dist : r.topk_direct ? r.map_dist : static_cast<double*>(r.tdist.p);
       const int32_t* cnt = counts_ptr(r);
       for (int64_t row = 0; row < r.q && n < kMaxRows; ++row, ++n)
         topk_host[slot][n] = TopkRow{cnt + (size_t)row * pg.n * 4, oi + row * r.k, od + row * r.k, r.k, 0};
     }
-    if (n > 0) {
+    if (n > 0 && few) {
+      launch_topk_few(topk_host[slot], n, pg.n, stream);
+    } else if (n > 0) {
       cudaMemcpyAsync(topk_dev[slot].p, topk_host[slot], (size_t)n * sizeof(TopkRow), cudaMemcpyHostToDevice, stream);
       launch_topk_rows(static_cast<const TopkRow*>(topk_dev[slot].p), n, pg.n, stream);
     }
@@ -303,7 +360,7 @@ class ServeEngine {
     cudaStreamWaitEvent(side, fin_ev[slot], 0);
     for (auto& rp : done) {
       Request& r = *rp;
-      if (!r.topk_on_dev && r.k > 0) {
+      if (!r.topk_on_dev && !r.topk_direct && r.k > 0) {
         cudaMemcpyAsync(r.user_idx, r.tidx.p, (size_t)r.q * r.k * 4, cudaMemcpyDeviceToHost, side);
         cudaMemcpyAsync(r.user_dist, r.tdist.p, (size_t)r.q * r.k * 8, cudaMemcpyDeviceToHost, side);
       }
@@ -513,9 +570,7 @@ class ServeEngine {
       }
     }
     if (t > 0) {
-      if (few) {
-        cudaMemcpyAsync(rows_dev[slot].p, rows_host[slot], n_rows * sizeof(RowSrc), cudaMemcpyHostToDevice, stream);
-      } else if (gathered_version != set_version) {
+      if (!few && gathered_version != set_version) {
         for (auto& r : active) {
           if (r->planes_built) continue;
           build_planes(static_cast<const uint8_t*>(r->packed.p), r->q, r->planes.p, stream);
@@ -534,13 +589,19 @@ class ServeEngine {
                              static_cast<uint32_t*>(step_planes.p), stream);
         gathered_version = set_version;
       }
-      cudaMemcpyAsync(outs_dev[slot].p, outs_host[slot], n_rows * sizeof(int32_t*), cudaMemcpyHostToDevice, stream);
+      if (!few)
+        cudaMemcpyAsync(outs_dev[slot].p, outs_host[slot], n_rows * sizeof(int32_t*), cudaMemcpyHostToDevice, stream);
       if (few) {
         const int64_t samples[2][2] = {{cols[0][0] * blk, std::min<int64_t>(cols[0][1] * blk, pg.n)},
                                        {0, std::min<int64_t>(cols[1][1] * blk, pg.n)}};
-        launch_few_rows(static_cast<const RowSrc*>(rows_dev[slot].p), n_rows,
+        FewTables tab;
+        for (int64_t r = 0; r < n_rows; ++r) {
+          tab.rows[r] = rows_host[slot][r];
+          tab.out[r] = outs_host[slot][r];
+        }
+        launch_few_rows(tab, n_rows,
                         static_cast<const uint32_t*>(panel_words.p), pg.n, pg.m, samples, few_words.p, sweep_part.p,
-                        sweep_part.cap, ctx->num_sms, outs_d, stream);
+                        sweep_part.cap, ctx->num_sms, stream);
         words_lk.unlock();
       } else if (sweep) {
         run_sweep(pl, static_cast<const uint8_t*>(step_planes.p), kMaxRows / 64, outs_d, n_rows, items_host[slot],
@@ -606,6 +667,7 @@ class ServeEngine {
         std::lock_guard<std::mutex> lk(mu);
         r->status = st == kDevTimeout ? IBS_ETIMEOUT : IBS_OK;
         release(*r, stream);
+        if (r->early) early_rows -= r->q;
         r->state = RState::Done;
         stats.requests_done++;
         any = true;
@@ -639,10 +701,23 @@ class ServeEngine {
           stats.peak_rows = std::max<uint64_t>(stats.peak_rows, (uint64_t)rows);
         }
         if (active.empty()) {
-          if (finishing.empty())
+          if (finishing.empty()) {
             cv_work.wait(lk, [&] { return stop || !pending.empty(); });
-          else
+          } else if (!pending.empty()) {  // (it waits for memory)
             cv_work.wait_for(lk, std::chrono::microseconds(200));
+          } else {
+            // the last results are a few hundred microseconds away: poll (a timed
+            // wait would add its period to every lone request's latency)
+            const auto t0 = std::chrono::steady_clock::now();
+            do {
+              lk.unlock();
+              const bool done = cudaEventQuery(finishing.front()->done_ev) != cudaErrorNotReady;
+              lk.lock();
+              if (done || stop || !pending.empty()) break;
+            } while (std::chrono::steady_clock::now() - t0 < std::chrono::milliseconds(2));
+            if (!stop && pending.empty() && cudaEventQuery(finishing.front()->done_ev) == cudaErrorNotReady)
+              cv_work.wait_for(lk, std::chrono::microseconds(200));
+          }
           continue;
         }
       }
@@ -704,6 +779,11 @@ class ServeEngine {
     }
     if (stream) cudaStreamDestroy(stream);
     if (side) cudaStreamDestroy(side);
+    {
+      std::unique_lock<std::shared_mutex> in_lk(in_mu);  // a call may still be copying
+      if (in) cudaStreamDestroy(in);
+      in = nullptr;
+    }
     stream = nullptr;
     side = nullptr;
   }
@@ -873,6 +953,10 @@ ibs_status serve_panel_load(ibs_ctx* ctx, const uint8_t* panel, int64_t n_panel,
   }
   eng->fixed_bytes = eng->panel_planes.cap + eng->step_planes.cap + eng->counter.cap + 2 * (eng->sweep_scratch.cap + eng->sweep_part.cap) +
                      2 * (eng->rows_dev[0].cap + eng->outs_dev[0].cap);
+  if (cudaStreamCreateWithFlags(&eng->in, cudaStreamNonBlocking) != cudaSuccess) {
+    cudaGetLastError();
+    eng->in = nullptr;  // requests are kept on the host
+  }
   eng->start();
   std::lock_guard<std::mutex> lk(ctx->mu);
   ctx->serve = std::move(eng);
@@ -937,11 +1021,36 @@ ibs_status serve_query(ibs_ctx* ctx, const uint8_t* q, int64_t nq, int k, int32_
   r->user_dist = od;
   r->counts_on_dev = counts_dev;
   r->topk_on_dev = topk_dev;
-  r->host_packed = copy_query(q, (size_t)e.pg.m * (size_t)((nq + 3) / 4));
+  if (k > 0 && !topk_dev) {
+    r->map_idx = static_cast<int32_t*>(mapped(oi));
+    r->map_dist = static_cast<double*>(mapped(od));
+  }
+  // A request that the engine can admit at once goes straight to the device;
+  // one behind others that wait for memory, or past the rows of a step, is kept
+  // on the host.  (20 requests with 75 MB of pinned samples: HOSTTIMES.)
+  const size_t bytes = (size_t)e.pg.m * (size_t)((nq + 3) / 4);
+  bool early = false;
+  if (ctx->ws_limit == 0) {
+    std::lock_guard<std::mutex> lk(e.mu);
+    early = !e.stop && e.early_rows + nq <= kMaxRows;
+    for (const auto& p : e.pending) early = early && p->early;
+    if (early) e.early_rows += nq;
+  }
+  if (early) {
+    r->early = e.copy_in(*r, q, bytes, need);
+    if (!r->early) {
+      std::lock_guard<std::mutex> lk(e.mu);
+      e.early_rows -= nq;
+    }
+  }
+  if (!r->early) r->host_packed = copy_query(q, bytes);
   r->id = e.next_id.fetch_add(1);
   {
     std::lock_guard<std::mutex> lk(e.mu);
-    if (e.stop) return fail(IBS_ECANCELLED, "engine is shutting down");
+    if (e.stop) {
+      if (r->early) e.release(*r, nullptr);
+      return fail(IBS_ECANCELLED, "engine is shutting down");
+    }
     e.all[r->id] = r;
     e.pending.push_back(r);
   }
