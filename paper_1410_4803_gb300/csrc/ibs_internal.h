@@ -174,6 +174,7 @@ cudaError_t launch_tc_planes(const uint8_t* packed, int64_t n, int64_t m, uint8_
 cudaError_t launch_tc_pairs(const uint8_t* planes, int64_t n, int64_t m, int fmt, int splits, int32_t* out_counts,
                             double* out_dist, int32_t* partial, bool square, int* status, const int2* tile_list,
                             cudaStream_t st);
+cudaError_t tc_pairs_load();  // the E2M1 kernels of launch_tc_planes and launch_tc_pairs, ahead of their first launch
 void tc_tile_order(int64_t T, int G, std::vector<int2>& out);
 int64_t tc_gather_ctas(int64_t n, int64_t nc);  // CTAs of one job of the gather launch
 // map_dev[c] = {job, sample block, chunk group, -} of gather CTA c; chunk groups

@@ -48,6 +48,9 @@ ibs_status setup_device(int dev) {
   g_status_addr[dev] = static_cast<int*>(p);
   e = cudaDeviceGetAttribute(&g_sms[dev], cudaDevAttrMultiProcessorCount, dev);
   if (e != cudaSuccess) return fail(IBS_ECUDA, "cudaDeviceGetAttribute failed: %s", cudaGetErrorString(e));
+  // loaded now: a call recorded into a graph may be the first to use them
+  if ((e = tc_pairs_load()) != cudaSuccess)
+    return fail(IBS_ECUDA, "tensor-core kernels could not be loaded: %s", cudaGetErrorString(e));
   g_ready[dev] = true;
   return IBS_OK;
 }
@@ -94,6 +97,28 @@ extern "C" ibs_status ibs_compute_noalloc(const uint8_t* packed, int64_t n, int6
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   // The status word must start at zero; the planes are fully rewritten by the transpose.
   IBS_CUDA_TRY(cudaMemsetAsync(g_status_addr[dev], 0, sizeof(int) * 4, st));
+  // Tensor-core tiles where their operand planes (2 bytes per genotype against
+  // 3 bits) and, with the marker axis split, the partial counts fit the scratch,
+  // and where there is enough to multiply: splitting costs them about 60 us,
+  // and tiles of few markers are bound by their epilogue.  Integer pipe against
+  // tensor core: 1,000 x 20,000 236 us and 93, 2,000 x 2,000 138 and 66, 300 x
+  // 50,000 94 and 76; but 400 x 8,000 49 and 88, 1,000 x 1,000 50 and 56, 4,000 x
+  // 1,000 198 and 196, 5,000 x 100 166 and 254.
+  const int64_t tc_nc = tc_chunks(m, kTcFp4);
+  const int tc_splits = tc_splits_for(tc_tiles(n), tc_nc, g_sms[dev]);
+  const size_t tc_bytes = (tc_planes_bytes(n, m, kTcFp4) + 255) / 256 * 256;
+  const size_t tc_partial = tc_splits > 1 ? (size_t)(n * (n + 1) / 2) * 16 : 0;
+  const bool tc = m >= 1536 && n * (n + 1) / 2 >= ((int64_t)1 << 31) / m;
+  if (tc && tc_bytes + tc_partial <= kNoAllocScratchBytes && tc_nc <= tc_max_chunks(kTcFp4)) {
+    uint8_t* planes = reinterpret_cast<uint8_t*>(g_planes_addr[dev]);
+    int32_t* sums = tc_splits > 1 ? reinterpret_cast<int32_t*>(planes + tc_bytes) : nullptr;
+    IBS_CUDA_TRY(launch_tc_planes(packed, n, m, planes, kTcFp4, st));
+    if (sums) IBS_CUDA_TRY(cudaMemsetAsync(sums, 0, tc_partial, st));
+    IBS_CUDA_TRY(launch_tc_pairs(planes, n, m, kTcFp4, tc_splits, out_counts, out_dist, sums, false,
+                                 g_status_addr[dev], nullptr, st));
+    if (sums) IBS_CUDA_TRY(launch_finalize(sums, n, out_counts, out_dist, false, st));
+    return IBS_OK;
+  }
   BedSource src;
   src.packed = packed;
   src.row_bytes = (n + 3) / 4;

@@ -1520,6 +1520,12 @@ cudaError_t launch_tc_pairs(const uint8_t* planes, int64_t n, int64_t m, int fmt
   return cudaGetLastError();
 }
 
+cudaError_t tc_pairs_load() {
+  cudaFuncAttributes a;
+  if (cudaError_t e = cudaFuncGetAttributes(&a, tc_planes_kernel<kTcFp4>)) return e;
+  return cudaFuncGetAttributes(&a, tc_tri_kernel<kTcFp4>);
+}
+
 // Grouped tile order: the upper triangle of T x T tiles in bands of G tile
 // rows; inside a band, column by column.  The CTAs running at the same time
 // then cover about G rows x (SMs / G) columns, so each block of planes they

@@ -68,6 +68,18 @@ def test_noalloc_matches_ibs_compute_on_two_calls():
         assert_dist_close(got_d, ora_d)
 
 
+# either side of the tensor-core rule (2^31 pair-variants; 1,536 variants), and a
+# split whose partial counts just fit the scratch beside the operand planes
+@pytest.mark.parametrize("n,m", [(1000, 4290), (1000, 4291), (1700, 1535), (1700, 1536), (2000, 8512), (2000, 8513)])
+def test_noalloc_tensor_core_rule(n, m):
+    rng = np.random.default_rng(n + m)
+    packed = pack_codes(random_codes(rng, n, m, miss=0.04), garbage_rng=rng)
+    got_c, got_d = _noalloc(packed, n, m)
+    want_c, want_d = _regular(packed, n, m)
+    assert (got_c == want_c).all()
+    assert_dist_close(got_d, want_d)
+
+
 def test_noalloc_rejects_host_buffers_before_any_work():
     import torch
     from paper_1410_4803_gb300 import ibs
