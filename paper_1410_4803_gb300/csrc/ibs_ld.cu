@@ -31,7 +31,7 @@
 // half-block) items of the band |b - a| <= window from a counter and streams
 // each item's sample chunks through a ring of 3 stages x 3 chunks (one copy of
 // the A block's 3 planes x 4 KiB per chunk, one of the B half-block's 3 planes
-// x 2 KiB per chunk, from a second copy of the planes laid out for it); two
+// x 2 KiB per chunk, from a second copy of the planes laid out for it); three
 // MMA warps issue 3 MMAs (M = 128, N = 192, 128 and 64, K = 64) per chunk into
 // six FP32 accumulators (64 tensor-memory columns each; unit scale factors at
 // 384..511); warps 4..19 read the accumulators back (four warps per lane
@@ -68,7 +68,7 @@ constexpr int kLdN = 64;                             // B rows (markers) per ite
 // (4,096 samples x 100,000 markers, window 1,000).
 constexpr uint32_t kLdSy = 0, kLdCnt = 64, kLdSyy = 128, kLdSxy = 192, kLdSx = 256, kLdSxx = 320;
 constexpr int kLdQueue = 8;
-// warps 0 (copies), 1 and 2 (MMAs), 3 idle, 4..19 epilogue: four warps per TMEM
+// warps 0 (copies), 1, 2 and 3 (MMAs), 4..19 epilogue: four warps per TMEM
 // lane quarter, each reading 16 of the item's 64 accumulator columns
 constexpr int kLdThreads = (4 + kLdEpiWarps) * 32;
 
@@ -259,7 +259,7 @@ __device__ __forceinline__ void tmem_ld8(uint32_t taddr, uint32_t (&r)[8]) {
 // arithmetic is integer and FP32 only, and the stores go through shared memory.
 // With FP64 arithmetic on held accumulators and one lane per marker row the
 // call took 2.33 ms (4,096 samples x 100,000 markers, window 1,000); 1.74 with
-// 8 epilogue warps, 1.67 with 16.
+// 8 epilogue warps, 1.67 with 16 (and 1.58 with three MMA warps instead of two).
 template <bool kSmall>
 __global__ void __launch_bounds__(kLdThreads, 1) tc_ld_kernel(const LdArgs args) {
   extern __shared__ __align__(1024) uint8_t smem_raw[];
@@ -274,15 +274,15 @@ __global__ void __launch_bounds__(kLdThreads, 1) tc_ld_kernel(const LdArgs args)
   if (threadIdx.x == 0) {
     for (int s = 0; s < kLdStages; ++s) {
       mbar_init(&full[s], 1);
-      mbar_init(&empty[s], 2);  // both MMA warps' commits
+      mbar_init(&empty[s], 3);  // the MMA warps' commits
     }
     for (int s = 0; s < kLdQueue; ++s) {
       mbar_init(&qfull[s], 1);
-      mbar_init(&qempty[s], 2 + kLdEpiWarps);  // the MMA warps and the epilogue warps
+      mbar_init(&qempty[s], 3 + kLdEpiWarps);  // the MMA warps and the epilogue warps
     }
-    mbar_init(&tfull, 2);
+    mbar_init(&tfull, 3);
     mbar_init(&tempty, kLdEpiWarps);
-    mbar_init(&drain, 2);
+    mbar_init(&drain, 3);
     mbar_fence_init();
     abort_flag = 0;
   }
@@ -357,11 +357,10 @@ __global__ void __launch_bounds__(kLdThreads, 1) tc_ld_kernel(const LdArgs args)
         mbar_wait_bounded(&full[j % kLdStages], (j / kLdStages) & 1u);
     }
     __syncwarp();
-  } else if (warp == 1 || warp == 2) {
-    // Two MMA warps with accumulators and products of their own, of the same
-    // cost: V_a times the three planes of B, and X_a times two and H_a times one.
-    // One warp's MMAs run while the other commits a stage and waits for the
-    // next (the tensor core queues hardly more than the MMA it runs).  Each waits
+  } else if (warp < 4) {
+    // Three MMA warps with accumulators and products of their own: V_a times the
+    // three planes of B, X_a times two, H_a times one.  One warp's MMAs run while
+    // another commits a stage and waits for the next (the tensor core queues hardly more than the MMA it runs).  Each waits
     // (bounded), at an item's start, until the epilogue has read the previous
     // item's accumulators, and for each stage until its operands have landed;
     // after a failed wait or another role's abort nothing more is issued.
@@ -388,8 +387,9 @@ __global__ void __launch_bounds__(kLdThreads, 1) tc_ld_kernel(const LdArgs args)
             const uint32_t acc = k0 + c > 0 ? 1u : 0u;
             if (warp == 1) {
               umma<kTcFp4, 3 * kLdN>(tmem + kLdSy, umma_desc(a0 + kTileBytes), umma_desc(b0), acc, sf);
-            } else {
+            } else if (warp == 2) {
               umma<kTcFp4, 2 * kLdN>(tmem + kLdSxy, umma_desc(a0), umma_desc(b0), acc, sf);
+            } else {
               umma<kTcFp4, kLdN>(tmem + kLdSxx, umma_desc(a0 + 2 * kTileBytes), umma_desc(b0 + kLdHalfBytes), acc, sf);
             }
           }

@@ -150,8 +150,10 @@ __device__ __forceinline__ uint32_t tc_transpose32(uint32_t x, int lane) {
   return x;
 }
 
-// A ring barrier's wait: one probe on the usual path; past it, bounded by
-// limit_ns and ended by another role's abort.
+// A ring barrier's wait: non-blocking probes on the usual path (a thread that
+// has suspended in try_wait wakes late: 76.6 ms against 73.8 for 20,000 samples
+// x 500,000 markers); past a few hundred, bounded by limit_ns and ended by
+// another role's abort.
 __device__ __noinline__ bool ring_wait_slow(uint64_t* bar, uint32_t parity, unsigned long long limit_ns,
                                              const int* abort_flag) {
   const unsigned long long t0 = globaltimer_ns();
@@ -167,7 +169,10 @@ __device__ __noinline__ bool ring_wait_slow(uint64_t* bar, uint32_t parity, unsi
 }
 __device__ __forceinline__ bool ring_wait(uint64_t* bar, uint32_t parity, unsigned long long limit_ns,
                                            const int* abort_flag) {
-  if (limit_ns >= 1000000ull && mbar_try_wait(bar, parity)) return true;
+  if (limit_ns >= 1000000ull) {
+    for (int i = 0; i < 400; ++i)
+      if (mbar_test_wait(bar, parity)) return true;
+  }
   return ring_wait_slow(bar, parity, limit_ns, abort_flag);
 }
 
