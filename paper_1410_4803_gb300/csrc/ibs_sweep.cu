@@ -824,7 +824,7 @@ SweepItem whole_item(const Tile& t, int wave) {
 // ends at the same time: each takes the next stretch, a few pieces of
 // neighbouring tiles.  A stretch has at least a few stages (a piece costs about
 // kMin stages of its own: pipeline fill, read-back, a part to add up), so a
-// small problem leaves clusters idle.  Then the lists, cluster by cluster.
+// small problem leaves clusters idle.
 void cut_rest(const std::vector<Tile>& rest, std::vector<std::vector<SweepItem>>& own, std::vector<double>& load,
               SweepPlan& pl) {
   const int C = (int)own.size();
@@ -885,6 +885,69 @@ void cut_rest(const std::vector<Tile>& rest, std::vector<std::vector<SweepItem>>
     }
     if (gr.pieces[0] + gr.pieces[1] + gr.pieces[2] > 0) pl.groups.push_back(gr);
   }
+}
+
+// The same in rounds: every tile of `rest` (one subset) is cut into 4 h equal
+// pieces, h each of V V^T and U U^T and 2 h of the third product, and the
+// clusters take the pieces in turn, all tiles' first pieces, then all second
+// ones: the tiles of a round run over the same markers and share operand
+// blocks through L2, which cut_rest's shares, each at a place of its own, do
+// not.  The cheaper of the two by a model in cycles: 620 a stage, 4 stages to
+// fill a piece's pipeline, 160 to write and add up a part; cut_rest's shares at
+// least the time of their operands, 3.4 KB a cycle from HBM or, where the
+// `operands` stay in L2, 5.7.  False where that is cut_rest.  Measured, rounds
+// against shares: 1,501 samples x 30,011 markers 101 us and 111, 2,500 x 100,000
+// 507 and 755, the square of 3,001 x 60,000 404 and 587, 6,000 x 200,000 3.46 ms
+// and 3.91, 20 served requests of 3,003 rows 8.9 and 11.8.
+constexpr int kPartsPerCluster = 6;
+bool cut_rounds(const std::vector<Tile>& rest, std::vector<std::vector<SweepItem>>& own, size_t operands,
+                SweepPlan& pl) {
+  const int64_t C = (int64_t)own.size(), R = (int64_t)rest.size();
+  if (R < 4) return false;
+  const int S = rest[0].stages;
+  constexpr double kFill = 4, kPart = 160, kHbm = 3400, kL2 = 5700;
+  constexpr size_t kL2Bytes = (size_t)129 << 20;
+  double even = 0, bytes = 0;
+  for (const Tile& t : rest) {
+    even += tile_cost(t) / (double)C;
+    bytes += 8.0 * t.stages * (kSwABytes + t.w * (kSwBBytes / 3));
+  }
+  double best = std::max(even, bytes / (operands > kL2Bytes ? kHbm : kL2)) + kPart * (double)(C + 2 * R);
+  int h = 0;
+  for (int k = 1; k <= 8 && S >= 8 * k && 4 * k * R <= kPartsPerCluster * C; ++k) {
+    const double cost = (double)((4 * k * R + C - 1) / C) * ((double)S / k + kFill) * stage_cost(3) + kPart * (double)(4 * k * R);
+    if (cost < best) {
+      best = cost;
+      h = k;
+    }
+  }
+  if (h == 0) return false;
+  for (int64_t t = 0; t < R; ++t) {
+    SweepGroup gr{};
+    gr.I = rest[(size_t)t].I;
+    gr.J = rest[(size_t)t].J;
+    gr.w = rest[(size_t)t].w;
+    gr.subset = rest[(size_t)t].subset;
+    gr.slot = pl.slots + (int)(4 * h * t);
+    gr.pieces[0] = gr.pieces[1] = h;
+    gr.pieces[2] = 2 * h;
+    pl.groups.push_back(gr);
+  }
+  for (int k = 0; k < 4 * h; ++k)
+    for (int64_t t = 0; t < R; ++t) {
+      SweepItem it = whole_item(rest[(size_t)t], -1);
+      it.q0 = (int)((int64_t)S * k / h);
+      it.q1 = (int)((int64_t)S * (k + 1) / h);
+      it.slot = pl.slots + (int)(4 * h * t) + k;
+      own[(size_t)((k * R + t) % C)].push_back(it);
+    }
+  pl.slots += (int)(4 * h * R);
+  return true;
+}
+
+// The clusters' lists, one after the other.
+void lay_out(const std::vector<std::vector<SweepItem>>& own, SweepPlan& pl) {
+  const int C = (int)own.size();
   pl.first.assign((size_t)C + 1, 0);
   for (int c = 0; c < C; ++c) {
     for (const SweepItem& it : own[(size_t)c]) {
@@ -901,7 +964,7 @@ void cut_rest(const std::vector<Tile>& rest, std::vector<std::vector<SweepItem>>
 // One matrix or one step: the full-width tiles run whole, one per cluster and
 // wave, as many full waves as there are; the last partial wave and the
 // narrower tiles are cut into equal shares.
-SweepPlan schedule(std::vector<Tile>& full, const std::vector<Tile>& narrow, int clusters) {
+SweepPlan schedule(std::vector<Tile>& full, const std::vector<Tile>& narrow, int clusters, size_t operands) {
   SweepPlan pl;
   const size_t C = (size_t)std::max(1, clusters), whole = full.size() / C * C;
   std::vector<std::vector<SweepItem>> own(C);
@@ -914,7 +977,8 @@ SweepPlan schedule(std::vector<Tile>& full, const std::vector<Tile>& narrow, int
   pl.waves = (int)(whole / C);
   std::vector<Tile> rest(full.begin() + (long)whole, full.end());
   rest.insert(rest.end(), narrow.begin(), narrow.end());
-  cut_rest(rest, own, load, pl);
+  if (!cut_rounds(rest, own, operands, pl)) cut_rest(rest, own, load, pl);
+  lay_out(own, pl);
   return pl;
 }
 
@@ -1031,7 +1095,7 @@ bool sweep_usable(int64_t n, int64_t m) {
 SweepPlan sweep_plan(int64_t n, int64_t m, int clusters) {
   std::vector<Tile> full, narrow;
   triangle_tiles(n, sweep_stages(m), 0, full, narrow);
-  return schedule(full, narrow, clusters);
+  return schedule(full, narrow, clusters, sweep_planes_bytes(n, m));
 }
 
 // Batched subsets, by decreasing marker count: each tile in turn to the least
@@ -1061,6 +1125,7 @@ SweepPlan sweep_plan_batch(const std::vector<std::pair<int64_t, int64_t>>& shape
     load[c] += tile_cost(all[t]);
   }
   cut_rest(std::vector<Tile>(all.begin() + (long)lead, all.end()), own, load, pl);
+  lay_out(own, pl);
   return pl;
 }
 
@@ -1069,12 +1134,13 @@ SweepPlan sweep_plan_batch(const std::vector<std::pair<int64_t, int64_t>>& shape
 SweepPlan sweep_plan_cross(int64_t row_blocks, const int64_t (&cols)[2][2], int64_t m, int clusters) {
   std::vector<Tile> full, narrow;
   const int S = sweep_stages(m);
+  const int64_t blocks = cols[0][1] - cols[0][0] + cols[1][1] - cols[1][0];
   for (const auto& r : cols)
     for (int64_t J = r[0]; J < r[1]; J += 3) {
       const int w = (int)std::min<int64_t>(3, r[1] - J);
       for (int64_t I = 0; I < row_blocks; I += 2) (w == 3 ? full : narrow).push_back({(int)I, (int)J, w, 0, S});
     }
-  return schedule(full, narrow, clusters);
+  return schedule(full, narrow, clusters, sweep_planes_bytes(kTB * (row_blocks + blocks), m));
 }
 
 bool sweep_encode_maps(void* maps, const void* planes, int64_t n, int64_t m) {
