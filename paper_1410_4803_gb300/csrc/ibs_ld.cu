@@ -30,8 +30,9 @@
 // One persistent CTA per SM, 20 warps: the copy warp claims (A block, B
 // half-block) items of the band |b - a| <= window from a counter and streams
 // each item's sample chunks through a ring of 3 stages x 3 chunks (one copy of
-// the A block's 3 planes x 4 KiB per chunk, one of the B half-block's 3 planes
-// x 2 KiB per chunk, from a second copy of the planes laid out for it); three
+// the A block's 3 planes x 4 KiB per chunk, one tensor copy of the B
+// half-block's 3 x 2 KiB per chunk out of the same planes: a second copy of
+// them laid out for B took as long to write as the first); three
 // MMA warps issue 3 MMAs (M = 128, N = 192, 128 and 64, K = 64) per chunk into
 // six FP32 accumulators (64 tensor-memory columns each; unit scale factors at
 // 384..511); warps 4..19 read the accumulators back (four warps per lane
@@ -85,14 +86,12 @@ __device__ __forceinline__ uint32_t even_bits(uint64_t x) {
 
 // Operand rows: CTA = (sample chunk c, marker block b), thread (row r, half):
 // marker b*128 + r, samples c*64 + 32*half .. +31 (8 bytes of the .bed row).
-// Writes 16 bytes of each of X, V, H (E2M1: +1 = 0x2, -1 = 0xA) twice: into
-// the A layout [block][chunk][plane][128 rows] and into the B layout
-// [half-block][chunk][plane][64 rows], so that an item's B operand for a run
-// of chunks is one contiguous copy; adds the marker's #hom A1 - #hom A2 over
+// Writes 16 bytes of each of X, V, H (E2M1: +1 = 0x2, -1 = 0xA) into
+// [block][chunk][plane][128 rows]; adds the marker's #hom A1 - #hom A2 over
 // these samples to diff.
 __global__ void __launch_bounds__(256) ld_planes_kernel(const uint8_t* __restrict__ packed, int64_t row_bytes,
                                                         int64_t n, int64_t m, uint8_t* __restrict__ planes,
-                                                        uint8_t* __restrict__ planes_b, int64_t n_chunks,
+                                                        int64_t n_chunks,
                                                         int32_t* __restrict__ diff) {
   const int64_t c = blockIdx.x, b = blockIdx.y;
   const int r = threadIdx.x >> 1, half = threadIdx.x & 1;
@@ -104,8 +103,12 @@ __global__ void __launch_bounds__(256) ld_planes_kernel(const uint8_t* __restric
     const uint8_t* row = packed + k * row_bytes + (s0 >> 2);
     const int64_t left = row_bytes - (s0 >> 2);
     uint64_t w = 0;
+    if (left >= 8 && (reinterpret_cast<uintptr_t>(row) & 7) == 0) {
+      w = __ldg(reinterpret_cast<const unsigned long long*>(row));
+    } else {
 #pragma unroll
-    for (int q = 0; q < 8; ++q) w |= (uint64_t)(q < left ? __ldg(row + q) : 0x55u) << (8 * q);
+      for (int q = 0; q < 8; ++q) w |= (uint64_t)(q < left ? __ldg(row + q) : 0x55u) << (8 * q);
+    }
     const uint32_t lo = even_bits(w), hi = even_bits(w >> 1);  // code bit 0, code bit 1 of 32 samples
     const uint32_t valid = n - s0 >= 32 ? 0xFFFFFFFFu : ((1u << (uint32_t)(n - s0)) - 1u);
     pres = (hi | ~lo) & valid;   // code != 1
@@ -127,10 +130,6 @@ __global__ void __launch_bounds__(256) ld_planes_kernel(const uint8_t* __restric
   *reinterpret_cast<uint4*>(base + 0 * kTileBytes) = make_uint4(wx[0], wx[1], wx[2], wx[3]);
   *reinterpret_cast<uint4*>(base + 1 * kTileBytes) = make_uint4(wv[0], wv[1], wv[2], wv[3]);
   *reinterpret_cast<uint4*>(base + 2 * kTileBytes) = make_uint4(wh[0], wh[1], wh[2], wh[3]);
-  uint8_t* bb = planes_b + (size_t)((b * 2 + (r >> 6)) * n_chunks + c) * kLdHalfChunkBytes + tile_off(r & 63, 16 * half);
-  *reinterpret_cast<uint4*>(bb + 0 * kLdHalfBytes) = make_uint4(wx[0], wx[1], wx[2], wx[3]);
-  *reinterpret_cast<uint4*>(bb + 1 * kLdHalfBytes) = make_uint4(wv[0], wv[1], wv[2], wv[3]);
-  *reinterpret_cast<uint4*>(bb + 2 * kLdHalfBytes) = make_uint4(wh[0], wh[1], wh[2], wh[3]);
 }
 
 // r from the six exact sums, oriented by the two markers' signs; NaN when N = 0
@@ -235,7 +234,6 @@ __device__ __forceinline__ double ld_r_value(int32_t N, int32_t sx, int32_t sy, 
 
 struct LdArgs {
   const uint8_t* planes;    // A layout
-  const uint8_t* planes_b;  // B layout
   int64_t n_chunks, m, window;
   const int2* items;  // (A marker block, B half-block)
   int64_t n_items;
@@ -245,6 +243,15 @@ struct LdArgs {
   int* counter;
   int* status;
 };
+
+__device__ __forceinline__ void tma_load_4d(void* dst, const CUtensorMap* map, int x0, int x1, int x2, int x3,
+                                            uint64_t* bar) {
+  asm volatile(
+      "cp.async.bulk.tensor.4d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4, %5}], "
+      "[%6];" ::"r"(smem_addr(dst)),
+      "l"(reinterpret_cast<uint64_t>(map)), "r"(x0), "r"(x1), "r"(x2), "r"(x3), "r"(smem_addr(bar))
+      : "memory");
+}
 
 __device__ __forceinline__ void tmem_ld8(uint32_t taddr, uint32_t (&r)[8]) {
   asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
@@ -261,7 +268,7 @@ __device__ __forceinline__ void tmem_ld8(uint32_t taddr, uint32_t (&r)[8]) {
 // call took 2.33 ms (4,096 samples x 100,000 markers, window 1,000); 1.74 with
 // 8 epilogue warps, 1.67 with 16 (and 1.58 with three MMA warps instead of two).
 template <bool kSmall>
-__global__ void __launch_bounds__(kLdThreads, 1) tc_ld_kernel(const LdArgs args) {
+__global__ void __launch_bounds__(kLdThreads, 1) tc_ld_kernel(const __grid_constant__ CUtensorMap bmap, const LdArgs args) {
   extern __shared__ __align__(1024) uint8_t smem_raw[];
   uint8_t* ring = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   __shared__ __align__(8) uint64_t full[kLdStages], empty[kLdStages], tfull, tempty, drain;
@@ -334,8 +341,8 @@ __global__ void __launch_bounds__(kLdThreads, 1) tc_ld_kernel(const LdArgs args)
         if (it < 0) break;
         const int2 item = args.items[it];
         const uint8_t* a = args.planes + (size_t)item.x * nk * kLdChunkBytes;
-        const uint8_t* b = args.planes_b + (size_t)item.y * nk * kLdHalfChunkBytes;
-        for (int64_t k = 0; k < nk; k += kLdPer, a += kLdPer * kLdChunkBytes, b += kLdPer * kLdHalfChunkBytes) {
+        int b = (int)((item.y >> 1) * nk);  // chunk of the B half-block's block
+        for (int64_t k = 0; k < nk; k += kLdPer, a += kLdPer * kLdChunkBytes, b += kLdPer) {
           if (g >= (uint32_t)kLdStages && !ring_wait(&empty[s], ph, kWaitLimitNs, &abort_flag)) {
             ok = false;
             break;
@@ -343,7 +350,7 @@ __global__ void __launch_bounds__(kLdThreads, 1) tc_ld_kernel(const LdArgs args)
           uint8_t* dst = ring + (size_t)s * kLdStageBytes;
           mbar_arrive_expect_tx(&full[s], kLdStageBytes);
           bulk_g2s(dst, a, kLdPer * kLdChunkBytes, &full[s]);
-          bulk_g2s(dst + kLdPer * kLdChunkBytes, b, kLdPer * kLdHalfChunkBytes, &full[s]);
+          tma_load_4d(dst + kLdPer * kLdChunkBytes, &bmap, 0, item.y & 1, 0, b, &full[s]);
           ++g;
           if (++s == kLdStages) {
             s = 0;
@@ -517,13 +524,27 @@ __global__ void ld_fill_tail_kernel(int64_t m, int64_t window, double* __restric
   }
 }
 
+// The planes as 64-bit elements, [block x chunk][plane][half-block][256]: a box is
+// one half-block's rows of kLdPer chunks.
+bool encode_ld_map(CUtensorMap* map, const void* planes, int64_t chunks) {
+  const EncodeTiledFn fn = encode_tiled_fn();
+  if (!fn) return false;
+  const cuuint64_t dims[4] = {256, 2, kLdPlanes, (cuuint64_t)chunks};
+  const cuuint64_t strides[3] = {(cuuint64_t)kLdHalfBytes, (cuuint64_t)kTileBytes, (cuuint64_t)kLdChunkBytes};
+  const cuuint32_t box[4] = {256, 1, kLdPlanes, kLdPer};
+  const cuuint32_t elem[4] = {1, 1, 1, 1};
+  return fn(map, CU_TENSOR_MAP_DATA_TYPE_UINT64, 4, const_cast<void*>(planes), dims, strides, box, elem,
+            CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+            CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
 }  // namespace
 
 // Sample chunks: ceil(n / 64), padded to a multiple of kLdPer with zero chunks.
 static int64_t ld_chunks(int64_t n) { return ((n + 63) / 64 + kLdPer - 1) / kLdPer * kLdPer; }
 
-size_t ld_planes_bytes(int64_t n, int64_t m) {  // A layout, then B layout
-  return (size_t)((m + kTB - 1) / kTB) * (size_t)ld_chunks(n) * (kLdChunkBytes + 2 * kLdHalfChunkBytes);
+size_t ld_planes_bytes(int64_t n, int64_t m) {
+  return (size_t)((m + kTB - 1) / kTB) * (size_t)ld_chunks(n) * kLdChunkBytes;
 }
 
 // Items of the band: (A block I of 128 markers, B half-block j of 64 markers)
@@ -543,20 +564,20 @@ cudaError_t launch_ld(const uint8_t* packed, int64_t n, int64_t m, int64_t windo
                       const int2* items, int64_t n_items, int* counter, double* out_r, int32_t* out_n,
                       int* status, int num_sms, cudaStream_t st) {
   const int64_t nc = ld_chunks(n), nb = (m + kTB - 1) / kTB;
-  if (nc > 2147483647LL || nb > 65535 || n_items > 2147483647LL - num_sms) return cudaErrorInvalidValue;
-  uint8_t* planes_b = planes + (size_t)nb * nc * kLdChunkBytes;
+  if (nc > 2147483647LL || nb > 65535 || nb * nc > 2147483647LL || n_items > 2147483647LL - num_sms) return cudaErrorInvalidValue;
   cudaError_t e = cudaMemsetAsync(diff, 0, (size_t)m * sizeof(int32_t), st);
   if (e != cudaSuccess) return e;
-  ld_planes_kernel<<<dim3((unsigned)nc, (unsigned)nb), 256, 0, st>>>(packed, (n + 3) / 4, n, m, planes, planes_b, nc,
-                                                                      diff);
+  ld_planes_kernel<<<dim3((unsigned)nc, (unsigned)nb), 256, 0, st>>>(packed, (n + 3) / 4, n, m, planes, nc, diff);
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
   if ((e = cudaMemsetAsync(counter, 0, sizeof(int), st)) != cudaSuccess) return e;
   auto kern = n < (1 << 15) ? tc_ld_kernel<true> : tc_ld_kernel<false>;
   if ((e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kLdSmem)) != cudaSuccess)
     return e;
-  LdArgs args{planes, planes_b, nc, m, window, items, n_items, diff, out_r, out_n, counter, status};
+  LdArgs args{planes, nc, m, window, items, n_items, diff, out_r, out_n, counter, status};
   if (n_items > 0) {
-    kern<<<(int)std::min<int64_t>(num_sms, n_items), kLdThreads, kLdSmem, st>>>(args);
+    CUtensorMap bmap;
+    if (!encode_ld_map(&bmap, planes, nb * nc)) return cudaErrorInvalidValue;
+    kern<<<(int)std::min<int64_t>(num_sms, n_items), kLdThreads, kLdSmem, st>>>(bmap, args);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
   }
   ld_fill_tail_kernel<<<64, 256, 0, st>>>(m, window, out_r, out_n);
