@@ -1598,7 +1598,7 @@ extern "C" ibs_status ibs_cluster_complete(ibs_ctx* ctx, const double* dist, int
   if (ibs_status s = ensure_buf(ctx, ctx->cluster_work, cluster_workspace_bytes(n))) return s;
   IBS_CUDA_TRY(launch_cluster_complete(dist, n, out_z, ctx->cluster_work.p, ctx->num_sms,
                                        static_cast<cudaStream_t>(stream)));
-  ctx->last_info[0] = 4;
+  ctx->last_info[0] = cluster_launches(n);
   ctx->last_info[1] = n - 1;
   ctx->last_info[2] = 1;
   return IBS_OK;

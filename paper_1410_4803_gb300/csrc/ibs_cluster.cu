@@ -23,7 +23,8 @@
 //      unrelated samples).  A rescan needs nothing of the update: by symmetry
 //      row r holds both D[r][i] and D[r][j], whose max it takes in column i's
 //      place.  So a merge waits for memory once, for both together.
-// The steps form one persistent CTA of 1,024 threads (32 warps); phases are
+// The steps form one CTA of 1,024 threads (32 warps), launched again each time a
+// quarter of the rows and columns has been merged away and dropped; phases are
 // separated by block barriers, which also order the memory updates.  Up to
 // kClSmemRows samples the row minima and flags sit in shared memory.  The
 // working matrix is square and symmetric in HBM.  It holds order-preserving
@@ -34,11 +35,12 @@
 //
 // What bounds it: latency.  The merges are a serial chain, each one round of
 // loads (700 cycles from L2, more from HBM) and four block barriers.
-// Measured, n = 4,096 unrelated samples: 31.3 ms, 7.6 us per merge (34.3 ms with the
-// rescans after the update); 125.1 ms with one warp per
-// rescanned row, a check of every flag before the next load of a row, FP64
-// shuffle trees and rescans after the update.
+// Measured, n = 4,096 unrelated samples: 24.2 ms, 5.9 us per merge; 31.4 ms over
+// all columns to the end (see cl_next); 34.3 ms with the rescans after the
+// update; 125.1 ms with one warp per rescanned row, a check of every flag before
+// the next load of a row, FP64 shuffle trees and rescans after the update.
 #include <cstdint>
+#include <type_traits>
 
 #include "ibs_device.cuh"
 #include "ibs_internal.h"
@@ -135,19 +137,22 @@ __global__ void cl_rowmin_kernel(const uint64_t* __restrict__ D, int64_t n, uint
 
 struct ClArgs {
   uint64_t* D;
-  int64_t n;
+  int64_t ld;     // row stride: the samples of the call
+  int64_t n;      // rows and columns still there
+  int32_t step0, steps;  // merges before this launch, and of it
   uint64_t* rk;   // row minima: key (kNoKey: merged away, or no active column to the right)
   uint32_t* rj;   // and column
   uint8_t* active;
-  uint32_t* list;  // rows to rescan after a merge
+  uint32_t* list;  // rows to rescan after a merge (not kSmem)
+  uint16_t* phys;  // kSmem: row r of the n is row phys[r] of D
   int32_t* id;
   int32_t* size;
   double* Z;  // [n-1][4]
 };
 
-// Row minima, activity flags and the rescan list live in shared memory when
-// they fit (17 bytes per sample, up to kClSmemRows samples), so that the
-// per-step argmin and the rescan checks touch no global memory.
+// Row minima, activity flags, the rescan list and the rows' places live in
+// shared memory when they fit (17 bytes per sample, up to kClSmemRows samples),
+// so that the per-step argmin and the rescan checks touch no global memory.
 constexpr int64_t kClSmemRows = 12000;
 constexpr size_t cl_smem_bytes(int64_t n) { return n <= kClSmemRows ? (size_t)n * 17 + 16 : 0; }
 
@@ -164,17 +169,22 @@ __global__ void __launch_bounds__(kClThreads, 1) cl_main_kernel(ClArgs a) {
   __shared__ uint32_t s_cnt[2];
   const int n = (int)a.n;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  using List = std::conditional_t<kSmem, uint16_t, uint32_t>;
   uint64_t* rk;
-  uint32_t *rj, *list;
+  uint32_t* rj;
+  List* list;
+  uint16_t* phys = nullptr;
   uint8_t* active;
   if constexpr (kSmem) {
     rk = reinterpret_cast<uint64_t*>(cl_smem);
     rj = reinterpret_cast<uint32_t*>(cl_smem + (size_t)n * 8);
-    list = reinterpret_cast<uint32_t*>(cl_smem + (size_t)n * 12);
+    list = reinterpret_cast<uint16_t*>(cl_smem + (size_t)n * 12);
+    phys = reinterpret_cast<uint16_t*>(cl_smem + (size_t)n * 14);
     active = cl_smem + (size_t)n * 16;
     for (int r = tid; r < n; r += kClThreads) {
       rk[r] = a.rk[r];
       rj[r] = a.rj[r];
+      phys[r] = a.phys[r];
       active[r] = a.active[r];
     }
   } else {
@@ -183,9 +193,10 @@ __global__ void __launch_bounds__(kClThreads, 1) cl_main_kernel(ClArgs a) {
     list = a.list;
     active = a.active;
   }
+  auto row_of = [&](int r) { return a.D + (size_t)(kSmem ? (int)phys[r] : r) * a.ld; };
   if (tid < 2) s_cnt[tid] = 0;
   __syncthreads();
-  for (int step = 0; step + 1 < n; ++step) {
+  for (int step = 0; step < a.steps; ++step) {
     // 1. global minimum over the row minima: (value, row) lexicographic
     uint64_t k = kNoKey;
     uint32_t b = kNoIdx;
@@ -207,8 +218,8 @@ __global__ void __launch_bounds__(kClThreads, 1) cl_main_kernel(ClArgs a) {
     b = s_i[lane];
     warp_best(k, b);  // every warp has the result
     const int i0 = (int)b, j0 = (int)rj[b];
-    const uint64_t* Di = a.D + (size_t)i0 * n;
-    const uint64_t* Dj = a.D + (size_t)j0 * n;
+    uint64_t* Di = row_of(i0);
+    const uint64_t* Dj = row_of(j0);
     // the update's first loads, in flight while the list is made
     uint64_t di[kClUpd], dj[kClUpd];
     auto load_update = [&](int c0) {
@@ -228,7 +239,7 @@ __global__ void __launch_bounds__(kClThreads, 1) cl_main_kernel(ClArgs a) {
 #pragma unroll 4
     for (int c = tid; c < n; c += kClThreads) {
       const int cj = (int)rj[c];
-      if ((cj == j0 && c != i0) || cj == i0) list[atomicAdd(cnt, 1u)] = (uint32_t)c;
+      if ((cj == j0 && c != i0) || cj == i0) list[atomicAdd(cnt, 1u)] = (List)c;
     }
     __syncthreads();
     const uint32_t L = *cnt;
@@ -237,7 +248,7 @@ __global__ void __launch_bounds__(kClThreads, 1) cl_main_kernel(ClArgs a) {
     const int gw = L <= 4 ? 8 : (L <= 8 ? 4 : (L <= 16 ? 2 : 1));
     for (uint32_t t = (uint32_t)(warp / gw); t < L; t += kWarps / gw) {
       const int r = (int)list[t];
-      const uint64_t* Dr = a.D + (size_t)r * n;
+      const uint64_t* Dr = row_of(r);
       const int stride = 32 * gw;
       uint64_t sk = kNoKey;
       uint32_t si = kNoIdx;
@@ -285,8 +296,8 @@ __global__ void __launch_bounds__(kClThreads, 1) cl_main_kernel(ClArgs a) {
         const int c = c0 + q * kClThreads;
         const uint64_t d = di[q] > dj[q] ? di[q] : dj[q];
         if (d != di[q]) {
-          a.D[(size_t)i0 * n + c] = d;
-          st_shared_entry(a.D + (size_t)c * n + i0, d);
+          Di[c] = d;
+          st_shared_entry(row_of(c) + i0, d);
         }
         if (c > i0 && d < uk) {
           uk = d;
@@ -333,23 +344,115 @@ __global__ void __launch_bounds__(kClThreads, 1) cl_main_kernel(ClArgs a) {
     }
     if (tid == kClThreads - 64) {  // the merge itself, off the critical path
       const int32_t ia = a.id[i0], ib = a.id[j0], sz = a.size[i0] + a.size[j0];
-      double* z = a.Z + (size_t)step * 4;
+      double* z = a.Z + (size_t)(a.step0 + step) * 4;
       z[0] = (double)(ia < ib ? ia : ib);
       z[1] = (double)(ia < ib ? ib : ia);
       z[2] = cl_value(k);
       z[3] = (double)sz;
-      a.id[i0] = (int32_t)(n + step);
+      a.id[i0] = (int32_t)(a.ld + a.step0 + step);
       a.size[i0] = sz;
+    }
+    __syncthreads();
+  }
+  if constexpr (kSmem) {  // for cl_compact_kernel
+    for (int r = tid; r < n; r += kClThreads) {
+      a.rk[r] = rk[r];
+      a.rj[r] = rj[r];
+      a.active[r] = active[r];
+    }
+  }
+}
+
+// Between launches of the main kernel: rows and columns merged away are dropped
+// (in order, so ties fall as before).  The arrays move down in place, a chunk at
+// a time: an entry never moves up, so a chunk is read before anything is written
+// over it.  act[c] = old column of new column c.
+__global__ void __launch_bounds__(kClThreads, 1) cl_compact_kernel(ClArgs a, uint16_t* __restrict__ act) {
+  extern __shared__ __align__(16) uint8_t cl_smem[];
+  uint16_t* to = reinterpret_cast<uint16_t*>(cl_smem);  // new index of an old one
+  __shared__ uint32_t s_sum[kClThreads / 32];
+  const int n = (int)a.n, tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  uint32_t before = 0;
+  for (int r0 = 0; r0 < n; r0 += kClThreads) {
+    const int r = r0 + tid;
+    const bool on = r < n && a.active[r] != 0;
+    const uint32_t ballot = __ballot_sync(0xffffffffu, on);
+    if (lane == 0) s_sum[warp] = __popc(ballot);
+    __syncthreads();
+    uint32_t at = before;
+    for (int w = 0; w < kClThreads / 32; ++w) {
+      if (w < warp) at += s_sum[w];
+      before += s_sum[w];
+    }
+    at += __popc(ballot & ((1u << lane) - 1u));
+    if (on) {
+      to[r] = (uint16_t)at;
+      act[at] = (uint16_t)r;
+    }
+    __syncthreads();
+  }
+  for (int r0 = 0; r0 < n; r0 += kClThreads) {
+    const int r = r0 + tid;
+    const bool on = r < n && a.active[r] != 0;
+    uint64_t k = 0;
+    uint32_t j = 0;
+    int32_t id = 0, size = 0;
+    uint16_t phys = 0;
+    if (on) {
+      k = a.rk[r];
+      j = a.rj[r];
+      id = a.id[r];
+      size = a.size[r];
+      phys = a.phys[r];
+    }
+    __syncthreads();
+    if (on) {
+      const int t = to[r];
+      a.rk[t] = k;
+      a.rj[t] = j < (uint32_t)n ? to[j] : j;
+      a.id[t] = id;
+      a.size[t] = size;
+      a.phys[t] = phys;
+    }
+    __syncthreads();
+  }
+  for (int r = tid; r < (int)before; r += kClThreads) a.active[r] = 1;
+}
+
+// ... and the columns of the `left` rows that stay, CTA = row.
+__global__ void __launch_bounds__(256) cl_compact_rows_kernel(ClArgs a, const uint16_t* __restrict__ act, int left) {
+  uint64_t* row = a.D + (size_t)a.phys[blockIdx.x] * a.ld;
+  constexpr int kPer = 8;
+  for (int c0 = threadIdx.x; c0 - (int)threadIdx.x < left; c0 += kPer * 256) {
+    uint64_t v[kPer];
+#pragma unroll
+    for (int q = 0; q < kPer; ++q) {
+      const int c = c0 + q * 256;
+      if (c < left) v[q] = row[act[c]];
+    }
+    __syncthreads();
+#pragma unroll
+    for (int q = 0; q < kPer; ++q) {
+      const int c = c0 + q * 256;
+      if (c < left) row[c] = v[q];
     }
     __syncthreads();
   }
 }
 
-__global__ void cl_state_init_kernel(int64_t n, uint8_t* active, int32_t* id, int32_t* size) {
+// Rows and columns after the next compaction: three quarters, down to 512 (and
+// only where the main kernel's state is in shared memory).  A merge costs 2.9
+// us on average from 256 columns down, 3.7 from 1,024 and 7.7 from 4,096 when
+// none are dropped.  4,096 samples: 24.2 ms against 31.4 (halves: 26.0; seven
+// eighths: 23.7, but more launches for the smaller matrices).
+int64_t cl_next(int64_t n) { return n <= 512 || n > kClSmemRows ? 1 : n * 3 / 4; }
+
+__global__ void cl_state_init_kernel(int64_t n, uint8_t* active, int32_t* id, int32_t* size, uint16_t* phys) {
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
     active[i] = 1;
     id[i] = (int32_t)i;
     size[i] = 1;
+    if (phys != nullptr) phys[i] = (uint16_t)i;
   }
 }
 
@@ -381,18 +484,38 @@ cudaError_t launch_cluster_complete(const double* tri, int64_t n, double* Z, voi
   cl_init_kernel<<<dim3(T, T), 256, 0, st>>>(tri, n, D);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
-  cl_state_init_kernel<<<grid, 256, 0, st>>>(n, active, id, size);
+  // (kSmem does not use the list in global memory)
+  const bool small = n <= kClSmemRows;
+  uint16_t *phys = small ? reinterpret_cast<uint16_t*>(list) : nullptr, *act = small ? phys + n : nullptr;
+  cl_state_init_kernel<<<grid, 256, 0, st>>>(n, active, id, size, phys);
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
   cl_rowmin_kernel<<<grid, 256, 0, st>>>(D, n, rk, rj);
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
-  ClArgs args{D, n, rk, rj, active, list, id, size, Z};
-  const size_t smem = cl_smem_bytes(n);
-  auto kern = n <= kClSmemRows ? cl_main_kernel<true> : cl_main_kernel<false>;
-  if (smem > 48 * 1024 &&
-      (e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) != cudaSuccess)
+  auto kern = small ? cl_main_kernel<true> : cl_main_kernel<false>;
+  if (cl_smem_bytes(n) > 48 * 1024 &&
+      (e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)cl_smem_bytes(n))) != cudaSuccess)
     return e;
-  kern<<<1, kClThreads, smem, st>>>(args);
-  return cudaGetLastError();
+  for (int64_t left = n; left > 1;) {
+    const int64_t next = cl_next(left);
+    const ClArgs args{D, n, left, (int32_t)(n - left), (int32_t)(left - next), rk, rj, active, list, phys, id, size, Z};
+    kern<<<1, kClThreads, cl_smem_bytes(left), st>>>(args);
+    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    if (next > 1) {
+      cl_compact_kernel<<<1, kClThreads, (size_t)left * 2, st>>>(args, act);
+      if ((e = cudaGetLastError()) != cudaSuccess) return e;
+      cl_compact_rows_kernel<<<(unsigned)next, 256, 0, st>>>(args, act, (int)next);
+      if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    }
+    left = next;
+  }
+  return cudaSuccess;
+}
+
+// Kernel launches of a call.
+int cluster_launches(int64_t n) {
+  int k = 3;
+  for (int64_t left = n; left > 1; left = cl_next(left)) k += cl_next(left) > 1 ? 3 : 1;
+  return k;
 }
 
 }  // namespace ibs

@@ -400,6 +400,7 @@ cudaError_t launch_grm(const uint8_t* packed, int64_t n, int64_t m, double* out,
 // triangle (ibs_compute's layout), into Z [n-1][4] on the device; `work` holds
 // cluster_workspace_bytes(n).
 size_t cluster_workspace_bytes(int64_t n);
+int cluster_launches(int64_t n);
 cudaError_t launch_cluster_complete(const double* tri, int64_t n, double* Z, void* work, int num_sms,
                                     cudaStream_t st);
 

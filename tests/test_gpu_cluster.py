@@ -72,6 +72,19 @@ def test_larger_matrix(ctx):
     np.testing.assert_array_equal(_gpu(ctx, tri, n), oracle.complete_linkage(tri, n))
 
 
+# around the sizes where merged rows and columns are dropped (three quarters left,
+# down to 512), with ties, infinities and rows that drop out of the last chunk
+@pytest.mark.parametrize("n", [512, 513, 514, 683, 684, 685, 1025, 1367])
+def test_compaction(ctx, n):
+    rng = np.random.default_rng(n)
+    D = np.round(rng.random((n, n)), 2)
+    D = np.maximum(D, D.T)
+    D[:, 5] = D[5, :] = np.nan
+    np.fill_diagonal(D, 0)
+    tri = _tri(D)
+    np.testing.assert_array_equal(_gpu(ctx, tri, n), oracle.complete_linkage(tri, n))
+
+
 def test_rejects(ctx):
     import torch
     from paper_1410_4803_gb300 import ibs
