@@ -330,7 +330,8 @@ def run_matrix(args, rank, world, local, name: str, full: bool = True):
     probe = ibs.ibs_probe_int_pipes(ctx)
     kinfo = ibs.ibs_kernel_info(ctx)
     kname = ibs.ibs_compute_kernel(ctx, n, m)
-    two_sm = use_tc and kname == "tc-pair"  # cta_group::2 kernel for long items
+    sweep = use_tc and kinfo["tc_format"] == "e2m1" and m < 1 << 21  # the marker-sweep kernel
+    two_sm = use_tc and kname == "tc-pair"  # without it: the cta_group::2 kernel for long items
     mma_probe = ibs.ibs_probe_mma(ctx) if use_tc else None
 
     with torch.cuda.stream(stream):
@@ -458,9 +459,10 @@ def run_matrix(args, rank, world, local, name: str, full: bool = True):
         mode = "tc-fp4" if fp4 else "tc-fp8"
     # transpose: read the 2-bit input once, write the operand planes (4 planes of one
     # byte (FP8) or half a byte (FP4) per padded genotype)
-    k = 64 if fp4 else 32
-    transpose_bytes = m * ((n + 3) // 4) + ((n + 127) // 128) * 128 * ((m + k - 1) // k) * k * 4 // (2 if fp4 else 1)
-    profile = f"{'tc_pair_kernel' if two_sm else 'tc_kernel_fp4' if fp4 else 'tc_kernel_fp8'}_{name}.md"
+    rows, k = (64, 288) if sweep else (128, 64 if fp4 else 32)
+    transpose_bytes = (m * ((n + 3) // 4) +
+                       ((n + rows - 1) // rows) * rows * ((m + k - 1) // k) * k * 4 // (2 if fp4 else 1))
+    profile = f"{'sweep_kernel' if sweep else 'tc_pair_kernel' if two_sm else 'tc_kernel_fp4' if fp4 else 'tc_kernel_fp8'}_{name}.md"
 
     # oracle block: the CPU baseline and the spot check of the last result
     exact = None
@@ -524,8 +526,11 @@ def run_matrix(args, rank, world, local, name: str, full: bool = True):
                      if not use_tc else
                      {"bound": "tensor", "achieved": 8.0 * achieved / 1e12, "peak": tc_tflops, "unit": "TFLOP/s",
                       "frac": 8.0 * achieved / 1e12 / tc_tflops,
-                      "traffic": profiled_traffic(profile, ("ibs_tc.cu", "ibs_device.cuh", "ibs_tc_common.cuh")),
-                      "kernel": ("tc_pair_kernel (tcgen05 cta_group::2, M = 256 over two SMs, E2M1 kind::mxf4 "
+                      "traffic": profiled_traffic(profile, ("ibs_sweep.cu" if sweep else "ibs_tc.cu", "ibs_device.cuh",
+                                                            "ibs_tc_common.cuh")),
+                      "kernel": ("sweep_kernel (tcgen05 cta_group::2, M = 256 over two SMs, N = 192, K = 96, E2M1 "
+                                 "kind::mxf4 indicator GEMMs)" if sweep else
+                                 "tc_pair_kernel (tcgen05 cta_group::2, M = 256 over two SMs, E2M1 kind::mxf4 "
                                  "indicator GEMMs)" if two_sm else
                                  f"tc_persistent_kernel (tcgen05 {'E2M1 kind::mxf4' if fp4 else 'E4M3 kind::f8f6f4'} "
                                  f"indicator GEMMs)"), "kernel_ms": pairs_ms,
@@ -536,8 +541,9 @@ def run_matrix(args, rank, world, local, name: str, full: bool = True):
                       "mma_probe": {"unit": "TFLOP/s",
                                     "measured": mma_probe["e2m1_tflops" if fp4 else "e4m3_tflops"],
                                     "frac": 8.0 * achieved / 1e12 / mma_probe["e2m1_tflops" if fp4 else "e4m3_tflops"],
-                                    "basis": "ibs_probe_mma: back-to-back 128x128 MMAs of this kind from "
-                                             "shared-memory tiles on all SMs, measured live"}}),
+                                    "basis": "ibs_probe_mma: back-to-back 128x128 MMAs of this kind (E2M1: K = 64) from "
+                                             "shared-memory tiles on all SMs, measured live; the sweep kernel's MMAs "
+                                             "(256x192 over two SMs, K = 96) run at up to 1.5 times that rate"}}),
         "integer_kernel": None if popc is None else {
             "kernel": "tri_kernel, carry-save LOP3/POPC over bit planes (IBS_KERNEL_CSA)",
             "kernel_ms": popc, "value": comps / (popc * 1e-3), "unit": UNIT,

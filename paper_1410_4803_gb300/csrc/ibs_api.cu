@@ -1437,8 +1437,9 @@ extern "C" ibs_status ibs_compute_batch(ibs_ctx* ctx, const uint8_t* pool, int64
                                  : -1;
     // The sweep kernel takes the place of policy 2's launches wherever it can run
     // every subset and no workspace limit is set, and nothing is timed (24
-    // subsets of 100 to 3,000 samples and 5,000 to 80,000 markers: 2.97 ms against
-    // 3.76 with the best of the other policies).
+    // subsets of 100 to 3,000 samples and 5,000 to 80,000 markers: 2.6 ms against
+    // 3.8 with the best of the other policies; 64 of 200 to 8,000 samples and
+    // 10,000 to 200,000 markers: 79 ms against 134).
     bool sweep = tc && ctx->ws_limit == 0 && tc_format_for(ctx) == kTcFp4 && tc_pair_mode() >= 0 && !tc_tile_kernel_forced() &&
                  (fixed_policy < 0 || fixed_policy == 2) &&
                  (te == ctx->tune.end() || te->second.split_policy == 2 || fixed_policy == 2);

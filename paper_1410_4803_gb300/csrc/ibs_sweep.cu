@@ -1098,27 +1098,37 @@ SweepPlan sweep_plan(int64_t n, int64_t m, int clusters) {
   return schedule(full, narrow, clusters, sweep_planes_bytes(n, m));
 }
 
-// Batched subsets, by decreasing marker count: each tile in turn to the least
-// loaded cluster, so that a subset's tiles run at the same time over the same
-// markers and share its planes through L2 (in shares of tiles laid end to
-// end the clusters ran all subsets at once, from HBM: 3.8 ms for 24 subsets of
-// a 10,000 x 200,000 pool); the last tiles, about one per cluster, are cut to
-// even out the end.
+// Batched subsets, by decreasing marker count.  First the whole waves of every
+// subset that has any, one tile per cluster and in lockstep as for one matrix;
+// then the other tiles, each in turn to the least loaded cluster, so that a
+// subset's tiles run at about the same time and share some of its planes through
+// L2 (in shares of tiles laid end to end the clusters ran all subsets at once,
+// from HBM: 3.8 ms for 24 subsets of a 10,000 x 200,000 pool); the last tiles,
+// about one per cluster, are cut to even out the end.  64 subsets of up to 8,000
+// samples and 200,000 markers: 79 ms against 125 without the waves.
 SweepPlan sweep_plan_batch(const std::vector<std::pair<int64_t, int64_t>>& shapes, int clusters) {
   std::vector<size_t> order(shapes.size());
   for (size_t k = 0; k < order.size(); ++k) order[k] = k;
   std::stable_sort(order.begin(), order.end(), [&](size_t a, size_t b) { return shapes[a].second > shapes[b].second; });
+  SweepPlan pl;
+  const size_t C = (size_t)std::max(1, clusters);
+  std::vector<std::vector<SweepItem>> own(C);
+  std::vector<double> load(C, 0.0);
   std::vector<Tile> all;
   for (size_t k : order) {
     std::vector<Tile> full, narrow;
     triangle_tiles(shapes[k].first, sweep_stages(shapes[k].second), (int)k, full, narrow);
-    all.insert(all.end(), full.begin(), full.end());
+    const size_t whole = full.size() / C * C;
+    for (size_t t = 0; t < whole; ++t) {
+      own[t % C].push_back(whole_item(full[t], pl.waves + (int)(t / C)));
+      load[t % C] += tile_cost(full[t]);
+      pl.wave_stages = std::max(pl.wave_stages, 4 * full[t].stages);
+    }
+    pl.waves += (int)(whole / C);
+    all.insert(all.end(), full.begin() + (long)whole, full.end());
     all.insert(all.end(), narrow.begin(), narrow.end());
   }
-  SweepPlan pl;
-  const size_t C = (size_t)std::max(1, clusters), lead = all.size() > C ? all.size() - C : 0;
-  std::vector<std::vector<SweepItem>> own(C);
-  std::vector<double> load(C, 0.0);
+  const size_t lead = all.size() > C ? all.size() - C : 0;
   for (size_t t = 0; t < lead; ++t) {
     const size_t c = (size_t)(std::min_element(load.begin(), load.end()) - load.begin());
     own[c].push_back(whole_item(all[t], -1));
