@@ -83,6 +83,14 @@ __device__ __forceinline__ uint64_t sweep_desc(uint32_t saddr, uint32_t col) {
          (uint64_t)1 << 46;
 }
 
+// Programmatic dependent launch: the operand builder, the sweeps and the sums of
+// a call follow each other without draining the machine in between; each starts
+// its set-up when the one before lets it and waits here until that one's results
+// are complete.  256 samples x 4,096 markers: 47 -> 42 us from Python, 1,501 x
+// 30,011 101 -> 98.
+__device__ __forceinline__ void wait_for_previous() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void let_next_start() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
 // The 16 bytes (64 samples) from byte0 on of marker row `marker` of `m`: any
 // alignment; beyond the row or the matrix, missing.
 __device__ __forceinline__ void sweep_row64(const uint8_t* __restrict__ packed, int64_t row_bytes, int64_t marker,
@@ -134,6 +142,7 @@ __device__ __forceinline__ void sweep_row64(const uint8_t* __restrict__ packed, 
 __global__ void __launch_bounds__(256) sweep_planes_kernel(const uint8_t* __restrict__ packed, int64_t row_bytes,
                                                            int64_t n, int64_t m, uint8_t* __restrict__ planes,
                                                            int64_t n_half, int64_t n_cols) {
+  let_next_start();
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int64_t c = blockIdx.x, h = (int64_t)blockIdx.y * 8 + warp;
   if (h >= n_half) return;
@@ -351,6 +360,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kSwThreads, 1)
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   cluster_sync_all();  // both CTAs' barriers initialised and scale factors stored
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+  wait_for_previous();
 
   // S stages of V V^T, S of U U^T, 2 S of Q R^T + R Q^T: the end of stage q's
   // product, or of the item
@@ -566,6 +576,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kSwThreads, 1)
       }
     }
   }
+  let_next_start();
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncthreads();
   cluster_sync_all();  // both CTAs have issued their last copy and the even CTA's MMAs are drained
@@ -604,6 +615,7 @@ __global__ void __launch_bounds__(128) sweep_finalize_kernel(const SweepGroup* _
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int t = blockIdx.y * 4 + warp;  // 2 CTAs x 4 row quarters x 24 column pieces
   const int ct = t % 24, quarter = (t / 24) & 3, rank = t / 96;
+  wait_for_previous();
   if (ct >= 8 * gr.w) return;
   const float* src = part + (size_t)(2 * gr.slot + rank) * kSwHalfTile + (size_t)ct * 16 * kTB + quarter * 32 + lane;
   const int first[3] = {0, gr.pieces[0], gr.pieces[0] + gr.pieces[1]};
@@ -988,14 +1000,25 @@ cudaError_t launch_sweep_w(const W& work, const SweepLaunch& l, cudaStream_t st)
   cudaError_t e = cudaFuncSetAttribute(sweep_kernel<W>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSwSmem);
   if (e != cudaSuccess) return e;
   const SweepArgs args{l.items, l.first, l.scratch, l.part, l.status, l.wait_ns, l.sync};
-  sweep_kernel<W><<<2 * l.clusters, kSwThreads, kSwSmem, st>>>(work, args);
-  if ((e = cudaGetLastError()) != cudaSuccess || l.n_groups <= 0) return e;
+  cudaLaunchAttribute early = {};
+  early.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  early.val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)(2 * l.clusters));
+  cfg.blockDim = dim3(kSwThreads);
+  cfg.dynamicSmemBytes = kSwSmem;
+  cfg.stream = st;
+  cfg.attrs = &early;
+  cfg.numAttrs = 1;
+  if ((e = cudaLaunchKernelEx(&cfg, sweep_kernel<W>, work, args)) != cudaSuccess || l.n_groups <= 0) return e;
   if (l.between) {
     e = cudaEventRecord(l.between, st);
     if (e != cudaSuccess) return e;
   }
-  sweep_finalize_kernel<W><<<dim3((unsigned)l.n_groups, 48), 128, 0, st>>>(l.groups, l.part, work);
-  return cudaGetLastError();
+  cfg.gridDim = dim3((unsigned)l.n_groups, 48);
+  cfg.blockDim = dim3(128);
+  cfg.dynamicSmemBytes = 0;
+  return cudaLaunchKernelEx(&cfg, sweep_finalize_kernel<W>, l.groups, l.part, work);
 }
 
 }  // namespace
