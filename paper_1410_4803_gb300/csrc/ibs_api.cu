@@ -266,9 +266,10 @@ static ibs_status compute_sweep(ibs_ctx* ctx, const uint8_t* packed, int64_t n, 
     rec.n = split ? 4 : 3;
     IBS_CUDA_TRY(cudaEventRecord(rec.ev[0], st));
   }
+  // (the counters first: the sweeps' programmatic launch follows a kernel)
+  if (sync_bytes > 0) IBS_CUDA_TRY(cudaMemsetAsync(sync.ctr, 0, sync_bytes, st));
   IBS_CUDA_TRY(launch_sweep_planes(packed, n, m, static_cast<uint8_t*>(ctx->planes.p), st));
   if (timing) IBS_CUDA_TRY(cudaEventRecord(rec.ev[1], st));
-  if (sync_bytes > 0) IBS_CUDA_TRY(cudaMemsetAsync(sync.ctr, 0, sync_bytes, st));
   SweepLaunch l;
   l.items = static_cast<const SweepItem*>(ctx->sweep_items.p);
   l.first = static_cast<const int32_t*>(ctx->sweep_first.p);

@@ -176,17 +176,6 @@ __device__ __forceinline__ bool ring_wait(uint64_t* bar, uint32_t parity, unsign
   return ring_wait_slow(bar, parity, limit_ns, abort_flag);
 }
 
-// A waiter warp's release of a ring slot to the MMA warp: one hardware barrier
-// per slot, on which the waiter arrives without blocking and the MMA warp
-// waits.  The waiter cannot arrive on a slot's barrier again before the MMA
-// warp has passed it: the slot is filled again only after its MMAs.
-__device__ __forceinline__ void ring_release(uint32_t id) {
-  asm volatile("barrier.cta.arrive %0, 64;" ::"r"(id) : "memory");
-}
-__device__ __forceinline__ void ring_acquire(uint32_t id) {
-  asm volatile("barrier.cta.sync %0, 64;" ::"r"(id) : "memory");
-}
-
 // ---------------------------------------------------------------------------
 // Clusters of two CTAs (the two-SM kernels).
 __device__ __forceinline__ uint32_t cluster_rank() {

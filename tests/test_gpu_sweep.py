@@ -107,3 +107,27 @@ def test_square(ctx, n, m):
     c = tri_c.astype(np.float64)
     with np.errstate(invalid="ignore"):
         np.testing.assert_array_equal(tri_d, (c[:, 1] + 2 * c[:, 0]) / (2 * c[:, 3]))
+
+
+@pytest.mark.parametrize("n,m", [(130, 1_000), (3201, 600)])  # parts only; whole waves with lockstep counters
+def test_recorded_into_a_graph(ctx, n, m):
+    """A call of a shape seen before, captured and replayed on new genotypes."""
+    import torch
+    from paper_1410_4803_gb300 import ibs
+    rng = np.random.default_rng(n)
+    packed = torch.from_numpy(pack_codes(random_codes(rng, n, m))).cuda()
+    counts = torch.empty((n * (n + 1) // 2, 4), dtype=torch.int32, device="cuda")
+    dist = torch.empty(n * (n + 1) // 2, dtype=torch.float64, device="cuda")
+    ibs.ibs_compute(ctx, packed, n, m, counts, dist)
+    ibs.ibs_synchronize(ctx)
+    graph, stream = torch.cuda.CUDAGraph(), torch.cuda.Stream()
+    with torch.cuda.graph(graph, stream=stream, capture_error_mode="thread_local"):
+        ibs.ibs_compute(ctx, packed, n, m, counts, dist, stream=stream)
+    again = pack_codes(random_codes(rng, n, m, miss=0.1))
+    packed.copy_(torch.from_numpy(again))
+    counts.fill_(-7)
+    graph.replay()
+    torch.cuda.synchronize()
+    want_c, want_d = oracle.ibs_triangle(again, n, m)
+    assert (counts.cpu().numpy() == want_c).all()
+    assert_dist_close(dist.cpu().numpy(), want_d)
