@@ -30,16 +30,14 @@
 // (128 x 32-byte FP16 tiles) and V' of its 32 markers as one E4M3 tile, in
 // the canonical K-major layout (20 KiB).  Tensor memory: numerator banks at
 // columns 0 and 128, the count at 256, the float-float high words at 384.
-// One persistent CTA per SM, 19 warps: warp 16 claims triangle tiles in the
+// One persistent CTA per SM, 10 warps: warp 8 claims triangle tiles in the
 // grouped order and streams both blocks' chunks through a ring of two stages
 // of four chunks (one 40 KiB bulk copy per block and stage: the copy engine
 // spends a fixed time per copy, measured near 340 cycles, so one chunk per
-// stage ran 1.6x slower); warp 17 issues 3 kind::f16 MMAs per chunk and one
-// kind::f8f6f4 MMA (the counts) per pair, released per stage by warp 18, which
-// waits on memory for it; warps 0..15 fold segments (warp w: TMEM lanes of
-// quarter w % 4, columns 32 (w / 4) .. +31) and store A.  With 8 warps of 64
-// columns a fold outlasts a segment's MMAs: 6.24 ms a call against 6.02 (4,096
-// samples x 100,000 markers).  Every wait is bounded (2 s of %globaltimer).
+// stage ran 1.6x slower); warp 9 issues 3 kind::f16 MMAs per chunk and one
+// kind::f8f6f4 MMA (the counts) per pair; warps 0..7 fold segments (warp w:
+// TMEM lanes of quarter w % 4, columns 64 (w / 4) .. +63) and store A.  Every
+// wait is bounded (2 s of %globaltimer).
 #include <algorithm>
 #include <cuda_fp16.h>
 #include <vector>
@@ -62,7 +60,7 @@ constexpr int kGrmPad = 4;                               // chunk count padded t
 constexpr int kGrmQueue = 8;
 constexpr int kGrmSeg = 8;                               // chunks per numerator segment
 static_assert(kGrmSeg % kGrmPad == 0, "a ring stage never straddles two segments");
-constexpr int kGrmEpiWarps = 16;
+constexpr int kGrmEpiWarps = 8;
 constexpr int kGrmThreads = (kGrmEpiWarps + 3) * 32;
 constexpr int kGrmCopyWarp = kGrmEpiWarps, kGrmMmaWarp = kGrmEpiWarps + 1, kGrmWaitWarp = kGrmEpiWarps + 2;
 // Hardware barrier between the waiter warp and the MMA warp (barrier 0 is
@@ -474,7 +472,7 @@ __global__ void __launch_bounds__(kGrmThreads, 1) tc_grm_kernel(const GrmArgs ar
   } else if (warp < kGrmEpiWarps) {
     const int quarter = warp & 3, half = warp >> 2;
     const int row = quarter * 32 + lane;
-    const uint32_t tl = tmem + ((uint32_t)(quarter * 32) << 16) + 32u * half;
+    const uint32_t tl = tmem + ((uint32_t)(quarter * 32) << 16) + 64u * half;
     uint32_t gs = 0;
     bool stop = false;
     for (uint32_t e = 0; !stop; ++e) {
@@ -486,9 +484,7 @@ __global__ void __launch_bounds__(kGrmThreads, 1) tc_grm_kernel(const GrmArgs ar
       if (it < 0) break;
       const GrmItem t = args.items[it];
       const int64_t nseg = (t.c1 - t.c0 + kGrmSeg - 1) / kGrmSeg;
-      float lo[32];
-#pragma unroll
-      for (int j = 0; j < 32; ++j) lo[j] = 0.0f;
+      float lo[64];
       for (int64_t sg = 0; sg < nseg; ++sg, ++gs) {
         const uint32_t b = gs & 1u;
         const bool ok = mbar_wait_bounded(&seg_full[b], (gs >> 1) & 1u);
@@ -498,15 +494,18 @@ __global__ void __launch_bounds__(kGrmThreads, 1) tc_grm_kernel(const GrmArgs ar
         }
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
 #pragma unroll
-        for (int h = 0; h < 2; ++h) {  // 16 columns at a time
+        for (int h = 0; h < 4; ++h) {  // 16 columns at a time
           uint32_t vn[16], vh[16];
           tmem_ld16(tl + kColNum + 128u * b + 16 * h, vn);
           if (sg > 0) tmem_ld16(tl + kColHi + 16 * h, vh);
           asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-          if (h == 1) arrive(&seg_free[b]);
+          if (h == 3) arrive(&seg_free[b]);
           if (sg == 0) {
 #pragma unroll
-            for (int j = 0; j < 16; ++j) vh[j] = vn[j];
+            for (int j = 0; j < 16; ++j) {
+              vh[j] = vn[j];
+              lo[16 * h + j] = 0.0f;
+            }
           } else {
 #pragma unroll
             for (int j = 0; j < 16; ++j) {
@@ -526,24 +525,19 @@ __global__ void __launch_bounds__(kGrmThreads, 1) tc_grm_kernel(const GrmArgs ar
       // the item's last segment is folded: read the counts, hand the count
       // accumulator back, then divide and store (a split item stores its sums)
       const int64_t gi = (int64_t)t.I * kTB + row;
-      const int64_t j0 = (int64_t)t.J * kTB + 32 * half;
-      // (through local memory: an unrolled loop would keep the quotients of many
-      // columns in registers)
-      float low[32];
+      const int64_t j0 = (int64_t)t.J * kTB + 64 * half;
 #pragma unroll
-      for (int j = 0; j < 32; ++j) low[j] = lo[j];
-#pragma unroll 1
-      for (int h = 0; h < 2; ++h) {
+      for (int h = 0; h < 4; ++h) {
         uint32_t vc[16], vh[16];
         tmem_ld16(tl + kColCnt + 16 * h, vc);
         tmem_ld16(tl + kColHi + 16 * h, vh);
         asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-        if (h == 1) arrive(&cnt_free);
+        if (h == 3) arrive(&cnt_free);
         if (t.part >= 0) {
-          const size_t base = (size_t)t.part * kTB * kTB + (size_t)row * kTB + 32 * half + 16 * h;
+          const size_t base = (size_t)t.part * kTB * kTB + (size_t)row * kTB + 64 * half + 16 * h;
 #pragma unroll
           for (int j = 0; j < 16; ++j) {
-            args.part_num[base + j] = (double)__uint_as_float(vh[j]) + (double)low[16 * h + j];
+            args.part_num[base + j] = (double)__uint_as_float(vh[j]) + (double)lo[16 * h + j];
             args.part_cnt[base + j] = __uint_as_float(vc[j]);
           }
         } else if (gi < args.n) {
@@ -552,7 +546,7 @@ __global__ void __launch_bounds__(kGrmThreads, 1) tc_grm_kernel(const GrmArgs ar
             const int64_t gj = j0 + 16 * h + j;
             if (gj >= args.n || gj < gi) continue;
             const float cnt = __uint_as_float(vc[j]);
-            const double num = (double)__uint_as_float(vh[j]) + (double)low[16 * h + j];
+            const double num = (double)__uint_as_float(vh[j]) + (double)lo[16 * h + j];
             args.out[tri_index(gi, gj, args.n)] =
                 cnt == 0.0f ? __longlong_as_double(0x7ff8000000000000LL) : div_count(num, cnt);
           }
