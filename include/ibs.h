@@ -373,8 +373,9 @@ ibs_status ibs_kernel_info(ibs_ctx* ctx, int64_t out[4]);
  * variants (E2M1 operands, triangle output), 4 tensor core with square output.
  * With E2M1 operands these three classes run on the two-SM kernel that sweeps
  * the markers once per product (clusters of two CTAs, tcgen05 cta_group::2);
- * where its workspace does not fit, with 2^21 or more variants and with E4M3
- * operands, class 2 runs one persistent CTA per SM, class 3 the two-SM kernel
+ * where its workspace does not fit, with few samples over many variants (up to
+ * 128 over 16,384, up to 256 over 49,152), with 2^21 or more variants and with
+ * E4M3 operands, class 2 runs one persistent CTA per SM, class 3 the two-SM kernel
  * over 256 x 128 tiles and class 4 one CTA per tile.
  * IBS_TC_PAIR=1 in the environment reports class 3 for every size of 129 or
  * more samples, IBS_TC_PAIR=0 runs (and reports) one CTA per SM always.  Host

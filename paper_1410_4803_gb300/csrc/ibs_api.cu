@@ -207,13 +207,17 @@ static bool tc_tile_kernel_forced() {
   return v;
 }
 
-// The sweep kernel (ibs_sweep.cu) computes E2M1 inputs, triangle or square: at
-// every size the faster one (256 x 4,096: 33 us a call against 82 on the kernels
-// below; 4,096 x 100,000: 979 against 1,564; 20,000 x 500,000: 77 against 142
-// ms; the square of 3,001 x 60,000: 583 us against 786).
+// The sweep kernel (ibs_sweep.cu) computes E2M1 inputs, triangle or square, except
+// one or two blocks of samples over many markers: there every stage of every
+// piece multiplies a narrow tile, and the pieces' sums are most of the call.
+// Sweep kernel against the kernels below: 256 x 4,096 27 us and 82, 200 x 20,000 42
+// and 59, 300 x 100,000 76 and 90, 4,096 x 100,000 935 and 1,566, 20,000 x 500,000
+// 74 and 142 ms, the square of 3,001 x 60,000 386 us and 788; but 64 x 20,000 36
+// and 33, 85 x 100,000 76 and 43, 200 x 100,000 86 and 65, 40 x 400,000 94 and 72.
 static bool use_sweep(const ibs_ctx* ctx, int64_t n, int64_t m, bool square) {
   return tc_format_for(ctx) == kTcFp4 && tc_pair_mode() >= 0 && !tc_tile_kernel_forced() &&
-         sweep_usable(n, m) && ctx->sweep_refused != std::vector<int64_t>{n, m, square ? 1 : 0};
+         !(n <= 128 && m > 16384) && !(n <= 256 && m > 49152) && sweep_usable(n, m) &&
+         ctx->sweep_refused != std::vector<int64_t>{n, m, square ? 1 : 0};
 }
 
 // ibs_compute on the sweep kernel: operand planes, the sweeps over the shape's

@@ -21,7 +21,10 @@
 // At most two steps are in flight, so admission and completion are handled
 // between steps while the GPU stays busy.
 //
-// Tensor-core form: a step with two or more query blocks runs on the two-SM
+// E2M1 without a workspace limit: steps run on the sweep kernel (ibs_sweep.cu),
+// over its own planes; a step of at most kFewRows rows runs on the integer pipe
+// over the panel's code bits (ibs_rows.cu), a second, small copy of the panel.
+// Otherwise a tensor-core step with two or more query blocks runs on the two-SM
 // kernel (items of two query blocks x one panel block; the faster kernel for
 // panels of at least 1,024 chunks), a step of one query block on the one-SM
 // kernel.  The step length is rounded so that its last wave of items is as
@@ -30,13 +33,13 @@
 // device step by step on a second stream (the panel columns each step wrote),
 // so those copies overlap the following steps instead of trailing them.  The
 // top-k of all requests that finish in a step runs as one launch.
-#include <shared_mutex>
 #include <algorithm>
 #include <atomic>
 #include <chrono>
 #include <condition_variable>
 #include <cstring>
 #include <deque>
+#include <shared_mutex>
 #include <thread>
 #include <unordered_map>
 

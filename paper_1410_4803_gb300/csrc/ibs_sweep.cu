@@ -45,10 +45,12 @@ namespace ibs {
 namespace {
 
 // A ring stage is kSwCols columns (three K steps): 18 KiB of A and up to 27
-// KiB of B.  A stage costs about 500 cycles whatever its size (barrier wait,
-// two copies, release; measured with copies alone: 31, 62 and 95 B/clk per SM
-// for stages of 3, 6 and 9 columns, 95 B/clk also for 12), and the MMAs of
-// three K steps take 576, so this is the smallest stage that does not bind.
+// KiB of B.  With one copying thread a stage costs about 500 cycles whatever its
+// size (barrier wait, two copies, release; copies alone: 31, 62 and 95 B/clk per
+// SM for stages of 3, 6 and 9 columns, 95 B/clk also for 12), and the MMAs of
+// three K steps take 576.  As built (a copying thread per operand), 4,096 x
+// 100,000 takes 1,033 us with 4 stages of 9 columns, 1,089 with 6 of 6 and 1,065
+// with 3 of 12.
 constexpr int kSwCols = 9;
 constexpr int kSwMarkers = 32 * kSwCols;  // 288
 constexpr int kSwStages = 4;
@@ -636,7 +638,7 @@ __global__ void __launch_bounds__(128) sweep_finalize_kernel(const SweepGroup* _
 // [begin, end) regrouped by sample, words[c][sample] = the low and the high code
 // bits of markers begin + 32 c ...  The gather below then reads 8 bytes per
 // sample and column; out of the rows it reads single bytes of 32 lines, which
-// took 1.8 ms of a 4 ms batch (24 subsets of 100 to 4000 samples, 10,000 x
+// took 1.8 ms of a 4 ms batch (24 subsets of 100 to 3,000 samples, 10,000 x
 // 200,000 pool).  Warp = one column of 64 samples, transposed by shuffles;
 // 512 neighbouring samples per CTA.  A fixed grid (the launch is in a graph and
 // the window is known per call); HBM-bound: the pool read once and written once.
@@ -815,8 +817,9 @@ void triangle_tiles(int64_t n, int stages, int subset, std::vector<Tile>& full, 
       }
 }
 
-// Cost of a tile's ring stage: about 620 cycles measured at full width, the fixed
-// cost of a stage for the narrow tiles.
+// Cost of a tile's ring stage in cycles: about 620 at full width with the operands
+// in L2 (715 in a long lockstep wave), the fixed cost of a stage for the narrow
+// tiles.
 double stage_cost(int w) { return w == 3 ? 620.0 : (w == 2 ? 520.0 : 500.0); }
 double tile_cost(const Tile& t) { return stage_cost(t.w) * 4 * t.stages; }
 
@@ -975,7 +978,7 @@ void lay_out(const std::vector<std::vector<SweepItem>>& own, SweepPlan& pl) {
 
 // One matrix or one step: the full-width tiles run whole, one per cluster and
 // wave, as many full waves as there are; the last partial wave and the
-// narrower tiles are cut into equal shares.
+// narrower tiles are cut into pieces, in rounds or in equal shares.
 SweepPlan schedule(std::vector<Tile>& full, const std::vector<Tile>& narrow, int clusters, size_t operands) {
   SweepPlan pl;
   const size_t C = (size_t)std::max(1, clusters), whole = full.size() / C * C;

@@ -43,6 +43,12 @@ def test_parts_and_waves(ctx, n, m):
     _check(ctx, n, m, n + m)
 
 
+# either side of the sizes that leave the sweep kernel: one block of samples, two
+@pytest.mark.parametrize("n,m", [(128, 16_384), (128, 16_385), (129, 16_385), (256, 49_152), (256, 49_153), (257, 49_153)])
+def test_narrow_inputs(ctx, n, m):
+    _check(ctx, n, m, n + m)
+
+
 def test_no_room_for_the_workspace():
     """A workspace bound that holds operand planes and partial counts but not
     the sweep kernel's scratch and parts: the call still computes."""
