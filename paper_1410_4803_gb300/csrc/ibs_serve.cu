@@ -98,8 +98,10 @@ PtrKind ptr_kind(const void* p) {
   return PtrKind::Pageable;
 }
 
-// The device's address of pinned host memory, or null.
-void* mapped(void* p) {
+// The device's address of pinned host memory aligned for a kernel's stores of
+// elements of `size` bytes, or null (a copy takes any alignment).
+void* mapped(void* p, size_t size) {
+  if (reinterpret_cast<uintptr_t>(p) % size != 0) return nullptr;
   cudaPointerAttributes a;
   if (cudaPointerGetAttributes(&a, p) != cudaSuccess) {
     cudaGetLastError();
@@ -1025,8 +1027,8 @@ ibs_status serve_query(ibs_ctx* ctx, const uint8_t* q, int64_t nq, int k, int32_
   r->counts_on_dev = counts_dev;
   r->topk_on_dev = topk_dev;
   if (k > 0 && !topk_dev) {
-    r->map_idx = static_cast<int32_t*>(mapped(oi));
-    r->map_dist = static_cast<double*>(mapped(od));
+    r->map_idx = static_cast<int32_t*>(mapped(oi, sizeof(int32_t)));
+    r->map_dist = static_cast<double*>(mapped(od, sizeof(double)));
   }
   // A request that the engine can admit at once goes straight to the device;
   // one behind others that wait for memory, or past the rows of a step, is kept

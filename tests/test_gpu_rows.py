@@ -66,3 +66,25 @@ def test_few_rows(q, n, m):
 def test_topk_ties(q, n, k):
     rng = np.random.default_rng(q + n + k)
     _run(random_codes(rng, n, 2, miss=0.3), random_codes(rng, q, 2, miss=0.3), k)
+
+
+@pytest.mark.parametrize("skew", [1, 4])
+def test_topk_lists_at_any_alignment(skew):
+    """Pinned lists that a kernel could not store to element by element are still copied there."""
+    import torch
+    from paper_1410_4803_gb300 import ibs
+    rng = np.random.default_rng(skew)
+    n, m, q, k = 300, 700, 3, 8
+    panel, rows = random_codes(rng, n, m), random_codes(rng, q, m)
+    ctx = ibs.ibs_init(0, flags=ibs.IBS_KERNEL_TC | ibs.IBS_TC_FP4)
+    try:
+        ibs.ibs_panel_load(ctx, pack_codes(panel), n, m)
+        idx = torch.zeros(q * k * 4 + 16, dtype=torch.uint8).pin_memory()
+        dist = torch.zeros(q * k * 8 + 16, dtype=torch.uint8).pin_memory()
+        packed = torch.from_numpy(pack_codes(rows)).pin_memory()
+        ibs.ibs_wait(ctx, ibs.ibs_query(ctx, packed, q, k, None, idx.data_ptr() + skew, dist.data_ptr() + skew))
+        got_i = np.frombuffer(idx.numpy().tobytes()[skew:skew + q * k * 4], np.int32).reshape(q, k)
+        got_d = np.frombuffer(dist.numpy().tobytes()[skew:skew + q * k * 8], np.float64).reshape(q, k)
+        _check_topk(_expected(panel, rows), got_i, got_d, k)
+    finally:
+        ibs.ibs_shutdown(ctx)
