@@ -129,7 +129,7 @@ class ServeEngine {
   DevBuf panel_planes, counter;
   cudaStream_t stream = nullptr;
   cudaStream_t in = nullptr;  // ibs_query's copies
-  std::shared_mutex in_mu;    // in used, or destroyed
+  std::shared_mutex in_mu;    // shared by ibs_query while it brings a request in; shutdown waits for it
   int64_t early_rows = 0;     // rows of the unfinished requests copied to the device by ibs_query (mu)
   std::thread worker;
   std::mutex mu;
@@ -272,11 +272,10 @@ class ServeEngine {
   }
 
   // The samples of a request from the caller's memory into device memory
-  // (caller's thread; done on return).  Device memory is read in the legacy
-  // stream's order, as by a plain copy.  The calls are allowed while a thread
-  // captures a graph elsewhere.
+  // (caller's thread, which holds in_mu; done on return).  Device memory is read
+  // in the legacy stream's order, as by a plain copy.  The calls are allowed
+  // while a thread captures a graph elsewhere.
   bool copy_in(Request& r, const uint8_t* q, size_t bytes, size_t need) {
-    std::shared_lock<std::shared_mutex> in_lk(in_mu);
     if (!in) return false;
     cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
     cudaThreadExchangeStreamCaptureMode(&mode);
@@ -739,6 +738,13 @@ class ServeEngine {
     }
     cv_work.notify_all();
     if (worker.joinable()) worker.join();
+    {
+      // A call that is bringing its request in uses the engine's memory and the
+      // context: it has returned before either goes.
+      std::unique_lock<std::shared_mutex> in_lk(in_mu);
+      if (in) cudaStreamDestroy(in);
+      in = nullptr;
+    }
     cudaStreamSynchronize(stream);
     if (side) cudaStreamSynchronize(side);
     std::lock_guard<std::mutex> lk(mu);
@@ -784,11 +790,6 @@ class ServeEngine {
     }
     if (stream) cudaStreamDestroy(stream);
     if (side) cudaStreamDestroy(side);
-    {
-      std::unique_lock<std::shared_mutex> in_lk(in_mu);  // a call may still be copying
-      if (in) cudaStreamDestroy(in);
-      in = nullptr;
-    }
     stream = nullptr;
     side = nullptr;
   }
@@ -1008,6 +1009,11 @@ ibs_status serve_query(ibs_ctx* ctx, const uint8_t* q, int64_t nq, int k, int32_
   auto eng = engine_of(ctx);
   if (ibs_status s = validate_query(eng, q, nq, k, oc, oi, od, counts_dev, topk_dev)) return s;
   ServeEngine& e = *eng;
+  std::shared_lock<std::shared_mutex> in_lk(e.in_mu);  // until return: neither engine nor context goes away
+  {
+    std::lock_guard<std::mutex> lk(e.mu);
+    if (e.stop) return fail(IBS_ECANCELLED, "engine is shutting down");
+  }
   const size_t need = e.mem_need(nq, k, counts_dev, topk_dev);
   // The engine's own buffers (panel planes, step tables) are always held, so a
   // request is refused at once when it could not fit even beside them alone.
@@ -1035,7 +1041,7 @@ ibs_status serve_query(ibs_ctx* ctx, const uint8_t* q, int64_t nq, int k, int32_
   // on the host.  (20 requests with 75 MB of pinned samples: 12.3 ms against 13.0.)
   const size_t bytes = (size_t)e.pg.m * (size_t)((nq + 3) / 4);
   bool early = false;
-  if (ctx->ws_limit == 0) {
+  if (e.in && ctx->ws_limit == 0) {
     std::lock_guard<std::mutex> lk(e.mu);
     early = !e.stop && e.early_rows + nq <= kMaxRows;
     for (const auto& p : e.pending) early = early && p->early;

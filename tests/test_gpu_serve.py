@@ -211,6 +211,48 @@ def test_shutdown_cancels_pending(panel):
     assert all(s in (ibs.IBS_OK, ibs.IBS_ECANCELLED) for s in statuses)
 
 
+@pytest.mark.parametrize("stop", ["shutdown", "reload"])
+def test_stop_while_a_call_brings_its_request_in(stop):
+    """ibs_query of device samples waits for the legacy stream with the engine's
+    memory in hand; a shutdown or a new panel meanwhile lets the call return
+    IBS_ECANCELLED first, and the context it uses outlives it."""
+    import torch
+    from paper_1410_4803_gb300 import ibs
+    from helpers import pack_codes, random_codes
+    rng = np.random.default_rng(8)
+    n_panel, m, q, k = 300, 700, 40, 4
+    pp = pack_codes(random_codes(rng, n_panel, m))
+    qp = torch.from_numpy(pack_codes(random_codes(rng, q, m))).cuda()
+    oi, od = _pinned((q, k), torch.int32), _pinned((q, k), torch.float64)
+    for _ in range(5):
+        ctx = ibs.ibs_init(0)
+        ibs.ibs_panel_load(ctx, pp, n_panel, m)
+        ended = []
+
+        def call():
+            try:
+                ibs.ibs_query(ctx, qp, q, k, None, oi, od)
+                ended.append(ibs.IBS_OK)
+            except ibs.IbsError as e:
+                ended.append(e.status)
+
+        t = threading.Thread(target=call)
+        torch.cuda._sleep(400_000_000)  # 0.2 s of the legacy stream
+        t.start()
+        time.sleep(0.05)
+        assert not ended
+        if stop == "reload":
+            ibs.ibs_panel_load(ctx, pp, n_panel, m)
+        else:
+            ibs.ibs_shutdown(ctx)
+        t.join(timeout=20)
+        assert ended == [ibs.IBS_ECANCELLED]
+        if stop == "reload":
+            rid = ibs.ibs_query(ctx, qp, q, k, None, oi, od)
+            ibs.ibs_wait(ctx, rid, timeout_ms=20000)
+            ibs.ibs_shutdown(ctx)
+
+
 SERVE_TWO_SM = r"""
 import sys
 import numpy as np
