@@ -399,6 +399,12 @@ ibs_status ibs_last_launch_info(ibs_ctx* ctx, int64_t out[3]);
  * IBS_EINVAL. */
 ibs_status ibs_test_set_wait_limit(ibs_ctx* ctx, int64_t ns);
 
+/* Testing hook of the serving engine's admission (the paper has no
+ * counterpart): the device memory, in bytes, that the requests in flight on
+ * the loaded panel may hold together, in place of what was free when the panel
+ * was loaded.  IBS_ESTATE without a panel, IBS_EINVAL for bytes < 1. */
+ibs_status ibs_test_set_serving_budget(ibs_ctx* ctx, int64_t bytes);
+
 #ifdef __cplusplus
 }
 #endif

@@ -1704,6 +1704,13 @@ extern "C" ibs_status ibs_test_set_wait_limit(ibs_ctx* ctx, int64_t ns) {
   return IBS_OK;
 }
 
+extern "C" ibs_status ibs_test_set_serving_budget(ibs_ctx* ctx, int64_t bytes) {
+  clear_error();
+  if (ibs_status s = check_ctx(ctx)) return s;
+  if (bytes < 1) return fail(IBS_EINVAL, "serving budget of %lld bytes", (long long)bytes);
+  return serve_set_budget(ctx, (size_t)bytes);
+}
+
 extern "C" ibs_status ibs_kernel_info(ibs_ctx* ctx, int64_t out[4]) {
   clear_error();
   if (ibs_status s = check_ctx(ctx)) return s;

@@ -78,7 +78,8 @@ struct Request {
   int32_t* map_idx = nullptr;  // pinned top-k outputs as the device sees them
   double* map_dist = nullptr;
   bool topk_direct = false;    // written there by the kernel
-  bool early = false;  // reserved and on the device since ibs_query
+  bool early = false;     // took its memory with its place in the queue
+  bool arriving = false;  // in the queue, its samples still on their way
   int64_t blocks_done = 0;  // panel blocks processed since admission
   cudaEvent_t done_ev = nullptr;  // recorded on the engine's copy stream after the request's last output
   ibs_status status = IBS_OK;
@@ -130,7 +131,7 @@ class ServeEngine {
   cudaStream_t stream = nullptr;
   cudaStream_t in = nullptr;  // ibs_query's copies
   std::shared_mutex in_mu;    // shared by ibs_query while it brings a request in; shutdown waits for it
-  int64_t early_rows = 0;     // rows of the unfinished requests copied to the device by ibs_query (mu)
+  int64_t early_rows = 0;     // rows of the unfinished early requests (mu)
   std::thread worker;
   std::mutex mu;
   std::condition_variable cv_work, cv_done;
@@ -275,46 +276,70 @@ class ServeEngine {
   // (caller's thread, which holds in_mu; done on return).  Device memory is read
   // in the legacy stream's order, as by a plain copy.  The calls are allowed
   // while a thread captures a graph elsewhere.
-  bool copy_in(Request& r, const uint8_t* q, size_t bytes, size_t need) {
-    if (!in) return false;
+  bool copy_in(Request& r, const uint8_t* q, size_t bytes) {
     cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
     cudaThreadExchangeStreamCaptureMode(&mode);
-    bool ok = reserve_request(r, need);
-    if (ok && alloc(r.packed, bytes, in) == IBS_OK) {
+    bool ok = alloc(r.packed, bytes, in) == IBS_OK;
+    if (ok) {
       const cudaStream_t s = ptr_kind(q) == PtrKind::Device ? cudaStreamLegacy : in;
       ok = cudaStreamSynchronize(in) == cudaSuccess &&
            cudaMemcpyAsync(r.packed.p, q, bytes, cudaMemcpyDefault, s) == cudaSuccess &&
            cudaStreamSynchronize(s) == cudaSuccess;
-      if (!ok) cudaGetLastError();
-    } else {
-      ok = false;
+      if (!ok) {
+        cudaGetLastError();
+        cudaFreeAsync(r.packed.p, in);
+        r.packed = DevBuf{};
+      }
     }
-    if (!ok) release(r, in);
     cudaThreadExchangeStreamCaptureMode(&mode);
     return ok;
   }
 
-  // Try to admit r (engine thread).  Returns false if it must wait.
+  // Try to admit r (engine thread).  Returns false if it must wait; it then
+  // keeps what it brought along (its memory in the budget, its samples).
   bool admit(const std::shared_ptr<Request>& r, int64_t active_rows) {
     if (active_rows + r->q > kMaxRows && active_rows > 0) return false;
     const size_t need = mem_need(r->q, r->k, r->counts_on_dev, r->topk_on_dev);
     if (!r->early && !reserve_request(*r, need)) return false;
     const size_t pk = (size_t)pg.m * (size_t)((r->q + 3) / 4);
-    if ((!r->early && alloc(r->packed, pk, stream)) || alloc(r->planes, geo(r->q).bytes, stream) ||
+    const bool host = r->packed.p == nullptr;  // the samples are in host_packed
+    if ((host && alloc(r->packed, pk, stream)) || alloc(r->planes, geo(r->q).bytes, stream) ||
         (!r->counts_on_dev && alloc(r->counts, (size_t)r->q * pg.n * 16, stream)) ||
         (!r->topk_on_dev && r->k > 0 &&
          (alloc(r->tidx, (size_t)r->q * r->k * 4, stream) || alloc(r->tdist, (size_t)r->q * r->k * 8, stream)))) {
       if (r->early)
-        free_async(*r, false, stream);  // it keeps its reservation and its samples
+        free_async(*r, host, stream);
       else
         release(*r, stream);
       return false;
     }
-    if (!r->early) cudaMemcpyAsync(r->packed.p, r->host_packed.data(), pk, cudaMemcpyHostToDevice, stream);
+    if (host) cudaMemcpyAsync(r->packed.p, r->host_packed.data(), pk, cudaMemcpyHostToDevice, stream);
     cudaEventCreateWithFlags(&r->done_ev, cudaEventDisableTiming);
     r->blocks_done = 0;
     r->state = RState::Active;
     return true;
+  }
+
+  // The samples of the early requests behind the first in line go back to the
+  // host (nothing is on the GPU, and the first found no device memory beside
+  // them); true if there were any.  lk holds mu.
+  bool take_back(std::unique_lock<std::mutex>& lk) {
+    std::vector<std::shared_ptr<Request>> behind;
+    bool first = true;
+    for (const auto& r : pending) {
+      if (r->arriving) continue;
+      if (!first && r->packed.p) behind.push_back(r);
+      first = false;
+    }
+    lk.unlock();
+    for (const auto& r : behind) {
+      r->host_packed.resize((size_t)pg.m * (size_t)((r->q + 3) / 4));
+      cudaMemcpyAsync(r->host_packed.data(), r->packed.p, r->host_packed.size(), cudaMemcpyDeviceToHost, stream);
+      free_async(*r, true, stream);
+    }
+    cudaStreamSynchronize(stream);
+    lk.lock();
+    return !behind.empty();
   }
 
   int32_t* counts_ptr(Request& r) { return r.counts_on_dev ? r.user_counts : static_cast<int32_t*>(r.counts.p); }
@@ -692,22 +717,34 @@ class ServeEngine {
         if (stop) break;
         int64_t rows = 0;
         for (auto& r : active) rows += r->q;
-        while (!pending.empty()) {
-          auto r = pending.front();
+        // In the order of the queue, past the requests whose samples are still on
+        // their way; callers only add at its end.
+        for (size_t i = 0; i < pending.size();) {
+          auto r = pending[i];
+          if (r->arriving) {
+            ++i;
+            continue;
+          }
           lk.unlock();
           const bool ok = admit(r, rows);
           lk.lock();
           if (!ok) break;
-          pending.pop_front();
+          pending.erase(pending.begin() + (std::ptrdiff_t)i);
           active.push_back(r);
           ++set_version;
           rows += r->q;
           stats.peak_rows = std::max<uint64_t>(stats.peak_rows, (uint64_t)rows);
         }
         if (active.empty()) {
+          auto waiting = [&] {
+            return std::any_of(pending.begin(), pending.end(), [](const auto& r) { return !r->arriving; });
+          };
           if (finishing.empty()) {
-            cv_work.wait(lk, [&] { return stop || !pending.empty(); });
-          } else if (!pending.empty()) {  // (it waits for memory)
+            if (!waiting())
+              cv_work.wait(lk, [&] { return stop || waiting(); });
+            else if (!take_back(lk))  // the first in line waits for memory held elsewhere
+              cv_work.wait_for(lk, std::chrono::microseconds(200));
+          } else if (waiting()) {  // (for memory)
             cv_work.wait_for(lk, std::chrono::microseconds(200));
           } else {
             // the last results are a few hundred microseconds away: poll (a timed
@@ -717,9 +754,9 @@ class ServeEngine {
               lk.unlock();
               const bool done = cudaEventQuery(finishing.front()->done_ev) != cudaErrorNotReady;
               lk.lock();
-              if (done || stop || !pending.empty()) break;
+              if (done || stop || waiting()) break;
             } while (std::chrono::steady_clock::now() - t0 < std::chrono::milliseconds(2));
-            if (!stop && pending.empty() && cudaEventQuery(finishing.front()->done_ev) == cudaErrorNotReady)
+            if (!stop && !waiting() && cudaEventQuery(finishing.front()->done_ev) == cudaErrorNotReady)
               cv_work.wait_for(lk, std::chrono::microseconds(200));
           }
           continue;
@@ -1017,7 +1054,11 @@ ibs_status serve_query(ibs_ctx* ctx, const uint8_t* q, int64_t nq, int k, int32_
   const size_t need = e.mem_need(nq, k, counts_dev, topk_dev);
   // The engine's own buffers (panel planes, step tables) are always held, so a
   // request is refused at once when it could not fit even beside them alone.
-  size_t avail = e.pool_budget;
+  size_t avail;
+  {
+    std::lock_guard<std::mutex> lk(e.budget_mu);
+    avail = e.pool_budget;
+  }
   if (ctx->ws_limit) avail = std::min(avail, ctx->ws_limit > e.fixed_bytes ? ctx->ws_limit - e.fixed_bytes : 0);
   if (need > avail) {
     std::lock_guard<std::mutex> lk(e.mu);
@@ -1036,37 +1077,45 @@ ibs_status serve_query(ibs_ctx* ctx, const uint8_t* q, int64_t nq, int k, int32_
     r->map_idx = static_cast<int32_t*>(mapped(oi, sizeof(int32_t)));
     r->map_dist = static_cast<double*>(mapped(od, sizeof(double)));
   }
-  // A request that the engine can admit at once goes straight to the device;
-  // one behind others that wait for memory, or past the rows of a step, is kept
-  // on the host.  (20 requests with 75 MB of pinned samples: 12.3 ms against 13.0.)
+  // A request that the engine can admit at once goes straight to the device (20
+  // requests with 75 MB of pinned samples: 12.3 ms against 13.0); one behind
+  // others that wait for memory, or past the rows of a step, is kept on the
+  // host.  The early ones take their memory and their places together, so no
+  // request holds memory that one ahead of it in the queue waits for.
   const size_t bytes = (size_t)e.pg.m * (size_t)((nq + 3) / 4);
-  bool early = false;
+  r->id = e.next_id.fetch_add(1);
   if (e.in && ctx->ws_limit == 0) {
     std::lock_guard<std::mutex> lk(e.mu);
-    early = !e.stop && e.early_rows + nq <= kMaxRows;
+    bool early = !e.stop && e.early_rows + nq <= kMaxRows;
     for (const auto& p : e.pending) early = early && p->early;
-    if (early) e.early_rows += nq;
-  }
-  if (early) {
-    r->early = e.copy_in(*r, q, bytes, need);
-    if (!r->early) {
-      std::lock_guard<std::mutex> lk(e.mu);
-      e.early_rows -= nq;
+    if (early && e.reserve_request(*r, need)) {
+      r->early = r->arriving = true;
+      e.early_rows += nq;
+      e.all[r->id] = r;
+      e.pending.push_back(r);
     }
   }
-  if (!r->early) r->host_packed = copy_query(q, bytes);
-  r->id = e.next_id.fetch_add(1);
+  if (!r->early || !e.copy_in(*r, q, bytes)) r->host_packed = copy_query(q, bytes);
   {
     std::lock_guard<std::mutex> lk(e.mu);
-    if (e.stop) {
-      if (r->early) e.release(*r, nullptr);
-      return fail(IBS_ECANCELLED, "engine is shutting down");
+    if (e.stop) return fail(IBS_ECANCELLED, "engine is shutting down");
+    if (r->early) {
+      r->arriving = false;
+    } else {
+      e.all[r->id] = r;
+      e.pending.push_back(r);
     }
-    e.all[r->id] = r;
-    e.pending.push_back(r);
   }
   e.cv_work.notify_all();
   *id = r->id;
+  return IBS_OK;
+}
+
+ibs_status serve_set_budget(ibs_ctx* ctx, size_t bytes) {
+  auto eng = engine_of(ctx);
+  if (!eng) return fail(IBS_ESTATE, "no panel loaded");
+  std::lock_guard<std::mutex> lk(eng->budget_mu);
+  eng->pool_budget = bytes;
   return IBS_OK;
 }
 

@@ -100,6 +100,7 @@ def load():
             "ibs_compute_noalloc": [p, i64, i64, p, p, p],
             "ibs_noalloc_status": [p],
             "ibs_test_set_wait_limit": [p, i64],
+            "ibs_test_set_serving_budget": [p, i64],
         }
         for name, args in sig.items():
             f = getattr(lib, name)
@@ -345,6 +346,11 @@ def ibs_test_set_wait_limit(ctx: Context, ns: int):
     """Testing hook: bound (ns) of the pipeline waits of ibs_compute's
     persistent pair kernels on this context; 0 restores the 2 s default."""
     _check(load().ibs_test_set_wait_limit(ctx._h, ns), "ibs_test_set_wait_limit")
+
+
+def ibs_test_set_serving_budget(ctx: Context, nbytes: int):
+    """Testing hook: device memory that the requests in flight on the loaded panel may hold together."""
+    _check(load().ibs_test_set_serving_budget(ctx._h, nbytes), "ibs_test_set_serving_budget")
 
 
 def ibs_batch_plan_info(ctx: Context) -> dict:

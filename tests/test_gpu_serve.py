@@ -253,6 +253,102 @@ def test_stop_while_a_call_brings_its_request_in(stop):
             ibs.ibs_shutdown(ctx)
 
 
+def _tight_engine(n_panel, m, q, k, rng):
+    """A context with a panel whose serving budget holds one request of q rows, not two."""
+    from paper_1410_4803_gb300 import ibs
+    from helpers import pack_codes, random_codes
+    codes = random_codes(rng, n_panel, m)
+    ctx = ibs.ibs_init(0)
+    ibs.ibs_panel_load(ctx, pack_codes(codes), n_panel, m)
+    planes = -(-q // 64) * (-(-m // 288) * 9) * 4096
+    need = m * -(-q // 4) + planes + q * n_panel * 16 + q * k * 12 + 4096
+    ibs.ibs_test_set_serving_budget(ctx, need * 3 // 2)
+    return ctx, codes
+
+
+def _check_request(panel_codes, codes, idx, dist, k):
+    wd = oracle.ibs_block(codes, panel_codes)[1]
+    for t in range(codes.shape[0]):
+        ti, td = oracle.topk(wd[t], k)
+        assert (idx.numpy()[t] == ti).all()
+        np.testing.assert_allclose(dist.numpy()[t], td, rtol=1e-12, atol=0)
+
+
+@pytest.mark.parametrize("first", ["device", "host"])
+def test_two_callers_and_a_budget_for_one(first):
+    """A call whose samples wait for the legacy stream holds the budget that the
+    other one needs: both are served, in either order of arrival."""
+    import torch
+    from paper_1410_4803_gb300 import ibs
+    from helpers import pack_codes, random_codes
+    rng = np.random.default_rng(17)
+    n_panel, m, q, k = 300, 3000, 200, 4
+    ctx, panel_codes = _tight_engine(n_panel, m, q, k, rng)
+    try:
+        codes = [random_codes(rng, q, m) for _ in range(2)]
+        packed = [torch.from_numpy(pack_codes(codes[0])).cuda(), torch.from_numpy(pack_codes(codes[1])).pin_memory()]
+        outs = [(_pinned((q, k), torch.int32), _pinned((q, k), torch.float64)) for _ in range(2)]
+        ids = [None, None]
+
+        def call(i):
+            ids[i] = ibs.ibs_query(ctx, packed[i], q, k, None, *outs[i])
+
+        torch.cuda._sleep(600_000_000)  # 0.3 s of the legacy stream, which the device samples wait for
+        order = (0, 1) if first == "device" else (1, 0)
+        threads = [threading.Thread(target=call, args=(i,)) for i in order]
+        for t in threads:
+            t.start()
+            time.sleep(0.05)
+        for t in threads:
+            t.join(timeout=20)
+        for rid in ids:
+            ibs.ibs_wait(ctx, rid, timeout_ms=20000)
+        for c, (oi, od) in zip(codes, outs):
+            _check_request(panel_codes, c, oi, od, k)
+    finally:
+        ibs.ibs_shutdown(ctx)
+
+
+def test_many_callers_and_a_tight_budget():
+    """Six threads, requests of 1 to 200 rows from the device and the host, with a budget for one or two at a time."""
+    import torch
+    from paper_1410_4803_gb300 import ibs
+    from helpers import pack_codes, random_codes
+    rng = np.random.default_rng(18)
+    n_panel, m, k = 300, 3000, 4
+    ctx, panel_codes = _tight_engine(n_panel, m, 200, k, rng)
+    try:
+        reqs = []
+        for i in range(36):
+            q = int(rng.integers(1, 201))
+            c = random_codes(rng, q, m)
+            t = torch.from_numpy(pack_codes(c))
+            reqs.append((q, c, t.cuda() if i % 3 == 0 else t.pin_memory() if i % 3 == 1 else t,
+                         _pinned((q, k), torch.int32), _pinned((q, k), torch.float64)))
+        torch.cuda.synchronize()
+        errors = []
+
+        def serve(mine):
+            try:
+                ids = [ibs.ibs_query(ctx, p, q, k, None, oi, od) for q, _, p, oi, od in mine]
+                for rid in ids:
+                    ibs.ibs_wait(ctx, rid, timeout_ms=30000)
+            except Exception as e:
+                errors.append(e)
+
+        threads = [threading.Thread(target=serve, args=(reqs[j::6],)) for j in range(6)]
+        for t in threads:
+            t.start()
+        for t in threads:
+            t.join(timeout=120)
+        assert not errors, errors
+        assert ibs.ibs_serve_stats_get(ctx)["requests_done"] == len(reqs)
+        for q, c, _, oi, od in reqs:
+            _check_request(panel_codes, c, oi, od, k)
+    finally:
+        ibs.ibs_shutdown(ctx)
+
+
 SERVE_TWO_SM = r"""
 import sys
 import numpy as np
