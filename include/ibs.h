@@ -405,6 +405,12 @@ ibs_status ibs_test_set_wait_limit(ibs_ctx* ctx, int64_t ns);
  * was loaded.  IBS_ESTATE without a panel, IBS_EINVAL for bytes < 1. */
 ibs_status ibs_test_set_serving_budget(ibs_ctx* ctx, int64_t bytes);
 
+/* Testing hook of the serving engine's error path (the paper has no
+ * counterpart): the next `steps` steps of the loaded panel's engine enqueue no
+ * pair kernel and count as failed launches, so the requests in them end with
+ * IBS_ECUDA.  IBS_ESTATE without a panel, IBS_EINVAL outside 0 .. 1000. */
+ibs_status ibs_test_fail_serving_steps(ibs_ctx* ctx, int64_t steps);
+
 #ifdef __cplusplus
 }
 #endif

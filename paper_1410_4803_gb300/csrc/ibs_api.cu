@@ -1711,6 +1711,13 @@ extern "C" ibs_status ibs_test_set_serving_budget(ibs_ctx* ctx, int64_t bytes) {
   return serve_set_budget(ctx, (size_t)bytes);
 }
 
+extern "C" ibs_status ibs_test_fail_serving_steps(ibs_ctx* ctx, int64_t steps) {
+  clear_error();
+  if (ibs_status s = check_ctx(ctx)) return s;
+  if (steps < 0 || steps > 1000) return fail(IBS_EINVAL, "%lld failing steps", (long long)steps);
+  return serve_fail_steps(ctx, (int)steps);
+}
+
 extern "C" ibs_status ibs_kernel_info(ibs_ctx* ctx, int64_t out[4]) {
   clear_error();
   if (ibs_status s = check_ctx(ctx)) return s;

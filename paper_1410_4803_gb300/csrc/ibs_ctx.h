@@ -203,6 +203,7 @@ ibs_status serve_wait(ibs_ctx* ctx, uint64_t id, int64_t timeout_ms);
 ibs_status serve_poll(ibs_ctx* ctx, uint64_t id);
 ibs_status serve_stats(ibs_ctx* ctx, ibs_serve_stats* out);
 ibs_status serve_set_budget(ibs_ctx* ctx, size_t bytes);
+ibs_status serve_fail_steps(ibs_ctx* ctx, int steps);
 void serve_stop(ibs_ctx* ctx);
 std::shared_ptr<ServeEngine> engine_of(ibs_ctx* ctx);
 

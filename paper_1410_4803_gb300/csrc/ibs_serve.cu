@@ -164,6 +164,7 @@ class ServeEngine {
   size_t items_cap = 0;
   cudaEvent_t step_ev[2] = {nullptr, nullptr};
   int64_t step_no = 0;
+  int failing_steps = 0;  // the next steps to fail (mu; serve_fail_steps)
   DevBuf step_planes, rows_dev[2], outs_dev[2];
   std::mutex budget_mu;
   size_t pool_budget = 0;  // bytes the requests may hold together
@@ -358,8 +359,11 @@ class ServeEngine {
   // Top-k of the requests that saw their last panel block in this step (on
   // the engine stream, after the step), then their top-k lists to the host
   // and their completion events on the copy stream (after their last counts
-  // columns).
-  void finish(const std::vector<std::shared_ptr<Request>>& done, int slot) {
+  // columns).  After a step that failed: the events only.
+  void finish(const std::vector<std::shared_ptr<Request>>& done, int slot, cudaError_t err) {
+    auto ok = [&](cudaError_t e) {
+      if (err == cudaSuccess) err = e;
+    };
     // every row of every finishing request in one launch (at most kMaxRows
     // rows: the admitted set never holds more)
     int64_t n = 0;
@@ -378,24 +382,28 @@ class ServeEngine {
       for (int64_t row = 0; row < r.q && n < kMaxRows; ++row, ++n)
         topk_host[slot][n] = TopkRow{cnt + (size_t)row * pg.n * 4, oi + row * r.k, od + row * r.k, r.k, 0};
     }
-    if (n > 0 && few) {
-      launch_topk_few(topk_host[slot], n, pg.n, stream);
-    } else if (n > 0) {
-      cudaMemcpyAsync(topk_dev[slot].p, topk_host[slot], (size_t)n * sizeof(TopkRow), cudaMemcpyHostToDevice, stream);
-      launch_topk_rows(static_cast<const TopkRow*>(topk_dev[slot].p), n, pg.n, stream);
+    if (err == cudaSuccess && n > 0 && few) {
+      ok(launch_topk_few(topk_host[slot], n, pg.n, stream));
+    } else if (err == cudaSuccess && n > 0) {
+      ok(cudaMemcpyAsync(topk_dev[slot].p, topk_host[slot], (size_t)n * sizeof(TopkRow), cudaMemcpyHostToDevice,
+                         stream));
+      ok(launch_topk_rows(static_cast<const TopkRow*>(topk_dev[slot].p), n, pg.n, stream));
     }
     if (!fin_ev[slot]) cudaEventCreateWithFlags(&fin_ev[slot], cudaEventDisableTiming);
     cudaEventRecord(fin_ev[slot], stream);
     cudaStreamWaitEvent(side, fin_ev[slot], 0);
     for (auto& rp : done) {
       Request& r = *rp;
-      if (!r.topk_on_dev && !r.topk_direct && r.k > 0) {
-        cudaMemcpyAsync(r.user_idx, r.tidx.p, (size_t)r.q * r.k * 4, cudaMemcpyDeviceToHost, side);
-        cudaMemcpyAsync(r.user_dist, r.tdist.p, (size_t)r.q * r.k * 8, cudaMemcpyDeviceToHost, side);
+      if (err == cudaSuccess && !r.topk_on_dev && !r.topk_direct && r.k > 0) {
+        ok(cudaMemcpyAsync(r.user_idx, r.tidx.p, (size_t)r.q * r.k * 4, cudaMemcpyDeviceToHost, side));
+        ok(cudaMemcpyAsync(r.user_dist, r.tdist.p, (size_t)r.q * r.k * 8, cudaMemcpyDeviceToHost, side));
       }
       cudaEventRecord(r.done_ev, side);
       r.state = RState::Finishing;
     }
+    if (err == cudaSuccess) return;
+    cudaGetLastError();
+    for (auto& rp : done) rp->status = IBS_ECUDA;
   }
 
   // Rows against panel blocks [cols[0][0], cols[0][1]) and [cols[1][0], cols[1][1])
@@ -444,17 +452,23 @@ class ServeEngine {
   // most three products.
   size_t sweep_part_bytes() const { return (size_t)6 * (size_t)std::max(1, clusters) * sweep_slot_bytes(); }
 
-  void ensure_items(size_t n) {
-    if (n <= items_cap) return;
+  cudaError_t ensure_items(size_t n) {
+    if (n <= items_cap) return cudaSuccess;
     const size_t each = std::max(std::max(sizeof(CrossItem), sizeof(PairItem)), sizeof(SweepItem));
+    items_cap = 0;
+    cudaError_t err = cudaSuccess;
     for (int s = 0; s < 2; ++s) {
       if (step_ev[s]) cudaEventSynchronize(step_ev[s]);
       if (items_dev[s].p) cudaFree(items_dev[s].p);
       if (items_host[s]) cudaFreeHost(items_host[s]);
-      cudaMalloc(&items_dev[s].p, n * each);
-      cudaHostAlloc(reinterpret_cast<void**>(&items_host[s]), n * each, cudaHostAllocDefault);
+      items_dev[s].p = nullptr;
+      items_host[s] = nullptr;
+      if (err == cudaSuccess) err = cudaMalloc(&items_dev[s].p, n * each);
+      if (err == cudaSuccess)
+        err = cudaHostAlloc(reinterpret_cast<void**>(&items_host[s]), n * each, cudaHostAllocDefault);
     }
-    items_cap = n;
+    if (err == cudaSuccess) items_cap = n;
+    return err;
   }
 
   // K-lockstep of a two-SM launch of n_items equal items (whole waves of one
@@ -525,8 +539,20 @@ class ServeEngine {
   }
 
   // One step: every active request's rows, packed densely into query blocks,
-  // against the current panel chunk.
+  // against the current panel chunk.  When a copy or a launch of it fails, the
+  // requests in it end with IBS_ECUDA; the engine goes on.
   void run_step() {
+    cudaError_t err = cudaSuccess;
+    auto ok = [&](cudaError_t e) {
+      if (err == cudaSuccess) err = e;
+    };
+    {
+      std::lock_guard<std::mutex> lk(mu);
+      if (failing_steps > 0) {
+        --failing_steps;
+        err = cudaErrorLaunchFailure;
+      }
+    }
     const int slot = (int)(step_no & 1);
     if (step_ev[slot]) cudaEventSynchronize(step_ev[slot]);  // slot's host tables are free again
     int64_t n_rows = 0;
@@ -559,13 +585,15 @@ class ServeEngine {
     const int64_t cols[2][2] = {{cursor, std::min(end, pgeo.blocks)}, {0, std::max<int64_t>(0, end - pgeo.blocks)}};
     if (sweep && n_rows > 0 && !few) {
       pl = sweep_plan_cross(qblocks, cols, pg.m, clusters);
-      ensure_items(std::max<size_t>(sweep_list_bytes(pl) / sizeof(SweepItem) + 1, n_items));
+      ok(ensure_items(std::max<size_t>(sweep_list_bytes(pl) / sizeof(SweepItem) + 1, n_items)));
     } else {
-      ensure_items(std::max<size_t>(n_items, 1));
+      ok(ensure_items(std::max<size_t>(n_items, 1)));
     }
     size_t t = 0;
     int32_t** outs_d = static_cast<int32_t**>(outs_dev[slot].p);
-    if (few) {
+    if (err != cudaSuccess) {
+      // nothing to list
+    } else if (few) {
       t = 1;
     } else if (sweep) {
       t = pl.items.size();
@@ -602,25 +630,27 @@ class ServeEngine {
       if (!few && gathered_version != set_version) {
         for (auto& r : active) {
           if (r->planes_built) continue;
-          build_planes(static_cast<const uint8_t*>(r->packed.p), r->q, r->planes.p, stream);
+          ok(build_planes(static_cast<const uint8_t*>(r->packed.p), r->q, r->planes.p, stream));
           r->planes_built = true;
         }
         // the admitted set changed: pack its rows into the step planes again
-        cudaMemcpyAsync(rows_dev[slot].p, rows_host[slot], n_rows * sizeof(RowSrc), cudaMemcpyHostToDevice, stream);
+        ok(cudaMemcpyAsync(rows_dev[slot].p, rows_host[slot], n_rows * sizeof(RowSrc), cudaMemcpyHostToDevice, stream));
         if (sweep)
-          launch_sweep_gather_rows(static_cast<const RowSrc*>(rows_dev[slot].p), n_rows, pgeo.chunks,
-                                   static_cast<uint8_t*>(step_planes.p), kMaxRows / 64, stream);
+          ok(launch_sweep_gather_rows(static_cast<const RowSrc*>(rows_dev[slot].p), n_rows, pgeo.chunks,
+                                      static_cast<uint8_t*>(step_planes.p), kMaxRows / 64, stream));
         else if (tc)
-          launch_tc_gather_rows(static_cast<const RowSrc*>(rows_dev[slot].p), n_rows, pgeo.chunks,
-                                static_cast<uint8_t*>(step_planes.p), stream);
+          ok(launch_tc_gather_rows(static_cast<const RowSrc*>(rows_dev[slot].p), n_rows, pgeo.chunks,
+                                   static_cast<uint8_t*>(step_planes.p), stream));
         else
-          launch_gather_rows(static_cast<const RowSrc*>(rows_dev[slot].p), n_rows, pg.n_chunks,
-                             static_cast<uint32_t*>(step_planes.p), stream);
+          ok(launch_gather_rows(static_cast<const RowSrc*>(rows_dev[slot].p), n_rows, pg.n_chunks,
+                                static_cast<uint32_t*>(step_planes.p), stream));
         gathered_version = set_version;
       }
       if (!few)
-        cudaMemcpyAsync(outs_dev[slot].p, outs_host[slot], n_rows * sizeof(int32_t*), cudaMemcpyHostToDevice, stream);
-      if (few) {
+        ok(cudaMemcpyAsync(outs_dev[slot].p, outs_host[slot], n_rows * sizeof(int32_t*), cudaMemcpyHostToDevice, stream));
+      if (err != cudaSuccess) {
+        // nothing reads what may not be there
+      } else if (few) {
         const int64_t samples[2][2] = {{cols[0][0] * blk, std::min<int64_t>(cols[0][1] * blk, pg.n)},
                                        {0, std::min<int64_t>(cols[1][1] * blk, pg.n)}};
         FewTables tab;
@@ -628,27 +658,26 @@ class ServeEngine {
           tab.rows[r] = rows_host[slot][r];
           tab.out[r] = outs_host[slot][r];
         }
-        launch_few_rows(tab, n_rows,
-                        static_cast<const uint32_t*>(panel_words.p), pg.n, pg.m, samples, few_words.p, sweep_part.p,
-                        sweep_part.cap, ctx->num_sms, stream);
-        words_lk.unlock();
+        ok(launch_few_rows(tab, n_rows,
+                           static_cast<const uint32_t*>(panel_words.p), pg.n, pg.m, samples, few_words.p, sweep_part.p,
+                           sweep_part.cap, ctx->num_sms, stream));
       } else if (sweep) {
-        run_sweep(pl, static_cast<const uint8_t*>(step_planes.p), kMaxRows / 64, outs_d, n_rows, items_host[slot],
-                  static_cast<uint8_t*>(items_dev[slot].p), static_cast<float*>(sweep_scratch.p),
-                  static_cast<float*>(sweep_part.p), sync_ctr, true, stream);
+        ok(run_sweep(pl, static_cast<const uint8_t*>(step_planes.p), kMaxRows / 64, outs_d, n_rows, items_host[slot],
+                     static_cast<uint8_t*>(items_dev[slot].p), static_cast<float*>(sweep_scratch.p),
+                     static_cast<float*>(sweep_part.p), sync_ctr, true, stream));
       } else if (two_sm) {
-        cudaMemcpyAsync(items_dev[slot].p, items_host[slot], t * sizeof(PairItem), cudaMemcpyHostToDevice, stream);
-        launch_tc_pair_cross(static_cast<const uint8_t*>(panel_planes.p), pg.n, pgeo.chunks,
-                             static_cast<const uint8_t*>(step_planes.p), geo(kMaxRows).blocks, outs_d, n_rows,
-                             static_cast<const PairItem*>(items_dev[slot].p), (int64_t)t, ctx->status_dev, stream,
-                             pair_sync((int64_t)t, sync_ctr, true, stream));
+        ok(cudaMemcpyAsync(items_dev[slot].p, items_host[slot], t * sizeof(PairItem), cudaMemcpyHostToDevice, stream));
+        ok(launch_tc_pair_cross(static_cast<const uint8_t*>(panel_planes.p), pg.n, pgeo.chunks,
+                                static_cast<const uint8_t*>(step_planes.p), geo(kMaxRows).blocks, outs_d, n_rows,
+                                static_cast<const PairItem*>(items_dev[slot].p), (int64_t)t, ctx->status_dev, stream,
+                                pair_sync((int64_t)t, sync_ctr, true, stream)));
       } else {
-        cudaMemcpyAsync(items_dev[slot].p, items_host[slot], t * sizeof(CrossItem), cudaMemcpyHostToDevice, stream);
-        cross(static_cast<const CrossItem*>(items_dev[slot].p), (int64_t)t, stream);
+        ok(cudaMemcpyAsync(items_dev[slot].p, items_host[slot], t * sizeof(CrossItem), cudaMemcpyHostToDevice, stream));
+        ok(cross(static_cast<const CrossItem*>(items_dev[slot].p), (int64_t)t, stream));
       }
       // this step's panel columns of requests whose counts go to host memory
       bool any_host = false;
-      for (auto& r : active) any_host |= !r->counts_on_dev && r->user_counts;
+      for (auto& r : active) any_host |= err == cudaSuccess && !r->counts_on_dev && r->user_counts;
       if (any_host) {
         if (!kern_ev[slot]) cudaEventCreateWithFlags(&kern_ev[slot], cudaEventDisableTiming);
         cudaEventRecord(kern_ev[slot], stream);
@@ -661,14 +690,15 @@ class ServeEngine {
         }
       }
     }
+    if (few) words_lk.unlock();
     cursor = (cursor + len) % pgeo.blocks;
     std::vector<std::shared_ptr<Request>> still, done;
     for (auto& r : active) {
       // A request joined at some cursor position and is done once it has seen
       // every panel block (blocks seen twice near the end are rewritten with
-      // the same counts).
+      // the same counts), or when its step failed.
       r->blocks_done += len;
-      if (r->blocks_done >= pgeo.blocks) {
+      if (r->blocks_done >= pgeo.blocks || err != cudaSuccess) {
         done.push_back(r);
         finishing.push_back(r);
       } else {
@@ -676,7 +706,7 @@ class ServeEngine {
       }
     }
     if (!done.empty()) {
-      finish(done, slot);
+      finish(done, slot, err);
       ++set_version;
     }
     active.swap(still);
@@ -691,10 +721,12 @@ class ServeEngine {
     std::vector<std::shared_ptr<Request>> still;
     bool any = false;
     for (auto& r : finishing) {
-      if (cudaEventQuery(r->done_ev) == cudaSuccess) {
+      const cudaError_t q = cudaEventQuery(r->done_ev);
+      if (q != cudaErrorNotReady) {
         const int st = __atomic_load_n(ctx->status_host, __ATOMIC_SEQ_CST);
         std::lock_guard<std::mutex> lk(mu);
-        r->status = st == kDevTimeout ? IBS_ETIMEOUT : IBS_OK;
+        if (q != cudaSuccess) r->status = IBS_ECUDA;
+        if (r->status == IBS_OK && st == kDevTimeout) r->status = IBS_ETIMEOUT;
         release(*r, stream);
         if (r->early) early_rows -= r->q;
         r->state = RState::Done;
@@ -1108,6 +1140,14 @@ ibs_status serve_query(ibs_ctx* ctx, const uint8_t* q, int64_t nq, int k, int32_
   }
   e.cv_work.notify_all();
   *id = r->id;
+  return IBS_OK;
+}
+
+ibs_status serve_fail_steps(ibs_ctx* ctx, int steps) {
+  auto eng = engine_of(ctx);
+  if (!eng) return fail(IBS_ESTATE, "no panel loaded");
+  std::lock_guard<std::mutex> lk(eng->mu);
+  eng->failing_steps = steps;
   return IBS_OK;
 }
 

@@ -101,6 +101,7 @@ def load():
             "ibs_noalloc_status": [p],
             "ibs_test_set_wait_limit": [p, i64],
             "ibs_test_set_serving_budget": [p, i64],
+            "ibs_test_fail_serving_steps": [p, i64],
         }
         for name, args in sig.items():
             f = getattr(lib, name)
@@ -351,6 +352,11 @@ def ibs_test_set_wait_limit(ctx: Context, ns: int):
 def ibs_test_set_serving_budget(ctx: Context, nbytes: int):
     """Testing hook: device memory that the requests in flight on the loaded panel may hold together."""
     _check(load().ibs_test_set_serving_budget(ctx._h, nbytes), "ibs_test_set_serving_budget")
+
+
+def ibs_test_fail_serving_steps(ctx: Context, steps: int):
+    """Testing hook: the next steps of the loaded panel's engine count as failed launches."""
+    _check(load().ibs_test_fail_serving_steps(ctx._h, steps), "ibs_test_fail_serving_steps")
 
 
 def ibs_batch_plan_info(ctx: Context) -> dict:

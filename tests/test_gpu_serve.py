@@ -349,6 +349,32 @@ def test_many_callers_and_a_tight_budget():
         ibs.ibs_shutdown(ctx)
 
 
+@pytest.mark.parametrize("q,flags", [(1, "IBS_KERNEL_TC"), (40, "IBS_KERNEL_TC"), (300, "IBS_KERNEL_TC"), (40, "IBS_KERNEL_CSA")])
+def test_failed_step_ends_its_requests(q, flags):
+    """A step whose launches fail gives its requests IBS_ECUDA, not counts that
+    nothing wrote; the engine serves the next request."""
+    import torch
+    from paper_1410_4803_gb300 import ibs
+    from helpers import pack_codes, random_codes
+    rng = np.random.default_rng(q)
+    n_panel, m, k = 300, 700, 4
+    panel_codes, codes = random_codes(rng, n_panel, m), random_codes(rng, q, m)
+    ctx = ibs.ibs_init(0, flags=getattr(ibs, flags))
+    try:
+        ibs.ibs_panel_load(ctx, pack_codes(panel_codes), n_panel, m)
+        packed = pack_codes(codes)
+        oi, od = _pinned((q, k), torch.int32), _pinned((q, k), torch.float64)
+        for _ in range(2):
+            ibs.ibs_test_fail_serving_steps(ctx, 1)
+            with pytest.raises(ibs.IbsError) as ei:
+                ibs.ibs_wait(ctx, ibs.ibs_query(ctx, packed, q, k, None, oi, od), timeout_ms=20000)
+            assert ei.value.status == ibs.IBS_ECUDA
+            ibs.ibs_wait(ctx, ibs.ibs_query(ctx, packed, q, k, None, oi, od), timeout_ms=20000)
+            _check_request(panel_codes, codes, oi, od, k)
+    finally:
+        ibs.ibs_shutdown(ctx)
+
+
 SERVE_TWO_SM = r"""
 import sys
 import numpy as np
