@@ -336,6 +336,7 @@ size_t sweep_slot_bytes();
 SweepSync sweep_sync(int waves, int stages, int2 setting);
 SweepPlan sweep_plan(int64_t n, int64_t m, int clusters);
 SweepPlan sweep_plan_batch(const std::vector<std::pair<int64_t, int64_t>>& shapes, int clusters);  // {n, m}
+int64_t sweep_step_blocks(int64_t panel_blocks, int64_t row_blocks, int64_t left, int clusters);
 SweepPlan sweep_plan_cross(int64_t row_blocks, const int64_t (&cols)[2][2], int64_t m, int clusters);
 cudaError_t launch_sweep_planes(const uint8_t* packed, int64_t n, int64_t m, uint8_t* planes, cudaStream_t st);
 // One matrix: the triangle or the square of n samples.

@@ -54,8 +54,9 @@ constexpr int kMaxQuery = 4096;     // rows per request
 constexpr int kMaxK = 64;           // top-k limit of the kernel
 constexpr int64_t kMaxRows = 4096;  // query rows admitted at once (slot limit)
 constexpr int64_t kStepWaves = 16;  // a step aims at this many waves of (query block, panel block) tiles
-constexpr int64_t kStepWavesTc = 8; // ... of the tensor-core form (a request of one query block then takes
-                                    // one step over a 100,000-sample panel; two steps cost it about 3 ms)
+constexpr int64_t kStepWavesTc = 8; // ... of the tensor-core form without the sweep kernel (a request of one query
+                                    // block then takes one step over a 100,000-sample panel; two steps cost it
+                                    // about 3 ms); with it: sweep_step_blocks
 constexpr int64_t kMinStepDiv = 32; // ... and covers at least 1/32 of the panel
 constexpr size_t kMemMargin = (size_t)1 << 30;
 constexpr int64_t kTcBlock = 128;          // samples per tensor-core block
@@ -578,7 +579,11 @@ class ServeEngine {
     // shorter steps that new requests can join between.
     const bool two_sm = pair && qblocks >= 2;
     const int64_t units = two_sm || sweep ? (qblocks + 1) / 2 : qblocks;
-    const int64_t len = step_len(units, two_sm || sweep ? clusters : grid_ctas);
+    int64_t left = 0;  // panel blocks that some request still has to see
+    for (auto& r : active) left = std::max(left, pgeo.blocks - r->blocks_done);
+    const int64_t len = few     ? left
+                        : sweep ? sweep_step_blocks(pgeo.blocks, qblocks, left, clusters)
+                                : step_len(units, two_sm ? clusters : grid_ctas);
     const size_t n_items = (size_t)units * (size_t)len;
     SweepPlan pl;
     const int64_t end = cursor + len;  // wraps around the panel at most once

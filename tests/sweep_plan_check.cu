@@ -89,6 +89,22 @@ void check(const ibs::SweepPlan& p, const std::vector<std::pair<int64_t, int64_t
   if (cover.size() != blocks) fail("blocks", n, m, C);
 }
 
+// Steps of serving: whole tiles up to the last, no block more than is needed,
+// one step for a lone request of one or two blocks over up to 155,000 samples
+// (76 clusters), no more steps over a panel than the shortest allowed length gives.
+void check_steps(int64_t panel, int64_t rows, int c) {
+  using namespace ibs;
+  const int64_t pairs = (rows + 1) / 2;
+  int64_t steps = 0, left = panel;
+  for (; left > 0; ++steps) {
+    const int64_t len = sweep_step_blocks(panel, rows, left, c);
+    if (len < 1 || len > left || (len < left && len % 3 != 0)) return fail("step length", panel, rows, c);
+    left -= len;
+  }
+  if (pairs == 1 && panel <= 16 * c && steps != 1) fail("steps of a lone request", panel, rows, c);
+  if (steps > std::max<int64_t>(33, panel * pairs / (8 * c) + 2)) fail("steps over the panel", panel, rows, c);
+}
+
 }  // namespace
 
 int main() {
@@ -108,6 +124,9 @@ int main() {
       ++lists;
     }
   }
+  for (int64_t panel : {1, 2, 3, 4, 40, 156, 157, 607, 608, 609, 782, 1215, 1216, 1217, 1563, 16384})
+    for (int64_t rows = 1; rows <= 32; ++rows)
+      for (int c : {1, 5, 76}) check_steps(panel, rows, c);
   printf("checked %d lists, %d failures\n", lists, failures);
   return failures == 0 ? 0 : 1;
 }
