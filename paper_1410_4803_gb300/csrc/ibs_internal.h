@@ -104,6 +104,15 @@ struct RowSrc {
 // [samples[0][0], samples[0][1]) and [samples[1][0], samples[1][1]).  `words`
 // holds few_rows_bytes; `part` at least 12 bytes per row and panel sample.
 constexpr int kFewRows = 16;
+// Up to 8 rows are one pass of population counts, less than the tensor-core step
+// takes to read the panel's operand planes; 9 to 16 are two, which only a small
+// panel's fixed costs outweigh.  One request, code bits and operand planes, us:
+// 8 rows and 17 against 20,000 x 100,000: 617 and 786, 77,000 x 200,000: 3,336 and
+// 4,659; 16 and 17 against 5,000 x 20,000: 166 and 185, 20,000 x 20,000: 321 and
+// 315, 20,000 x 50,000: 620 and 493, 77,000 x 200,000: 6,223 and 4,659.
+inline bool few_rows_pay(int64_t rows, int64_t n_panel, int64_t m) {
+  return rows >= 1 && (rows <= 8 || (rows <= kFewRows && n_panel * m <= 400000000));
+}
 size_t few_rows_bytes(int64_t n_cols);
 struct FewTables {  // by value: no copies in front of the kernels
   RowSrc rows[kFewRows];

@@ -22,7 +22,7 @@
 // between steps while the GPU stays busy.
 //
 // E2M1 without a workspace limit: steps run on the sweep kernel (ibs_sweep.cu),
-// over its own planes; a step of at most kFewRows rows runs on the integer pipe
+// over its own planes; a step of few rows (few_rows_pay) runs on the integer pipe
 // over the panel's code bits (ibs_rows.cu), a second, small copy of the panel.
 // Otherwise a tensor-core step with two or more query blocks runs on the two-SM
 // kernel (items of two query blocks x one panel block; the faster kernel for
@@ -558,11 +558,9 @@ class ServeEngine {
     if (step_ev[slot]) cudaEventSynchronize(step_ev[slot]);  // slot's host tables are free again
     int64_t n_rows = 0;
     for (auto& r : active) n_rows += r->q;
-    // Up to kFewRows rows: the panel's code bits instead of its operand planes
-    // (one row against a 20,000 x 100,000 panel: 0.35 ms a request against 1.15;
-    // 16 rows cost two passes of about 0.3 ms, the tensor-core step 1 ms).
+    // Few rows: the panel's code bits instead of its operand planes
     std::unique_lock<std::mutex> words_lk(words_mu);
-    const bool few = n_rows > 0 && n_rows <= kFewRows && panel_words.p;
+    const bool few = few_rows_pay(n_rows, pg.n, pg.m) && panel_words.p;
     if (!few) words_lk.unlock();
     n_rows = 0;
     for (auto& r : active)

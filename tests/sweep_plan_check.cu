@@ -124,6 +124,12 @@ int main() {
       ++lists;
     }
   }
+  for (int64_t rows = 0; rows <= 18; ++rows)  // serving steps on the panel's code bits
+    for (int64_t n : {int64_t{300}, int64_t{20000}, int64_t{20001}, int64_t{2147483647}}) {
+      const bool small = n <= 20000;  // panels of 20,000 markers
+      if (ibs::few_rows_pay(rows, n, 20000) != (rows >= 1 && (rows <= 8 || (small && rows <= 16))))
+        fail("few rows", n, rows, 0);
+    }
   for (int64_t panel : {1, 2, 3, 4, 40, 156, 157, 607, 608, 609, 782, 1215, 1216, 1217, 1563, 16384})
     for (int64_t rows = 1; rows <= 32; ++rows)
       for (int c : {1, 5, 76}) check_steps(panel, rows, c);

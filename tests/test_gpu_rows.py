@@ -60,6 +60,26 @@ def test_few_rows(q, n, m):
     _run(random_codes(rng, n, m, miss=0.05), random_codes(rng, q, m, miss=0.05), min(16, 2 * n))
 
 
+# 8 rows on the code bits, 9 on the operand planes of a panel past the size for more
+@pytest.mark.parametrize("q", [8, 9])
+def test_few_rows_of_a_larger_panel(q):
+    import torch
+    from paper_1410_4803_gb300 import ibs
+    rng = np.random.default_rng(q)
+    n, m = 2003, 200_003
+    packed = rng.integers(0, 256, (m, (n + 3) // 4), dtype=np.uint8)
+    rows = rng.integers(0, 256, (m, (q + 3) // 4), dtype=np.uint8)
+    ctx = ibs.ibs_init(0, flags=ibs.IBS_KERNEL_TC | ibs.IBS_TC_FP4)
+    try:
+        ibs.ibs_panel_load(ctx, torch.from_numpy(packed).cuda(), n, m)
+        got, idx, dist = _query(ctx, rows, q, n, 16)
+    finally:
+        ibs.ibs_shutdown(ctx)
+    want = oracle.ibs_block(oracle.unpack(rows, q, m), oracle.unpack(packed, n, m))[0]
+    assert (got == want).all()
+    _check_topk(want, idx, dist, 16)
+
+
 # two markers: few distinct distances, and rows without a common call
 @pytest.mark.parametrize("q", [1, 40])
 @pytest.mark.parametrize("n,k", [(3, 64), (127, 64), (600, 1), (3000, 64), (3000, 16)])
