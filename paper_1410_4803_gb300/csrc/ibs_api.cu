@@ -1089,6 +1089,7 @@ ibs_status plan_upload(ibs_ctx* ctx, BatchPlan& plan, const uint8_t* pool, int64
   IBS_CUDA_TRY(cudaMemcpyAsync(plan.subsets.p, sd.data(), sizeof(SubsetDev) * k, cudaMemcpyHostToDevice, st));
   if (plan.sweep) {
     SweepPool sp;
+    plan.uses_words = false;
     sp.packed = pool;
     sp.row_bytes = (pool_n + 3) / 4;
     sp.n = pool_n;
@@ -1105,11 +1106,13 @@ ibs_status plan_upload(ibs_ctx* ctx, BatchPlan& plan, const uint8_t* pool, int64
       const size_t bytes = (size_t)cols * (size_t)pool_n * 8;
       size_t free_b = 0, total_b = 0;
       // (without room, or as more than a quarter of what is free: not regrouped)
-      if (plan.words.cap >= bytes ||
+      if (ctx->pool_words.cap >= bytes ||
           (cudaMemGetInfo(&free_b, &total_b) == cudaSuccess && bytes <= free_b / 4 &&
-           ensure_buf(ctx, plan.words, bytes) == IBS_OK)) {
+           ensure_buf(ctx, ctx->pool_words, bytes) == IBS_OK)) {
         sp.cols = cols;
-        sp.words = static_cast<uint32_t*>(plan.words.p);
+        sp.words = static_cast<uint32_t*>(ctx->pool_words.p);
+        plan.uses_words = true;
+        if (ctx->words_ev) IBS_CUDA_TRY(cudaStreamWaitEvent(st, ctx->words_ev, 0));
       }
       clear_error();
     }
@@ -1349,7 +1352,7 @@ void plan_free(ibs_ctx* ctx, BatchPlan& plan) {
   plan.graph = nullptr;
   for (DevBuf* b : {&plan.planes, &plan.partial, &plan.subsets, &plan.jobs, &plan.items, &plan.split_ids,
                     &plan.counter, &plan.tc_planes, &plan.tc_jobs, &plan.split_tiles, &plan.gather_map, &plan.pitems,
-                    &plan.units, &plan.unit_counter, &plan.ready, &plan.need, &plan.pair_sync, &plan.words})
+                    &plan.units, &plan.unit_counter, &plan.ready, &plan.need, &plan.pair_sync})
     free_buf(ctx, *b);
 }
 
@@ -1560,8 +1563,16 @@ extern "C" ibs_status ibs_compute_batch(ibs_ctx* ctx, const uint8_t* pool, int64
     it = ctx->plans.emplace(key, std::move(plan)).first;
   }
   BatchPlan& plan = *it->second;
-  if (ibs_status s = plan_upload(ctx, plan, pool, pool_n, pool_m, subs, shapes, st)) return s;
-  IBS_CUDA_TRY(cudaGraphLaunch(plan.exec, st));
+  {
+    // The regrouped pool is one buffer of the context: a batch on another stream
+    // waits for the last one that used it.
+    if (ibs_status s = plan_upload(ctx, plan, pool, pool_n, pool_m, subs, shapes, st)) return s;
+    IBS_CUDA_TRY(cudaGraphLaunch(plan.exec, st));
+    if (plan.uses_words) {
+      if (!ctx->words_ev) IBS_CUDA_TRY(cudaEventCreateWithFlags(&ctx->words_ev, cudaEventDisableTiming));
+      IBS_CUDA_TRY(cudaEventRecord(ctx->words_ev, st));
+    }
+  }
   int64_t own_gathers = 0;  // policy 5: subsets no two-SM launch gathered
   if (plan.split_policy == 5) {
     int64_t upto = 0;
@@ -1772,6 +1783,8 @@ extern "C" ibs_status ibs_shutdown(ibs_ctx* ctx) {
     cudaDeviceSynchronize();
     for (auto& kv : ctx->plans) plan_free(ctx, *kv.second);
     ctx->plans.clear();
+    free_buf(ctx, ctx->pool_words);
+    if (ctx->words_ev) cudaEventDestroy(ctx->words_ev);
     free_buf(ctx, ctx->planes);
     free_buf(ctx, ctx->partial);
     free_buf(ctx, ctx->tile_list);

@@ -86,12 +86,12 @@ struct BatchPlan {
   // split policy 2 on the sweep kernel (E2M1): tc_planes holds sweep planes,
   // units the subsets' tensor maps, counter the items' offsets per cluster,
   // split_tiles the split tiles, planes the scratch of whole tiles, partial the
-  // parts, jobs the SweepPool, words its regrouped rows
+  // parts, jobs the SweepPool
   bool sweep = false;
+  bool uses_words = false;  // the last call regrouped its pool
   int sweep_clusters = 0;
   int64_t sweep_groups = 0;
   SweepSync sweep_sync;
-  DevBuf words;
   cudaStream_t side = nullptr;
   std::vector<cudaEvent_t> stage_ev;
   cudaEvent_t fork_ev = nullptr, join_ev = nullptr;  // policy 3: the side stream's gather
@@ -173,6 +173,10 @@ struct ibs_ctx {
   };
   std::vector<TimingRec> timing_used, timing_free;
 
+  // batches on the sweep kernel: the pool's rows in use, regrouped by sample on
+  // every call; one buffer for all plans
+  ibs::DevBuf pool_words;
+  cudaEvent_t words_ev = nullptr;  // after the last batch that used it
   std::map<std::vector<int64_t>, std::unique_ptr<ibs::BatchPlan>> plans;
   std::map<std::string, ibs::TuneEntry> tune;
 

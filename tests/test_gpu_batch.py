@@ -236,6 +236,72 @@ def test_batch_windows_move_between_calls(pool):
         ibs.ibs_shutdown(ctx)
 
 
+def _random_pool(n, m, seed):
+    import torch
+    g = torch.Generator(device="cuda").manual_seed(seed)
+    return torch.randint(0, 256, (m, (n + 3) // 4), dtype=torch.uint8, device="cuda", generator=g)
+
+
+def _subset_args(pool_n, n, vb, vl, seed):
+    import torch
+    idx = np.sort(np.random.default_rng(seed).choice(pool_n, size=n, replace=False)).astype(np.int64)
+    P = n * (n + 1) // 2
+    return [(torch.from_numpy(idx).cuda(), vb, vl, torch.full((P, 4), -7, dtype=torch.int32, device="cuda"), None)]
+
+
+def test_plans_share_the_regrouped_pool():
+    """Batches of other sizes of one pool: each plan keeps planes and parts of
+    its own, but not another copy of the pool (0.8 GB here)."""
+    import torch
+    from paper_1410_4803_gb300 import ibs
+    pool_n, m = 4096, 800_000
+    pool = _random_pool(pool_n, m, 1)
+    calls = [_subset_args(pool_n, n, 0, m, n) for n in (1025, 1026, 1027)]
+    ctx = ibs.ibs_init(0, flags=ibs.IBS_KERNEL_TC | ibs.IBS_TC_FP4)
+    try:
+        held = []
+        for subs in calls:
+            torch.cuda.synchronize()
+            before = torch.cuda.mem_get_info()[0]
+            ibs.ibs_compute_batch(ctx, pool, pool_n, m, subs)
+            ibs.ibs_synchronize(ctx)
+            held.append(before - torch.cuda.mem_get_info()[0])
+        planes = 17 * 64 * 2 * m
+        assert held[0] > planes + 0.8e9  # the pool is regrouped
+        assert max(held[1:]) < planes + 0.5e9, held
+    finally:
+        ibs.ibs_shutdown(ctx)
+
+
+def test_batches_on_two_streams():
+    """Two plans whose pools are regrouped, back to back on two streams: the
+    results of each alone."""
+    import torch
+    from paper_1410_4803_gb300 import ibs
+    pool_n, m = 2048, 60_000
+    pool = _random_pool(pool_n, m, 2)
+    calls = [_subset_args(pool_n, 900, 0, 30_000, 1), _subset_args(pool_n, 700, 29_001, 30_999, 2)]
+    ctx = ibs.ibs_init(0, flags=ibs.IBS_KERNEL_TC | ibs.IBS_TC_FP4)
+    try:
+        want = []
+        for subs in calls:
+            ibs.ibs_compute_batch(ctx, pool, pool_n, m, subs)
+            ibs.ibs_synchronize(ctx)
+            want.append(subs[0][3].clone())
+        streams = [torch.cuda.Stream() for _ in calls]
+        for _ in range(5):
+            for subs in calls:
+                subs[0][3].fill_(-7)
+            torch.cuda.synchronize()
+            for subs, st in zip(calls, streams):
+                ibs.ibs_compute_batch(ctx, pool, pool_n, m, subs, stream=st)
+            torch.cuda.synchronize()
+            for subs, w in zip(calls, want):
+                assert torch.equal(subs[0][3], w)
+    finally:
+        ibs.ibs_shutdown(ctx)
+
+
 POLICY5_CHILD = r"""
 import sys
 import numpy as np
