@@ -42,6 +42,13 @@ void release_bytes(ibs_ctx* ctx, size_t bytes) {
   ctx->owned_bytes = bytes > ctx->owned_bytes ? 0 : ctx->owned_bytes - bytes;
 }
 
+bool drop_pool_words(ibs_ctx* ctx) {
+  std::lock_guard<std::mutex> lk(ctx->words_mu);
+  if (!ctx->pool_words.p) return false;
+  free_buf(ctx, ctx->pool_words);  // waits for the launches that read it
+  return true;
+}
+
 ibs_status ensure_buf(ibs_ctx* ctx, DevBuf& b, size_t need) {
   if (need == 0) need = 16;
   if (b.cap >= need) return IBS_OK;
@@ -55,6 +62,12 @@ ibs_status ensure_buf(ibs_ctx* ctx, DevBuf& b, size_t need) {
     return fail(IBS_ENOMEM, "workspace limit %zu bytes would be exceeded (need %zu more)", ctx->ws_limit, need);
   void* p = nullptr;
   cudaError_t e = cudaMalloc(&p, need);
+  // (the regrouped copies of genotypes only save time: they go first, but not
+  // one for the other)
+  if (e != cudaSuccess && &b != &ctx->pool_words) {
+    if (drop_pool_words(ctx)) e = cudaMalloc(&p, need);
+    if (e != cudaSuccess && serve_give_back_words(ctx)) e = cudaMalloc(&p, need);
+  }
   if (e != cudaSuccess) {
     release_bytes(ctx, need);
     cudaGetLastError();
@@ -1565,7 +1578,10 @@ extern "C" ibs_status ibs_compute_batch(ibs_ctx* ctx, const uint8_t* pool, int64
   BatchPlan& plan = *it->second;
   {
     // The regrouped pool is one buffer of the context: a batch on another stream
-    // waits for the last one that used it.
+    // waits for the last one that used it, and it is not given back before the
+    // launch that reads it is enqueued.
+    std::unique_lock<std::mutex> words_lk(ctx->words_mu, std::defer_lock);
+    if (plan.sweep) words_lk.lock();
     if (ibs_status s = plan_upload(ctx, plan, pool, pool_n, pool_m, subs, shapes, st)) return s;
     IBS_CUDA_TRY(cudaGraphLaunch(plan.exec, st));
     if (plan.uses_words) {
@@ -1783,7 +1799,7 @@ extern "C" ibs_status ibs_shutdown(ibs_ctx* ctx) {
     cudaDeviceSynchronize();
     for (auto& kv : ctx->plans) plan_free(ctx, *kv.second);
     ctx->plans.clear();
-    free_buf(ctx, ctx->pool_words);
+    drop_pool_words(ctx);
     if (ctx->words_ev) cudaEventDestroy(ctx->words_ev);
     free_buf(ctx, ctx->planes);
     free_buf(ctx, ctx->partial);

@@ -174,7 +174,8 @@ struct ibs_ctx {
   std::vector<TimingRec> timing_used, timing_free;
 
   // batches on the sweep kernel: the pool's rows in use, regrouped by sample on
-  // every call; one buffer for all plans
+  // every call; one buffer for all plans, given back when memory runs short
+  std::mutex words_mu;  // pool_words: from its allocation to the launch that reads it
   ibs::DevBuf pool_words;
   cudaEvent_t words_ev = nullptr;  // after the last batch that used it
   std::map<std::vector<int64_t>, std::unique_ptr<ibs::BatchPlan>> plans;
@@ -187,6 +188,10 @@ namespace ibs {
 
 ibs_status ensure_buf(ibs_ctx* ctx, DevBuf& b, size_t need);
 void free_buf(ibs_ctx* ctx, DevBuf& b);
+// Memory that only saves time, given back when an allocation finds no room (true
+// if there was any): the batches' regrouped pool, the served panel's code bits.
+bool drop_pool_words(ibs_ctx* ctx);
+bool serve_give_back_words(ibs_ctx* ctx);
 bool reserve_bytes(ibs_ctx* ctx, size_t bytes);
 void release_bytes(ibs_ctx* ctx, size_t bytes);
 int pick_mode(const ibs_ctx* ctx);

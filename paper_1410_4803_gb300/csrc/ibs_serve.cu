@@ -248,6 +248,7 @@ class ServeEngine {
     if (bytes == 0) return IBS_OK;
     cudaError_t e = cudaMallocAsync(&b.p, bytes, s);
     if (e != cudaSuccess && give_back_words()) e = cudaMallocAsync(&b.p, bytes, s);
+    if (e != cudaSuccess && drop_pool_words(ctx)) e = cudaMallocAsync(&b.p, bytes, s);
     if (e != cudaSuccess) {
       cudaGetLastError();
       b.p = nullptr;
@@ -872,6 +873,11 @@ std::shared_ptr<ServeEngine> engine_of(ibs_ctx* ctx) {
   return ctx->serve;
 }
 
+bool serve_give_back_words(ibs_ctx* ctx) {
+  const auto e = engine_of(ctx);
+  return e && e->give_back_words();
+}
+
 void serve_stop(ibs_ctx* ctx) {
   std::shared_ptr<ServeEngine> e;
   {
@@ -945,6 +951,7 @@ ibs_status serve_panel_load(ibs_ctx* ctx, const uint8_t* panel, int64_t n_panel,
   void* tmp = nullptr;
   if (ptr_kind(panel) != PtrKind::Device) {
     cudaError_t e = cudaMalloc(&tmp, bytes);
+    if (e != cudaSuccess && drop_pool_words(ctx)) e = cudaMalloc(&tmp, bytes);
     if (e != cudaSuccess) {
       free_buf(ctx, eng->panel_planes);
       no_sweep();

@@ -375,6 +375,43 @@ def test_failed_step_ends_its_requests(q, flags):
         ibs.ibs_shutdown(ctx)
 
 
+def test_panel_words_make_room():
+    """The panel's code bits (1 GB here) only save time: a matrix whose operand
+    planes find no room beside them gets it, and queries go on without them."""
+    import torch
+    from paper_1410_4803_gb300 import ibs
+    g = torch.Generator(device="cuda").manual_seed(3)
+    rand = lambda n, m: torch.randint(0, 256, (m, (n + 3) // 4), dtype=torch.uint8, device="cuda", generator=g)  # noqa: E731
+    n_panel, m_panel, n, m, k = 40_000, 100_000, 6000, 150_000, 4
+    panel, packed = rand(n_panel, m_panel), rand(n, m)
+    row = rand(1, m_panel).cpu()
+    counts = torch.empty((n * (n + 1) // 2, 4), dtype=torch.int32, device="cuda")
+    ctx = ibs.ibs_init(0)
+    ibs.ibs_compute(ctx, packed, n, m, counts)
+    ibs.ibs_synchronize(ctx)
+    want = counts.clone()
+    ibs.ibs_shutdown(ctx)
+    ctx = ibs.ibs_init(0)
+    hold = None
+    try:
+        ibs.ibs_panel_load(ctx, panel, n_panel, m_panel)
+        outs = [(_pinned((1, k), torch.int32), _pinned((1, k), torch.float64)) for _ in range(2)]
+        ibs.ibs_wait(ctx, ibs.ibs_query(ctx, row, 1, k, None, *outs[0]), timeout_ms=60000)
+        torch.cuda.empty_cache()
+        hold = torch.empty(torch.cuda.mem_get_info()[0] - (3 << 29), dtype=torch.uint8, device="cuda")  # 1.5 GB left
+        counts.fill_(-7)
+        ibs.ibs_compute(ctx, packed, n, m, counts)  # 1.8 GB of planes
+        ibs.ibs_synchronize(ctx)
+        hold = None
+        torch.cuda.empty_cache()
+        assert torch.equal(counts, want)
+        ibs.ibs_wait(ctx, ibs.ibs_query(ctx, row, 1, k, None, *outs[1]), timeout_ms=60000)
+        assert torch.equal(outs[0][0], outs[1][0]) and torch.equal(outs[0][1], outs[1][1])
+    finally:
+        hold = None
+        ibs.ibs_shutdown(ctx)
+
+
 SERVE_TWO_SM = r"""
 import sys
 import numpy as np
