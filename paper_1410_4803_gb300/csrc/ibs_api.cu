@@ -95,6 +95,7 @@ using namespace ibs;
 
 namespace {
 
+constexpr char kTuneSweep[] = "_sweep";  // ends the tune keys of batches on the sweep kernel
 constexpr int kFlagPlain = 0x10;  // force the plain kernel (one POPC per count and word)
 constexpr int kFlagCsa = 0x20;    // force the carry-save kernel
 
@@ -203,7 +204,11 @@ ibs_status ibs_init(const ibs_config* cfg, ibs_ctx** out_ctx) {
       const int got = sscanf(line.c_str(),
                              "{\"key\": \"%511[^\"]\", \"mode\": %d, \"split\": %d, \"ms\": %lf, \"pair_min\": %lld}", key,
                              &t.mode, &t.split_policy, &t.ms, &pm);
-      if (got >= 4) {  // entries written before the size class was tuned lack pair_min
+      // (entries written before the size class was tuned lack pair_min; an untimed
+      // entry under a timed policy's key is none)
+      const std::string k = got >= 1 ? key : "";
+      const bool sweep = k.size() > strlen(kTuneSweep) && k.rfind(kTuneSweep) == k.size() - strlen(kTuneSweep);
+      if (got >= 4 && (t.ms > 0 || sweep)) {
         t.pair_min = pm;
         ctx->tune[key] = t;
       }
@@ -1462,8 +1467,7 @@ extern "C" ibs_status ibs_compute_batch(ibs_ctx* ctx, const uint8_t* pool, int64
     // 3.8 with the best of the other policies; 64 of 200 to 8,000 samples and
     // 10,000 to 200,000 markers: 79 ms against 134).
     bool sweep = tc && ctx->ws_limit == 0 && tc_format_for(ctx) == kTcFp4 && tc_pair_mode() >= 0 && !tc_tile_kernel_forced() &&
-                 (fixed_policy < 0 || fixed_policy == 2) &&
-                 (te == ctx->tune.end() || te->second.split_policy == 2 || fixed_policy == 2);
+                 (fixed_policy < 0 || fixed_policy == 2);
     for (const auto& sh : shapes) sweep = sweep && sweep_usable(sh.n, sh.m);
     auto plan = std::make_unique<BatchPlan>();
     if (sweep && plan_build(ctx, *plan, shapes, mode, 2, 1024, true) != IBS_OK) {
@@ -1474,11 +1478,13 @@ extern "C" ibs_status ibs_compute_batch(ibs_ctx* ctx, const uint8_t* pool, int64
       clear_error();
     }
     if (sweep) {
-      if (fixed_policy < 0 && te == ctx->tune.end() && !getenv("IBS_NO_AUTOTUNE")) {
+      // recorded under a key of its own: the entries of the timed policies neither
+      // keep a batch off the sweep kernel nor stand in for a measurement
+      if (fixed_policy < 0 && !getenv("IBS_NO_AUTOTUNE") && ctx->tune.count(tk + kTuneSweep) == 0) {
         TuneEntry t;
         t.mode = mode;
         t.split_policy = 2;
-        ctx->tune[tk] = t;
+        ctx->tune[tk + kTuneSweep] = t;
         save_tune(ctx);
       }
     } else if (fixed_policy >= 0) {

@@ -302,6 +302,50 @@ def test_batches_on_two_streams():
         ibs.ibs_shutdown(ctx)
 
 
+def test_tune_file_and_the_sweep_kernel(tmp_path):
+    """The sweep kernel's batches are not timed: an entry of another policy does
+    not keep a batch off it, and it leaves no entry that a context which cannot
+    take it (a workspace limit) would follow unmeasured."""
+    import json
+    from paper_1410_4803_gb300 import ibs
+    pool_n, m = 600, 3000
+    pool = _random_pool(pool_n, m, 3)
+    subs = [_subset_args(pool_n, n, 0, vl, n)[0] for n, vl in ((300, 3000), (150, 2000), (90, 2500), (200, 900))]
+    path = tmp_path / "tune.jsonl"
+
+    def run(**kw):
+        """Kernel launches of the batch on a new context, and the file's entries after it."""
+        for s in subs:
+            s[3].fill_(-7)
+        ctx = ibs.ibs_init(0, flags=ibs.IBS_KERNEL_TC | ibs.IBS_TC_FP4, autotune_cache_path=str(path), **kw)
+        try:
+            ibs.ibs_compute_batch(ctx, pool, pool_n, m, subs)
+            ibs.ibs_synchronize(ctx)
+            launches = ibs.ibs_last_launch_info(ctx)["launches"]
+        finally:
+            ibs.ibs_shutdown(ctx)
+        return launches, [json.loads(x) for x in path.read_text().splitlines()]
+
+    launches, entries = run()
+    assert launches <= 3  # gather, sweeps, sums
+    want = [s[3].clone() for s in subs]
+    assert all(e["ms"] == 0 for e in entries)
+    _, entries = run(workspace_bytes=256 << 20)
+    timed = [e for e in entries if e["ms"] > 0]
+    assert len(timed) == 1
+    for s, w in zip(subs, want):
+        assert (s[3] == w).all()
+    # the entry of another policy
+    path.write_text(json.dumps(dict(timed[0], split=0)) + "\n")
+    launches, entries = run()
+    assert launches <= 3
+    assert [e for e in entries if e["ms"] > 0] == [dict(timed[0], split=0)]
+    # an untimed entry under a timed policy's key is measured anew
+    path.write_text(json.dumps(dict(timed[0], ms=0.0, split=2)) + "\n")
+    _, entries = run(workspace_bytes=256 << 20)
+    assert len([e for e in entries if e["ms"] > 0]) == 1
+
+
 POLICY5_CHILD = r"""
 import sys
 import numpy as np
