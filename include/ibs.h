@@ -188,7 +188,8 @@ typedef struct {
  *      windows reach the two-SM size (see ibs_compute_kernel) run the two-SM
  *      kernel.  With E2M1 operands, the sweep kernel allowed and no workspace
  *      limit set, this policy is one gather and one sweep-kernel launch over
- *      all subsets instead, and it is taken without timing the others;
+ *      all subsets instead, and it is taken without timing the others (but for
+ *      a lone subset of up to 128 samples over many variants);
  *   3  one two-SM persistent launch over every subset's two-SM work list,
  *      concatenated, with the gather fused: a concurrent gather kernel fills
  *      the operand planes unit by unit and per-subset readiness counters hold

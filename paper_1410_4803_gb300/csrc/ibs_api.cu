@@ -1465,8 +1465,15 @@ extern "C" ibs_status ibs_compute_batch(ibs_ctx* ctx, const uint8_t* pool, int64
     // every subset and no workspace limit is set, and nothing is timed (24
     // subsets of 100 to 3,000 samples and 5,000 to 80,000 markers: 2.6 ms against
     // 3.8 with the best of the other policies; 64 of 200 to 8,000 samples and
-    // 10,000 to 200,000 markers: 79 ms against 134).
-    bool sweep = tc && ctx->ws_limit == 0 && tc_format_for(ctx) == kTcFp4 && tc_pair_mode() >= 0 && !tc_tile_kernel_forced() &&
+    // 10,000 to 200,000 markers: 79 ms against 134).  A lone subset of one block of
+    // samples stays with the timed policies where its markers are many, as in
+    // ibs_compute: sweep kernel and best policy, 16 x 10,000 47 us and 49, 16 x
+    // 14,000 52 and 47, 64 x 18,000 57 and 57, 85 x 25,000 62 and 63, 85 x 100,000
+    // 116 and 94, 120 x 35,000 76 and 78, 128 x 100,000 117 and 114; but two of 40 x
+    // 100,000 126 and 139, four of 85 x 100,000 218 and 287.
+    const bool narrow = n_subsets == 1 && shapes[0].n <= 128 &&
+                        shapes[0].m > std::max<int64_t>(12000, 4000 + 280 * shapes[0].n);
+    bool sweep = !narrow && tc && ctx->ws_limit == 0 && tc_format_for(ctx) == kTcFp4 && tc_pair_mode() >= 0 && !tc_tile_kernel_forced() &&
                  (fixed_policy < 0 || fixed_policy == 2);
     for (const auto& sh : shapes) sweep = sweep && sweep_usable(sh.n, sh.m);
     auto plan = std::make_unique<BatchPlan>();

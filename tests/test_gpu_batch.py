@@ -346,6 +346,30 @@ def test_tune_file_and_the_sweep_kernel(tmp_path):
     assert len([e for e in entries if e["ms"] > 0]) == 1
 
 
+@pytest.mark.parametrize("n,m,timed", [(16, 12_000, False), (16, 12_001, True), (100, 32_000, False),
+                                       (100, 32_001, True), (128, 39_841, True), (129, 39_841, False)])
+def test_lone_narrow_subset(tmp_path, n, m, timed):
+    """Either side of the sizes at which a lone subset of one block of samples
+    goes to the timed policies."""
+    import json
+    from paper_1410_4803_gb300 import ibs
+    pool_n = 150
+    pool = _random_pool(pool_n, m, n)
+    subs = _subset_args(pool_n, n, 0, m, n)
+    path = tmp_path / "tune.jsonl"
+    ctx = ibs.ibs_init(0, flags=ibs.IBS_KERNEL_TC | ibs.IBS_TC_FP4, autotune_cache_path=str(path))
+    try:
+        for _ in range(2):
+            subs[0][3].fill_(-7)
+            ibs.ibs_compute_batch(ctx, pool, pool_n, m, subs)
+            ibs.ibs_synchronize(ctx)
+            G = oracle.unpack_subset(pool.cpu().numpy(), pool_n, m, subs[0][0].cpu().numpy(), 0, m)
+            assert (subs[0][3].cpu().numpy() == oracle.ibs_triangle_from_codes(G)[0]).all()
+    finally:
+        ibs.ibs_shutdown(ctx)
+    assert any(json.loads(x)["ms"] > 0 for x in path.read_text().splitlines()) == timed
+
+
 POLICY5_CHILD = r"""
 import sys
 import numpy as np
