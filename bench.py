@@ -330,7 +330,7 @@ def run_matrix(args, rank, world, local, name: str, full: bool = True):
     probe = ibs.ibs_probe_int_pipes(ctx)
     kinfo = ibs.ibs_kernel_info(ctx)
     kname = ibs.ibs_compute_kernel(ctx, n, m)
-    sweep = use_tc and kinfo["tc_format"] == "e2m1" and n > 256 and m < 1 << 21  # the marker-sweep kernel
+    sweep = ibs.ibs_compute_sweep_kernel(ctx, n, m)
     two_sm = use_tc and kname == "tc-pair"  # without it: the cta_group::2 kernel for long items
     mma_probe = ibs.ibs_probe_mma(ctx) if use_tc else None
 

@@ -368,8 +368,8 @@ ibs_status ibs_grm(ibs_ctx* ctx, const uint8_t* packed, int64_t n_samples, int64
  * operand format (0 E4M3, 1 E2M1), out[2] = SMs of the device, out[3] = device. */
 ibs_status ibs_kernel_info(ibs_ctx* ctx, int64_t out[4]);
 
-/* The pair kernel ibs_compute runs on this context for an n_samples x
- * n_variants matrix, written to *out: 0 POPC plain, 1 POPC carry-save,
+/* The class of pair kernel that ibs_compute runs on this context for an n_samples
+ * x n_variants matrix, written to *out: 0 POPC plain, 1 POPC carry-save,
  * 2 tensor core, 3 tensor core with 129 or more samples and at least 65,536
  * variants (E2M1 operands, triangle output), 4 tensor core with square output.
  * With E2M1 operands these three classes run on the two-SM kernel that sweeps
@@ -378,11 +378,19 @@ ibs_status ibs_kernel_info(ibs_ctx* ctx, int64_t out[4]);
  * 128 over 16,384, up to 256 over 49,152), with 2^21 or more variants and with
  * E4M3 operands, class 2 runs one persistent CTA per SM, class 3 the two-SM kernel
  * over 256 x 128 tiles and class 4 one CTA per tile.
- * IBS_TC_PAIR=1 in the environment reports class 3 for every size of 129 or
- * more samples, IBS_TC_PAIR=0 runs (and reports) one CTA per SM always.  Host
+ * ibs_compute_sweep_kernel says which of the two.
+ * IBS_TC_PAIR=1 in the environment makes class 3 of every size of 129 or more
+ * samples, IBS_TC_PAIR=0 runs (and reports) one CTA per SM always; IBS_SWEEP=0,
+ * read by ibs_init, keeps every path of the context off the sweep kernel.  Host
  * only, no device work; IBS_EINVAL for sizes ibs_compute
  * refuses or out == NULL. */
 ibs_status ibs_compute_kernel(ibs_ctx* ctx, int64_t n_samples, int64_t n_variants, int64_t* out);
+
+/* 1 in *out when ibs_compute on this context runs the sweep kernel for an
+ * n_samples x n_variants matrix, 0 when it runs the kernel of the class that
+ * ibs_compute_kernel reports (also once the sweep kernel's workspace has found
+ * no room for this shape).  IBS_EINVAL as there. */
+ibs_status ibs_compute_sweep_kernel(ibs_ctx* ctx, int64_t n_samples, int64_t n_variants, int64_t* out);
 
 /* Counters of the last ibs_compute / ibs_compute_batch on this context:
  * out[0] = kernel launches enqueued, out[1] = pair tiles, out[2] = K splits. */

@@ -179,6 +179,8 @@ ibs_status ibs_init(const ibs_config* cfg, ibs_ctx** out_ctx) {
   ctx->cc_minor = prop.minor;
   const char* tcenv = getenv("IBS_DEFAULT_KERNEL");
   ctx->default_tc = !(tcenv && strcmp(tcenv, "popc") == 0);
+  const char* senv = getenv("IBS_SWEEP");
+  ctx->sweep_on = !(senv && strcmp(senv, "0") == 0);
   const char* env = getenv("IBS_PAIR_MODE");
   if (env && env[0] >= '0' && env[0] <= '2' && env[1] == 0) ctx->default_mode = env[0] - '0';
   e = cudaHostAlloc(reinterpret_cast<void**>(&ctx->status_host), sizeof(int), cudaHostAllocMapped);
@@ -233,7 +235,7 @@ static bool tc_tile_kernel_forced() {
 // 74 and 142 ms, the square of 3,001 x 60,000 386 us and 788; but 64 x 20,000 36
 // and 33, 85 x 100,000 76 and 43, 200 x 100,000 86 and 65, 40 x 400,000 94 and 72.
 static bool use_sweep(const ibs_ctx* ctx, int64_t n, int64_t m, bool square) {
-  return tc_format_for(ctx) == kTcFp4 && tc_pair_mode() >= 0 && !tc_tile_kernel_forced() &&
+  return ctx->sweep_on && tc_format_for(ctx) == kTcFp4 && tc_pair_mode() >= 0 && !tc_tile_kernel_forced() &&
          !(n <= 128 && m > 16384) && !(n <= 256 && m > 49152) && sweep_usable(n, m) &&
          ctx->sweep_refused != std::vector<int64_t>{n, m, square ? 1 : 0};
 }
@@ -1473,7 +1475,7 @@ extern "C" ibs_status ibs_compute_batch(ibs_ctx* ctx, const uint8_t* pool, int64
     // 100,000 126 and 139, four of 85 x 100,000 218 and 287.
     const bool narrow = n_subsets == 1 && shapes[0].n <= 128 &&
                         shapes[0].m > std::max<int64_t>(12000, 4000 + 280 * shapes[0].n);
-    bool sweep = !narrow && tc && ctx->ws_limit == 0 && tc_format_for(ctx) == kTcFp4 && tc_pair_mode() >= 0 && !tc_tile_kernel_forced() &&
+    bool sweep = ctx->sweep_on && !narrow && tc && ctx->ws_limit == 0 && tc_format_for(ctx) == kTcFp4 && tc_pair_mode() >= 0 && !tc_tile_kernel_forced() &&
                  (fixed_policy < 0 || fixed_policy == 2);
     for (const auto& sh : shapes) sweep = sweep && sweep_usable(sh.n, sh.m);
     auto plan = std::make_unique<BatchPlan>();
@@ -1783,6 +1785,15 @@ extern "C" ibs_status ibs_compute_kernel(ibs_ctx* ctx, int64_t n, int64_t m, int
   } else {
     *out = tc_pair_usable(n, m, tc_format_for(ctx)) ? 3 : 2;
   }
+  return IBS_OK;
+}
+
+extern "C" ibs_status ibs_compute_sweep_kernel(ibs_ctx* ctx, int64_t n, int64_t m, int64_t* out) {
+  int64_t kernel = 0;
+  if (ibs_status s = ibs_compute_kernel(ctx, n, m, &kernel)) return s;
+  if (!out) return fail(IBS_EINVAL, "out is NULL");
+  DeviceGuard g(ctx->device);
+  *out = use_tc(ctx) && use_sweep(ctx, n, m, (ctx->flags & IBS_OUT_SQUARE) != 0) ? 1 : 0;
   return IBS_OK;
 }
 

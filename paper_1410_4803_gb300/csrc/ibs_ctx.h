@@ -127,6 +127,7 @@ struct ibs_ctx {
   int cc_major = 0, cc_minor = 0;
   int default_mode = 1;
   bool default_tc = true;         // ibs_compute uses the tensor-core form unless told otherwise
+  bool sweep_on = true;           // the sweep kernel where it can run (IBS_SWEEP=0: never)
 
   std::mutex mu;                  // guards memory accounting
   size_t owned_bytes = 0;

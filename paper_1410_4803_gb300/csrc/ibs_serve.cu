@@ -912,7 +912,7 @@ ibs_status serve_panel_load(ibs_ctx* ctx, const uint8_t* panel, int64_t n_panel,
     eng->clusters = 0;
     eng->pgeo = eng->geo(n_panel);
   };
-  if (eng->tc && eng->fmt == kTcFp4 && ctx->ws_limit == 0 && tc_pair_mode() >= 0 && sweep_usable(std::max<int64_t>(n_panel, kMaxRows), m)) {
+  if (ctx->sweep_on && eng->tc && eng->fmt == kTcFp4 && ctx->ws_limit == 0 && tc_pair_mode() >= 0 && sweep_usable(std::max<int64_t>(n_panel, kMaxRows), m)) {
     eng->clusters = sweep_clusters();
     eng->sweep = true;
     for (DevBuf* b : {&eng->sweep_scratch, &eng->sync_scratch})

@@ -92,6 +92,7 @@ def load():
             "ibs_batch_plan_info": [p, ctypes.POINTER(ctypes.c_int64)],
             "ibs_kernel_info": [p, ctypes.POINTER(ctypes.c_int64)],
             "ibs_compute_kernel": [p, i64, i64, ctypes.POINTER(ctypes.c_int64)],
+            "ibs_compute_sweep_kernel": [p, i64, i64, ctypes.POINTER(ctypes.c_int64)],
             "ibs_ld_r": [p, p, i64, i64, i64, p, p, p],
             "ibs_cluster_complete": [p, p, i64, p, p],
             "ibs_grm": [p, p, i64, i64, p, p],
@@ -341,6 +342,15 @@ def ibs_compute_kernel(ctx: Context, n_samples: int, n_variants: int) -> str:
     out = ctypes.c_int64()
     _check(load().ibs_compute_kernel(ctx._h, n_samples, n_variants, ctypes.byref(out)), "ibs_compute_kernel")
     return COMPUTE_KERNELS[out.value]
+
+
+def ibs_compute_sweep_kernel(ctx: Context, n_samples: int, n_variants: int) -> bool:
+    """True when ibs_compute runs the sweep kernel for this shape, in place of
+    the kernel of the class that ibs_compute_kernel names."""
+    out = ctypes.c_int64()
+    _check(load().ibs_compute_sweep_kernel(ctx._h, n_samples, n_variants, ctypes.byref(out)),
+           "ibs_compute_sweep_kernel")
+    return out.value != 0
 
 
 def ibs_test_set_wait_limit(ctx: Context, ns: int):

@@ -173,6 +173,29 @@ def test_batch_each_policy(pool, policy, fmt, monkeypatch):
         ibs.ibs_shutdown(ctx)
 
 
+def test_batch_policy2_without_the_sweep_kernel(pool, monkeypatch):
+    """Policy 2's launches per subset, which the sweep kernel stands in for where it can run."""
+    import torch
+    from paper_1410_4803_gb300 import ibs
+    monkeypatch.setenv("IBS_BATCH_POLICY", "2")
+    monkeypatch.setenv("IBS_SWEEP", "0")
+    w, codes = pool
+    subs = _make_subsets(np.random.default_rng(9), w.n, w.m)
+    ctx = ibs.ibs_init(0, flags=_flags(ibs, "IBS_KERNEL_TC|IBS_TC_FP4"))
+    try:
+        dev = torch.from_numpy(w.packed).cuda()
+        for _ in range(2):
+            res = _run_batch(ctx, w, subs, dev)
+            assert ibs.ibs_last_launch_info(ctx)["launches"] > len(subs)
+            for (idx, vb, vl), (c, d) in zip(subs, res):
+                G = oracle.unpack_subset(w.packed, w.n, w.m, idx, vb, vl)
+                oc, od, _ = oracle.ibs_triangle_from_codes(G)
+                assert (c == oc).all(), f"n={idx.size} window={vb}+{vl}"
+                assert_dist_close(d, od)
+    finally:
+        ibs.ibs_shutdown(ctx)
+
+
 def test_batch_out_of_range_index_is_reported(pool):
     """A corrupted sample index is not read: the kernel treats that sample as
     all-missing and ibs_synchronize reports IBS_EINVAL."""

@@ -1,8 +1,10 @@
 """The two-SM pair kernel (tcgen05 cta_group::2) through ibs_compute, forced
-on for every size with IBS_TC_PAIR=1: bit-exact counts and distances within
-1e-12 against the oracle.  The switch is read once per process, so each case
-runs in a child process.  Also the default choice (ibs_compute_kernel): the
-pair kernel for 65,536 or more variants, the one-SM kernel otherwise.
+on for every size with IBS_TC_PAIR=1, and with IBS_SWEEP=0 so that the sweep
+kernel does not take its place: bit-exact counts and distances within 1e-12
+against the oracle.  IBS_TC_PAIR is read once per process, so each case
+runs in a child process.  Also the class of each size (ibs_compute_kernel): the
+pair kernel for 65,536 or more variants, the one-SM kernel otherwise; and the
+sizes that run the sweep kernel instead (ibs_compute_sweep_kernel).
 Shapes: two blocks with a ragged marker tail, a lone diagonal tile per column
 pair, garbage in the padding bits, every tile split over K (fewer pair items
 than clusters), and whole waves plus an unsplit tail; every ring variant.
@@ -28,7 +30,7 @@ from paper_1410_4803_gb300 import ibs
 ctx = ibs.ibs_init(0, flags=ibs.IBS_KERNEL_TC | ibs.IBS_TC_FP4)
 rng = np.random.default_rng({seed})
 for n, m, miss, garbage in {shapes!r}:
-    assert ibs.ibs_compute_kernel(ctx, n, m) == "tc-pair", (n, m)
+    assert ibs.ibs_compute_kernel(ctx, n, m) == "tc-pair" and not ibs.ibs_compute_sweep_kernel(ctx, n, m), (n, m)
     codes = random_codes(rng, n, m, miss=miss)
     packed = pack_codes(codes, garbage_rng=np.random.default_rng(7) if garbage else None)
     want_c, want_d = oracle.ibs_triangle(packed, n, m)
@@ -52,7 +54,7 @@ SHAPES = {
 @pytest.mark.parametrize("ring", sorted(SHAPES))
 def test_pair_kernel_matches_oracle(ring):
     code = CHILD.format(tests=os.path.join(ROOT, "tests"), root=ROOT, seed=11, shapes=SHAPES[ring])
-    env = dict(os.environ, IBS_TC_PAIR="1", IBS_TC_PAIR_RING=ring)
+    env = dict(os.environ, IBS_TC_PAIR="1", IBS_SWEEP="0", IBS_TC_PAIR_RING=ring)
     r = subprocess.run([sys.executable, "-c", code], env=env, capture_output=True, text=True, timeout=600)
     assert r.returncode == 0, r.stdout + r.stderr
     assert r.stdout.count("ok n=") == len(SHAPES[ring])
@@ -90,6 +92,24 @@ def test_default_kernel_choice(mode):
     assert r.returncode == 0 and "ok" in r.stdout, r.stdout + r.stderr
 
 
+def test_sizes_of_the_sweep_kernel(monkeypatch):
+    """Where the sweep kernel runs, and the switch that keeps a context off it."""
+    from paper_1410_4803_gb300 import ibs
+    tc4, tc8 = ibs.IBS_KERNEL_TC | ibs.IBS_TC_FP4, ibs.IBS_KERNEL_TC | ibs.IBS_TC_FP8
+    want = [(tc4, 4096, 100_000, True), (tc4, 256, 4096, True), (tc4, 1, 1, True), (tc4, 300, 2_097_151, True),
+            (tc4, 300, 2_097_152, False), (tc4, 128, 16_384, True), (tc4, 128, 16_385, False),
+            (tc4, 200, 70_000, False), (tc4 | ibs.IBS_OUT_SQUARE, 3001, 60_000, True), (tc8, 4096, 100_000, False),
+            (ibs.IBS_KERNEL_CSA, 4096, 100_000, False)]
+    monkeypatch.delenv("IBS_SWEEP", raising=False)
+    for flags, n, m, sweep in want:
+        with ibs.ibs_init(0, flags=flags) as ctx:
+            assert ibs.ibs_compute_sweep_kernel(ctx, n, m) == sweep, (flags, n, m)
+    monkeypatch.setenv("IBS_SWEEP", "0")
+    for flags, n, m, _ in want:
+        with ibs.ibs_init(0, flags=flags) as ctx:
+            assert not ibs.ibs_compute_sweep_kernel(ctx, n, m)
+
+
 # K-lockstep of full waves with short segments, so that the bounded waits run
 # many times per item: shapes with at least one full wave of pair items (76
 # clusters; 2,200 samples = 18 blocks = 90 pair items) and hundreds of chunks,
@@ -100,7 +120,7 @@ SYNC_SHAPES = [(2200, 20_000, 0.02, True), (2500, 9_001, 0.05, False), (700, 30_
 @pytest.mark.parametrize("sync", ["16,2", "16,3"])
 def test_pair_kernel_lockstep_matches_oracle(sync):
     code = CHILD.format(tests=os.path.join(ROOT, "tests"), root=ROOT, seed=12, shapes=SYNC_SHAPES)
-    env = dict(os.environ, IBS_TC_PAIR="1", IBS_TC_PAIR_SYNC=sync)
+    env = dict(os.environ, IBS_TC_PAIR="1", IBS_SWEEP="0", IBS_TC_PAIR_SYNC=sync)
     env.pop("IBS_TC_PAIR_RING", None)
     r = subprocess.run([sys.executable, "-c", code], env=env, capture_output=True, text=True, timeout=900)
     assert r.returncode == 0, r.stdout + r.stderr

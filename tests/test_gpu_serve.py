@@ -464,8 +464,8 @@ ibs.ibs_shutdown(ctx)
 
 def test_serving_two_sm_kernel_matches_oracle():
     """The engine's steps and the unbatched path on the two-SM kernel (forced
-    on for this small panel with IBS_TC_PAIR=1; the switch is read once per
-    process, so the case runs in a child): items of two query blocks x one
+    on for this small panel with IBS_TC_PAIR=1, the sweep kernel off; the first
+    switch is read once per process, so the case runs in a child): items of two query blocks x one
     panel block, a lone last block when the step's block count is odd, steps
     of one block on the one-SM kernel, counts columns copied to host memory
     step by step."""
@@ -474,7 +474,7 @@ def test_serving_two_sm_kernel_matches_oracle():
     import sys
     root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
     code = SERVE_TWO_SM.format(tests=os.path.join(root, "tests"), root=root)
-    env = dict(os.environ, IBS_TC_PAIR="1")
+    env = dict(os.environ, IBS_TC_PAIR="1", IBS_SWEEP="0")
     r = subprocess.run([sys.executable, "-c", code], env=env, capture_output=True, text=True, timeout=900)
     assert r.returncode == 0, r.stdout + r.stderr
     assert r.stdout.count("ok q=") == 8, r.stdout

@@ -44,23 +44,28 @@ def test_parts_and_waves(ctx, n, m):
 
 
 # either side of the sizes that leave the sweep kernel: one block of samples, two
-@pytest.mark.parametrize("n,m", [(128, 16_384), (128, 16_385), (129, 16_385), (256, 49_152), (256, 49_153), (257, 49_153)])
+# (the two-SM kernel from 65,536 markers on)
+@pytest.mark.parametrize("n,m", [(128, 16_384), (128, 16_385), (129, 16_385), (256, 49_152), (256, 49_153), (257, 49_153),
+                                 (200, 70_000)])
 def test_narrow_inputs(ctx, n, m):
     _check(ctx, n, m, n + m)
 
 
-def test_no_room_for_the_workspace():
+# planes 26 MB, partial counts 2.9 MB: the one-SM kernel; planes 51 MB: the two-SM kernel
+@pytest.mark.parametrize("n,m,limit,kernel", [(600, 20_000, 32 << 20, "tc-persistent"), (300, 66_000, 56 << 20, "tc-pair")])
+def test_no_room_for_the_workspace(n, m, limit, kernel):
     """A workspace bound that holds operand planes and partial counts but not
     the sweep kernel's scratch and parts: the call still computes."""
     from paper_1410_4803_gb300 import ibs
     rng = np.random.default_rng(3)
-    n, m = 600, 20_000
     packed = pack_codes(random_codes(rng, n, m))
     want_c, want_d = oracle.ibs_triangle(packed, n, m)
-    c = ibs.ibs_init(0, workspace_bytes=32 << 20)  # planes 26 MB, partial counts 2.9 MB
+    c = ibs.ibs_init(0, workspace_bytes=limit)
     try:
+        assert ibs.ibs_compute_kernel(c, n, m) == kernel and ibs.ibs_compute_sweep_kernel(c, n, m)
         for _ in range(2):
             got_c, got_d = gpu_compute(c, packed, n, m)
+            assert not ibs.ibs_compute_sweep_kernel(c, n, m)
             assert (got_c == want_c).all()
             assert_dist_close(got_d, want_d)
     finally:

@@ -6,9 +6,9 @@ the context's status word, stops issuing work, waits (with the full bound)
 for the copies and MMAs it already issued, frees its tensor memory and
 returns.  The test sets a 1 ns bound through the test hook, so the first
 wait that is not already over (an operand stage, the accumulators) runs out,
-in the one-SM persistent kernel and in the two-SM kernel (whose waiter warp
-then stops waiting but keeps releasing its MMA warp until the work list
-ends); ibs_synchronize must then
+in the one-SM persistent kernel, in the sweep kernel and in the two-SM kernel
+(whose waiter warp then stops waiting but keeps releasing its MMA warp until the
+work list ends); ibs_synchronize must then
 report IBS_ETIMEOUT, and the next call on the same context with the default
 bound must be bit-exact against the oracle.  The failure is made on the
 device with a short limit only: nothing faults, traps or hangs.
@@ -27,7 +27,8 @@ def _run(ctx, packed_dev, n, m):
     return counts, dist
 
 
-@pytest.mark.parametrize("n,m,kernel", [(200, 60_000, "tc-persistent"), (300, 200_000, "tc-pair")])
+@pytest.mark.parametrize("n,m,kernel", [(200, 60_000, "tc-persistent"), (300, 200_000, "tc-pair"),
+                                        (200, 200_000, "tc-pair")])
 def test_short_wait_limit_reports_timeout_and_context_recovers(n, m, kernel):
     import torch
     import oracle
@@ -38,6 +39,7 @@ def test_short_wait_limit_reports_timeout_and_context_recovers(n, m, kernel):
     ctx = ibs.ibs_init(0)
     try:
         assert ibs.ibs_compute_kernel(ctx, n, m) == kernel
+        assert ibs.ibs_compute_sweep_kernel(ctx, n, m) == (n == 300)
         dev = torch.from_numpy(packed).cuda()
         ibs.ibs_test_set_wait_limit(ctx, 1)  # 1 ns: the first wait that is not already over runs out
         _run(ctx, dev, n, m)
