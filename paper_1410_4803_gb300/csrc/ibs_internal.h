@@ -342,6 +342,7 @@ bool sweep_usable(int64_t n, int64_t m);
 size_t sweep_planes_bytes(int64_t n, int64_t m);
 size_t sweep_scratch_bytes(int clusters);
 size_t sweep_slot_bytes();
+int sweep_max_slots(int clusters);  // of sweep_plan and sweep_plan_cross
 SweepSync sweep_sync(int waves, int stages, int2 setting);
 SweepPlan sweep_plan(int64_t n, int64_t m, int clusters);
 SweepPlan sweep_plan_batch(const std::vector<std::pair<int64_t, int64_t>>& shapes, int clusters);  // {n, m}

@@ -417,8 +417,11 @@ class ServeEngine {
            (pl.first.size() + 8) * sizeof(int32_t);
   }
   cudaError_t run_sweep(const SweepPlan& pl, const uint8_t* row_planes, int64_t row_half, int32_t* const* row_out,
-                        int64_t n_rows, uint8_t* host, uint8_t* dev, float* scratch, float* part, DevBuf& ctr,
-                        bool library_buf, cudaStream_t s) {
+                        int64_t n_rows, uint8_t* host, uint8_t* dev, const DevBuf& scratch, const DevBuf& part,
+                        DevBuf& ctr, bool library_buf, cudaStream_t s) {
+    // (the kernel indexes both by the plan)
+    if (sweep_scratch_bytes(pl.clusters) > scratch.cap || (size_t)pl.slots * sweep_slot_bytes() > part.cap)
+      return cudaErrorInvalidValue;
     const size_t ib = pl.items.size() * sizeof(SweepItem), gb = pl.groups.size() * sizeof(SweepGroup);
     std::memcpy(host, pl.items.data(), ib);
     if (gb > 0) std::memcpy(host + ib, pl.groups.data(), gb);
@@ -431,8 +434,8 @@ class ServeEngine {
     l.first = reinterpret_cast<const int32_t*>(dev + ib + gb);
     l.n_groups = (int64_t)pl.groups.size();
     l.clusters = pl.clusters;
-    l.scratch = scratch;
-    l.part = part;
+    l.scratch = static_cast<float*>(scratch.p);
+    l.part = static_cast<float*>(part.p);
     l.status = ctx->status_dev;
     l.wait_ns = kWaitLimitNs;
     l.sync = sweep_sync(pl.waves, pl.wave_stages, tc_pair_sync_setting(0));
@@ -451,8 +454,8 @@ class ServeEngine {
 
   // Parts that a plan over C clusters can need: its shares meet at C - 1 cuts,
   // each the end of one piece and the start of another, and a piece touches at
-  // most three products.
-  size_t sweep_part_bytes() const { return (size_t)6 * (size_t)std::max(1, clusters) * sweep_slot_bytes(); }
+  // most three products; in rounds, at most as many by their own rule.
+  size_t sweep_part_bytes() const { return (size_t)sweep_max_slots(clusters) * sweep_slot_bytes(); }
 
   cudaError_t ensure_items(size_t n) {
     if (n <= items_cap) return cudaSuccess;
@@ -667,8 +670,7 @@ class ServeEngine {
                            sweep_part.cap, ctx->num_sms, stream));
       } else if (sweep) {
         ok(run_sweep(pl, static_cast<const uint8_t*>(step_planes.p), kMaxRows / 64, outs_d, n_rows, items_host[slot],
-                     static_cast<uint8_t*>(items_dev[slot].p), static_cast<float*>(sweep_scratch.p),
-                     static_cast<float*>(sweep_part.p), sync_ctr, true, stream));
+                     static_cast<uint8_t*>(items_dev[slot].p), sweep_scratch, sweep_part, sync_ctr, true, stream));
       } else if (two_sm) {
         ok(cudaMemcpyAsync(items_dev[slot].p, items_host[slot], t * sizeof(PairItem), cudaMemcpyHostToDevice, stream));
         ok(launch_tc_pair_cross(static_cast<const uint8_t*>(panel_planes.p), pg.n, pgeo.chunks,
@@ -1294,8 +1296,7 @@ ibs_status serve_query_sync(ibs_ctx* ctx, const uint8_t* q, int64_t nq, int k, i
     if (e.sweep)
       ce = e.run_sweep(pl, static_cast<const uint8_t*>(r.planes.p), (nq + 63) / 64,
                        static_cast<int32_t* const*>(outs_d.p), nq, sweep_host.data(),
-                       static_cast<uint8_t*>(items_dev.p), static_cast<float*>(e.sync_scratch.p),
-                       static_cast<float*>(e.sync_part.p), sync_d, false, s);
+                       static_cast<uint8_t*>(items_dev.p), e.sync_scratch, e.sync_part, sync_d, false, s);
     else if (two_sm)
       ce = launch_tc_pair_cross(static_cast<const uint8_t*>(e.panel_planes.p), pg.n, e.pgeo.chunks,
                                 static_cast<const uint8_t*>(r.planes.p), qg.blocks,

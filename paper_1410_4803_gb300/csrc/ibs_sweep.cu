@@ -1033,6 +1033,7 @@ size_t sweep_planes_bytes(int64_t n, int64_t m) { return (size_t)((n + 63) / 64)
 
 size_t sweep_scratch_bytes(int clusters) { return (size_t)clusters * 2 * 3 * kSwHalfTile * sizeof(float); }
 size_t sweep_slot_bytes() { return 2 * kSwHalfTile * sizeof(float); }
+int sweep_max_slots(int clusters) { return kPartsPerCluster * std::max(1, clusters); }
 
 // Lockstep of `waves` waves of whole tiles of at most `stages` ring stages, by
 // the two-SM kernels' setting {chunks of 64 markers, lag}; off: no counters.
