@@ -376,7 +376,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kSwThreads, 1)
       const uint32_t full0 = cluster_addr(&full[0], 0);  // the even CTA's ring barriers
       uint8_t* dst0 = ring + (is_b ? kSwABytes : 0);
       uint32_t g = 0, s = 0, ph = 1;  // stages issued, ring slot, parity of the slot's previous release
-      bool stop = false;
+      bool stop = false, keep = true;
       for (int e = it0; e < it1 && !stop; ++e) {
         const SweepItem it = args.items[e];
         const int h = is_b ? 2 * it.J + it.w * (int)rank : 2 * (it.I + (int)rank);
@@ -385,7 +385,10 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kSwThreads, 1)
         const uint32_t bytes = 2u * (uint32_t)(kSwABytes + kSwCols * 1024 * it.w);
         // lockstep: warp 0 announces every segment and holds back until the
         // whole wave has started the segment `lag` back (warp 3 follows
-        // through the ring)
+        // through the ring).  That only saves traffic: where the wave does not
+        // come within a quarter of the bound that the other roles wait with
+        // (another kernel holds an SM, as the clustering of a large matrix does
+        // for seconds), the CTA goes on alone.
         int* ctr = !is_b && args.sync.seg > 0 && it.wave >= 0 ? args.sync.ctr + (int64_t)it.wave * args.sync.n_seg : nullptr;
         int left = 0, sg = 0;
         int q = it.q0;
@@ -399,10 +402,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kSwThreads, 1)
             if (ctr != nullptr && left-- == 0) {
               left = args.sync.seg - 1;
               atomicAdd(ctr + sg, 1);
-              if (sg >= args.sync.lag && !wait_ready(ctr + sg - args.sync.lag, 2 * (int)cluster_total(), wait_ns)) {
-                stop = true;
-                break;
-              }
+              if (keep && sg >= args.sync.lag)
+                keep = wait_ready(ctr + sg - args.sync.lag, 2 * (int)cluster_total(), wait_ns / 4);
               ++sg;
             }
             if (g >= (uint32_t)kSwStages && !ring_wait(&empty[s], ph, wait_ns, &abort_flag)) {

@@ -13,6 +13,8 @@ report IBS_ETIMEOUT, and the next call on the same context with the default
 bound must be bit-exact against the oracle.  The failure is made on the
 device with a short limit only: nothing faults, traps or hangs.
 """
+import time
+
 import numpy as np
 import pytest
 
@@ -56,6 +58,39 @@ def test_short_wait_limit_reports_timeout_and_context_recovers(n, m, kernel):
     want_c, want_d = oracle.ibs_triangle(packed, n, m)
     assert (got_c == want_c).all()
     assert_dist_close(got_d, want_d)
+
+
+def test_sweep_goes_on_while_another_kernel_holds_an_sm():
+    """The sweep kernel's waves run in lockstep over all SMs.  Clustering holds one
+    for longer than the bound of the waits (a launch of about 20 ms and 8 ms here;
+    seconds and 2 s for larger matrices): the call takes longer, and is right."""
+    import torch
+    from paper_1410_4803_gb300 import ibs
+    rng = np.random.default_rng(5)
+    n, m = 4500, 3003  # two whole waves of tiles
+    packed = torch.from_numpy(pack_codes(random_codes(rng, n, m))).cuda()
+    rows = 8192
+    d = torch.rand(rows * (rows + 1) // 2, dtype=torch.float64, device="cuda")
+    link = torch.empty((rows - 1, 4), dtype=torch.float64, device="cuda")
+    counts = torch.empty((n * (n + 1) // 2, 4), dtype=torch.int32, device="cuda")
+    with ibs.ibs_init(0) as ctx, ibs.ibs_init(0) as other:
+        assert ibs.ibs_compute_sweep_kernel(ctx, n, m)
+        ibs.ibs_compute(ctx, packed, n, m, counts)
+        ibs.ibs_synchronize(ctx)
+        want = counts.clone()
+        ibs.ibs_cluster_complete(other, d, rows, link)
+        ibs.ibs_synchronize(other)
+        ibs.ibs_test_set_wait_limit(ctx, 8_000_000)
+        streams = [torch.cuda.Stream() for _ in range(2)]
+        for _ in range(3):
+            counts.fill_(-7)
+            torch.cuda.synchronize()
+            ibs.ibs_cluster_complete(other, d, rows, link, stream=streams[0])
+            time.sleep(0.004)  # past its initialisation, in the launch on one SM
+            ibs.ibs_compute(ctx, packed, n, m, counts, stream=streams[1])
+            ibs.ibs_synchronize(ctx, streams[1])
+            torch.cuda.synchronize()
+            assert torch.equal(counts, want)
 
 
 def test_wait_limit_argument_checks():
