@@ -31,6 +31,7 @@
 // an operand whose rows are one contiguous run per column.
 #include <algorithm>
 #include <atomic>
+#include <climits>
 #include <cstdio>
 #include <cstdlib>
 #include <cstring>
@@ -376,7 +377,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kSwThreads, 1)
       const uint32_t full0 = cluster_addr(&full[0], 0);  // the even CTA's ring barriers
       uint8_t* dst0 = ring + (is_b ? kSwABytes : 0);
       uint32_t g = 0, s = 0, ph = 1;  // stages issued, ring slot, parity of the slot's previous release
-      bool stop = false, keep = true;
+      int lag = args.sync.lag;
+      bool stop = false;
       for (int e = it0; e < it1 && !stop; ++e) {
         const SweepItem it = args.items[e];
         const int h = is_b ? 2 * it.J + it.w * (int)rank : 2 * (it.I + (int)rank);
@@ -402,8 +404,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kSwThreads, 1)
             if (ctr != nullptr && left-- == 0) {
               left = args.sync.seg - 1;
               atomicAdd(ctr + sg, 1);
-              if (keep && sg >= args.sync.lag)
-                keep = wait_ready(ctr + sg - args.sync.lag, 2 * (int)cluster_total(), wait_ns / 4);
+              if (sg >= lag && !wait_ready(ctr + sg - lag, 2 * (int)cluster_total(), wait_ns / 4)) lag = INT_MAX;
               ++sg;
             }
             if (g >= (uint32_t)kSwStages && !ring_wait(&empty[s], ph, wait_ns, &abort_flag)) {
