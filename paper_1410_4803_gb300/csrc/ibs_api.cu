@@ -1132,7 +1132,10 @@ ibs_status plan_upload(ibs_ctx* ctx, BatchPlan& plan, const uint8_t* pool, int64
         sp.cols = cols;
         sp.words = static_cast<uint32_t*>(ctx->pool_words.p);
         plan.uses_words = true;
-        if (ctx->words_ev) IBS_CUDA_TRY(cudaStreamWaitEvent(st, ctx->words_ev, 0));
+        unsigned long long id = 0;
+        IBS_CUDA_TRY(cudaStreamGetId(st, &id));
+        if (ctx->words_ev && id != ctx->words_stream) IBS_CUDA_TRY(cudaStreamWaitEvent(st, ctx->words_ev, 0));
+        ctx->words_stream = id;
       }
       clear_error();
     }

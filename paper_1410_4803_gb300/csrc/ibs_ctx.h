@@ -178,6 +178,7 @@ struct ibs_ctx {
   // every call; one buffer for all plans, given back when memory runs short
   std::mutex words_mu;  // pool_words: from its allocation to the launch that reads it
   ibs::DevBuf pool_words;
+  unsigned long long words_stream = 0;  // id of the stream of the last batch that used it
   cudaEvent_t words_ev = nullptr;  // after the last batch that used it
   std::map<std::vector<int64_t>, std::unique_ptr<ibs::BatchPlan>> plans;
   std::map<std::string, ibs::TuneEntry> tune;
