@@ -107,7 +107,12 @@ ibs_status ibs_init(const ibs_config* cfg, ibs_ctx** out_ctx);
  *   stream      cudaStream_t or NULL.
  * Transposes the matrix into library-owned sample-major bit planes, then runs
  * the triangular pair-count kernel with the fused count/distance epilogue;
- * which pair kernel a shape gets is given by ibs_compute_kernel. */
+ * which pair kernel a shape gets is given by ibs_compute_kernel and
+ * ibs_compute_sweep_kernel.  A call of the shape of the context's last one enqueues
+ * kernels and memsets only and may be recorded into a CUDA graph.  The recording
+ * uses the work list of that shape and the workspace, which belong to the context:
+ * replay it while no call of another shape, and none that needs more workspace, has
+ * been made on the context since, else record it again. */
 ibs_status ibs_compute(ibs_ctx* ctx, const uint8_t* packed, int64_t n_samples, int64_t n_variants,
                        int32_t* out_counts, double* out_dist, void* stream);
 
