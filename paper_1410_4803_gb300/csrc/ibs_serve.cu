@@ -39,6 +39,7 @@
 #include <condition_variable>
 #include <cstring>
 #include <deque>
+#include <new>
 #include <shared_mutex>
 #include <thread>
 #include <unordered_map>
@@ -335,14 +336,25 @@ class ServeEngine {
       first = false;
     }
     lk.unlock();
+    bool any = false;
     for (const auto& r : behind) {
-      r->host_packed.resize((size_t)pg.m * (size_t)((r->q + 3) / 4));
-      cudaMemcpyAsync(r->host_packed.data(), r->packed.p, r->host_packed.size(), cudaMemcpyDeviceToHost, stream);
+      try {
+        r->host_packed.resize((size_t)pg.m * (size_t)((r->q + 3) / 4));
+      } catch (const std::bad_alloc&) {
+        continue;
+      }
+      if (cudaMemcpyAsync(r->host_packed.data(), r->packed.p, r->host_packed.size(), cudaMemcpyDeviceToHost, stream) !=
+              cudaSuccess ||
+          cudaStreamSynchronize(stream) != cudaSuccess) {
+        cudaGetLastError();
+        r->host_packed.clear();
+        continue;  // its samples stay where they are
+      }
       free_async(*r, true, stream);
+      any = true;
     }
-    cudaStreamSynchronize(stream);
     lk.lock();
-    return !behind.empty();
+    return any;
   }
 
   int32_t* counts_ptr(Request& r) { return r.counts_on_dev ? r.user_counts : static_cast<int32_t*>(r.counts.p); }
@@ -547,6 +559,7 @@ class ServeEngine {
   // against the current panel chunk.  When a copy or a launch of it fails, the
   // requests in it end with IBS_ECUDA; the engine goes on.
   void run_step() {
+    cudaGetLastError();  // (a query of an event that is not ready leaves one: no launch reports it as its own)
     cudaError_t err = cudaSuccess;
     auto ok = [&](cudaError_t e) {
       if (err == cudaSuccess) err = e;
