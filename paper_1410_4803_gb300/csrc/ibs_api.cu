@@ -237,7 +237,7 @@ static bool tc_tile_kernel_forced() {
 static bool use_sweep(const ibs_ctx* ctx, int64_t n, int64_t m, bool square) {
   return ctx->sweep_on && tc_format_for(ctx) == kTcFp4 && tc_pair_mode() >= 0 && !tc_tile_kernel_forced() &&
          !(n <= 128 && m > 16384) && !(n <= 256 && m > 49152) && sweep_usable(n, m) &&
-         ctx->sweep_refused != std::vector<int64_t>{n, m, square ? 1 : 0};
+         (ctx->sweep_refused.empty() || ctx->sweep_refused.count({n, m, square ? 1 : 0}) == 0);
 }
 
 // ibs_compute on the sweep kernel: operand planes, the sweeps over the shape's
@@ -344,7 +344,8 @@ ibs_status ibs_compute(ibs_ctx* ctx, const uint8_t* packed, int64_t n, int64_t m
                       &ctx->sweep_groups, &ctx->single_sync})
       free_buf(ctx, *b);
     ctx->sweep_key.clear();
-    ctx->sweep_refused = {n, m, square ? 1 : 0};
+    if (ctx->sweep_refused.size() >= 64) ctx->sweep_refused.clear();
+    ctx->sweep_refused.insert({n, m, square ? 1 : 0});
     clear_error();
   }
   // Tensor-core form, triangle output: the persistent kernel over a work list

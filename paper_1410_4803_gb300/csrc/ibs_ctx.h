@@ -7,6 +7,7 @@
 #include <map>
 #include <memory>
 #include <mutex>
+#include <set>
 #include <string>
 #include <vector>
 
@@ -153,7 +154,8 @@ struct ibs_ctx {
   int single_clusters = 0;
   bool single_pair = false;  // single_items holds PairItem (two-SM kernel), else WorkItem
   // sweep kernel: work list of the last (n, m, clusters), scratch of whole tiles
-  std::vector<int64_t> sweep_key, sweep_refused;  // refused: the shape that found no room last
+  std::vector<int64_t> sweep_key;
+  std::set<std::vector<int64_t>> sweep_refused;  // shapes that found no room (a few dozen at most)
   ibs::DevBuf sweep_items, sweep_first, sweep_groups, sweep_scratch;
   int sweep_clusters = 0, sweep_waves = 0, sweep_wave_stages = 0, sweep_slots = 0;
   int64_t sweep_n_groups = 0;

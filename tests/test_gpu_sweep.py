@@ -72,6 +72,24 @@ def test_no_room_for_the_workspace(n, m, limit, kernel):
         ibs.ibs_shutdown(c)
 
 
+def test_shapes_without_room_are_remembered():
+    """Calls of two such shapes in turn try the sweep kernel's workspace once
+    each, not on every call (a device-wide free and allocation each time)."""
+    from paper_1410_4803_gb300 import ibs
+    rng = np.random.default_rng(4)
+    shapes = [(600, 20_000), (500, 20_000)]
+    packed = [pack_codes(random_codes(rng, n, m)) for n, m in shapes]
+    want = [oracle.ibs_triangle(p, n, m)[0] for p, (n, m) in zip(packed, shapes)]
+    c = ibs.ibs_init(0, workspace_bytes=32 << 20)
+    try:
+        for _ in range(2):
+            for p, (n, m), w in zip(packed, shapes, want):
+                assert (gpu_compute(c, p, n, m)[0] == w).all()
+        assert not any(ibs.ibs_compute_sweep_kernel(c, n, m) for n, m in shapes)
+    finally:
+        ibs.ibs_shutdown(c)
+
+
 @pytest.mark.parametrize("pool_n,n,vb,vl", [
     (1003, 1000, 0, 3001),   # the window regrouped by sample: from the first marker to the last
     (1003, 300, 37, 2593),   # from inside a column of the pool
