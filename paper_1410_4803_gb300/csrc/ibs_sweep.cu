@@ -837,15 +837,22 @@ SweepItem whole_item(const Tile& t, int wave) {
   return it;
 }
 
+constexpr int kPartsPerCluster = 6;
+
 // Lay the tiles of `rest` end to end and cut them so that every cluster's load
 // ends at the same time: each takes the next stretch, a few pieces of
 // neighbouring tiles.  A stretch has at least a few stages (a piece costs about
-// kMin stages of its own: pipeline fill, read-back, a part to add up), so a
-// small problem leaves clusters idle.
+// kMin stages of its own: pipeline fill, read-back, a part to add up) or a tile,
+// so a small problem leaves clusters idle.  A tile that is not cut goes to parts
+// too, as far as there are slots: two SMs take about 110 us to write the 256 x 384
+// pairs of a whole tile, the sums' grid has all of them.  With few markers that
+// is all there is: 300 x 50 42 us and 106 with whole tiles, 1,000 x 300 44 and 104,
+// 3,000 x 1,000 77 and 297 (the last share held 80 of its 900 stages).
 void cut_rest(const std::vector<Tile>& rest, std::vector<std::vector<SweepItem>>& own, std::vector<double>& load,
               SweepPlan& pl) {
-  const int C = (int)own.size();
+  const int C = (int)own.size(), R = (int)rest.size();
   constexpr double kMin = 8 * 620.0;
+  const bool parts = 3 * R + C <= sweep_max_slots(C);  // a cut adds at most one slot to its tile's three
   double total = 0;
   for (const Tile& t : rest) total += tile_cost(t);
   // the clusters that take part, the least loaded first, and the common end
@@ -857,13 +864,22 @@ void cut_rest(const std::vector<Tile>& rest, std::vector<std::vector<SweepItem>>
   for (int k = 1; k <= C; ++k) {
     held += load[(size_t)by[(size_t)k - 1]];
     const double e = (held + total) / k;  // if k clusters share the rest
-    if (k > 1 && e - load[(size_t)by[(size_t)k - 1]] < kMin) break;
+    if (k > std::max(1, R) && e - load[(size_t)by[(size_t)k - 1]] < kMin) break;
     shares = k;
     end = e;
   }
   std::sort(by.begin(), by.begin() + shares);  // in order, so that neighbours work on neighbouring tiles
   int share = 0;
+  double left = total;
   auto room = [&] { return end - load[(size_t)by[(size_t)share]]; };
+  // (the end of those that are left, anew: what the rules on slivers gave or took
+  // would otherwise all fall to the last one)
+  auto next_share = [&] {
+    ++share;
+    end = left;
+    for (int k = share; k < shares; ++k) end += load[(size_t)by[(size_t)k]];
+    end /= shares - share;
+  };
   for (const Tile& t : rest) {
     const int S = t.stages;
     const double cost = stage_cost(t.w);
@@ -879,13 +895,13 @@ void cut_rest(const std::vector<Tile>& rest, std::vector<std::vector<SweepItem>>
       int k = last ? 4 * S - q : (int)std::max(0.0, std::min((double)(4 * S - q), room() / cost + 0.5));
       if (4 * S - q - k > 0 && 4 * S - q - k < 3) k = 4 * S - q;  // no sliver left behind
       if (k < 3 && k < 4 * S - q) {                               // nor one begun
-        ++share;
+        next_share();
         continue;
       }
       SweepItem it = whole_item(t, -1);
       it.q0 = q;
       it.q1 = q + k;
-      if (q != 0 || k != 4 * S) {
+      if (parts || q != 0 || k != 4 * S) {
         it.slot = pl.slots;
         for (int pr = 0; pr < 3; ++pr) {
           const int a = pr == 0 ? 0 : pr * S, b = pr == 2 ? 4 * S : (pr + 1) * S;
@@ -897,8 +913,9 @@ void cut_rest(const std::vector<Tile>& rest, std::vector<std::vector<SweepItem>>
       }
       own[(size_t)by[(size_t)share]].push_back(it);
       load[(size_t)by[(size_t)share]] += cost * k;
+      left -= cost * k;
       q += k;
-      if (!last && room() < 0.5 * cost) ++share;
+      if (!last && room() < 0.5 * cost) next_share();
     }
     if (gr.pieces[0] + gr.pieces[1] + gr.pieces[2] > 0) pl.groups.push_back(gr);
   }
@@ -916,7 +933,6 @@ void cut_rest(const std::vector<Tile>& rest, std::vector<std::vector<SweepItem>>
 // against shares: 1,501 samples x 30,011 markers 101 us and 111, 2,500 x 100,000
 // 507 and 755, the square of 3,001 x 60,000 404 and 587, 6,000 x 200,000 3.46 ms
 // and 3.91, 20 served requests of 3,003 rows 8.9 and 11.8.
-constexpr int kPartsPerCluster = 6;
 bool cut_rounds(const std::vector<Tile>& rest, std::vector<std::vector<SweepItem>>& own, size_t operands,
                 SweepPlan& pl) {
   const int64_t C = (int64_t)own.size(), R = (int64_t)rest.size();

@@ -88,6 +88,28 @@ void check(const ibs::SweepPlan& p, const std::vector<Want>& want, int64_t n, in
       base += g->second.pieces[pr];
     }
   }
+  // one matrix or step: whole tiles in waves only, where the others have slots; and
+  // no cluster with twice its share of the work
+  if (one) {
+    std::set<std::pair<int, int>> rest;
+    bool whole = false;
+    double most = 0, total = 0;
+    for (int c = 0; c < p.clusters; ++c) {
+      double load = 0;
+      for (int i = p.first[(size_t)c]; i < p.first[(size_t)c + 1]; ++i) {
+        const SweepItem& it = p.items[(size_t)i];
+        load += stage_cost(it.w) * (it.q1 - it.q0);
+        if (it.wave < 0) {
+          rest.insert({it.I, it.J});
+          whole |= it.slot < 0;
+        }
+      }
+      most = std::max(most, load);
+      total += load;
+    }
+    if (whole && 3 * (int)rest.size() + C <= sweep_max_slots(C)) fail("whole tile outside the waves", n, m, C);
+    if (most > 2 * total / p.clusters + 8 * 620) fail("balance", n, m, C);
+  }
   for (int u : used)
     if (u != 1) fail("unused slot", n, m, C);
   for (int u : wave)
@@ -136,8 +158,8 @@ void check_steps(int64_t panel, int64_t rows, int c) {
 
 int main() {
   int lists = 0;
-  for (int64_t n : {1, 63, 64, 128, 129, 256, 257, 384, 385, 700, 1501, 4096, 5000, 9999, 20000})
-    for (int64_t m : {1, 288, 289, 1000, 30011, 100000, 500000, 2097151})
+  for (int64_t n : {1, 63, 64, 128, 129, 256, 257, 384, 385, 700, 1501, 3000, 4096, 5000, 9999, 20000})
+    for (int64_t m : {1, 288, 289, 577, 1000, 1500, 30011, 100000, 500000, 2097151})
       for (int c : {1, 5, 74, 76}) {
         check(ibs::sweep_plan(n, m, c), {triangle(n, m)}, n, m, c, true);
         ++lists;

@@ -36,9 +36,9 @@ def test_edges(ctx, n, m):
     _check(ctx, n, m, 1000 * n + m)
 
 
-# parts only (few tiles, many markers); one full wave of whole tiles (76 clusters) and
+# parts only (few tiles, many markers; many tiles, few markers); one full wave of whole tiles (76 clusters) and
 # a split rest; two waves, with more than one lockstep segment each
-@pytest.mark.parametrize("n,m", [(130, 60_000), (1100, 9_001), (3201, 2_000), (4500, 3_003)])
+@pytest.mark.parametrize("n,m", [(130, 60_000), (1100, 9_001), (3201, 2_000), (4500, 3_003), (3000, 1_000), (3000, 50)])
 def test_parts_and_waves(ctx, n, m):
     _check(ctx, n, m, n + m)
 
