@@ -380,7 +380,8 @@ ibs_status ibs_kernel_info(ibs_ctx* ctx, int64_t out[4]);
  * With E2M1 operands these three classes run on the two-SM kernel that sweeps
  * the markers once per product (clusters of two CTAs, tcgen05 cta_group::2);
  * where its workspace does not fit, with few samples over many variants (up to
- * 128 over 16,384, up to 256 over 49,152), with 2^21 or more variants and with
+ * 128 over 16,384, up to 256 over 49,152), without distances over few variants (a
+ * few thousand at most), with 2^21 or more variants and with
  * E4M3 operands, class 2 runs one persistent CTA per SM, class 3 the two-SM kernel
  * over 256 x 128 tiles and class 4 one CTA per tile.
  * ibs_compute_sweep_kernel says which of the two.
@@ -392,9 +393,10 @@ ibs_status ibs_kernel_info(ibs_ctx* ctx, int64_t out[4]);
 ibs_status ibs_compute_kernel(ibs_ctx* ctx, int64_t n_samples, int64_t n_variants, int64_t* out);
 
 /* 1 in *out when ibs_compute on this context runs the sweep kernel for an
- * n_samples x n_variants matrix, 0 when it runs the kernel of the class that
- * ibs_compute_kernel reports (also once the sweep kernel's workspace has found
- * no room for this shape).  IBS_EINVAL as there. */
+ * n_samples x n_variants matrix with distances (without them on a context with
+ * IBS_NO_DIST, where few variants stay off it), 0 when it runs the kernel of the
+ * class that ibs_compute_kernel reports (also once the sweep kernel's workspace has
+ * found no room for this shape).  IBS_EINVAL as there. */
 ibs_status ibs_compute_sweep_kernel(ibs_ctx* ctx, int64_t n_samples, int64_t n_variants, int64_t* out);
 
 /* Counters of the last ibs_compute / ibs_compute_batch on this context:

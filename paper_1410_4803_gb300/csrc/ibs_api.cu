@@ -234,9 +234,26 @@ static bool tc_tile_kernel_forced() {
 // and 59, 300 x 100,000 76 and 90, 4,096 x 100,000 935 and 1,566, 20,000 x 500,000
 // 74 and 142 ms, the square of 3,001 x 60,000 386 us and 788; but 64 x 20,000 36
 // and 33, 85 x 100,000 76 and 43, 200 x 100,000 86 and 65, 40 x 400,000 94 and 72.
-static bool use_sweep(const ibs_ctx* ctx, int64_t n, int64_t m, bool square) {
+// Without distances the kernels below have little to write per tile, and two
+// launches where they need not split over K; the sweep kernel's three take longer
+// over few markers (us, those kernels and the sweep kernel): 200 x 1,000 30 and 38,
+// 200 x 2,000 33 and 33, 1,000 x 1,600 36 and 38, 1,000 x 2,500 39 and 33, 2,048 x
+// 3,000 43 and 45, 3,072 x 4,000 77 and 80, 10,000 x 1,500 436 and 504; where they split
+// the last wave (more than one chunk, and at most 3/4 of the SMs in it), 2,300 x 64 43
+// and 45, 2,300 x 65 80 and 45, 15,000 x 100 1,050 and 998.  Squares: 500 x 700 35 and
+// 39, 500 x 1,300 39 and 36, 2,048 x 1,600 41 and 49, 2,048 x 2,500 49 and 48, 8,000 x
+// 1,300 390 and 389.
+static bool few_markers(const ibs_ctx* ctx, int64_t n, int64_t m, bool square) {
+  const int64_t T = (n + 127) / 128, tiles = T * (T + 1) / 2, rem = tiles % ctx->num_sms;
+  if (square) return m < (T >= 12 && T <= 17 ? 2000 : 1300);
+  if (tiles < ctx->num_sms) return m < (T == 1 ? 1300 : (T < 15 ? 2000 : 3500));
+  return m <= 64 || (m < 4000 && (rem == 0 || 4 * rem > 3 * ctx->num_sms));
+}
+
+static bool use_sweep(const ibs_ctx* ctx, int64_t n, int64_t m, bool square, bool dist) {
   return ctx->sweep_on && tc_format_for(ctx) == kTcFp4 && tc_pair_mode() >= 0 && !tc_tile_kernel_forced() &&
-         !(n <= 128 && m > 16384) && !(n <= 256 && m > 49152) && sweep_usable(n, m) &&
+         !(n <= 128 && m > 16384) && !(n <= 256 && m > 49152) && (dist || !few_markers(ctx, n, m, square)) &&
+         sweep_usable(n, m) &&
          (ctx->sweep_refused.empty() || ctx->sweep_refused.count({n, m, square ? 1 : 0}) == 0);
 }
 
@@ -335,7 +352,7 @@ ibs_status ibs_compute(ibs_ctx* ctx, const uint8_t* packed, int64_t n, int64_t m
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   const bool tc = use_tc(ctx);
   const int fmt = tc_format_for(ctx);
-  if (tc && use_sweep(ctx, n, m, square)) {
+  if (tc && use_sweep(ctx, n, m, square, out_dist != nullptr)) {
     const ibs_status s = compute_sweep(ctx, packed, n, m, out_counts, out_dist, square, st);
     if (s != IBS_ENOMEM) return s;
     // no room for its scratch and parts: nothing is enqueued, and the kernels
@@ -1797,7 +1814,7 @@ extern "C" ibs_status ibs_compute_sweep_kernel(ibs_ctx* ctx, int64_t n, int64_t 
   if (ibs_status s = ibs_compute_kernel(ctx, n, m, &kernel)) return s;
   if (!out) return fail(IBS_EINVAL, "out is NULL");
   DeviceGuard g(ctx->device);
-  *out = use_tc(ctx) && use_sweep(ctx, n, m, (ctx->flags & IBS_OUT_SQUARE) != 0) ? 1 : 0;
+  *out = use_tc(ctx) && use_sweep(ctx, n, m, (ctx->flags & IBS_OUT_SQUARE) != 0, (ctx->flags & IBS_NO_DIST) == 0);
   return IBS_OK;
 }
 

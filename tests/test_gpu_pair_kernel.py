@@ -100,6 +100,11 @@ def test_sizes_of_the_sweep_kernel(monkeypatch):
             (tc4, 300, 2_097_152, False), (tc4, 128, 16_384, True), (tc4, 128, 16_385, False),
             (tc4, 200, 70_000, False), (tc4 | ibs.IBS_OUT_SQUARE, 3001, 60_000, True), (tc8, 4096, 100_000, False),
             (ibs.IBS_KERNEL_CSA, 4096, 100_000, False)]
+    # without distances: one block, one wave, an unsplit last wave, a split one; squares
+    nd, sq = tc4 | ibs.IBS_NO_DIST, tc4 | ibs.IBS_NO_DIST | ibs.IBS_OUT_SQUARE
+    for flags, n, m in ((nd, 128, 1300), (nd, 129, 2000), (nd, 2048, 3500), (nd, 3072, 4000), (nd, 2300, 65),
+                        (sq, 128, 1300), (sq, 2048, 2000), (sq, 8000, 1300)):
+        want += [(flags, n, m, True), (flags, n, m - 1, False)]
     monkeypatch.delenv("IBS_SWEEP", raising=False)
     for flags, n, m, sweep in want:
         with ibs.ibs_init(0, flags=flags) as ctx:

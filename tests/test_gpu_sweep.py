@@ -51,6 +51,32 @@ def test_narrow_inputs(ctx, n, m):
     _check(ctx, n, m, n + m)
 
 
+# either side of the markers that a call without distances needs for the sweep kernel
+@pytest.mark.parametrize("n,m", [(128, 1300), (500, 2000), (2048, 3500), (2300, 65)])
+@pytest.mark.parametrize("square", [False, True])
+def test_counts_alone(n, m, square):
+    import torch
+    from paper_1410_4803_gb300 import ibs
+    c = ibs.ibs_init(0, flags=ibs.IBS_KERNEL_TC | ibs.IBS_TC_FP4 | (ibs.IBS_OUT_SQUARE if square else 0))
+    try:
+        for mm in (m - 1, m) if not square else (1299, 1300):
+            rng = np.random.default_rng(n + mm)
+            packed = pack_codes(random_codes(rng, n, mm, miss=0.05))
+            want = oracle.ibs_triangle(packed, n, mm)[0]
+            counts = torch.full((n * n if square else n * (n + 1) // 2, 4), -7, dtype=torch.int32, device="cuda")
+            ibs.ibs_compute(c, torch.from_numpy(packed).cuda(), n, mm, counts)
+            ibs.ibs_synchronize(c)
+            got = counts.cpu().numpy()
+            if square:
+                i, j = np.triu_indices(n)
+                got = got.reshape(n, n, 4)
+                assert (got[j, i] == want).all()
+                got = got[i, j]
+            assert (got == want).all(), mm
+    finally:
+        ibs.ibs_shutdown(c)
+
+
 # planes 26 MB, partial counts 2.9 MB: the one-SM kernel; planes 51 MB: the two-SM kernel
 @pytest.mark.parametrize("n,m,limit,kernel", [(600, 20_000, 32 << 20, "tc-persistent"), (300, 66_000, 56 << 20, "tc-pair")])
 def test_no_room_for_the_workspace(n, m, limit, kernel):
