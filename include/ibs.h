@@ -194,7 +194,8 @@ typedef struct {
  *      kernel.  With E2M1 operands, the sweep kernel allowed and no workspace
  *      limit set, this policy is one gather and one sweep-kernel launch over
  *      all subsets instead, and it is taken without timing the others (but for
- *      a lone subset of up to 128 samples over many variants);
+ *      a lone subset of up to 128 samples over many variants, and batches
+ *      without distances over few variants);
  *   3  one two-SM persistent launch over every subset's two-SM work list,
  *      concatenated, with the gather fused: a concurrent gather kernel fills
  *      the operand planes unit by unit and per-subset readiness counters hold

@@ -1465,6 +1465,22 @@ extern "C" ibs_status ibs_compute_batch(ibs_ctx* ctx, const uint8_t* pool, int64
                                                  : -1;
   key.push_back(forced);
   key.push_back(tc ? 1 : 0);
+  // Counts alone over few markers stay with the timed policies, as in ibs_compute:
+  // a tile has little to write there.  Best policy and sweep kernel, us: one of 2,000 x
+  // 3,000 59 and 66, 3 of 2,000 x 8,000 175 and 202, 20 of 500 x 8,000 193 and 232, 20
+  // of 1,000 x 8,000 368 and 387, 20 of 1,000 x 12,000 487 and 461, 64 of 300 x 5,000 304
+  // and 322; of more pairs, 64 of 1,000 x 3,000 574 and 676, 64 of 1,000 x 5,000 776
+  // and 781, 64 of 1,000 x 8,000 1,058 and 935, 200 of 300 x 5,000 776 and 749.
+  double pairs = 0, work = 0;
+  bool any_dist = false;
+  for (int i = 0; i < n_subsets; ++i) {
+    const double p = 0.5 * (double)shapes[i].n * (double)(shapes[i].n + 1);
+    pairs += p;
+    work += p * (double)shapes[i].m;
+    any_dist = any_dist || (!(ctx->flags & IBS_NO_DIST) && subs[i].out_dist);
+  }
+  const bool few = !any_dist && work < pairs * (pairs <= 1.2e7 ? 10000.0 : 5000.0);
+  key.push_back(few ? 1 : 0);
 
   auto it = ctx->plans.find(key);
   if (it == ctx->plans.end()) {
@@ -1496,7 +1512,7 @@ extern "C" ibs_status ibs_compute_batch(ibs_ctx* ctx, const uint8_t* pool, int64
     // 100,000 126 and 139, four of 85 x 100,000 218 and 287.
     const bool narrow = n_subsets == 1 && shapes[0].n <= 128 &&
                         shapes[0].m > std::max<int64_t>(12000, 4000 + 280 * shapes[0].n);
-    bool sweep = ctx->sweep_on && !narrow && tc && ctx->ws_limit == 0 && tc_format_for(ctx) == kTcFp4 && tc_pair_mode() >= 0 && !tc_tile_kernel_forced() &&
+    bool sweep = ctx->sweep_on && !narrow && !few && tc && ctx->ws_limit == 0 && tc_format_for(ctx) == kTcFp4 && tc_pair_mode() >= 0 && !tc_tile_kernel_forced() &&
                  (fixed_policy < 0 || fixed_policy == 2);
     for (const auto& sh : shapes) sweep = sweep && sweep_usable(sh.n, sh.m);
     auto plan = std::make_unique<BatchPlan>();

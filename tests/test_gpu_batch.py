@@ -265,11 +265,12 @@ def _random_pool(n, m, seed):
     return torch.randint(0, 256, (m, (n + 3) // 4), dtype=torch.uint8, device="cuda", generator=g)
 
 
-def _subset_args(pool_n, n, vb, vl, seed):
+def _subset_args(pool_n, n, vb, vl, seed, dist=True):
     import torch
     idx = np.sort(np.random.default_rng(seed).choice(pool_n, size=n, replace=False)).astype(np.int64)
     P = n * (n + 1) // 2
-    return [(torch.from_numpy(idx).cuda(), vb, vl, torch.full((P, 4), -7, dtype=torch.int32, device="cuda"), None)]
+    return [(torch.from_numpy(idx).cuda(), vb, vl, torch.full((P, 4), -7, dtype=torch.int32, device="cuda"),
+             torch.empty(P, dtype=torch.float64, device="cuda") if dist else None)]
 
 
 def test_plans_share_the_regrouped_pool():
@@ -367,6 +368,34 @@ def test_tune_file_and_the_sweep_kernel(tmp_path):
     path.write_text(json.dumps(dict(timed[0], ms=0.0, split=2)) + "\n")
     _, entries = run(workspace_bytes=256 << 20)
     assert len([e for e in entries if e["ms"] > 0]) == 1
+
+
+@pytest.mark.parametrize("m,dist,timed", [(9_999, False, True), (10_000, False, False), (300, True, False)])
+def test_batch_of_counts_alone(tmp_path, m, dist, timed):
+    """Batches without distances: either side of the mean marker count at which
+    they go to the timed policies; the plan of the same shapes with distances is
+    another."""
+    import json
+    import torch
+    from paper_1410_4803_gb300 import ibs
+    pool_n = 300
+    pool = _random_pool(pool_n, m, 5)
+    subs = [_subset_args(pool_n, n, 0, m, n, dist=False)[0] for n in (140, 150, 90)]
+    with_dist = [s[:4] + (torch.empty(s[3].shape[0], dtype=torch.float64, device="cuda"),) for s in subs]
+    path = tmp_path / "tune.jsonl"
+    ctx = ibs.ibs_init(0, flags=ibs.IBS_KERNEL_TC | ibs.IBS_TC_FP4, autotune_cache_path=str(path))
+    try:
+        for use in ((with_dist, with_dist) if dist else (subs, with_dist, subs)):
+            for s in subs:
+                s[3].fill_(-7)
+            ibs.ibs_compute_batch(ctx, pool, pool_n, m, use)
+            ibs.ibs_synchronize(ctx)
+            for s in subs:
+                G = oracle.unpack_subset(pool.cpu().numpy(), pool_n, m, s[0].cpu().numpy(), 0, m)
+                assert (s[3].cpu().numpy() == oracle.ibs_triangle_from_codes(G)[0]).all()
+    finally:
+        ibs.ibs_shutdown(ctx)
+    assert any(json.loads(x)["ms"] > 0 for x in path.read_text().splitlines()) == timed
 
 
 @pytest.mark.parametrize("n,m,timed", [(16, 12_000, False), (16, 12_001, True), (100, 32_000, False),
