@@ -381,8 +381,8 @@ ibs_status ibs_kernel_info(ibs_ctx* ctx, int64_t out[4]);
  * With E2M1 operands these three classes run on the two-SM kernel that sweeps
  * the markers once per product (clusters of two CTAs, tcgen05 cta_group::2);
  * where its workspace does not fit, with few samples over many variants (up to
- * 128 over 16,384, up to 256 over 49,152), without distances over few variants (a
- * few thousand at most), with 2^21 or more variants and with
+ * 128 over 10,368 or 16,384, up to 256 over 24,000 to 49,000), with up to 20
+ * samples over few, without distances over few variants (a few thousand at most), with 2^21 or more variants and with
  * E4M3 operands, class 2 runs one persistent CTA per SM, class 3 the two-SM kernel
  * over 256 x 128 tiles and class 4 one CTA per tile.
  * ibs_compute_sweep_kernel says which of the two.

@@ -227,13 +227,28 @@ static bool tc_tile_kernel_forced() {
   return v;
 }
 
-// The sweep kernel (ibs_sweep.cu) computes E2M1 inputs, triangle or square, except
-// one or two blocks of samples over many markers: there every stage of every
-// piece multiplies a narrow tile, and the pieces' sums are most of the call.
-// Sweep kernel against the kernels below: 256 x 4,096 27 us and 82, 200 x 20,000 42
-// and 59, 300 x 100,000 76 and 90, 4,096 x 100,000 935 and 1,566, 20,000 x 500,000
-// 74 and 142 ms, the square of 3,001 x 60,000 386 us and 788; but 64 x 20,000 36
-// and 33, 85 x 100,000 76 and 43, 200 x 100,000 86 and 65, 40 x 400,000 94 and 72.
+// The sweep kernel (ibs_sweep.cu) computes E2M1 inputs, triangle or square, with
+// these exceptions.  Sweep kernel against the kernels below: 256 x 4,096 27 us and
+// 82, 300 x 100,000 76 and 90, 4,096 x 100,000 935 and 1,566, 20,000 x 500,000 73 and 142
+// ms, the square of 3,001 x 60,000 386 us and 788.
+//
+// One or two blocks of samples over many markers: every stage of every piece
+// multiplies a narrow tile, and the pieces' sums are most of the call.  The one-SM
+// kernel splits a lone tile from 163 chunks (10,369 markers) on.  Those kernels and
+// the sweep kernel (us): 64 x 10,000 68 and 38, 64 x 12,000 36 and 39, 80 x 14,000 41
+// and 43, 128 x 16,000 51 and 43, 85 x 100,000 43 and 76, 129 x 30,000 62 and 62, 129 x
+// 40,000 64 and 69, 200 x 40,000 67 and 71, 256 x 49,000 81 and 78; squares 96 x 12,000
+// 38 and 42, 128 x 16,000 48 and 48, 129 x 25,000 57 and 60, 200 x 30,000 61 and 65, 230 x
+// 40,000 75 and 75, 256 x 49,000 83 and 82.
+static bool narrow_input(int64_t n, int64_t m, bool square) {
+  if (n <= 128) return m > (n <= (square ? 104 : 72) ? 10368 : 16384);
+  if (n > 256) return false;
+  return m > (square ? 24000 + 450 * std::max<int64_t>(0, n - 200) : 32000 + 135 * (n - 128));
+}
+
+// A few samples over few markers: three launches against two (20 x 1,000 34 and 32).
+static bool tiny_input(int64_t n, int64_t m) { return n <= 20 && m < 1300; }
+
 // Without distances the kernels below have little to write per tile, and two
 // launches where they need not split over K; the sweep kernel's three take longer
 // over few markers (us, those kernels and the sweep kernel): 200 x 1,000 30 and 38,
@@ -252,7 +267,7 @@ static bool few_markers(const ibs_ctx* ctx, int64_t n, int64_t m, bool square) {
 
 static bool use_sweep(const ibs_ctx* ctx, int64_t n, int64_t m, bool square, bool dist) {
   return ctx->sweep_on && tc_format_for(ctx) == kTcFp4 && tc_pair_mode() >= 0 && !tc_tile_kernel_forced() &&
-         !(n <= 128 && m > 16384) && !(n <= 256 && m > 49152) && (dist || !few_markers(ctx, n, m, square)) &&
+         !narrow_input(n, m, square) && !tiny_input(n, m) && (dist || !few_markers(ctx, n, m, square)) &&
          sweep_usable(n, m) &&
          (ctx->sweep_refused.empty() || ctx->sweep_refused.count({n, m, square ? 1 : 0}) == 0);
 }

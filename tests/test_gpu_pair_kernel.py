@@ -96,10 +96,15 @@ def test_sizes_of_the_sweep_kernel(monkeypatch):
     """Where the sweep kernel runs, and the switch that keeps a context off it."""
     from paper_1410_4803_gb300 import ibs
     tc4, tc8 = ibs.IBS_KERNEL_TC | ibs.IBS_TC_FP4, ibs.IBS_KERNEL_TC | ibs.IBS_TC_FP8
-    want = [(tc4, 4096, 100_000, True), (tc4, 256, 4096, True), (tc4, 1, 1, True), (tc4, 300, 2_097_151, True),
+    want = [(tc4, 4096, 100_000, True), (tc4, 256, 4096, True), (tc4, 21, 1, True), (tc4, 300, 2_097_151, True),
             (tc4, 300, 2_097_152, False), (tc4, 128, 16_384, True), (tc4, 128, 16_385, False),
             (tc4, 200, 70_000, False), (tc4 | ibs.IBS_OUT_SQUARE, 3001, 60_000, True), (tc8, 4096, 100_000, False),
             (ibs.IBS_KERNEL_CSA, 4096, 100_000, False)]
+    # few samples: over few markers, and one or two blocks over many
+    sq = tc4 | ibs.IBS_OUT_SQUARE
+    for flags, n, m in ((tc4, 20, 1300), (tc4, 72, 10_369), (tc4, 73, 16_385), (tc4, 129, 32_136), (tc4, 256, 49_281),
+                        (sq, 104, 10_369), (sq, 105, 16_385), (sq, 200, 24_001), (sq, 256, 49_201)):
+        want += [(flags, n, m, n == 20), (flags, n, m - 1, n != 20)]
     # without distances: one block, one wave, an unsplit last wave, a split one; squares
     nd, sq = tc4 | ibs.IBS_NO_DIST, tc4 | ibs.IBS_NO_DIST | ibs.IBS_OUT_SQUARE
     for flags, n, m in ((nd, 128, 1300), (nd, 129, 2000), (nd, 2048, 3500), (nd, 3072, 4000), (nd, 2300, 65),

@@ -46,7 +46,7 @@ def test_parts_and_waves(ctx, n, m):
 # either side of the sizes that leave the sweep kernel: one block of samples, two
 # (the two-SM kernel from 65,536 markers on)
 @pytest.mark.parametrize("n,m", [(128, 16_384), (128, 16_385), (129, 16_385), (256, 49_152), (256, 49_153), (257, 49_153),
-                                 (200, 70_000)])
+                                 (200, 70_000), (72, 10_368), (72, 10_369), (129, 32_135), (129, 32_136), (20, 1299)])
 def test_narrow_inputs(ctx, n, m):
     _check(ctx, n, m, n + m)
 
