@@ -60,6 +60,13 @@ constexpr int64_t kStepWavesTc = 8; // ... of the tensor-core form without the s
                                     // about 3 ms); with it: sweep_step_blocks
 constexpr int64_t kMinStepDiv = 32; // ... and covers at least 1/32 of the panel
 constexpr size_t kMemMargin = (size_t)1 << 30;
+// Samples of this size go to the device from ibs_query, smaller ones by way of host
+// memory: their copy to the device takes the caller 30 us, and a burst of them came
+// in one by one, each in a step of its own.  20 requests of 1 to 16 rows against 38,314
+// x 13,313: 1.6 ms with all sent to the device, 0.93 with 256 KiB (0.89 before any
+// was); 1 to 512 rows (3,003 in all) against 20,000 x 100,000: 7.4 ms, 6.8 with 256
+// KiB, 6.9 with 1 MiB.
+constexpr size_t kDirectBytes = (size_t)256 << 10;
 constexpr int64_t kTcBlock = 128;          // samples per tensor-core block
 constexpr size_t kTcChunkBytes = 16384;    // one (block, chunk) of operand planes
 
@@ -1134,14 +1141,14 @@ ibs_status serve_query(ibs_ctx* ctx, const uint8_t* q, int64_t nq, int k, int32_
     r->map_idx = static_cast<int32_t*>(mapped(oi, sizeof(int32_t)));
     r->map_dist = static_cast<double*>(mapped(od, sizeof(double)));
   }
-  // A request that the engine can admit at once goes straight to the device (20
-  // requests with 75 MB of pinned samples: 12.3 ms against 13.0); one behind
-  // others that wait for memory, or past the rows of a step, is kept on the
-  // host.  The early ones take their memory and their places together, so no
-  // request holds memory that one ahead of it in the queue waits for.
+  // A request that the engine can admit at once is early: it takes its memory and
+  // its place together, so no request holds memory that one ahead of it in the
+  // queue waits for, and its samples go straight to the device when they are many
+  // (kDirectBytes).  One behind others that wait for memory, or past the rows of
+  // a step, is kept on the host.
   const size_t bytes = (size_t)e.pg.m * (size_t)((nq + 3) / 4);
   r->id = e.next_id.fetch_add(1);
-  if (e.in && ctx->ws_limit == 0) {
+  if (ctx->ws_limit == 0) {
     std::lock_guard<std::mutex> lk(e.mu);
     bool early = !e.stop && e.early_rows + nq <= kMaxRows;
     for (const auto& p : e.pending) early = early && p->early;
@@ -1152,7 +1159,8 @@ ibs_status serve_query(ibs_ctx* ctx, const uint8_t* q, int64_t nq, int k, int32_
       e.pending.push_back(r);
     }
   }
-  if (!r->early || !e.copy_in(*r, q, bytes)) r->host_packed = copy_query(q, bytes);
+  const bool direct = r->early && e.in && bytes >= kDirectBytes;
+  if (!direct || !e.copy_in(*r, q, bytes)) r->host_packed = copy_query(q, bytes);
   {
     std::lock_guard<std::mutex> lk(e.mu);
     if (e.stop) return fail(IBS_ECANCELLED, "engine is shutting down");

@@ -211,8 +211,9 @@ def test_shutdown_cancels_pending(panel):
     assert all(s in (ibs.IBS_OK, ibs.IBS_ECANCELLED) for s in statuses)
 
 
+@pytest.mark.parametrize("m", [700, 30_000])  # by way of the host, and straight to the device
 @pytest.mark.parametrize("stop", ["shutdown", "reload"])
-def test_stop_while_a_call_brings_its_request_in(stop):
+def test_stop_while_a_call_brings_its_request_in(stop, m):
     """ibs_query of device samples waits for the legacy stream with the engine's
     memory in hand; a shutdown or a new panel meanwhile lets the call return
     IBS_ECANCELLED first, and the context it uses outlives it."""
@@ -220,7 +221,7 @@ def test_stop_while_a_call_brings_its_request_in(stop):
     from paper_1410_4803_gb300 import ibs
     from helpers import pack_codes, random_codes
     rng = np.random.default_rng(8)
-    n_panel, m, q, k = 300, 700, 40, 4
+    n_panel, q, k = 300, 40, 4
     pp = pack_codes(random_codes(rng, n_panel, m))
     qp = torch.from_numpy(pack_codes(random_codes(rng, q, m))).cuda()
     oi, od = _pinned((q, k), torch.int32), _pinned((q, k), torch.float64)
@@ -274,15 +275,16 @@ def _check_request(panel_codes, codes, idx, dist, k):
         np.testing.assert_allclose(dist.numpy()[t], td, rtol=1e-12, atol=0)
 
 
+@pytest.mark.parametrize("m", [3000, 6000])  # by way of the host, and straight to the device
 @pytest.mark.parametrize("first", ["device", "host"])
-def test_two_callers_and_a_budget_for_one(first):
+def test_two_callers_and_a_budget_for_one(first, m):
     """A call whose samples wait for the legacy stream holds the budget that the
     other one needs: both are served, in either order of arrival."""
     import torch
     from paper_1410_4803_gb300 import ibs
     from helpers import pack_codes, random_codes
     rng = np.random.default_rng(17)
-    n_panel, m, q, k = 300, 3000, 200, 4
+    n_panel, q, k = 300, 200, 4
     ctx, panel_codes = _tight_engine(n_panel, m, q, k, rng)
     try:
         codes = [random_codes(rng, q, m) for _ in range(2)]
@@ -315,7 +317,7 @@ def test_many_callers_and_a_tight_budget():
     from paper_1410_4803_gb300 import ibs
     from helpers import pack_codes, random_codes
     rng = np.random.default_rng(18)
-    n_panel, m, k = 300, 3000, 4
+    n_panel, m, k = 300, 8000, 4
     ctx, panel_codes = _tight_engine(n_panel, m, 200, k, rng)
     try:
         reqs = []
