@@ -154,8 +154,9 @@ class ServeEngine {
   int grid_ctas = 0;   // persistent cross-kernel CTAs (SMs x 2)
   bool sweep = false;  // the sweep kernel for every step (E2M1)
   DevBuf sweep_scratch, sweep_part;  // the steps'
-  DevBuf sync_scratch, sync_part;    // the unbatched path's, one call at a time
-  std::mutex sync_mu;
+  DevBuf sync_scratch, sync_part;    // the unbatched path's, one call's kernels at a time
+  std::mutex sync_mu;                // from the wait for the last call's kernels to the event after this one's
+  cudaEvent_t sync_ev = nullptr;     // after the last call's kernels
   DevBuf panel_words, few_words;     // sweep: the panel's code bits by sample, for steps of few rows; the rows'
   std::mutex words_mu;               // panel_words in use or given back
   bool pair = false;   // two-SM kernel for steps of two or more query blocks
@@ -885,6 +886,11 @@ class ServeEngine {
     }
     if (stream) cudaStreamDestroy(stream);
     if (side) cudaStreamDestroy(side);
+    {
+      std::lock_guard<std::mutex> sync_lk(sync_mu);
+      if (sync_ev) cudaEventDestroy(sync_ev);
+      sync_ev = nullptr;
+    }
     stream = nullptr;
     side = nullptr;
   }
@@ -1269,9 +1275,7 @@ ibs_status serve_query_sync(ibs_ctx* ctx, const uint8_t* q, int64_t nq, int k, i
   const bool two_sm = e.pair && qg.blocks >= 2;
   SweepPlan pl;
   std::vector<uint8_t> sweep_host;
-  std::unique_lock<std::mutex> sync_lk(e.sync_mu, std::defer_lock);
   if (e.sweep) {
-    sync_lk.lock();  // the scratch and parts, until the stream is waited for
     const int64_t cols[2][2] = {{0, e.pgeo.blocks}, {0, 0}};
     pl = sweep_plan_cross(qg.blocks, cols, pg.m, e.clusters);
     sweep_host.resize(ServeEngine::sweep_list_bytes(pl));
@@ -1314,11 +1318,23 @@ ibs_status serve_query_sync(ibs_ctx* ctx, const uint8_t* q, int64_t nq, int k, i
     ce = cudaMemcpyAsync(items_dev.p, item_src, item_bytes, cudaMemcpyHostToDevice, s);
   if (ce == cudaSuccess) ce = e.build_planes(static_cast<const uint8_t*>(r.packed.p), nq, r.planes.p, s);
   if (ce == cudaSuccess) {
-    if (e.sweep)
-      ce = e.run_sweep(pl, static_cast<const uint8_t*>(r.planes.p), (nq + 63) / 64,
-                       static_cast<int32_t* const*>(outs_d.p), nq, sweep_host.data(),
-                       static_cast<uint8_t*>(items_dev.p), e.sync_scratch, e.sync_part, sync_d, false, s);
-    else if (two_sm)
+    if (e.sweep) {
+      // The scratch and the parts pass from call to call in the streams' order, so
+      // that the copies and the operands of one call overlap the kernels of another.
+      std::lock_guard<std::mutex> lk(e.sync_mu);
+      if (!e.sync_ev)
+        ce = cudaEventCreateWithFlags(&e.sync_ev, cudaEventDisableTiming);
+      else
+        ce = cudaStreamWaitEvent(s, e.sync_ev, 0);
+      if (ce == cudaSuccess)
+        ce = e.run_sweep(pl, static_cast<const uint8_t*>(r.planes.p), (nq + 63) / 64,
+                         static_cast<int32_t* const*>(outs_d.p), nq, sweep_host.data(),
+                         static_cast<uint8_t*>(items_dev.p), e.sync_scratch, e.sync_part, sync_d, false, s);
+      if (e.sync_ev) {
+        const cudaError_t re = cudaEventRecord(e.sync_ev, s);
+        if (ce == cudaSuccess) ce = re;
+      }
+    } else if (two_sm)
       ce = launch_tc_pair_cross(static_cast<const uint8_t*>(e.panel_planes.p), pg.n, e.pgeo.chunks,
                                 static_cast<const uint8_t*>(r.planes.p), qg.blocks,
                                 static_cast<int32_t* const*>(outs_d.p), nq,

@@ -414,6 +414,49 @@ def test_panel_words_make_room():
         ibs.ibs_shutdown(ctx)
 
 
+def test_unbatched_calls_of_several_threads():
+    """ibs_query_sync from four threads at once, with parts and with whole waves of
+    tiles, counts on the device and on the host: the calls share the sweep kernel's
+    workspace in turn, and each result is the one of the call alone."""
+    import torch
+    from paper_1410_4803_gb300 import ibs
+    from helpers import pack_codes, random_codes
+    rng = np.random.default_rng(23)
+    n_panel, m, k = 5000, 900, 4
+    ctx = ibs.ibs_init(0)
+    try:
+        ibs.ibs_panel_load(ctx, pack_codes(random_codes(rng, n_panel, m)), n_panel, m)
+        reqs = []
+        for i, q in enumerate((1, 130, 700, 4096)):  # 4,096: 16 row pairs x 13 column groups, two whole waves
+            packed = torch.from_numpy(pack_codes(random_codes(rng, q, m))).pin_memory()
+            host = i % 2 == 0
+            counts = torch.empty((q, n_panel, 4), dtype=torch.int32, device="cpu" if host else "cuda")
+            outs = [counts.pin_memory() if host else counts, _pinned((q, k), torch.int32), _pinned((q, k), torch.float64)]
+            ibs.ibs_query_sync(ctx, packed, q, k, *outs)
+            reqs.append((q, packed, outs, [x.clone() for x in outs]))
+        errors = []
+
+        def work(q, packed, outs, want):
+            try:
+                for _ in range(8):
+                    outs[0].fill_(-7)
+                    torch.cuda.synchronize()
+                    ibs.ibs_query_sync(ctx, packed, q, k, *outs)
+                    for x, w in zip(outs, want):
+                        assert torch.equal(x, w), q
+            except Exception as e:
+                errors.append(e)
+
+        threads = [threading.Thread(target=work, args=r) for r in reqs]
+        for t in threads:
+            t.start()
+        for t in threads:
+            t.join(timeout=120)
+        assert not errors, errors
+    finally:
+        ibs.ibs_shutdown(ctx)
+
+
 SERVE_TWO_SM = r"""
 import sys
 import numpy as np
